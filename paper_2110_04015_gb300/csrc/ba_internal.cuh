@@ -139,7 +139,7 @@ struct System {
     float* S32 = nullptr;     // float(S^), tiled layout
     float* S32u = nullptr;    // its upper triangle (diagonal blocks included), tiled upper pattern
     double* lam = nullptr;    // 9 n_c: Lam
-    double* Dhat = nullptr;   // n_c x 81: inverses of the diagonal blocks of S^
+    double* Dhat = nullptr;   // n_c x 81: inverses of the diagonal blocks of S^, in double-float (float2)
     float* lam32 = nullptr;   // 9 n_c: float(Lam)
     float* G32 = nullptr;     // n_o x 36: G_o = J_p^T A_o in float32 (from the float32 Jacobians), rows
                               // 3P..3P+2 at offset 12 P (three 16-byte aligned parts)

@@ -1268,7 +1268,8 @@ __global__ void k_df_to_double(double* __restrict__ buf, int64_t n) {
 
 // D_j^{-1} = (S_jj)^{-1} = L^{-T} L^{-1} from the Cholesky factor of the diagonal block.
 // With lam != nullptr the block is first scaled by its diagonal, B^ = s B s with s_a = B_aa^{-1/2};
-// Dinv then receives (B^)^{-1}, lam the scale factors and lam32 their float32 roundings.
+// Dinv then receives (B^)^{-1} in double-float (hi, lo in the 8 bytes of a float64), lam the scale
+// factors and lam32 their float32 roundings.
 __global__ void k_block_jacobi(int32_t n_c, const double* __restrict__ Sd, double* __restrict__ Dinv,
                                double* __restrict__ lam, float* __restrict__ lam32, int* status) {
     for (int64_t j = gtid(); j < n_c; j += gstride()) {
@@ -1316,8 +1317,14 @@ __global__ void k_block_jacobi(int32_t n_c, const double* __restrict__ Sd, doubl
             for (int b = a; b < 9; ++b) {
                 double v = 0.0;
                 for (int k = b; k < 9; ++k) v += Li[9 * k + a] * Li[9 * k + b];
-                D[9 * a + b] = v;
-                D[9 * b + a] = v;
+                if (lam) {
+                    const df64 d = df_from(v);
+                    df_st(reinterpret_cast<float2*>(D) + 9 * a + b, d);
+                    df_st(reinterpret_cast<float2*>(D) + 9 * b + a, d);
+                } else {
+                    D[9 * a + b] = v;
+                    D[9 * b + a] = v;
+                }
             }
         }
     }

@@ -48,8 +48,11 @@ namespace {
 constexpr int kGramMax = kMaxDirs * kMaxDirs + kMaxDirs;   // Delta (w x w) and gamma (w)
 constexpr int kChunkCams = 112;                             // cameras per Phi partial
 constexpr double kStagnation = 1e-4;                        // float32 sweep stop on t_i (see Ctl::stag)
-constexpr int kTotals = 16;                                 // per-problem grid totals
-constexpr int kUpdCams = 28;                                // cameras per CTA of the update kernels (252 rows)
+// Cameras and threads per CTA of the update kernels (126 rows).  Their time is a chain of latencies
+// (the camera sums, D^{-1} r, the CTA sum, the arrival of the last CTA), so the CTAs are small: 72 of
+// them for 1000 cameras; with 252 rows each, half as many SMs carried twice the arithmetic.
+constexpr int kUpdCams = 14;
+constexpr int kUpdThreads = 128;
 
 // Where one problem of the batch lives (fixed for a solve).
 struct Layout {
@@ -110,6 +113,7 @@ struct Outer {
     double tr;         // |-b~ - S x|^2 of the current x
     double tr_prev;    // the same before the last sweep (scales that sweep's residual history)
     double tol_in;     // relative tolerance of the next inner sweep
+    double unit;       // power of two near |-b~ - S x|: the sweep solves for the residual divided by it
     int status;
     int active;        // still refining
     int swept;         // takes part in the sweep being run
@@ -194,6 +198,19 @@ __device__ __forceinline__ void load_partial(ExactSum<float>& s, const double* s
     s.add_pair(v.x, v.y);
 }
 
+// the partial at *slot, written by another CTA of this launch (read past L1)
+__device__ __forceinline__ void load_partial_cg(ExactSum<double>& s, const double* slot) { s.s += __ldcg(slot); }
+__device__ __forceinline__ void load_partial_cg(ExactSum<float>& s, const double* slot) {
+    const float2 v = __ldcg(reinterpret_cast<const float2*>(slot));
+    s.add_pair(v.x, v.y);
+}
+template <typename T>
+__device__ __forceinline__ ExactSum<T> warp_total(ExactSum<T> s) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) combine_shfl(s, o);
+    return s;
+}
+
 // Value k of the kThreads / 32 warp sums in red (row stride nv), added as a fixed tree
 // ((w0 + w1) + (w2 + w3)) + ((w4 + w5) + (w6 + w7)): three dependent float64 additions.
 __device__ __forceinline__ double sum_warps(const double* red, int nv, int k) {
@@ -217,6 +234,14 @@ __device__ __forceinline__ void cta_sum_write(double (&v)[NV], double* out) {
     __syncthreads();
     if (threadIdx.x < NV) out[threadIdx.x] = sum_warps(&red[0][0], NV, threadIdx.x);
     __syncthreads();
+}
+
+// Sum of the Gram-style partials slots[0 .. np) in a fixed order (one warp; every lane returns it).
+template <typename T>
+__device__ __forceinline__ ExactSum<T> warp_sum_slots(const double* slots, int np) {
+    ExactSum<T> s;
+    for (int p = threadIdx.x & 31; p < np; p += 32) load_partial(s, slots + p);
+    return warp_total(s);
 }
 
 // Sum partial[p * stride + k] over p < np in a fixed order (called by one warp; every lane returns it).
@@ -291,42 +316,86 @@ __device__ __forceinline__ bool nothing_selected(const Ctl* ctl, const ItemList&
     return !__any_sync(0xffffffffu, any);
 }
 
-// Sum the CTA's NV values, publish them as partial[blockIdx.x], and let the last CTA of the grid
-// row to finish write the row's totals (in CTA order) to totals[0..NV).  Every CTA of the grid
-// row must call it.  Returns true (in every thread) in the CTA that wrote the totals, after they
-// are visible to the whole CTA.
-template <int NV>
-__device__ __forceinline__ bool grid_sum_finalize(double (&v)[NV], double* partial, int* cnt, double* totals) {
-    __shared__ double red[kThreads / 32][NV];
+// Sum the CTA's NV values (kUpdThreads threads), publish them as partial[blockIdx.x], and let the last
+// CTA of the grid row to finish write the row's totals (in CTA order) to totals[0..NV) (shared
+// memory).  Every CTA of the grid row must call it.  Returns true (in every thread) in the CTA that
+// wrote the totals, after they are visible to the whole CTA.  Warp k adds value k, so the CTA's sum
+// takes 3 additions and a shuffle tree in one warp per value instead of a tree in every warp.
+template <typename T, int NV>
+__device__ __forceinline__ bool grid_sum_finalize(const ExactSum<T> (&v)[NV], double* partial, int* cnt, double* totals) {
+    static_assert(NV <= kUpdThreads / 32, "one warp per value");
+    __shared__ double st[NV][kUpdThreads];   // slots of store_partial
     __shared__ int last;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        double s = warp_sum(v[k]);
-        if (lane == 0) red[wid][k] = s;
-    }
+    for (int k = 0; k < NV; ++k) store_partial(&st[k][threadIdx.x], v[k]);
     __syncthreads();
-    if (threadIdx.x < NV) partial[int64_t(blockIdx.x) * NV + threadIdx.x] = sum_warps(&red[0][0], NV, threadIdx.x);
-    __threadfence();
+    if (wid < NV) {
+        ExactSum<T> s;
+#pragma unroll
+        for (int u = 0; u < kUpdThreads / 32; ++u) load_partial(s, &st[wid][lane + 32 * u]);
+        s = warp_total(s);
+        if (lane == 0) {
+            store_partial(partial + int64_t(blockIdx.x) * NV + wid, s);
+            __threadfence();
+        }
+    }
     __syncthreads();
     if (threadIdx.x == 0) last = (atomicAdd(cnt, 1) == int(gridDim.x) - 1);
     __syncthreads();
     if (!last) return false;
     __threadfence();
     // warp k adds value k over the CTA partials: lane l takes partials l, l + 32, ... (independent
-    // loads, short float64 chains), then the fixed shuffle tree; partials of CTAs without rows are
-    // exact zeros, so the sum does not depend on the grid width
-    static_assert(NV <= kThreads / 32, "one warp per value");
+    // loads, short chains), then the fixed shuffle tree; partials of CTAs without rows are exact
+    // zeros, so the sum does not depend on the grid width
     if (wid < NV) {
-        double s = 0.0;
-        for (int b = lane; b < int(gridDim.x); b += 32) s += __ldcg(partial + int64_t(b) * NV + wid);
-        s = warp_sum(s);
-        if (lane == 0) totals[wid] = s;
+        ExactSum<T> s;
+        for (int b = lane; b < int(gridDim.x); b += 32) load_partial_cg(s, partial + int64_t(b) * NV + wid);
+        s = warp_total(s);
+        if (lane == 0) totals[wid] = s.value();
     }
     if (threadIdx.x == 0) *cnt = 0;
     __syncthreads();
     return true;
 }
+
+// Row of a camera's D^{-1} block, and its product with the camera's residual.  The float32 sweeps keep
+// the blocks in double-float (k_block_jacobi) and form the product with error-free transformations,
+// rounded once to float32, like the float64 product that it replaces: nine dependent float64
+// multiply-adds and nine conversions per row held the update at 12 us on 1000 cameras.
+template <typename T>
+struct DinvRow;
+template <>
+struct DinvRow<double> {
+    double d[9];
+    __device__ __forceinline__ void load(const double* row, bool act) {
+#pragma unroll
+        for (int b = 0; b < 9; ++b) d[b] = act ? row[b] : 0.0;
+    }
+    __device__ __forceinline__ double dot(const double* r) const {
+        double s = 0.0;
+#pragma unroll
+        for (int b = 0; b < 9; ++b) s += d[b] * r[b];
+        return s;
+    }
+};
+template <>
+struct DinvRow<float> {
+    float2 d[9];
+    __device__ __forceinline__ void load(const double* row, bool act) {
+#pragma unroll
+        for (int b = 0; b < 9; ++b) d[b] = act ? reinterpret_cast<const float2*>(row)[b] : make_float2(0.f, 0.f);
+    }
+    __device__ __forceinline__ float dot(const float* r) const {
+        ExactSum<float> s;
+#pragma unroll
+        for (int b = 0; b < 9; ++b) {
+            s.add(d[b].x, r[b]);
+            s.lo = __fmaf_rn(d[b].y, r[b], s.lo);
+        }
+        return __fadd_rn(s.hi, s.lo);
+    }
+};
 
 // ---- bulk copies (cp.async.bulk + mbarrier) --------------------------------------------
 
@@ -414,6 +483,24 @@ constexpr size_t spmv_smem() {
 // never fills a partly written sector from DRAM) and value 8 at tb[8 n_slots + e].
 constexpr int kTbHead = 8;
 
+
+// One camera's sums q^T p and p^T r (a warp; lanes 0..8 hold the rows, the others zeros) into the two
+// slots at camdot.
+template <typename T>
+__device__ __forceinline__ void camera_dots(int lane, T q, T p, T r, double* camdot) {
+    ExactSum<T> dq, dr;
+    dq.add(q, p);
+    dr.add(p, r);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {   // lanes 16..31 hold zeros
+        combine_shfl(dq, o);
+        combine_shfl(dr, o);
+    }
+    if (lane == 0) {
+        store_partial(camdot, dq);
+        store_partial(camdot + 1, dr);
+    }
+}
 
 // Tile cursor of a warp: the tiles of its selected items (WarpItems) in order, skipping empty
 // items.  The consumer loop selects items with the same predicate, which no kernel changes while
@@ -629,20 +716,9 @@ __global__ void __launch_bounds__(SpmvShape<T, CFG>::kWarps * 32, 1) k_spmv(
         if (fin) {
             const int64_t rowi = 9 * int64_t(it.row) + lane;
             if (lane < 9) out[ooff + rowi] = val;
-            if (MODE == 1 && !SYM) {
-                double dq = 0.0, dr = 0.0;
-                if (lane < 9) {
-                    const double pv = double(z[zoff + rowi]);
-                    dq = double(val) * pv;
-                    dr = pv * double(rvec[rowi]);
-                }
-                dq = warp_sum(dq);
-                dr = warp_sum(dr);
-                if (lane == 0) {
-                    camdot[2 * int64_t(it.row)] = dq;
-                    camdot[2 * int64_t(it.row) + 1] = dr;
-                }
-            }
+            if (MODE == 1 && !SYM)
+                camera_dots(lane, lane < 9 ? val : T(0), lane < 9 ? z[zoff + rowi] : T(0),
+                            lane < 9 ? rvec[rowi] : T(0), camdot + 2 * int64_t(it.row));
         }
     }
     if (bad) {
@@ -730,20 +806,9 @@ __global__ void __launch_bounds__(kColWarps * 32, 12) k_spmv_col(const int64_t* 
                 val = out[ooff + rowi] + val;
                 out[ooff + rowi] = val;
             }
-            if (MODE == 1) {
-                double dq = 0.0, dr = 0.0;
-                if (lane < 9) {
-                    const double pv = double(z[zoff + rowi]);
-                    dq = double(val) * pv;
-                    dr = pv * double(rvec[rowi]);
-                }
-                dq = warp_sum(dq);
-                dr = warp_sum(dr);
-                if (lane == 0) {
-                    camdot[2 * j] = dq;
-                    camdot[2 * j + 1] = dr;
-                }
-            }
+            if (MODE == 1)
+                camera_dots(lane, lane < 9 ? val : T(0), lane < 9 ? z[zoff + rowi] : T(0),
+                            lane < 9 ? rvec[rowi] : T(0), camdot + 2 * j);
         }
         __syncthreads();
     }
@@ -958,46 +1023,57 @@ __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
 
 // ---------------------------------------------------------------------------------------
 // initialisation shared by both algorithms: x = 0, r = sign * rhs, z = D^{-1} r, P_0 = z
-// (grid: CTAs x problems; thread = camera of the problem)
+// (grid: update CTAs x problems; thread = row, as in the update kernels; partial: one slot per CTA).
+// outer (mixed precision, may be null): r is divided by the sweep's unit, a power of two, so that the
+// float32 sums of a sweep start near one whatever the residual's size (their error terms would
+// otherwise leave the float32 range on late sweeps).
 
 template <typename T>
-__global__ void k_init_vec(const Layout* __restrict__ lay, const double* __restrict__ rhs, double sign,
-                           const double* __restrict__ scale, const double* __restrict__ Dinv, T* __restrict__ x,
-                           T* __restrict__ r, T* __restrict__ z, T* __restrict__ P, double* __restrict__ partial) {
+__global__ void __launch_bounds__(kUpdThreads) k_init_vec(const Layout* __restrict__ lay, const double* __restrict__ rhs,
+                                                          double sign, const double* __restrict__ scale,
+                                                          const double* __restrict__ Dinv, const Outer* __restrict__ outer,
+                                                          T* __restrict__ x, T* __restrict__ r, T* __restrict__ z,
+                                                          T* __restrict__ P, double* __restrict__ partial) {
     const Layout L = lay[blockIdx.y];
-    double v[1] = {0.0};
-    for (int64_t jl = gtid(); jl < L.nc; jl += gstride()) {
-        const int64_t j = L.c0 + jl;
-        double rv[9];
-#pragma unroll
-        for (int a = 0; a < 9; ++a) {
-            const double sa = scale ? scale[9 * j + a] : 1.0;
-            const T ra = T(sign * sa * rhs[9 * j + a]);
-            r[9 * j + a] = ra;
-            x[9 * j + a] = T(0);
-            rv[a] = double(ra);
-            v[0] += rv[a] * rv[a];
-        }
-        const double* D = Dinv + 81 * j;
-#pragma unroll
-        for (int a = 0; a < 9; ++a) {
-            double s = 0.0;
-#pragma unroll
-            for (int b = 0; b < 9; ++b) s += D[9 * a + b] * rv[b];
-            z[9 * j + a] = T(s);
-            P[L.hoff + 9 * jl + a] = T(s);
-        }
+    __shared__ T sr[kUpdCams * 9];
+    __shared__ double st[kUpdThreads];
+    const int t = threadIdx.x, cl = t / 9, a = t - 9 * (t / 9);
+    const int64_t jl = int64_t(blockIdx.x) * kUpdCams + cl;
+    const bool act = t < kUpdCams * 9 && jl < L.nc;
+    const int64_t i = 9 * (L.c0 + jl) + a;
+    if (outer) sign /= outer[blockIdx.y].unit;
+    DinvRow<T> D;
+    D.load(Dinv + 9 * i, act);
+    T rv = T(0);
+    if (act) {
+        rv = T(sign * (scale ? scale[i] : 1.0) * rhs[i]);
+        r[i] = rv;
+        x[i] = T(0);
     }
-    cta_sum_write<1>(v, partial + int64_t(blockIdx.y) * gridDim.x + blockIdx.x);
+    if (t < kUpdCams * 9) sr[t] = rv;
+    ExactSum<T> v;
+    v.add(rv, rv);
+    store_partial(&st[t], v);
+    __syncthreads();
+    if (act) {
+        const T zs = D.dot(sr + 9 * cl);
+        z[i] = zs;
+        P[L.hoff + 9 * jl + a] = zs;
+    }
+    if (t < 32) {
+        const ExactSum<T> s = warp_sum_slots<T>(st, kUpdThreads);
+        if (t == 0) store_partial(partial + int64_t(blockIdx.y) * gridDim.x + blockIdx.x, s);
+    }
 }
 
 // One warp per problem.  outer (mixed precision, may be null) supplies the sweep's tolerance and
 // iteration budget and leaves the problems that are not refined any more done from the start.
+template <typename T>
 __global__ void k_init_ctl(Ctl* ctl, const Layout* __restrict__ lay, const double* __restrict__ partial, int np,
                            const Params* __restrict__ prm, double stag, int direct_q,
                            const Outer* __restrict__ outer, int* blk_off, int* blk_w, int mi1) {
     const int p = blockIdx.x;
-    const double rr0 = sum_partials(partial + int64_t(p) * np, np, 1, 0);
+    const double rr0 = warp_sum_slots<T>(partial + int64_t(p) * np, np).value();
     if (threadIdx.x == 0) {
         Ctl c;
         memset(&c, 0, sizeof(c));
@@ -1093,106 +1169,105 @@ __device__ __forceinline__ double fast_rcp(double p) {
 // ---------------------------------------------------------------------------------------
 // Algorithm 1 (grid: CTAs x problems)
 
-// This thread's share of the per-camera sums (Delta, gamma) of cameras [0, nc): cameras
-// threadIdx.x + k blockDim.x, four at a time in interleaved sums (their loads in flight together),
-// added as (0 + 1) + (2 + 3).
-__device__ __forceinline__ void sum_camdot(const double* cd, int nc, double (&d)[2]) {
-    const int bd = blockDim.x;
-    double a0[4] = {0.0, 0.0, 0.0, 0.0}, a1[4] = {0.0, 0.0, 0.0, 0.0};
-    int j = threadIdx.x;
-    for (; j + 3 * bd < nc; j += 4 * bd)
+// The sums over cameras [0, nc) of the per-camera sums (Delta, gamma), returned to every thread of
+// the CTA: warp w takes value w mod 2 over the cameras of half w / 2 (64-camera stride, four
+// interleaved sums with their loads in flight together), then a shuffle tree and the two halves.
+template <typename T>
+__device__ __forceinline__ void sum_camdot(const double* cd, int nc, ExactSum<T>& Delta, ExactSum<T>& gamma) {
+    static_assert(kUpdThreads == 128, "two values x two halves");
+    __shared__ double sh[4];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    ExactSum<T> a[4];
+    const double* c = cd + (wid & 1);
+    int j = 32 * (wid >> 1) + lane;
+    for (; j + 192 < nc; j += 256)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            a0[u] += cd[2 * int64_t(j + u * bd)];
-            a1[u] += cd[2 * int64_t(j + u * bd) + 1];
-        }
+        for (int u = 0; u < 4; ++u) load_partial(a[u], c + 2 * int64_t(j + 64 * u));
 #pragma unroll
     for (int u = 0; u < 3; ++u)
-        if (j + u * bd < nc) {
-            a0[u] += cd[2 * int64_t(j + u * bd)];
-            a1[u] += cd[2 * int64_t(j + u * bd) + 1];
-        }
-    d[0] = (a0[0] + a0[1]) + (a0[2] + a0[3]);
-    d[1] = (a1[0] + a1[1]) + (a1[2] + a1[3]);
+        if (j + 64 * u < nc) load_partial(a[u], c + 2 * int64_t(j + 64 * u));
+    combine(a[0], a[1]);
+    combine(a[2], a[3]);
+    combine(a[0], a[2]);
+    a[0] = warp_total(a[0]);
+    if (lane == 0) store_partial(&sh[wid], a[0]);
+    __syncthreads();
+    load_partial(Delta, &sh[0]);
+    load_partial(Delta, &sh[2]);
+    load_partial(gamma, &sh[1]);
+    load_partial(gamma, &sh[3]);
 }
 
-__device__ void pcg_decide(Ctl* c, const double* tot, double* hist, int p, int nb);
+__device__ void pcg_decide(Ctl* c, double D, double g, const double* tot, double* hist, int p, int nb);
 
 // alpha = gamma / Delta; x += alpha p; r -= alpha q; z = D^{-1} r; totals of |r|^2, q^T z, r^T z,
 // then (the CTA that finalises the totals) the stop test and beta.
 // Delta and gamma are the sums over the problem's cameras (camera order) of the per-camera sums
-// of the product; every CTA forms them the same way, CTA 0 stores them for the decide step.
+// of the product; every CTA forms them the same way.
 // Thread = one row (9 per camera, kUpdCams cameras per CTA); the rows of a camera meet in
 // shared memory for z = D^{-1} r.  CTA b of a problem takes its cameras [b kUpdCams, ...), so the
 // partition depends on the problem alone (the grid has a CTA for every chunk of the largest).
+// Bound by latency: on 1000 cameras 12 us of a 22 us iteration when the sums ran in float64 (whose
+// pipe does 1.7 lanes per clock and SM, so each warp-wide addition of a shuffle tree costs as much as
+// a full one); 8.6 us with the float32 sweeps' sums as float pairs (the solve of that
+// case 13.4 -> 11.2 ms).
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_pcg_update(const double* __restrict__ Dinv, const T* __restrict__ P,
-                                                         const T* __restrict__ Q, T* __restrict__ x,
-                                                         T* __restrict__ r, T* __restrict__ z,
-                                                         const double* __restrict__ camdot,
-                                                         double* __restrict__ totals, double* __restrict__ dpart,
-                                                         int* __restrict__ dcnt, double* __restrict__ hist,
-                                                         Ctl* ctl) {
+__global__ void __launch_bounds__(kUpdThreads) k_pcg_update(const double* __restrict__ Dinv, const T* __restrict__ P,
+                                                            const T* __restrict__ Q, T* __restrict__ x,
+                                                            T* __restrict__ r, T* __restrict__ z,
+                                                            const double* __restrict__ camdot,
+                                                            double* __restrict__ dpart, int* __restrict__ dcnt,
+                                                            double* __restrict__ hist, Ctl* ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const int p = blockIdx.y;
     const Ctl& c = ctl[p];
     if (c.done) return;
     const int64_t c0 = c.lay.c0;
     const int nc = c.lay.nc;
-    __shared__ double dg[2];
     __shared__ T sr[kUpdCams * 9];
+    __shared__ double tot[3];
     const int t = threadIdx.x, cl = t / 9, a = t - 9 * (t / 9);
     const int64_t jl = int64_t(blockIdx.x) * kUpdCams + cl;
     const bool act = t < kUpdCams * 9 && jl < nc;
-    double drow[9];   // this row of the camera's D^{-1} block, requested before the CTA sum waits
-    {
-        double d[2];
-        sum_camdot(camdot + 2 * c0, nc, d);
-#pragma unroll
-        for (int b = 0; b < 9; ++b) drow[b] = act ? Dinv[81 * (c0 + jl) + 9 * a + b] : 0.0;
-        cta_sum_write<2>(d, dg);
-    }
-    double* tot = totals + int64_t(p) * kTotals;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        tot[0] = dg[0];
-        tot[1] = dg[1];
-    }
+    const int64_t hb = c.lay.hoff - 9 * c0;
+    const int64_t i = 9 * (c0 + jl) + a;
+    // this row's operands, requested before the CTA waits for the camera sums
+    DinvRow<T> D;
+    D.load(Dinv + 9 * i, act);
+    const T pv = act ? P[hb + i] : T(0), qv = act ? Q[hb + i] : T(0);
+    const T xv = act ? x[i] : T(0), r0 = act ? r[i] : T(0);
+    ExactSum<T> Delta, gamma;
+    sum_camdot<T>(camdot + 2 * c0, nc, Delta, gamma);
     // alpha = gamma / Delta; the float32 sweeps divide the rounded operands in float32 (a float64
     // division is a long dependent chain on this GPU's narrow float64 pipe)
     T alpha;
-    if constexpr (sizeof(T) == 4) alpha = __fdiv_rn(float(dg[1]), float(dg[0]));
-    else alpha = dg[1] * fast_rcp<2>(dg[0]);
-    const int64_t hb = c.lay.hoff - 9 * c0;
-    const int64_t i = 9 * (c0 + jl) + a;
-    double v[3] = {0.0, 0.0, 0.0};
-    T rv = T(0), qv = T(0);
+    if constexpr (sizeof(T) == 4) alpha = __fdiv_rn(__fadd_rn(gamma.hi, gamma.lo), __fadd_rn(Delta.hi, Delta.lo));
+    else alpha = gamma.s * fast_rcp<2>(Delta.s);
+    ExactSum<T> v[3];
+    T rv = T(0);
     if (act) {
-        x[i] = x[i] + alpha * P[hb + i];
-        qv = Q[hb + i];
-        rv = r[i] - alpha * qv;
+        x[i] = xv + alpha * pv;
+        rv = r0 - alpha * qv;
         r[i] = rv;
-        v[0] = double(rv) * double(rv);
+        v[0].add(rv, rv);
     }
     if (t < kUpdCams * 9) sr[t] = rv;
     __syncthreads();
     if (act) {
-        double s = 0.0;
-#pragma unroll
-        for (int b = 0; b < 9; ++b) s += drow[b] * double(sr[9 * cl + b]);
-        const T zs = T(s);
+        const T zs = D.dot(sr + 9 * cl);
         z[i] = zs;
-        v[1] = double(qv) * double(zs);
-        v[2] = double(rv) * double(zs);
+        v[1].add(qv, zs);
+        v[2].add(rv, zs);
     }
-    if (grid_sum_finalize<3>(v, dpart + int64_t(p) * gridDim.x * 3, dcnt + 4 * p, tot + 2) && threadIdx.x == 0)
-        pcg_decide(ctl + p, tot, hist, p, gridDim.y);
+    if (grid_sum_finalize<T, 3>(v, dpart + int64_t(p) * gridDim.x * 3, dcnt + 4 * p, tot) && threadIdx.x == 0)
+        pcg_decide(ctl + p, Delta.value(), gamma.value(), tot, hist, p, gridDim.y);
 }
 
 // stop test and beta = Phi / Delta for problem p (one thread, after the update's totals are in);
 // hist is iteration-major (it x nb)
-__device__ void pcg_decide(Ctl* c, const double* tot, double* hist, int p, int nb) {
+__device__ void pcg_decide(Ctl* c, double D, double g, const double* tot, double* hist, int p, int nb) {
     if (c->status == BA_ERR_TIMEOUT) { c->done = 1; return; }
-    const double D = tot[0], g = tot[1], rr = tot[2], phi = tot[3];
+    const double rr = tot[0], phi = tot[1];
     const int it = c->it + 1;
     c->it = it;
     c->Delta = D;
@@ -1208,7 +1283,7 @@ __device__ void pcg_decide(Ctl* c, const double* tot, double* hist, int p, int n
     } else if (it >= c->max_iters) {
         c->done = 1;
         c->status = BA_ERR_NOT_CONVERGED;
-    } else if (c->stag > 0.0 && g * g < c->stag * tot[4] * D) {   // (g^2 / D) / tot[4] < stag
+    } else if (c->stag > 0.0 && g * g < c->stag * tot[2] * D) {   // (g^2 / D) / r^T z < stag
         c->done = 1;          // no measurable progress left at this precision: end the sweep
         c->status = BA_OK;
     } else {
@@ -1570,16 +1645,15 @@ __global__ void __launch_bounds__(kSmallThreads) k_mcg_small(Ctl* ctl, const dou
 __device__ void mcg_decide(Ctl* c, const double* tot, double* hist, int* blk_off, int* blk_w, int mi1, int p, int nb);
 
 // x += P_i alpha; r -= Q_i alpha; z = D^{-1} r; totals of |r|^2 and r^T z, then (last CTA) the
-// decide step (grid: CTAs x problems;
-// thread = one row, as in k_pcg_update).
+// decide step (grid: CTAs x problems; thread = one row, as in k_pcg_update).  The columns of the block
+// are requested together (up to 16 of P and of Q per row).
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_mcg_update(const double* __restrict__ Dinv, const T* __restrict__ P,
-                                                         const T* __restrict__ Q, T* __restrict__ x,
-                                                         T* __restrict__ r, T* __restrict__ z,
-                                                         double* __restrict__ dpart, int* __restrict__ dcnt,
-                                                         double* __restrict__ totals, double* __restrict__ hist,
-                                                         int* __restrict__ blk_off, int* __restrict__ blk_w, int mi1,
-                                                         Ctl* ctl) {
+__global__ void __launch_bounds__(kUpdThreads) k_mcg_update(const double* __restrict__ Dinv, const T* __restrict__ P,
+                                                            const T* __restrict__ Q, T* __restrict__ x,
+                                                            T* __restrict__ r, T* __restrict__ z,
+                                                            double* __restrict__ dpart, int* __restrict__ dcnt,
+                                                            double* __restrict__ hist, int* __restrict__ blk_off,
+                                                            int* __restrict__ blk_w, int mi1, Ctl* ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const int p = blockIdx.y;
     const Ctl& c = ctl[p];
@@ -1592,40 +1666,46 @@ __global__ void __launch_bounds__(kThreads) k_mcg_update(const double* __restric
     const T* Qp = Q + c.lay.hoff + int64_t(off) * n;
     __shared__ T sal[kMaxDirs];
     __shared__ T sr[kUpdCams * 9];
+    __shared__ double tot[2];
     const int t = threadIdx.x, cl = t / 9, a = t - 9 * (t / 9);
     const int64_t jl = int64_t(blockIdx.x) * kUpdCams + cl;
     const bool act = t < kUpdCams * 9 && jl < nc;
-    double drow[9];   // this row of the camera's D^{-1} block, requested early
+    const int64_t il = 9 * jl + a, i = 9 * c0 + il;
+    DinvRow<T> D;
+    D.load(Dinv + 9 * i, act);
+    T pv[kMaxDirs], qv[kMaxDirs];
 #pragma unroll
-    for (int b = 0; b < 9; ++b) drow[b] = act ? Dinv[81 * (c0 + jl) + 9 * a + b] : 0.0;
+    for (int b = 0; b < kMaxDirs; ++b) {
+        const bool in = act && b < w;
+        pv[b] = in ? Pp[int64_t(b) * n + il] : T(0);
+        qv[b] = in ? Qp[int64_t(b) * n + il] : T(0);
+    }
+    const T xv = act ? x[i] : T(0), r0 = act ? r[i] : T(0);
     if (threadIdx.x < kMaxDirs) sal[threadIdx.x] = int(threadIdx.x) < w ? T(c.alpha_v[threadIdx.x]) : T(0);
     __syncthreads();
-    const int64_t il = 9 * jl + a, i = 9 * c0 + il;
-    double v[2] = {0.0, 0.0};
+    ExactSum<T> v[2];
     T rv = T(0);
     if (act) {
         T dx = T(0), dr = T(0);
-        for (int b = 0; b < w; ++b) {
-            dx += Pp[int64_t(b) * n + il] * sal[b];
-            dr += Qp[int64_t(b) * n + il] * sal[b];
-        }
-        x[i] = x[i] + dx;
-        rv = r[i] - dr;
+#pragma unroll
+        for (int b = 0; b < kMaxDirs; ++b)
+            if (b < w) {   // columns past w may hold anything (alpha there is 0)
+                dx += pv[b] * sal[b];
+                dr += qv[b] * sal[b];
+            }
+        x[i] = xv + dx;
+        rv = r0 - dr;
         r[i] = rv;
-        v[0] = double(rv) * double(rv);
+        v[0].add(rv, rv);
     }
     if (t < kUpdCams * 9) sr[t] = rv;
     __syncthreads();
     if (act) {
-        double s = 0.0;
-#pragma unroll
-        for (int b = 0; b < 9; ++b) s += drow[b] * double(sr[9 * cl + b]);
-        const T zs = T(s);
+        const T zs = D.dot(sr + 9 * cl);
         z[i] = zs;
-        v[1] = double(rv) * double(zs);
+        v[1].add(rv, zs);
     }
-    double* tot = totals + int64_t(p) * kTotals + 8;
-    if (grid_sum_finalize<2>(v, dpart + int64_t(p) * gridDim.x * 2, dcnt + 4 * p + 1, tot) && threadIdx.x == 0)
+    if (grid_sum_finalize<T, 2>(v, dpart + int64_t(p) * gridDim.x * 2, dcnt + 4 * p + 1, tot) && threadIdx.x == 0)
         mcg_decide(ctl + p, tot, hist, blk_off, blk_w, mi1, p, gridDim.y);
 }
 
@@ -1997,13 +2077,17 @@ __global__ void k_true_reduce(Ctl* ctl, const double* __restrict__ partial) {
     }
 }
 
-// mixed precision: x64 += Lam (double) d32, the inner solution mapped back from the scaled system
-// x += Lam d (a float32 sweep's correction, unscaled), and x split into double-float for the true
-// residual that follows (its per-observation products take no float64 input)
-__global__ void k_accumulate(int64_t n, const float* __restrict__ d, const double* __restrict__ lam,
-                             double* __restrict__ x, float2* __restrict__ xd) {
-    for (int64_t i = gtid(); i < n; i += gstride()) {
-        const double v = x[i] + lam[i] * double(d[i]);
+// mixed precision: x += unit Lam d, a float32 sweep's correction mapped back from the scaled system,
+// and x split into double-float for the true residual that follows (its per-observation products take
+// no float64 input); grid: CTAs x problems
+__global__ void k_accumulate(const Layout* __restrict__ lay, const Outer* __restrict__ outer,
+                             const float* __restrict__ d, const double* __restrict__ lam, double* __restrict__ x,
+                             float2* __restrict__ xd) {
+    const Layout L = lay[blockIdx.y];
+    const double unit = outer[blockIdx.y].unit;
+    for (int64_t il = gtid(); il < 9 * int64_t(L.nc); il += gstride()) {
+        const int64_t i = 9 * int64_t(L.c0) + il;
+        const double v = x[i] + lam[i] * (unit * double(d[i]));
         x[i] = v;
         const float h = __double2float_rn(v);
         xd[i] = make_float2(h, __double2float_rn(v - double(h)));
@@ -2034,6 +2118,7 @@ __global__ void k_outer_init(const Layout* __restrict__ lay, const double* __res
         o.bb = s[0];
         o.tr = s[0];
         o.tr_prev = s[0];
+        o.unit = 1.0;
         o.status = s[0] == 0.0 ? BA_OK : BA_ERR_NOT_CONVERGED;
         o.active = s[0] == 0.0 ? 0 : 1;
         outer[blockIdx.x] = o;
@@ -2063,6 +2148,7 @@ __global__ void k_refine_plan(Outer* outer, int nb, const Params* __restrict__ p
         double t = need > 0.1 * inner_tol ? fmax(0.3 * need, 0.1 * inner_tol) : inner_tol;
         if (t >= 1.0) t = 0.5;
         o->tol_in = t;
+        o->unit = ldexp(1.0, max(-900, min(900, ilogb(sqrt(o->tr)))));
         o->max_in = prm->max_iters - o->iters;
         o->swept = 1;
         mine = 1;
@@ -2147,7 +2233,7 @@ struct Solver {
     int nb = 0;               // problems
     int64_t n = 0;            // 9 n_c over all problems
     int mi1 = 0;              // per-problem stride of the per-step arrays (max_iters + 1)
-    int gx = 1;               // grid width of the per-camera kernels
+    int gx = 1;               // grid width of the kernels over all rows of a problem (x += d)
     int gu = 1;               // grid width of the update kernels (kUpdCams cameras per CTA)
     int gg = 1;               // Gram grid width
     int gq = 1;               // grid width of the per-row kernels
@@ -2156,7 +2242,7 @@ struct Solver {
     int gcol = 1;             // grid width of the column pass of the symmetric product (a CTA per camera)
     std::vector<Layout> lay;  // of the current solve
     Buf P, Q, r, z, xw, PT, part_a, part_b, part_cam, dpinv, beta, betaf, phip, hist, blk_off, blk_w, ctl, outer, rt,
-        lay_d, totals, dpart, dcnt, camdot, params, loops;
+        lay_d, dpart, dcnt, camdot, params, loops;
     Ctl* h_ctl = nullptr;     // pinned, nb
     Outer* h_outer = nullptr; // pinned, nb
     Params* h_params = nullptr;   // pinned staging of the per-solve arguments
@@ -2436,8 +2522,8 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     w->nb = nb;
     w->n = n;
     w->mi1 = std::max(w->mi1, a.max_iters + 1);
-    w->gx = int(std::min<int64_t>(G, (nc_max + kThreads - 1) / kThreads));
-    if ((int64_t(nc_max) + kUpdCams - 1) / kUpdCams > 65535) throw Error(BA_ERR_INVALID_ARG, "too many cameras in one problem");
+    w->gx = int(std::min<int64_t>(std::max(1, 4 * G / nb), (9 * int64_t(nc_max) + kThreads - 1) / kThreads));
+    if ((int64_t(nc_max) + 27) / 28 > 65535) throw Error(BA_ERR_INVALID_ARG, "too many cameras in one problem");
     w->gu = (nc_max + kUpdCams - 1) / kUpdCams;
     w->gg = int(std::min<int64_t>(G, (9 * int64_t(nc_max) + 127) / 128));
     w->gq = std::max(1, G / nb);
@@ -2465,7 +2551,7 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     grow(w->xw, size_t(n) * elt);
     grow(w->PT, size_t(n) * kMaxDirs * elt);
     grow(w->part_a, size_t(nb) * w->gg * kGramMax * sizeof(double));
-    grow(w->part_b, size_t(nb) * w->gx * sizeof(double));
+    grow(w->part_b, size_t(nb) * w->gu * sizeof(double));
     grow(w->part_cam, size_t(s.n_c) * 2 * sizeof(double));
     grow(w->dpinv, size_t(nb) * w->mi1 * kMaxDirs * kMaxDirs * sizeof(double));
     grow(w->beta, size_t(boff) * kMaxDirs * sizeof(double));
@@ -2478,7 +2564,6 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     grow(w->outer, size_t(nb) * sizeof(Outer));
     grow(w->rt, size_t(n) * sizeof(double));
     grow(w->lay_d, size_t(nb) * sizeof(Layout));
-    grow(w->totals, size_t(nb) * kTotals * sizeof(double));
     grow(w->dpart, size_t(nb) * w->gu * 5 * sizeof(double));
     grow(w->camdot, size_t(s.n_c) * 2 * sizeof(double));
     grow(w->params, sizeof(Params));
@@ -2515,7 +2600,7 @@ void solver_destroy(Solver* w) {
     if (!w) return;
     Buf* bufs[] = {&w->P, &w->Q, &w->r, &w->z, &w->xw, &w->PT, &w->part_a, &w->part_b, &w->part_cam, &w->dpinv,
                    &w->beta, &w->betaf, &w->phip, &w->hist, &w->blk_off, &w->blk_w, &w->ctl, &w->outer, &w->rt,
-                   &w->lay_d, &w->totals, &w->dpart, &w->dcnt, &w->camdot, &w->params, &w->loops};
+                   &w->lay_d, &w->dpart, &w->dcnt, &w->camdot, &w->params, &w->loops};
     for (Buf* b : bufs) free_buf(*b);
     for (SolveExec* e : w->execs) {
         cudaGraphExecDestroy(e->exec);
@@ -2618,21 +2703,20 @@ static int enqueue_iteration(Solver* w, const Structure& s, const T* S, const T*
     T* r = ptr<T>(w->r);
     T* z = ptr<T>(w->z);
     Ctl* ctl = ptr<Ctl>(w->ctl);
-    double* totals = ptr<double>(w->totals);
     int* dcnt = ptr<int>(w->dcnt);
     const int Gt = num_sms();   // tile-streaming products: one CTA per SM
     if (!mcg) {
         const int np = enqueue_product<T, 1>(w, s, S, Su, P, kSelLive, Q, r, st);
-        launch_chained(k_pcg_update<T>, dim3(w->gu, nb), dim3(kThreads), 0, st, Dinv, P, Q, x, r, z,
-                       ptr<double>(w->camdot), totals, ptr<double>(w->dpart), dcnt, ptr<double>(w->hist), ctl);
+        launch_chained(k_pcg_update<T>, dim3(w->gu, nb), dim3(kUpdThreads), 0, st, Dinv, P, Q, x, r, z,
+                       ptr<double>(w->camdot), ptr<double>(w->dpart), dcnt, ptr<double>(w->hist), ctl);
         launch_chained(k_pcg_dir<T>, dim3(w->gq, nb), dim3(kThreads), 0, st, z, P, ctl);
         return np + 2;
     } else {
         launch_chained(k_mcg_gram<T>, dim3(w->gg, nb), dim3(kThreads), 0, st, P, Q, r, ptr<double>(w->part_a), ctl);
         launch_chained(k_mcg_small<T>, dim3(nb), dim3(kSmallThreads), 0, st, ctl, ptr<double>(w->part_a), w->gg,
                        ptr<double>(w->dpinv), w->mi1);
-        launch_chained(k_mcg_update<T>, dim3(w->gu, nb), dim3(kThreads), 0, st, Dinv, P, Q, x, r, z,
-                       ptr<double>(w->dpart) + 3 * size_t(nb) * w->gu, dcnt, totals, ptr<double>(w->hist),
+        launch_chained(k_mcg_update<T>, dim3(w->gu, nb), dim3(kUpdThreads), 0, st, Dinv, P, Q, x, r, z,
+                       ptr<double>(w->dpart) + 3 * size_t(nb) * w->gu, dcnt, ptr<double>(w->hist),
                        ptr<int>(w->blk_off), ptr<int>(w->blk_w), w->mi1, ctl);
         launch_chained(k_mcg_phi<T>, dim3(w->gphi, nb), dim3(kThreads), 0, st, Q, z, ptr<double>(w->phip), ctl);
         T* betat = sizeof(T) == 8 ? ptr<T>(w->beta) : ptr<T>(w->betaf);
@@ -2669,9 +2753,10 @@ template <typename T>
 static int krylov_init(Solver* w, const Structure& s, const T* S, const T* Su, const double* Dinv, const double* rhs,
                        double sign, const double* scale, T* x, const Outer* outer, cudaStream_t st, bool q0 = true) {
     const int nb = w->nb;
-    k_init_vec<T><<<dim3(w->gx, nb), kThreads, 0, st>>>(ptr<Layout>(w->lay_d), rhs, sign, scale, Dinv, x, ptr<T>(w->r),
-                                                         ptr<T>(w->z), ptr<T>(w->P), ptr<double>(w->part_b));
-    k_init_ctl<<<nb, 32, 0, st>>>(ptr<Ctl>(w->ctl), ptr<Layout>(w->lay_d), ptr<double>(w->part_b), w->gx,
+    k_init_vec<T><<<dim3(w->gu, nb), kUpdThreads, 0, st>>>(ptr<Layout>(w->lay_d), rhs, sign, scale, Dinv, outer, x,
+                                                            ptr<T>(w->r), ptr<T>(w->z), ptr<T>(w->P),
+                                                            ptr<double>(w->part_b));
+    k_init_ctl<T><<<nb, 32, 0, st>>>(ptr<Ctl>(w->ctl), ptr<Layout>(w->lay_d), ptr<double>(w->part_b), w->gu,
                                   ptr<Params>(w->params), sizeof(T) == 4 ? kStagnation : 0.0, sizeof(T) == 4 ? 1 : 0,
                                   outer, ptr<int>(w->blk_off), ptr<int>(w->blk_w), w->mi1);
     return 2 + (q0 ? enqueue_product<T, 0>(w, s, S, Su, ptr<T>(w->P), kSelLive, ptr<T>(w->Q), nullptr, st) : 0);
@@ -2778,7 +2863,8 @@ static cudaGraphExec_t build_solve_graph(Solver* w, const Structure& s, const Sy
             int kpre = 0;
             capture_krylov<float>(w, s, y.S32, y.S32u, y.Dhat, ptr<double>(w->rt), 1.0, y.lam, ptr<float>(w->xw),
                                   ptr<Outer>(w->outer), mcg, a.chunk, c2, w->cap3, &kpre, &gc.body);
-            k_accumulate<<<grid_for_host(n), kThreads, 0, c2>>>(n, ptr<float>(w->xw), y.lam, x, y.xd);
+            k_accumulate<<<dim3(w->gx, nb), kThreads, 0, c2>>>(ptr<Layout>(w->lay_d), ptr<Outer>(w->outer),
+                                                               ptr<float>(w->xw), y.lam, x, y.xd);
             const int tr = true_residual(w, s, y, x, ptr<double>(w->rt), c2);
             k_refine_after<<<nb, 32, 0, c2>>>(ptr<Ctl>(w->ctl), ptr<Outer>(w->outer), ptr<Params>(w->params));
             k_refine_plan<<<1, kThreads, 0, c2>>>(ptr<Outer>(w->outer), nb, ptr<Params>(w->params), ho, 1,
@@ -2879,7 +2965,8 @@ static void run_host_loops(Solver* w, const Structure& s, const System& y, const
                                            ptr<float>(w->xw), ptr<Outer>(w->outer), st, a.mcg != 0);
             k_loop_cond<<<1, kThreads, 0, st>>>(none, 0, ptr<Ctl>(w->ctl), nb, lp, 1, a.chunk, prm);
             launches += 1 + host_krylov_loop(w, chunk_exec, gc, a, st, waits);
-            k_accumulate<<<grid_for_host(n), kThreads, 0, st>>>(n, ptr<float>(w->xw), y.lam, x, y.xd);
+            k_accumulate<<<dim3(w->gx, nb), kThreads, 0, st>>>(ptr<Layout>(w->lay_d), ptr<Outer>(w->outer),
+                                                               ptr<float>(w->xw), y.lam, x, y.xd);
             launches += 1 + true_residual(w, s, y, x, ptr<double>(w->rt), st);
             k_refine_after<<<nb, 32, 0, st>>>(ptr<Ctl>(w->ctl), ptr<Outer>(w->outer), prm);
             k_refine_plan<<<1, kThreads, 0, st>>>(ptr<Outer>(w->outer), nb, prm, none, 0, lp, 1);
