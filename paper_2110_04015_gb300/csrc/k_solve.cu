@@ -397,6 +397,16 @@ struct DinvRow<float> {
     }
 };
 
+// 16-byte asynchronous copies global -> shared (both addresses 16-byte aligned)
+template <typename T>
+__device__ __forceinline__ void cp_async16(T* dst, const T* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+                 "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
+
 // ---- bulk copies (cp.async.bulk + mbarrier) --------------------------------------------
 
 // Bounded mbarrier waits: after `polls` unsuccessful polls a wait gives up (polls = 0: at once); the
@@ -1768,250 +1778,316 @@ __device__ void mcg_decide(Ctl* c, const double* tot, double* hist, int* blk_off
 }
 
 // partial sums of Q[:, c]^T z over row chunks inside each subset:
-// phip[(c * n_eff + s) * K + k] for c < hist_cols (one warp per entry; grid: CTAs x problems)
-template <typename T>
-__global__ void k_mcg_phi(const T* __restrict__ Q, const T* __restrict__ z, double* __restrict__ phip,
-                          const Ctl* __restrict__ ctl) {
-    wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
-    const Ctl& c = ctl[blockIdx.y];
-    if (c.done) return;
+// phip[(c * n_eff + s) * K + k] for c < hist_cols, as store_partial slots (grid: CTAs x problems).
+// Reads the whole history once, so it is bound by memory (L2 while the history fits): a warp takes one
+// row chunk of up to kPhiCols columns at once, 8 rows of each in flight (32 loads a lane), and reads z
+// once for all of them.  A column at a time with float64 shuffle trees ran at 2.1 TB/s (34 us on
+// 2000 columns of 9000 rows; now 21 us).  Fewer columns at once when there are not enough chunks for
+// the warps; a column's sum does not depend on it.
+constexpr int kPhiCols = 4;
+template <typename T, int NC>
+__device__ __forceinline__ void phi_columns(const T* __restrict__ qc, int64_t n, const T* __restrict__ zp, int r0, int r1,
+                                            double* __restrict__ out, int64_t ostride) {
     const int lane = threadIdx.x & 31;
-    const int nc = c.lay.nc;
-    const int64_t n = int64_t(nc) * 9;
-    const int n_eff = c.n_eff, sz = c.sz, K = c.K;
-    const int cz = (sz + K - 1) / K;
-    const int64_t items = int64_t(c.hist_cols) * n_eff * K;
-    const T* Qp = Q + c.lay.hoff;
-    const T* zp = z + 9 * int64_t(c.lay.c0);
-    double* ph = phip + c.lay.phoff;
-    for (int64_t it = gtid() >> 5; it < items; it += gstride() >> 5) {
-        const int k = int(it % K);
-        const int64_t cs = it / K;
-        const int s = int(cs % n_eff);
-        const int64_t cc = cs / n_eff;
-        int j0 = s * sz + k * cz;
-        int j1 = j0 + cz;
-        const int send = (s + 1) * sz < nc ? (s + 1) * sz : nc;
-        if (j1 > send) j1 = send;
-        const T* qc = Qp + cc * n;
-        ExactSum<T> acc;
-        for (int64_t row = int64_t(j0) * 9 + lane; row < int64_t(j1) * 9; row += 32) acc.add(qc[row], zp[row]);
-        const double sum = warp_sum(acc.value());
-        if (lane == 0) ph[it] = sum;
+    constexpr int U = 8;
+    ExactSum<T> acc[NC];
+    for (int base = r0 + lane; base < r1; base += 32 * U) {
+        T zv[U], qv[NC][U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int row = base + 32 * u;
+            const bool in = row < r1;
+            zv[u] = in ? zp[row] : T(0);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) qv[c][u] = in ? qc[c * n + row] : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) acc[c].add(qv[c][u], zv[u]);
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        acc[c] = warp_total(acc[c]);
+        if (lane == 0) store_partial(out + c * ostride, acc[c]);
     }
 }
 
-// beta_{i,j} = Delta_j^+ Phi_{i,j} for every history block j, into beta rows (one warp per block);
-// betat receives the same rows in the Krylov storage type (float32 sweeps), so the
-// reorthogonalisation reads them without conversions.  Float64 additions form long dependent
-// chains on this GPU, so the sums are interleaved: with 32 or more entries a lane carries up to 8
-// entries side by side; with fewer, G lanes share an entry's partials (lane g of the group takes
-// k = g, g + G, ... into 4 interleaved sums) and add them in a fixed shuffle tree.
 template <typename T>
-__global__ void k_mcg_beta(const double* __restrict__ phip, const double* __restrict__ dpinv,
-                           const int* __restrict__ blk_off, const int* __restrict__ blk_w, double* __restrict__ beta,
-                           T* __restrict__ betat, const Ctl* __restrict__ ctl, int mi1) {
+__global__ void __launch_bounds__(kThreads) k_mcg_phi(const T* __restrict__ Q, const T* __restrict__ z,
+                                                      double* __restrict__ phip, const Ctl* __restrict__ ctl) {
+    wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
+    const Ctl& c = ctl[blockIdx.y];
+    if (c.done) return;
+    const int nc = c.lay.nc;
+    const int64_t n = int64_t(nc) * 9;
+    const int sz = c.sz, K = c.K, hist = c.hist_cols, chunks = c.n_eff * K;
+    const int cz = (sz + K - 1) / K;
+    const T* Qp = Q + c.lay.hoff;
+    const T* zp = z + 9 * int64_t(c.lay.c0);
+    double* ph = phip + c.lay.phoff;
+    const int64_t warps = gstride() >> 5;
+    const int nb = 2 * int64_t(hist) * chunks >= kPhiCols * warps ? kPhiCols : 1;   // columns at once
+    const int64_t items = int64_t((hist + nb - 1) / nb) * chunks;
+    for (int64_t it = gtid() >> 5; it < items; it += warps) {
+        const int ch = int(it % chunks), c0 = int(it / chunks) * nb;
+        const int s = ch / K, k = ch - s * K;
+        int j0 = s * sz + k * cz, j1 = j0 + cz;
+        const int send = (s + 1) * sz < nc ? (s + 1) * sz : nc;
+        if (j1 > send) j1 = send;
+        const T* qc = Qp + int64_t(c0) * n;
+        double* out = ph + int64_t(c0) * chunks + ch;
+        const int m = hist - c0 < nb ? hist - c0 : nb;
+        if (m == kPhiCols) phi_columns<T, kPhiCols>(qc, n, zp, 9 * j0, 9 * j1, out, chunks);
+        else
+            for (int u = 0; u < m; ++u) phi_columns<T, 1>(qc + u * n, n, zp, 9 * j0, 9 * j1, out + int64_t(u) * chunks, chunks);
+    }
+}
+
+// Phi_j (wj x w) of one history block, entry e = a w + s: the partials of history column off + a over
+// subset s (local block) or over every subset (global block); they are contiguous.  nt threads
+// (t = 0 .. nt - 1, whole warps): G of them share an entry, each adds every G-th partial into two
+// interleaved sums, and the group's sums meet in a fixed shuffle tree.
+template <typename T>
+__device__ __forceinline__ void phi_block(const double* ph, int off, int w, int ne, int m, int n_eff, int K, bool local,
+                                          int t, int nt, double* sphi) {
+    int G = 1;
+    while (G < 32 && 2 * G * ne <= nt) G *= 2;
+    const int e = t / G, g = t % G;
+    if (t - (t & 31) >= ne * G) return;   // warps without an entry (their shuffles go whole)
+    ExactSum<T> a0, a1;
+    if (e < ne) {
+        const int a = e / w, s2 = e - w * (e / w);
+        const int64_t cc = off + a;
+        const double* sp = local ? ph + (cc * n_eff + s2) * K : ph + cc * n_eff * K;
+        int k = g;
+        for (; k + G < m; k += 2 * G) {
+            load_partial(a0, sp + k);
+            load_partial(a1, sp + k + G);
+        }
+        if (k < m) load_partial(a0, sp + k);
+    }
+    combine(a0, a1);
+    for (int o = G / 2; o > 0; o >>= 1) combine_shfl(a0, o);
+    if (e < ne && g == 0) sphi[e] = a0.value();
+}
+
+// Entry (a, s) of Delta_j^+ Phi_j in float64, four interleaved sums (a float64 operation has a long
+// latency on this GPU).
+__device__ __forceinline__ double beta_entry(const double* Dp, const double* sphi, int a, int s, int w, int wj) {
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int b = 0; b < kMaxDirs; b += 4)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (b + u < wj) v[u] += Dp[a * kMaxDirs + b + u] * sphi[(b + u) * w + s];
+    return (v[0] + v[1]) + (v[2] + v[3]);
+}
+
+// beta_{i,j} = Delta_j^+ Phi_{i,j} for every history block j, into beta rows in the Krylov storage type
+// (the float64 product rounded once).  Blocks go round the CTAs (block jb to CTA jb mod gridDim.x),
+// so consecutive ones run on different SMs; a block of 64 entries or more takes the whole CTA (a
+// thread per entry), smaller ones a warp each.  With a warp per 16 x 16 block the 128 float64
+// multiply-adds of a warp were a chain of 13 us (2000 columns); 4.8 us with the CTA.
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_mcg_beta(const double* __restrict__ phip, const double* __restrict__ dpinv,
+                                                       const int* __restrict__ blk_off, const int* __restrict__ blk_w,
+                                                       T* __restrict__ beta, const Ctl* __restrict__ ctl, int mi1) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const int p = blockIdx.y;
     const Ctl& c = ctl[p];
     if (c.done) return;
-    __shared__ double sphi[kThreads / 32][kMaxDirs * kMaxDirs];
+    constexpr int NW = kThreads / 32;
+    constexpr int kBig = 64;                          // entries from which a block takes the CTA
+    __shared__ double sphi[kMaxDirs * kMaxDirs];
+    __shared__ double swarp[NW][kBig];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nblk = c.it;   // blocks 0..it-1 are the history
-    const int n_eff = c.n_eff, K = c.K, w = c.w_new, local = c.local;
+    const int n_eff = c.n_eff, K = c.K, w = c.w_new;
+    const bool local = c.local != 0;
     const int m = local ? K : n_eff * K;   // partials per Phi entry
     const double* ph = phip + c.lay.phoff;
     const int* bo = blk_off + int64_t(p) * mi1;
     const int* bw = blk_w + int64_t(p) * mi1;
-    double* Bp = beta + c.lay.boff * kMaxDirs;
-    T* Bt = betat + c.lay.boff * kMaxDirs;
-    // block jb goes to warp (jb / gridDim.x) of CTA (jb mod gridDim.x): consecutive blocks on
-    // different SMs, so their float64 products share no SM's float64 pipe
-    for (int64_t jb = blockIdx.x + int64_t(gridDim.x) * wid; jb < nblk; jb += int64_t(gridDim.x) * (blockDim.x >> 5)) {
-        const int off = bo[jb], wj = bw[jb];
-        const int ne = wj * w;
-        // entries e = lane + 32 u of this lane: (a, s) = (e / w, e mod w)
-        int ea[8], es[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int e = lane + 32 * u;
-            ea[u] = e / w;
-            es[u] = e - w * ea[u];
-        }
-        // Phi_j (wj x w): entry (a, s) adds the partials of history column off + a over subset s
-        // (local block) or over every subset (global block); they are contiguous
-        auto src = [&](int a, int s2) -> const double* {
-            const int64_t cc = off + a;
-            return local ? ph + (cc * n_eff + s2) * K : ph + cc * n_eff * K;
-        };
-        if (ne >= 32) {
-            double v[8];
-            const double* sp[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                v[u] = 0.0;
-                sp[u] = src(ea[u], es[u]);
-            }
-            for (int k = 0; k < m; ++k)
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (lane + 32 * u < ne) v[u] += sp[u][k];
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (lane + 32 * u < ne) sphi[wid][lane + 32 * u] = v[u];
-        } else {
-            int G = 1;
-            while (2 * G * ne <= 32) G *= 2;
-            const int e = lane / G, g = lane % G;
-            double v0 = 0.0, v1 = 0.0, v2 = 0.0, v3 = 0.0;
-            if (e < ne) {
-                const double* sp = src(e / w, e % w);
-                int k = g;
-                for (; k + 3 * G < m; k += 4 * G) {
-                    v0 += sp[k];
-                    v1 += sp[k + G];
-                    v2 += sp[k + 2 * G];
-                    v3 += sp[k + 3 * G];
+    T* Bp = beta + c.lay.boff * kMaxDirs;
+    for (int64_t j0 = blockIdx.x; j0 < nblk; j0 += int64_t(gridDim.x) * NW) {
+        const int64_t jw = j0 + int64_t(gridDim.x) * wid;   // this warp's block
+        if (jw < nblk && bw[jw] * w < kBig) {
+            const int off = bo[jw], ne = bw[jw] * w;
+            // a warp has no more lanes than it needs for 32 entries at a time
+            for (int e0 = 0; e0 < ne; e0 += 32) {
+                const int part = ne - e0 < 32 ? ne - e0 : 32;
+                if (e0 == 0 && part == ne) phi_block<T>(ph, off, w, ne, m, n_eff, K, local, lane, 32, swarp[wid]);
+                else if (lane < part) {
+                    const int e = e0 + lane, a = e / w, s2 = e - w * (e / w);
+                    const double* sp = local ? ph + (int64_t(off + a) * n_eff + s2) * K : ph + int64_t(off + a) * n_eff * K;
+                    ExactSum<T> a0;
+                    for (int k = 0; k < m; ++k) load_partial(a0, sp + k);
+                    swarp[wid][e] = a0.value();
                 }
-                if (k < m) v0 += sp[k];
-                if (k + G < m) v1 += sp[k + G];
-                if (k + 2 * G < m) v2 += sp[k + 2 * G];
             }
-            double v = (v0 + v1) + (v2 + v3);
-            for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (e < ne && g == 0) sphi[wid][e] = v;
+            __syncwarp();
+            const double* Dp = dpinv + (int64_t(p) * mi1 + jw) * kMaxDirs * kMaxDirs;
+            for (int e = lane; e < ne; e += 32)
+                Bp[int64_t(off + e / w) * kMaxDirs + e % w] = T(beta_entry(Dp, swarp[wid], e / w, e % w, w, bw[jw]));
+            __syncwarp();
         }
-        __syncwarp();
-        const double* Dp = dpinv + (int64_t(p) * mi1 + jb) * kMaxDirs * kMaxDirs;
-        double v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = 0.0;
-        for (int b2 = 0; b2 < wj; ++b2)
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (lane + 32 * u < ne) v[u] += Dp[ea[u] * kMaxDirs + b2] * sphi[wid][b2 * w + es[u]];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if (lane + 32 * u < ne) {
-                const int64_t o = int64_t(off + ea[u]) * kMaxDirs + es[u];
-                Bp[o] = v[u];
-                Bt[o] = T(v[u]);
-            }
+        for (int u = 0; u < NW; ++u) {
+            const int64_t jb = j0 + int64_t(gridDim.x) * u;
+            if (jb >= nblk) break;
+            const int wj = bw[jb], ne = wj * w;
+            if (ne < kBig) continue;
+            const int off = bo[jb], t = threadIdx.x;
+            phi_block<T>(ph, off, w, ne, m, n_eff, K, local, t, kThreads, sphi);
+            __syncthreads();
+            const double* Dp = dpinv + (int64_t(p) * mi1 + jb) * kMaxDirs * kMaxDirs;
+            if (t < ne) Bp[int64_t(off + t / w) * kMaxDirs + t % w] = T(beta_entry(Dp, sphi, t / w, t % w, w, wj));
+            __syncthreads();
         }
-        __syncwarp();
     }
 }
 
-// P_new = Z - P_hist beta, Q_new = (S Z) - Q_hist beta (Eq. 18; Q only when Q is updated rather than
-// recomputed).  A tall-skinny product over the history: a CTA takes 32 consecutive rows of one
-// problem, its kPqSlices warps split each 64-column tile of the history (warp k takes columns
-// k, k + kPqSlices, ...; lane = row, so every column is read as 32 consecutive values), beta
-// tiles are staged in shared memory, and the slices are added in slice order at the end.
-// A one-column block (a global step) accumulates one column only.
-constexpr int kPqSlices = 4;
+// P_new = Z - P_hist beta, Q_new = (S Z) - Q_hist beta (Eq. 18; Q in float64 only: the float32 sweeps
+// recompute it).  A tall-skinny product over the history, bound by reading it once: a CTA takes
+// 32 consecutive rows of one problem, its kSlices warps split each tile of kTile columns (warp k takes
+// columns k, k + kSlices, ...; lane = row, so every column is read as 32 consecutive values, eight
+// columns in flight per lane), beta tiles are staged in shared memory, and the slices' sums meet
+// in shared memory, where warp s adds column s of the new block in slice order.  With 4 warps
+// per CTA and 4 columns in flight, 7 warps an SM kept 4 KB of loads in flight (131 us on 2000 columns
+// of 9000 rows, 0.55 TB/s; now 35 us).  A one-column block (a global step) accumulates one column
+// only.
 template <typename T>
-__global__ void __launch_bounds__(kPqSlices * 32) k_mcg_pq(T* __restrict__ P, T* __restrict__ Q,
-                                                            const T* __restrict__ z, const T* __restrict__ beta,
-                                                            T* __restrict__ PT, const Ctl* __restrict__ ctl) {
+struct PqShape;
+template <> struct PqShape<float> { static constexpr int kSlices = 16, kTile = 256; };
+template <> struct PqShape<double> { static constexpr int kSlices = 8, kTile = 128; };
+
+template <typename T>
+__global__ void __launch_bounds__(PqShape<T>::kSlices * 32, 2) k_mcg_pq(T* __restrict__ P, T* __restrict__ Q,
+                                                                     const T* __restrict__ z, const T* __restrict__ beta,
+                                                                     T* __restrict__ PT, const Ctl* __restrict__ ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const Ctl& c = ctl[blockIdx.y];
     if (c.done) return;
-    constexpr int TC = 64;
-    constexpr int kBPer = TC * kMaxDirs / (kPqSlices * 32);   // beta values a thread stages per tile
-    __shared__ __align__(16) T sB[TC][kMaxDirs];
-    __shared__ T red[2][kPqSlices][32][kMaxDirs + 1];
+    constexpr bool kUpdQ = sizeof(T) == 8;
+    constexpr int NS = PqShape<T>::kSlices, TC = PqShape<T>::kTile;
+    constexpr int U = kUpdQ ? 4 : 8;                   // columns in flight (of P, and of Q)
+    // two beta tiles during the loop over the history, then the slices' sums
+    __shared__ __align__(16) T smem[NS * 32 * (kMaxDirs + 1)];
+    static_assert(2 * TC * kMaxDirs <= NS * 32 * (kMaxDirs + 1), "beta tiles fit");
+    auto red = reinterpret_cast<T(*)[32][kMaxDirs + 1]>(smem);
     const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
     const int64_t n = int64_t(c.lay.nc) * 9;
     const int64_t r0g = 9 * int64_t(c.lay.c0);
-    const int w = c.w_new, off = c.new_off, hc = c.hist_cols, local = c.local, sz = c.sz;
-    const bool upd_q = !c.direct_q;
+    const int w = c.w_new, off = c.new_off, hc = c.hist_cols, sz = c.sz;
+    const bool local = c.local != 0;
     T* Pp = P + c.lay.hoff;
     T* Qp = Q + c.lay.hoff;
     const T* Bp = beta + c.lay.boff * kMaxDirs;
     for (int64_t base = int64_t(blockIdx.x) * 32; base < n; base += int64_t(gridDim.x) * 32) {
         const int64_t row = base + lane;
         const bool act = row < n;
-        T ap[kMaxDirs], aq[kMaxDirs];
+        T ap[kMaxDirs], aq[kUpdQ ? kMaxDirs : 1];
 #pragma unroll
         for (int s = 0; s < kMaxDirs; ++s) {
             ap[s] = T(0);
-            aq[s] = T(0);
+            if constexpr (kUpdQ) aq[s] = T(0);
         }
-        // beta tile c0 + TC is read into registers while tile c0 is used (its loads in flight)
-        T bnext[kBPer];
-        auto load_b = [&](int c0n) {
-#pragma unroll
-            for (int u = 0; u < kBPer; ++u) {
-                const int t = threadIdx.x + u * blockDim.x;
-                const int cc = t / kMaxDirs, s = t % kMaxDirs;
-                bnext[u] = (c0n + cc < hc && s < w) ? Bp[int64_t(c0n + cc) * kMaxDirs + s] : T(0);
-            }
+        // beta tile t + 1 is copied while tile t is used (rows of 16 values; past w they may hold
+        // anything, which reaches only sums that are not used)
+        auto copy_b = [&](int c0n) {
+            const int rows = hc - c0n < TC ? hc - c0n : TC;
+            constexpr int kPer = 16 / sizeof(T);
+            T* dst = smem + ((c0n / TC) & 1) * TC * kMaxDirs;
+            for (int t = threadIdx.x; t * kPer < rows * kMaxDirs; t += blockDim.x)
+                cp_async16(dst + t * kPer, Bp + int64_t(c0n) * kMaxDirs + t * kPer);
+            cp_async_commit();
         };
-        load_b(0);
+        copy_b(0);
         for (int c0 = 0; c0 < hc; c0 += TC) {
             const int tc = hc - c0 < TC ? hc - c0 : TC;
+            copy_b(c0 + TC);   // nothing past the last tile
+            cp_async_wait_prev();
             __syncthreads();
-#pragma unroll
-            for (int u = 0; u < kBPer; ++u) {
-                const int t = threadIdx.x + u * blockDim.x;
-                sB[t / kMaxDirs][t % kMaxDirs] = bnext[u];
-            }
-            __syncthreads();
-            if (c0 + TC < hc) load_b(c0 + TC);
-            if (!act) continue;
+            auto sB = reinterpret_cast<const T(*)[kMaxDirs]>(smem + ((c0 / TC) & 1) * TC * kMaxDirs);
             const T* pc = Pp + int64_t(c0) * n + row;
             const T* qc = Qp + int64_t(c0) * n + row;
-            if (w == 1) {
-#pragma unroll 4
-                for (int cl = k; cl < tc; cl += kPqSlices) {
-                    const T b0 = sB[cl][0];
-                    ap[0] += pc[int64_t(cl) * n] * b0;
-                    if (upd_q) aq[0] += qc[int64_t(cl) * n] * b0;
-                }
-            } else if (upd_q) {
-#pragma unroll 2
-                for (int cl = k; cl < tc; cl += kPqSlices) {
-                    const T pv = pc[int64_t(cl) * n], qv = qc[int64_t(cl) * n];
+            for (int cl = k; cl < tc; cl += NS * U) {
+                T pv[U], qv[U];
 #pragma unroll
-                    for (int s = 0; s < kMaxDirs; ++s) {
-                        ap[s] += pv * sB[cl][s];
-                        aq[s] += qv * sB[cl][s];
+                for (int u = 0; u < U; ++u) {
+                    const int cu = cl + u * NS;
+                    const bool in = act && cu < tc;
+                    pv[u] = in ? pc[int64_t(cu) * n] : T(0);
+                    if constexpr (kUpdQ) qv[u] = in ? qc[int64_t(cu) * n] : T(0);
+                }
+                if (w == 1) {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int cu = cl + u * NS;
+                        const T b0 = cu < tc ? sB[cu][0] : T(0);
+                        ap[0] += pv[u] * b0;
+                        if constexpr (kUpdQ) aq[0] += qv[u] * b0;
+                    }
+                } else {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int cu = cl + u * NS;
+                        if (cu >= tc) break;
+#pragma unroll
+                        for (int s = 0; s < kMaxDirs; s += 2) {
+                            if constexpr (kUpdQ) {
+                                ap[s] += pv[u] * sB[cu][s];
+                                ap[s + 1] += pv[u] * sB[cu][s + 1];
+                                aq[s] += qv[u] * sB[cu][s];
+                                aq[s + 1] += qv[u] * sB[cu][s + 1];
+                            } else {   // packed: each half rounds like a scalar fused multiply-add
+                                const float2 b2 = *reinterpret_cast<const float2*>(&sB[cu][s]);
+                                const float2 v = __ffma2_rn(make_float2(pv[u], pv[u]), b2, make_float2(ap[s], ap[s + 1]));
+                                ap[s] = v.x;
+                                ap[s + 1] = v.y;
+                            }
+                        }
                     }
                 }
-            } else {
-#pragma unroll 4
-                for (int cl = k; cl < tc; cl += kPqSlices) {
-                    const T pv = pc[int64_t(cl) * n];
-#pragma unroll
-                    for (int s = 0; s < kMaxDirs; ++s) ap[s] += pv * sB[cl][s];
-                }
             }
+            __syncthreads();
         }
+        // column s of the new block is added by warp s mod NS, over the slices in order
+        const int sub = act ? int(row / 9) / sz : 0;
+        const T zr = act ? z[r0g + row] : T(0);
+        auto slices = [&](const T* acc, auto&& put) {
+            __syncthreads();
 #pragma unroll
-        for (int s = 0; s < kMaxDirs; ++s) {
-            red[0][k][lane][s] = ap[s];
-            red[1][k][lane][s] = aq[s];
-        }
-        __syncthreads();
-        if (k == 0 && act) {
-            const int sub = int(row / 9) / sz;
-            const T zr = z[r0g + row];
+            for (int s = 0; s < kMaxDirs; ++s) red[k][lane][s] = acc[s];
+            __syncthreads();
+            for (int s = k; s < kMaxDirs; s += NS) {
+                T sum = T(0);
+                if (s < w)
 #pragma unroll
-            for (int s = 0; s < kMaxDirs; ++s) {
-                T sp = T(0), sq = T(0);
-#pragma unroll
-                for (int kk = 0; kk < kPqSlices; ++kk) {
-                    sp += red[0][kk][lane][s];
-                    sq += red[1][kk][lane][s];
-                }
-                const T pn = ((local ? (s == sub) : (s == 0)) ? zr : T(0)) - sp;
-                if (s < w) {
-                    Pp[int64_t(off + s) * n + row] = pn;
-                    if (upd_q) Qp[int64_t(off + s) * n + row] -= sq;
-                }
-                // row-major copy of the new block for the multi-column product (zero past w)
-                if (!upd_q) PT[(r0g + row) * kMaxDirs + s] = s < w ? pn : T(0);
+                    for (int kk = 0; kk < NS; ++kk) sum += red[kk][lane][s];
+                put(s, sum);
             }
+        };
+        if constexpr (kUpdQ) {
+            slices(ap, [&](int s, T sum) {
+                if (act && s < w) Pp[int64_t(off + s) * n + row] = (s == (local ? sub : 0) ? zr : T(0)) - sum;
+            });
+            slices(aq, [&](int s, T sum) {
+                if (act && s < w) Qp[int64_t(off + s) * n + row] -= sum;
+            });
+        } else {
+            T pn = T(0);
+            slices(ap, [&](int s, T sum) {   // NS = kMaxDirs: one column per warp
+                pn = s < w ? (s == (local ? sub : 0) ? zr : T(0)) - sum : T(0);
+                if (act && s < w) Pp[int64_t(off + s) * n + row] = pn;
+            });
+            // row-major copy of the new block for the multi-column product (zero past w)
+            static_assert(kUpdQ || NS == kMaxDirs, "one column per warp");
+            __syncthreads();
+            red[0][lane][k] = pn;
+            __syncthreads();
+            const int rr = threadIdx.x / kMaxDirs, ss = threadIdx.x % kMaxDirs;
+            if (base + rr < n) PT[(r0g + base) * kMaxDirs + threadIdx.x] = red[0][rr][ss];
         }
         __syncthreads();
     }
@@ -2241,7 +2317,7 @@ struct Solver {
     int gphi = 1, gb = 1;     // Phi and beta grid widths
     int gcol = 1;             // grid width of the column pass of the symmetric product (a CTA per camera)
     std::vector<Layout> lay;  // of the current solve
-    Buf P, Q, r, z, xw, PT, part_a, part_b, part_cam, dpinv, beta, betaf, phip, hist, blk_off, blk_w, ctl, outer, rt,
+    Buf P, Q, r, z, xw, PT, part_a, part_b, part_cam, dpinv, beta, phip, hist, blk_off, blk_w, ctl, outer, rt,
         lay_d, dpart, dcnt, camdot, params, loops;
     Ctl* h_ctl = nullptr;     // pinned, nb
     Outer* h_outer = nullptr; // pinned, nb
@@ -2555,7 +2631,6 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     grow(w->part_cam, size_t(s.n_c) * 2 * sizeof(double));
     grow(w->dpinv, size_t(nb) * w->mi1 * kMaxDirs * kMaxDirs * sizeof(double));
     grow(w->beta, size_t(boff) * kMaxDirs * sizeof(double));
-    grow(w->betaf, size_t(boff) * kMaxDirs * sizeof(float));
     grow(w->phip, size_t(phoff) * sizeof(double));
     grow(w->hist, size_t(nb) * w->mi1 * sizeof(double));
     grow(w->blk_off, size_t(nb) * w->mi1 * sizeof(int));
@@ -2599,7 +2674,7 @@ Solver* solver_create() { return new Solver(); }
 void solver_destroy(Solver* w) {
     if (!w) return;
     Buf* bufs[] = {&w->P, &w->Q, &w->r, &w->z, &w->xw, &w->PT, &w->part_a, &w->part_b, &w->part_cam, &w->dpinv,
-                   &w->beta, &w->betaf, &w->phip, &w->hist, &w->blk_off, &w->blk_w, &w->ctl, &w->outer, &w->rt,
+                   &w->beta, &w->phip, &w->hist, &w->blk_off, &w->blk_w, &w->ctl, &w->outer, &w->rt,
                    &w->lay_d, &w->dpart, &w->dcnt, &w->camdot, &w->params, &w->loops};
     for (Buf* b : bufs) free_buf(*b);
     for (SolveExec* e : w->execs) {
@@ -2719,10 +2794,9 @@ static int enqueue_iteration(Solver* w, const Structure& s, const T* S, const T*
                        ptr<double>(w->dpart) + 3 * size_t(nb) * w->gu, dcnt, ptr<double>(w->hist),
                        ptr<int>(w->blk_off), ptr<int>(w->blk_w), w->mi1, ctl);
         launch_chained(k_mcg_phi<T>, dim3(w->gphi, nb), dim3(kThreads), 0, st, Q, z, ptr<double>(w->phip), ctl);
-        T* betat = sizeof(T) == 8 ? ptr<T>(w->beta) : ptr<T>(w->betaf);
+        T* betat = ptr<T>(w->beta);
         launch_chained(k_mcg_beta<T>, dim3(w->gb, nb), dim3(kThreads), 0, st, ptr<double>(w->phip),
-                       ptr<double>(w->dpinv), ptr<int>(w->blk_off), ptr<int>(w->blk_w), ptr<double>(w->beta), betat,
-                       ctl, w->mi1);
+                       ptr<double>(w->dpinv), ptr<int>(w->blk_off), ptr<int>(w->blk_w), betat, ctl, w->mi1);
         if constexpr (sizeof(T) == 8) {
             // Eq. 18: Q_{i+1} = S Z_{i+1} - sum_j Q_j beta_{i,j}; S Z over whole rows for the
             // problems forming a global block, over the subset segments for the local ones
@@ -2731,12 +2805,12 @@ static int enqueue_iteration(Solver* w, const Structure& s, const T* S, const T*
             if (w->use_l)
                 launch_spmv<T, 0, false, false>(w->spmv_cfg, st, s.row_ptr, s.tile_ptr, s.col, S, z, w->items_l,
                                                 kSelLocal, Q, nullptr, nullptr, ctl, nullptr);
-            launch_chained(k_mcg_pq<T>, dim3(w->gpq, nb), dim3(kPqSlices * 32), 0, st, P, Q, z, betat, (T*)nullptr,
+            launch_chained(k_mcg_pq<T>, dim3(w->gpq, nb), dim3(PqShape<T>::kSlices * 32), 0, st, P, Q, z, betat, (T*)nullptr,
                            ctl);
             return w->use_l ? 8 : 7;
         } else {
             // Algorithm 2: Q_{i+1} = S P_{i+1}
-            launch_chained(k_mcg_pq<T>, dim3(w->gpq, nb), dim3(kPqSlices * 32), 0, st, P, Q, z, betat, ptr<T>(w->PT),
+            launch_chained(k_mcg_pq<T>, dim3(w->gpq, nb), dim3(PqShape<T>::kSlices * 32), 0, st, P, Q, z, betat, ptr<T>(w->PT),
                            ctl);
             const int np = enqueue_product<T, 2>(w, s, S, Su, P, kSelW1, Q, nullptr, st);
             launch_chained(k_spmm<T>, dim3(Gt), dim3(SpmmCfg::kWarps * 32), spmm_smem<T>(), st, s.row_ptr, s.tile_ptr,
