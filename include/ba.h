@@ -86,15 +86,16 @@ typedef struct ba_options {
                                   (default 1e-6: one sweep when float32 reaches the tolerance) */
     int32_t max_refine;        /* MIXED: maximum outer refinement sweeps (default 64) */
     int32_t item_blocks;       /* stored 9x9 blocks of S per work item of the block-sparse products
-                                  (longer rows are split): 0 (default) = 512, else a multiple of 32
-                                  in [32, 4096]; ba_autotune sets it */
+                                  (longer rows are split): 0 (default) = 512, or 256 below 1200
+                                  (float64: 800) cameras; else a multiple of 32 in [32, 4096];
+                                  ba_autotune sets it */
     int32_t wait_polls;        /* bounded device waits: polls of a tile copy's barrier before the
                                   solve gives up with BA_ERR_TIMEOUT (the kernel then waits for its
                                   own copies still in flight, with the default bound, and returns).
                                   0 (default) = 2^20; 1 .. 2^30; -1 = no poll at all, so every such
                                   wait gives up at once (tests the timeout path) */
     int32_t spmv_config;       /* warps x copy stages per CTA of the tile-streaming one-column product:
-                                  0 (default) = float32 16 x 1, float64 4 x 2; 1 = 8 x 2 / 8 x 1;
+                                  0 (default) = float32 16 x 1, float64 8 x 1; 1 = 8 x 2 / 4 x 2;
                                   2 = 10 x 2 / 2 x 4; ba_autotune sets it */
     int32_t host_loop;         /* 1: drive the iteration and refinement loops from the host (a plain
                                   graph of chunk_iters iterations per launch, the stop flags read back

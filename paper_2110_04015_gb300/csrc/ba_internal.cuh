@@ -208,7 +208,7 @@ struct SolveArgs {
     double inner_tol = 1e-3;
     int max_refine = 12;
     int64_t max_history = 0;
-    int item_blocks = 0;    // blocks per work item of the block-sparse products (0: 512)
+    int item_blocks = 0;    // blocks per work item of the block-sparse products (0: by the problem's size)
     int wait_polls = kDefaultWaitPolls;   // tile-copy waits: polls before giving up (0: give up at once)
     int host_loop = 0;      // 1: the loops run from the host (plain graphs), for profilers
     int spmv_cfg = 0;       // shape of the tile-streaming one-column products (0, 1, 2)

@@ -469,23 +469,55 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int po
 // Warps per CTA and copy stages of the tile-streaming one-column product, one CTA per SM.  Three
 // shapes per precision (ba_options.spmv_config, chosen by ba_autotune); shape 0 is the default:
 // float32 16 warps x 1 stage (measured faster than 8 x 2 for the full-pattern product: more warps
-// cover the gathers of p), float64 4 x 2.  The symmetric product does twice the arithmetic per tile,
-// so a second stage per warp keeps the next copy in flight during it (shapes 1 and 2).  Every shape
-// keeps its stages within 207 KB.
+// cover the gathers of p), float64 8 x 1: two warps per scheduler keep the float64 pipe busy while one
+// waits for its copy (1936 cameras: 0.566 ms, 0.94 of the pipe's rate, against 0.824 ms for 4 x 2 and
+// 1.59 ms for 2 x 4; 601 cameras 85 us against 129 us).  The symmetric product does twice the
+// arithmetic per tile, so a second stage per warp keeps the next copy in flight during it (shapes 1
+// and 2).  Every shape keeps its stages within 207 KB.
 template <typename T, int CFG>
 struct SpmvShape;
 template <> struct SpmvShape<float, 0> { static constexpr int kWarps = 16, kStages = 1; };
 template <> struct SpmvShape<float, 1> { static constexpr int kWarps = 8, kStages = 2; };
 template <> struct SpmvShape<float, 2> { static constexpr int kWarps = 10, kStages = 2; };
-template <> struct SpmvShape<double, 0> { static constexpr int kWarps = 4, kStages = 2; };
-template <> struct SpmvShape<double, 1> { static constexpr int kWarps = 8, kStages = 1; };
+template <> struct SpmvShape<double, 0> { static constexpr int kWarps = 8, kStages = 1; };
+template <> struct SpmvShape<double, 1> { static constexpr int kWarps = 4, kStages = 2; };
 template <> struct SpmvShape<double, 2> { static constexpr int kWarps = 2, kStages = 4; };
 constexpr int kSpmvShapes = 3;
-// Shared memory of k_spmv: the warps' tile stages, then the stages' barriers.
+// Shared memory of k_spmv: the warps' tile stages, the stages' barriers, then the warps' row sums.
+constexpr int kRowSums = 9 * 33;   // nine sums of 32 lanes, one bank apart
 template <typename T, int CFG>
 constexpr size_t spmv_smem() {
     return sizeof(T) * SpmvShape<T, CFG>::kWarps * SpmvShape<T, CFG>::kStages * kTileElems +
-           sizeof(uint64_t) * SpmvShape<T, CFG>::kWarps * SpmvShape<T, CFG>::kStages;
+           sizeof(uint64_t) * SpmvShape<T, CFG>::kWarps * SpmvShape<T, CFG>::kStages +
+           sizeof(T) * SpmvShape<T, CFG>::kWarps * kRowSums;
+}
+
+// Sum of acc[a] over the warp's lanes in lane a (a < 9; the other lanes return zero).  The sums meet in
+// shared memory: three lanes add 11, 11 and 10 of a row's 32 values (two interleaved chains), then
+// the three.  Nine shuffle trees cost 45 warp-wide additions, in float64 more than half of the 81
+// multiply-adds of a tile; this costs 12.
+template <typename T>
+__device__ __forceinline__ T row_sums(const T (&acc)[9], T* red) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int a = 0; a < 9; ++a) red[33 * a + lane] = acc[a];
+    __syncwarp();
+    T v0 = T(0), v1 = T(0);
+    if (lane < 27) {
+        const T* p = red + 33 * (lane / 3) + 11 * (lane % 3);
+#pragma unroll
+        for (int u = 0; u < 10; u += 2) {
+            v0 += p[u];
+            v1 += p[u + 1];
+        }
+        if (lane % 3 < 2) v0 += p[10];
+    }
+    __syncwarp();
+    const T v = v0 + v1;
+    const int from = lane < 9 ? 3 * lane : 0;
+    const T s0 = __shfl_sync(0xffffffffu, v, from), s1 = __shfl_sync(0xffffffffu, v, from + 1),
+            s2 = __shfl_sync(0xffffffffu, v, from + 2);
+    return lane < 9 ? (s0 + s1) + s2 : T(0);
 }
 
 // The transposed terms of the symmetric product, one slot per stored upper block: values 0..7 of slot
@@ -569,6 +601,7 @@ __global__ void __launch_bounds__(SpmvShape<T, CFG>::kWarps * 32, 1) k_spmv(
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     T* tiles = reinterpret_cast<T*>(smem_raw) + size_t(wid) * NS * kTileElems;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem_raw + sizeof(T) * NW * NS * kTileElems) + wid * NS;
+    T* red = reinterpret_cast<T*>(smem_raw + (sizeof(T) * kTileElems + sizeof(uint64_t)) * NW * NS) + wid * kRowSums;
     T* part = static_cast<T*>(L.part);
     constexpr uint32_t tile_bytes = sizeof(T) * kTileElems;
 
@@ -700,11 +733,7 @@ __global__ void __launch_bounds__(SpmvShape<T, CFG>::kWarps * 32, 1) k_spmv(
             }
             if (bad) break;
         }
-#pragma unroll
-        for (int a = 0; a < 9; ++a) acc[a] = warp_sum(acc[a]);
-        T val = acc[0];
-#pragma unroll
-        for (int a = 1; a < 9; ++a) if (lane == a) val = acc[a];
+        T val = row_sums(acc, red);
         bool fin = true;
         if (it.ng > 1) {
             if (lane < 9) part[int64_t(it.slot) * 9 + lane] = val;
@@ -2366,25 +2395,28 @@ static T* ptr(const Buf& b) {
     return static_cast<T*>(b.p);
 }
 
-// Default blocks per work item: 16 tiles.  Rows up to that length are one item; longer rows are
-// split, and the row's pieces combined by the last one to finish.  The rule depends on nothing
-// but the row, so a problem's products sum in the same order alone and in any batch.  (Measured
-// on GB300: 512 is within 2 % of the best of 32 .. 1024 for a 1936-camera problem and a 64-problem
-// batch; a rule that split small problems' rows finer was up to 3x slower on the batch.)
-constexpr int kItemBlocks = 512;
+// Default blocks per work item: 16 tiles, and 8 for problems whose rows are too few to keep every warp
+// busy with 16 (the longest item then sets the time).  Rows up to that length are one item; longer
+// rows are split, and the row's pieces combined by the last one to finish.  The rule depends on the
+// problem's own camera count alone, so its products sum in the same order alone and in any batch.
+// Measured on GB300, product at 512 / 256 blocks: float32 601 cameras 33.8 / 26.0 us (the solves 16 %
+// faster), 1000 cameras 43.4 / 41.9 us, 1936 cameras 118.1 / 119.1 us (MCG 2.5 % slower); float64 601
+// cameras 82.0 / 71.1 us, 1000 cameras 166 / 174 us.  64 and 128 blocks suit single problems of
+// 150 .. 300 cameras (up to 25 % of a product) and cost a batch of such problems as much.
+static int default_item_blocks(int n_cams, bool fp32) { return n_cams < (fp32 ? 1200 : 800) ? 256 : 512; }
 
 // Items of the block-sparse product, problem by problem: each (row, segment) split into chunks of
-// at most cb blocks (cb = forced_cb, else kItemBlocks).
+// at most cb blocks (cb = forced_cb, else default_item_blocks).
 // split = false: one segment per row; otherwise segment s of a row of problem b holds the blocks
 // whose column camera lies in [c0 + s sz, c0 + (s + 1) sz), for s < n_eff (empty segments get
 // one empty item, which writes zeros).
 static std::vector<SpItem> build_items(const std::vector<int64_t>& h_row_ptr, const std::vector<int32_t>& h_col,
-                                       const std::vector<Layout>& lay, bool split, int forced_cb) {
+                                       const std::vector<Layout>& lay, bool split, int forced_cb, bool fp32) {
     std::vector<SpItem> out;
     int grp = 0;
     for (size_t b = 0; b < lay.size(); ++b) {
         const Layout& L = lay[b];
-        const int cb = forced_cb > 0 ? forced_cb : kItemBlocks;
+        const int cb = forced_cb > 0 ? forced_cb : default_item_blocks(L.nc, fp32);
         const int nseg = split ? L.n_eff : 1;
         for (int32_t j = L.c0; j < L.c0 + L.nc; ++j) {
             const int64_t rj = h_row_ptr[j], nj = h_row_ptr[j + 1] - rj;
@@ -2534,14 +2566,14 @@ static void ensure_items(Solver* w, const Structure& s, int n_dirs, int forced_c
     const int64_t wg = sms * ng, wu = sms * nu, wl = sms * nl;
     const bool fresh = !w->items_g.items || w->items_cb != cb;
     if (fresh || w->items_g.nw != wg) {
-        upload_items(w->items_g, build_items(s.h_row_ptr, s.h_col, w->lay, false, cb), wg, ng);
+        upload_items(w->items_g, build_items(s.h_row_ptr, s.h_col, w->lay, false, cb, fp32), wg, ng);
         if (w->mm_part) cudaFree(w->mm_part);
         w->mm_part = nullptr;
         BA_CUDA_TRY(cudaMalloc(&w->mm_part, sizeof(double) * kMaxDirs * 9 * size_t(w->items_g.n > 0 ? w->items_g.n : 1)));
         ++w->epoch;
     }
     if (!s.h_row_ptr_u.empty() && (fresh || w->items_u.nw != wu)) {
-        upload_items(w->items_u, build_items(s.h_row_ptr_u, s.h_col_u, w->lay, false, cb), wu, nu);
+        upload_items(w->items_u, build_items(s.h_row_ptr_u, s.h_col_u, w->lay, false, cb, fp32), wu, nu);
         ++w->epoch;
     }
     if (fresh) {
@@ -2549,7 +2581,7 @@ static void ensure_items(Solver* w, const Structure& s, int n_dirs, int forced_c
         w->items_cb = cb;
     }
     if (n_dirs > 1 && (w->items_l_dirs != n_dirs || w->items_l.nw != wl)) {
-        upload_items(w->items_l, build_items(s.h_row_ptr, s.h_col, w->lay, true, cb), wl, nl);
+        upload_items(w->items_l, build_items(s.h_row_ptr, s.h_col, w->lay, true, cb, fp32), wl, nl);
         w->items_l_dirs = n_dirs;
         ++w->epoch;
     }
