@@ -4,8 +4,8 @@
 // Algorithm 1 (block-Jacobi PCG) and Algorithm 2 (MCG) run as a fixed sequence of kernels per
 // iteration.  All data-dependent control (the stop test, the tau-test and the width of the next
 // direction block, the history size) lives in one device struct Ctl per problem, written only by
-// the per-problem "decide" steps (run by the CTA that finalises an update kernel's sums, and by the
-// small solve) and read by the others.  A whole solve is one CUDA graph: a conditional WHILE node
+// the per-problem "decide" steps (run by one CTA of the kernel after an update, and by the small
+// solve) and read by the others.  A whole solve is one CUDA graph: a conditional WHILE node
 // repeats a body of `chunk` iterations while k_loop_cond finds a problem that is not done (the
 // float64 iterative refinement of mixed precision is an outer WHILE node around it), so the host
 // launches the graph once and reads the results once; nothing inside a solve waits on the host.
@@ -83,7 +83,8 @@ struct Ctl {
     int off_cur;
     double rr0, rr, rz, ga, tol2, tau;
     double rr0_inv;    // 1 / rr0: the residual history stores rr / rr0 without a division per step
-    double Delta, gamma, beta;          // PCG scalars
+    int live;          // the problem was not done at this iteration's update (read by the kernel whose
+                       // first CTA runs the decide step, which may set done meanwhile)
     double alpha_v[kMaxDirs];
     double true_rr, bb;                 // true residual and |rhs|^2
     double stag;       // float32 sweeps: stop when t_i (energy decrease / r^T D^-1 r) falls below this
@@ -171,12 +172,6 @@ struct ExactSum<float> {
     }
 };
 
-// s += sum_k x[k * xs] y[k * ys] for k < n
-template <typename T>
-__device__ __forceinline__ void dot_rows(ExactSum<T>& s, const T* x, int xs, const T* y, int ys, int n) {
-    for (int k = 0; k < n; ++k) s.add(x[k * xs], y[k * ys]);
-}
-
 // A Gram partial sum as stored between the Gram and the small-solve kernels: float64, or (for the
 // float32 sweeps) the float pair (hi, lo) in the same 8 bytes, so that adding the partials needs no
 // float64 arithmetic either.
@@ -198,11 +193,10 @@ __device__ __forceinline__ void load_partial(ExactSum<float>& s, const double* s
     s.add_pair(v.x, v.y);
 }
 
-// the partial at *slot, written by another CTA of this launch (read past L1)
-__device__ __forceinline__ void load_partial_cg(ExactSum<double>& s, const double* slot) { s.s += __ldcg(slot); }
-__device__ __forceinline__ void load_partial_cg(ExactSum<float>& s, const double* slot) {
-    const float2 v = __ldcg(reinterpret_cast<const float2*>(slot));
-    s.add_pair(v.x, v.y);
+// add the slot whose 8 bytes are in v (loaded earlier)
+__device__ __forceinline__ void add_slot(ExactSum<double>& s, double v) { s.s += v; }
+__device__ __forceinline__ void add_slot(ExactSum<float>& s, double v) {
+    s.add_pair(__int_as_float(__double2loint(v)), __int_as_float(__double2hiint(v)));
 }
 template <typename T>
 __device__ __forceinline__ ExactSum<T> warp_total(ExactSum<T> s) {
@@ -316,16 +310,14 @@ __device__ __forceinline__ bool nothing_selected(const Ctl* ctl, const ItemList&
     return !__any_sync(0xffffffffu, any);
 }
 
-// Sum the CTA's NV values (kUpdThreads threads), publish them as partial[blockIdx.x], and let the last
-// CTA of the grid row to finish write the row's totals (in CTA order) to totals[0..NV) (shared
-// memory).  Every CTA of the grid row must call it.  Returns true (in every thread) in the CTA that
-// wrote the totals, after they are visible to the whole CTA.  Warp k adds value k, so the CTA's sum
-// takes 3 additions and a shuffle tree in one warp per value instead of a tree in every warp.
+// Sum the CTA's NV values (kUpdThreads threads) into partial[blockIdx.x * NV ..] (store_partial slots).
+// Warp k adds value k: 3 additions and one shuffle tree per value instead of a tree in every warp.
+// The next kernel adds the CTAs' partials (total_of): with the last CTA to arrive doing it here, its
+// fences, its counter and a second round of loads held an update for 3 us.
 template <typename T, int NV>
-__device__ __forceinline__ bool grid_sum_finalize(const ExactSum<T> (&v)[NV], double* partial, int* cnt, double* totals) {
+__device__ __forceinline__ void cta_publish(const ExactSum<T> (&v)[NV], double* partial) {
     static_assert(NV <= kUpdThreads / 32, "one warp per value");
     __shared__ double st[NV][kUpdThreads];   // slots of store_partial
-    __shared__ int last;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < NV; ++k) store_partial(&st[k][threadIdx.x], v[k]);
@@ -335,28 +327,24 @@ __device__ __forceinline__ bool grid_sum_finalize(const ExactSum<T> (&v)[NV], do
 #pragma unroll
         for (int u = 0; u < kUpdThreads / 32; ++u) load_partial(s, &st[wid][lane + 32 * u]);
         s = warp_total(s);
-        if (lane == 0) {
-            store_partial(partial + int64_t(blockIdx.x) * NV + wid, s);
-            __threadfence();
-        }
+        if (lane == 0) store_partial(partial + int64_t(blockIdx.x) * NV + wid, s);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) last = (atomicAdd(cnt, 1) == int(gridDim.x) - 1);
-    __syncthreads();
-    if (!last) return false;
-    __threadfence();
-    // warp k adds value k over the CTA partials: lane l takes partials l, l + 32, ... (independent
-    // loads, short chains), then the fixed shuffle tree; partials of CTAs without rows are exact
-    // zeros, so the sum does not depend on the grid width
-    if (wid < NV) {
-        ExactSum<T> s;
-        for (int b = lane; b < int(gridDim.x); b += 32) load_partial_cg(s, partial + int64_t(b) * NV + wid);
-        s = warp_total(s);
-        if (lane == 0) totals[wid] = s.value();
+}
+
+// Total of value k over np CTA partials (one warp; every lane returns it): lane l adds partials
+// l, l + 32, ..., eight loads in flight, then the fixed shuffle tree.
+template <typename T, int NV>
+__device__ __forceinline__ ExactSum<T> total_of(const double* partial, int np, int k) {
+    ExactSum<T> s;
+    for (int b = threadIdx.x & 31; b < np; b += 8 * 32) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = b + 32 * u < np ? partial[int64_t(b + 32 * u) * NV + k] : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (b + 32 * u < np) add_slot(s, v[u]);
     }
-    if (threadIdx.x == 0) *cnt = 0;
-    __syncthreads();
-    return true;
+    return warp_total(s);
 }
 
 // Row of a camera's D^{-1} block, and its product with the camera's residual.  The float32 sweeps keep
@@ -373,10 +361,10 @@ struct DinvRow<double> {
         for (int b = 0; b < 9; ++b) d[b] = act ? row[b] : 0.0;
     }
     __device__ __forceinline__ double dot(const double* r) const {
-        double s = 0.0;
+        double s[3] = {0.0, 0.0, 0.0};   // a float64 operation takes about 150 cycles: short chains
 #pragma unroll
-        for (int b = 0; b < 9; ++b) s += d[b] * r[b];
-        return s;
+        for (int b = 0; b < 9; ++b) s[b % 3] += d[b] * r[b];
+        return (s[0] + s[1]) + s[2];
     }
 };
 template <>
@@ -1190,16 +1178,26 @@ __global__ void k_loop_cond(cudaGraphConditionalHandle h, int use_handle, const 
     }
 }
 
+// Nearest float32 of a float64 p > 0 in float32's normal range, and the float64 equal to such a float32,
+// from their bit patterns: the conversion instructions run on the float64 pipe (about 150 cycles each),
+// this on the integer pipe.
+__device__ __forceinline__ float bits_to_f32(double p) {
+    return __int_as_float(int(((__double_as_longlong(p) + (1ll << 28)) >> 29) - (896ll << 23)));
+}
+__device__ __forceinline__ double bits_to_f64(float r) {
+    return __longlong_as_double((static_cast<long long>(__float_as_int(r)) + (896ll << 23)) << 29);
+}
+
 // 1 / p in float64 without the long division chain (an exact float64 division is a dependent
 // sequence of about ten operations on this GPU's narrow float64 pipe): a float32 estimate
 // (relative error below 2^-23) refined by Newton steps r <- r + r (1 - p r), each of which
 // squares the error: one step leaves it below 2^-46 (about 1e-14), two reach float64 rounding.
-// Values outside the float32 range divide.
+// Values that are not positive or outside 2^-100 .. 2^100 divide.
 template <int kSteps = 1>
 __device__ __forceinline__ double fast_rcp(double p) {
-    const double ap = fabs(p);
-    if (!(ap > 1e-30 && ap < 1e30)) return 1.0 / p;
-    double r = double(__frcp_rn(float(p)));
+    const int e = __double2hiint(p);   // sign, exponent and high fraction bits
+    if (!(e >= ((1023 - 100) << 20) && e < ((1023 + 100) << 20))) return 1.0 / p;
+    double r = bits_to_f64(__frcp_rn(bits_to_f32(p)));
 #pragma unroll
     for (int k = 0; k < kSteps; ++k) r = fma(r, fma(-p, r, 1.0), r);
     return r;
@@ -1209,38 +1207,52 @@ __device__ __forceinline__ double fast_rcp(double p) {
 // Algorithm 1 (grid: CTAs x problems)
 
 // The sums over cameras [0, nc) of the per-camera sums (Delta, gamma), returned to every thread of
-// the CTA: warp w takes value w mod 2 over the cameras of half w / 2 (64-camera stride, four
-// interleaved sums with their loads in flight together), then a shuffle tree and the two halves.
+// the CTA: thread t takes cameras t + 128 k, eight loads in flight, then shuffle trees and the warps in
+// order.  (Four dependent rounds of loads, one value per warp, took 2.6 us for 1000 cameras.)
 template <typename T>
 __device__ __forceinline__ void sum_camdot(const double* cd, int nc, ExactSum<T>& Delta, ExactSum<T>& gamma) {
-    static_assert(kUpdThreads == 128, "two values x two halves");
-    __shared__ double sh[4];
+    __shared__ __align__(16) double sh[2 * (kUpdThreads / 32)];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    ExactSum<T> a[4];
-    const double* c = cd + (wid & 1);
-    int j = 32 * (wid >> 1) + lane;
-    for (; j + 192 < nc; j += 256)
+    ExactSum<T> d, g, d1, g1;
+    for (int j = threadIdx.x; j < nc; j += 8 * kUpdThreads) {
+        double2 v[8];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) load_partial(a[u], c + 2 * int64_t(j + 64 * u));
+        for (int u = 0; u < 8; ++u)
+            v[u] = j + u * kUpdThreads < nc ? *reinterpret_cast<const double2*>(cd + 2 * int64_t(j + u * kUpdThreads))
+                                            : make_double2(0.0, 0.0);
 #pragma unroll
-    for (int u = 0; u < 3; ++u)
-        if (j + 64 * u < nc) load_partial(a[u], c + 2 * int64_t(j + 64 * u));
-    combine(a[0], a[1]);
-    combine(a[2], a[3]);
-    combine(a[0], a[2]);
-    a[0] = warp_total(a[0]);
-    if (lane == 0) store_partial(&sh[wid], a[0]);
+        for (int u = 0; u < 8; u += 2) {
+            if (j + u * kUpdThreads < nc) {
+                add_slot(d, v[u].x);
+                add_slot(g, v[u].y);
+            }
+            if (j + (u + 1) * kUpdThreads < nc) {
+                add_slot(d1, v[u + 1].x);
+                add_slot(g1, v[u + 1].y);
+            }
+        }
+    }
+    combine(d, d1);
+    combine(g, g1);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        combine_shfl(d, o);
+        combine_shfl(g, o);
+    }
+    if (lane == 0) {
+        store_partial(&sh[2 * wid], d);
+        store_partial(&sh[2 * wid + 1], g);
+    }
     __syncthreads();
-    load_partial(Delta, &sh[0]);
-    load_partial(Delta, &sh[2]);
-    load_partial(gamma, &sh[1]);
-    load_partial(gamma, &sh[3]);
+#pragma unroll
+    for (int w = 0; w < kUpdThreads / 32; ++w) {
+        load_partial(Delta, &sh[2 * w]);
+        load_partial(gamma, &sh[2 * w + 1]);
+    }
 }
 
-__device__ void pcg_decide(Ctl* c, double D, double g, const double* tot, double* hist, int p, int nb);
-
-// alpha = gamma / Delta; x += alpha p; r -= alpha q; z = D^{-1} r; totals of |r|^2, q^T z, r^T z,
-// then (the CTA that finalises the totals) the stop test and beta.
+// alpha = gamma / Delta; x += alpha p; r -= alpha q; z = D^{-1} r; per CTA the sums of |r|^2, q^T z and
+// r^T z (dpart), from which k_pcg_dir takes the stop test and beta; dtot: Delta and gamma.
 // Delta and gamma are the sums over the problem's cameras (camera order) of the per-camera sums
 // of the product; every CTA forms them the same way.
 // Thread = one row (9 per camera, kUpdCams cameras per CTA); the rows of a camera meet in
@@ -1248,23 +1260,24 @@ __device__ void pcg_decide(Ctl* c, double D, double g, const double* tot, double
 // partition depends on the problem alone (the grid has a CTA for every chunk of the largest).
 // Bound by latency: on 1000 cameras 12 us of a 22 us iteration when the sums ran in float64 (whose
 // pipe does 1.7 lanes per clock and SM, so each warp-wide addition of a shuffle tree costs as much as
-// a full one); 8.6 us with the float32 sweeps' sums as float pairs (the solve of that
-// case 13.4 -> 11.2 ms).
+// a full one); 8.6 us with the float32 sweeps' sums as float pairs; 3.3 us with the camera sums' loads in
+// flight together and the decide step in k_pcg_dir.
 template <typename T>
 __global__ void __launch_bounds__(kUpdThreads) k_pcg_update(const double* __restrict__ Dinv, const T* __restrict__ P,
                                                             const T* __restrict__ Q, T* __restrict__ x,
                                                             T* __restrict__ r, T* __restrict__ z,
                                                             const double* __restrict__ camdot,
-                                                            double* __restrict__ dpart, int* __restrict__ dcnt,
-                                                            double* __restrict__ hist, Ctl* ctl) {
+                                                            double* __restrict__ dpart, double* __restrict__ dtot,
+                                                            Ctl* ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const int p = blockIdx.y;
     const Ctl& c = ctl[p];
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl[p].live = !c.done;
     if (c.done) return;
     const int64_t c0 = c.lay.c0;
     const int nc = c.lay.nc;
+    if (int64_t(blockIdx.x) * kUpdCams >= nc) return;   // no camera (a smaller problem of the batch)
     __shared__ T sr[kUpdCams * 9];
-    __shared__ double tot[3];
     const int t = threadIdx.x, cl = t / 9, a = t - 9 * (t / 9);
     const int64_t jl = int64_t(blockIdx.x) * kUpdCams + cl;
     const bool act = t < kUpdCams * 9 && jl < nc;
@@ -1298,19 +1311,19 @@ __global__ void __launch_bounds__(kUpdThreads) k_pcg_update(const double* __rest
         v[1].add(qv, zs);
         v[2].add(rv, zs);
     }
-    if (grid_sum_finalize<T, 3>(v, dpart + int64_t(p) * gridDim.x * 3, dcnt + 4 * p, tot) && threadIdx.x == 0)
-        pcg_decide(ctl + p, Delta.value(), gamma.value(), tot, hist, p, gridDim.y);
+    cta_publish<T, 3>(v, dpart + int64_t(p) * gridDim.x * 3);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        store_partial(dtot + 2 * int64_t(p), Delta);
+        store_partial(dtot + 2 * int64_t(p) + 1, gamma);
+    }
 }
 
-// stop test and beta = Phi / Delta for problem p (one thread, after the update's totals are in);
-// hist is iteration-major (it x nb)
+// stop test for problem p (one thread); hist is iteration-major (it x nb)
 __device__ void pcg_decide(Ctl* c, double D, double g, const double* tot, double* hist, int p, int nb) {
     if (c->status == BA_ERR_TIMEOUT) { c->done = 1; return; }
-    const double rr = tot[0], phi = tot[1];
+    const double rr = tot[0];
     const int it = c->it + 1;
     c->it = it;
-    c->Delta = D;
-    c->gamma = g;
     c->rr = rr;
     hist[int64_t(c->hist_off + it - 1) * nb + p] = rr * c->rr0_inv * c->hist_scale;   // squared relative residual
     if (!(D > 0.0) || !(rr == rr) || isinf(rr)) {
@@ -1325,86 +1338,154 @@ __device__ void pcg_decide(Ctl* c, double D, double g, const double* tot, double
     } else if (c->stag > 0.0 && g * g < c->stag * tot[2] * D) {   // (g^2 / D) / r^T z < stag
         c->done = 1;          // no measurable progress left at this precision: end the sweep
         c->status = BA_OK;
-    } else {
-        c->beta = phi * fast_rcp<2>(D);
     }
 }
 
-// p = z - beta p (rows of the problem)
+// beta = Phi / Delta and p = z - beta p (rows of the problem).  Every CTA adds the update's partials (gu
+// slots of three per problem) and forms beta; the first CTA of a problem also runs the stop test, in
+// another warp than beta (a problem that ends there gets one more direction, which nothing reads).
 template <typename T>
-__global__ void k_pcg_dir(const T* __restrict__ z, T* __restrict__ P, const Ctl* __restrict__ ctl) {
+__global__ void __launch_bounds__(kThreads) k_pcg_dir(const T* __restrict__ z, T* __restrict__ P,
+                                                      const double* __restrict__ dpart, int gu,
+                                                      const double* __restrict__ dtot, double* __restrict__ hist,
+                                                      Ctl* ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
-    const Ctl& c = ctl[blockIdx.y];
-    if (c.done) return;
-    const T beta = T(c.beta);
-    const int64_t n = int64_t(c.lay.nc) * 9, r0 = 9 * int64_t(c.lay.c0);
+    const int p = blockIdx.y;
+    const Ctl& c = ctl[p];
+    if (!c.live) return;
+    const int nc = c.lay.nc;
+    const int64_t n = int64_t(nc) * 9, r0 = 9 * int64_t(c.lay.c0);
+    if (int64_t(blockIdx.x) * blockDim.x >= n) return;
+    __shared__ double tot[3];
+    __shared__ T sbeta;
     T* Pp = P + c.lay.hoff;
-    for (int64_t i = gtid(); i < n; i += gstride()) Pp[i] = z[r0 + i] - beta * Pp[i];
+    int64_t i = gtid();
+    T zv = T(0), pv = T(0);
+    if (i < n) {   // requested before the CTA waits for the sums
+        zv = z[r0 + i];
+        pv = Pp[i];
+    }
+    ExactSum<T> D, g;
+    load_partial(D, dtot + 2 * int64_t(p));
+    load_partial(g, dtot + 2 * int64_t(p) + 1);
+    const int wid = threadIdx.x >> 5;
+    if (wid < 3) {
+        const ExactSum<T> s = total_of<T, 3>(dpart + int64_t(p) * gu * 3, (nc + kUpdCams - 1) / kUpdCams, wid);
+        if ((threadIdx.x & 31) == 0) tot[wid] = s.value();
+        if (wid == 1 && (threadIdx.x & 31) == 0) sbeta = T(s.value() * fast_rcp<2>(D.value()));
+    }
+    __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x == 32 * 7) pcg_decide(ctl + p, D.value(), g.value(), tot, hist, p, gridDim.y);
+    const T beta = sbeta;
+    if (i < n) Pp[i] = zv - beta * pv;
+    for (i += gstride(); i < n; i += gstride()) Pp[i] = z[r0 + i] - beta * Pp[i];
 }
 
 // ---------------------------------------------------------------------------------------
 // Algorithm 2
 
 // Gram partials of Delta_i = Q_i^T P_i (w x w) and gamma_i = P_i^T r (w) for the current block.
-// A problem of n rows uses min(gridDim.x, ceil(n / 128)) CTAs of its grid row (the rest return),
-// each a contiguous run of rows, so the partition depends on the problem alone.
-__device__ __forceinline__ int gram_ctas(int64_t n, int gx) {
-    const int64_t g = (n + 127) / 128;
-    return int(g < gx ? g : gx);
-}
+// The n rows of a problem fall into gram_parts runs of consecutive rows with a partial each, so the
+// partition depends on the problem alone.
+constexpr int kGramRows = 64;
+constexpr int kGramThreads = 1024;
+__device__ __forceinline__ int gram_parts(int n, int gmax) { return min((n + kGramRows - 1) / kGramRows, gmax); }
 
+// A CTA takes the runs blockIdx.x, blockIdx.x + gridDim.x, ... and stages kGramRows rows at a time, the
+// next ones in registers meanwhile.  Its threads split the rows over NG groups (4 to 16, as many as w x w
+// threads fit); a thread adds one entry of Delta over its group's rows in two interleaved sums, and a
+// row of gamma's products per half warp; the sums meet in shared memory.  Bound by the
+// float-pair additions (10 instructions a term): with one thread per entry over 128 rows the kernel took
+// 9 us on 1000 cameras (15.4k of its cycles staging and adding), now 4.7 us; more CTAs than SMs made a
+// batch of 16 problems pay each CTA's start in turn (14.1 us; looping CTAs 13.0 us).
 template <typename T>
-__global__ void k_mcg_gram(const T* __restrict__ P, const T* __restrict__ Q, const T* __restrict__ r,
-                           double* __restrict__ partial, const Ctl* __restrict__ ctl) {
+__global__ void __launch_bounds__(kGramThreads) k_mcg_gram(const T* __restrict__ P, const T* __restrict__ Q,
+                                                           const T* __restrict__ r, double* __restrict__ partial,
+                                                           int gmax, const Ctl* __restrict__ ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const int p = blockIdx.y;
     const Ctl& c = ctl[p];
     if (c.done) return;
-    const int64_t n = int64_t(c.lay.nc) * 9;
-    const int gp = gram_ctas(n, gridDim.x);
+    const int nr = c.lay.nc * 9;
+    const int64_t n = nr;
+    const int gp = gram_parts(nr, gmax);
     if (int(blockIdx.x) >= gp) return;
-    constexpr int TR = 128;   // rows staged at once: a problem's share of rows is usually one tile
+    constexpr int TR = kGramRows, NW = kGramThreads / 32;
+    static_assert(TR * kMaxDirs == kGramThreads && 2 * NW == TR, "a value of P and of Q per thread, a row per half warp");
     __shared__ T sP[TR][kMaxDirs + 1], sQ[TR][kMaxDirs + 1], sr[TR];
-    const int w = c.w_cur, off = c.off_cur;
-    const int ne = w * w + w;
-    const T* Pp = P + c.lay.hoff;
-    const T* Qp = Q + c.lay.hoff;
+    __shared__ double st[kGramThreads];      // the groups' sums, slot g w w + e
+    __shared__ double sg[NW][kMaxDirs];      // the warps' sums of gamma
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const int w = c.w_cur, off = c.off_cur, ww = w * w;
+    const T* Pp = P + c.lay.hoff + int64_t(off) * n;
+    const T* Qp = Q + c.lay.hoff + int64_t(off) * n;
     const T* rp = r + 9 * int64_t(c.lay.c0);
-    const int64_t per = (n + gp - 1) / gp;
-    const int64_t r0 = int64_t(blockIdx.x) * per;
-    const int64_t r1 = r0 + per < n ? r0 + per : n;
-    ExactSum<T> acc[2];   // entries threadIdx.x and threadIdx.x + 256
-    for (int64_t base = r0; base < r1; base += TR) {
-        const int rows = int(r1 - base < TR ? r1 - base : TR);
-        for (int t = threadIdx.x; t < TR * kMaxDirs; t += blockDim.x) {
-            const int rr = t % TR, cc = t / TR;   // a warp reads 32 consecutive rows of one column
-            T pv = T(0), qv = T(0);
-            if (rr < rows && cc < w) {
-                pv = Pp[int64_t(off + cc) * n + base + rr];
-                qv = Qp[int64_t(off + cc) * n + base + rr];
+    const int per = (nr + gp - 1) / gp;
+    int NG = 4;   // row groups; a group has kGramThreads / NG threads
+    while (NG < 16 && kGramThreads / (2 * NG) >= ww) NG *= 2;
+    const int gt = kGramThreads / NG, g = t / gt, e = t - g * gt, gr = TR / NG;
+    const int lr = t % TR, lc = t / TR;      // loads: a warp reads 32 rows of one column
+    T pn = T(0), qn = T(0), rn = T(0);
+    auto load = [&](int base, int end) {
+        const bool in = base + lr < end;
+        pn = in && lc < w ? Pp[lc * n + base + lr] : T(0);
+        qn = in && lc < w ? Qp[lc * n + base + lr] : T(0);
+        rn = in && lc == 0 ? rp[base + lr] : T(0);
+    };
+    int part = blockIdx.x, base = part * per;
+    load(base, min(base + per, nr));
+    while (part < gp) {
+        ExactSum<T> a0, a1, ag;
+        bool more = true;
+        while (more) {
+            sP[lr][lc] = pn;
+            sQ[lr][lc] = qn;
+            if (lc == 0) sr[lr] = rn;
+            __syncthreads();
+            // the next rows of this run, or the first of the CTA's next run
+            base += TR;
+            more = base < min((part + 1) * per, nr);
+            if (!more) base = (part + int(gridDim.x)) * per;
+            const int np = more ? part : part + int(gridDim.x);
+            if (np < gp) load(base, min((np + 1) * per, nr));
+            if (e < ww) {   // rows past the last one are zeros
+                const T* x = &sQ[g * gr][e / w];
+                const T* y = &sP[g * gr][e % w];
+#pragma unroll 4
+                for (int k = 0; k < gr; k += 2) {
+                    a0.add(x[k * (kMaxDirs + 1)], y[k * (kMaxDirs + 1)]);
+                    a1.add(x[(k + 1) * (kMaxDirs + 1)], y[(k + 1) * (kMaxDirs + 1)]);
+                }
             }
-            sP[rr][cc] = pv;
-            sQ[rr][cc] = qv;
-        }
-        if (threadIdx.x < TR) sr[threadIdx.x] = int(threadIdx.x) < rows ? rp[base + threadIdx.x] : T(0);
-        __syncthreads();
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int e = threadIdx.x + h * blockDim.x;
-            if (e < ne) {
-                const T* x = e < w * w ? &sQ[0][e / w] : &sP[0][e - w * w];
-                const T* y = e < w * w ? &sP[0][e % w] : &sr[0];
-                const int ys = e < w * w ? kMaxDirs + 1 : 1;
-                dot_rows(acc[h], x, kMaxDirs + 1, y, ys, rows);
+            {
+                const int row = 2 * wid + (lane >> 4);
+                ag.add(sP[row][lane & 15], sr[row]);
             }
+            __syncthreads();
         }
+        combine(a0, a1);
+        combine_shfl(ag, 16);
+        if (e < ww) store_partial(&st[g * ww + e], a0);
+        if (lane < kMaxDirs) store_partial(&sg[wid][lane], ag);
         __syncthreads();
-    }
-    double* out = partial + (int64_t(p) * gridDim.x + blockIdx.x) * kGramMax;
+        double* out = partial + (int64_t(p) * gmax + part) * kGramMax;
+        if (t < ww) {
+            ExactSum<T> a;
+            for (int k = 0; k < NG; ++k) load_partial(a, &st[k * ww + t]);
+            store_partial(out + t, a);
+        } else if (t >= kGramThreads - kMaxDirs && t - (kGramThreads - kMaxDirs) < w) {
+            const int cc = t - (kGramThreads - kMaxDirs);
+            ExactSum<T> a, b;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int e = threadIdx.x + h * blockDim.x;
-        if (e < ne) store_partial(out + e, acc[h]);
+            for (int k = 0; k < NW; k += 2) {
+                load_partial(a, &sg[k][cc]);
+                load_partial(b, &sg[k + 1][cc]);
+            }
+            combine(a, b);
+            store_partial(out + ww + cc, a);
+        }
+        part += gridDim.x;
+        // st and sg are written again only after the next run's first barrier
     }
 }
 
@@ -1522,177 +1603,212 @@ __device__ void pinv_sym_jacobi(double (*sA)[kMaxDirs + 1], double (*sV)[kMaxDir
 }
 
 
-// Inverse of the symmetric w x w matrix in sA by Gauss-Jordan sweeps on the diagonal (no
-// pivoting), accepted only when it equals the pseudo-inverse: every sweep pivot must be positive
-// (A positive definite), and with lambda_min(A) >= 1 / trace(A^{-1}) and lambda_max(A) <=
-// trace(A), 1 / trace(A^{-1}) exceeding 1e3 times the threshold w 2^-52 trace(A) means no
-// eigenvalue is dropped, so A^+ = A^{-1}.  Thread 16 i + j (of the first 256) owns entry (i, j);
-// a sweep updates every entry once, and the owner of the next pivot forms its reciprocal right
-// after its own update, so the dependent float64 chain is 16 reciprocals long and no other thread
-// spends the narrow float64 pipe on it.  sA is left intact; sX receives A^{-1} (symmetrised).
-// Returns false (sX undefined) when the certificate fails.
-__device__ bool inverse_certified(double (*sA)[kMaxDirs + 1], double (*sX)[kMaxDirs + 1], int w) {
-    __shared__ int ok;
-    __shared__ double tr, trinv;
-    __shared__ double rk[kMaxDirs];   // 1 / pivot k
+// Inverse of the symmetric w x w matrix in sA by symmetric Gauss-Jordan sweeps on the diagonal (no
+// pivoting), accepted (certified below) only when it equals the pseudo-inverse.  The first kInvThreads
+// threads of the CTA call it; thread t owns entry (i, j), i >= j, of the lower triangle (the diagonal
+// entries in warp 0), so a sweep costs 5 warps of float64 operations.  A dependent float64 operation
+// takes about 150 cycles here, so the chain of a sweep is kept to three of them: with t = x_ik x_kj formed
+// while the pivot's reciprocal r is (an estimate from the bit pattern and one Newton step), an entry
+// is x_ij - t r.  sX (full storage) receives A^{-1}; *bad is set when a pivot is not positive.
+// (16 x 16: 29k cycles with a mul, an fma and five operations for the reciprocal in the chain and two
+// barriers of 1024 threads per sweep.)  sA is symmetrised on the way.
+constexpr int kInvThreads = 160;
+__device__ __forceinline__ void inv_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(kInvThreads) : "memory"); }
+__device__ __forceinline__ void inverse_sweeps(double (*sA)[kMaxDirs + 1], double (*sX)[kMaxDirs + 1], int w, int* bad) {
+    __shared__ double rk;
     const int t = threadIdx.x;
-    const int i = t / kMaxDirs, j = t % kMaxDirs;
-    const bool in = t < kMaxDirs * kMaxDirs && i < w && j < w;
-    if (t < kMaxDirs * kMaxDirs) sX[i][j] = in ? sA[i][j] : 0.0;
-    if (t < 32) {
-        double d = t < w ? sA[t][t] : 0.0;
-        d = warp_sum(d);
-        if (t == 0) {
-            tr = d;
-            const double p0 = sA[0][0];
-            ok = p0 > 0.0;
-            rk[0] = fast_rcp(p0);
-        }
+    // entry of this thread: the diagonal first, then the strict lower triangle row by row
+    int i = t, j = t;
+    if (t >= kMaxDirs) {
+        int q = t - kMaxDirs;
+        i = 1;
+        while (q >= i) q -= i++;
+        j = q;
     }
-    __syncthreads();
+    const bool in = t < kMaxDirs * (kMaxDirs + 1) / 2 && i < w && j < w;
+    double x = 0.0;
+    if (in) {   // symmetrised, also for the eigen-decomposition
+        x = i == j ? sA[i][i] : 0.5 * (sA[i][j] + sA[j][i]);
+        sA[i][j] = sA[j][i] = x;
+        sX[i][j] = sX[j][i] = x;
+    }
     for (int k = 0; k < w; ++k) {
-        double v = 0.0;
-        if (in) {
-            const double r = rk[k];
-            if (i == k && j == k) v = r;
-            else if (i == k) v = sX[k][j] * r;
-            else if (j == k) v = -sX[i][k] * r;
-            else v = fma(-sX[i][k] * r, sX[k][j], sX[i][j]);
+        inv_barrier();   // sX holds the matrix after k sweeps
+        const double xik = in ? sX[i][k] : 0.0, xkj = in ? sX[k][j] : 0.0;
+        // the new entry is b - a r in every position: x_ij - x_ik x_kj r off the pivot's row and
+        // column, x_kj r and x_ik r on them, -r on the pivot
+        double a = xik * xkj, b = x;
+        if (i == k || j == k) {
+            a = i == j ? 1.0 : -x;
+            b = 0.0;
         }
-        __syncthreads();
-        if (in) {
-            sX[i][j] = v;
-            if (i == k + 1 && j == k + 1) {   // the next pivot
-                if (!(v > 0.0)) ok = 0;
-                rk[k + 1] = fast_rcp(v);
-            }
+        if (t == k) {
+            if (!(x > 0.0)) *bad = 1;
+            rk = fast_rcp(x);
         }
-        __syncthreads();
+        inv_barrier();
+        if (in) {
+            x = fma(-a, rk, b);
+            sX[i][j] = sX[j][i] = x;
+        }
     }
-    double sym = 0.0;
-    if (in) sym = 0.5 * (sX[i][j] + sX[j][i]);
-    __syncthreads();
-    if (in) sX[i][j] = sym;
-    __syncthreads();
-    if (t < 32) {
-        double d = t < w ? sX[t][t] : 0.0;
-        d = warp_sum(d);
-        if (t == 0) trinv = d;
-    }
-    __syncthreads();
-    if (!ok) return false;
-    // 1 / trace(A^{-1}) > 1e3 thr, i.e. 1e3 thr trace(A^{-1}) < 1 (false for a NaN)
-    const double thr = w * 2.220446049250313e-16 * tr;
-    return 1e3 * thr * trinv < 1.0;
+    if (in) sX[i][j] = sX[j][i] = -x;   // the sweeps leave -A^{-1}
 }
 
+// Distributed shared memory of a cluster: the same variable of CTA `rank`, and the cluster's barrier.
+__device__ __forceinline__ void store_remote(double* var, int rank, double v) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(var)), "r"(rank));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
 // Delta_i, gamma_i -> Delta_i^+ (stored for the reorthogonalisation), alpha_i, gamma^T alpha.
-// One CTA of kSmallThreads per problem (the matrix work uses the first 256); gx is the width of
-// the Gram grid.
+// One cluster of kSmallCtas CTAs per problem; gx is the stride of the Gram partials.  The CTAs share the
+// entries of the Gram sums (one SM reading the partials of 9000 rows took 7k cycles), whose totals meet in
+// the first CTA's shared memory; it does the rest.  A^{-1} is certified when every sweep pivot is
+// positive (A positive definite) and 1 / trace(A^{-1}) <= lambda_min exceeds 1e3 times the threshold
+// w 2^-52 trace(A) >= w 2^-52 lambda_max: no eigenvalue is dropped, so A^+ = A^{-1}.  Otherwise the
+// eigen-decomposition runs.  1000 cameras, w = 16: 20.5 us in one CTA with the longer inverse, now 12.4 us.
 constexpr int kSmallThreads = 1024;
+constexpr int kSmallCtas = 8;
+constexpr int kSmallGroups = 32;   // groups of threads that share the partials of an entry
 template <typename T>
-__global__ void __launch_bounds__(kSmallThreads) k_mcg_small(Ctl* ctl, const double* __restrict__ partial, int gx, double* __restrict__ dpinv,
-                            int mi1) {
+__global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThreads)
+    k_mcg_small(Ctl* ctl, const double* __restrict__ partial, int gx, double* __restrict__ dpinv, int mi1) {
+    cluster_arrive();    // waited for before the first store to another CTA: every CTA has started by then
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
-    const int p = blockIdx.x;
+    const int p = blockIdx.x / kSmallCtas, rank = blockIdx.x % kSmallCtas;
     Ctl* c = ctl + p;
-    if (c->done) return;
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const bool done = c->done != 0;
+    if (rank == 0 && t == 0) {
+        c->live = !done;
+        c->hist_cols = c->cols;   // the next reorthogonalisation runs over every column so far
+    }
+    if (done) {
+        cluster_wait();
+        return;
+    }
     __shared__ double sA[kMaxDirs][kMaxDirs + 1], sV[kMaxDirs][kMaxDirs + 1], sX[kMaxDirs][kMaxDirs + 1];
-    __shared__ double sg[kMaxDirs];
-    __shared__ double sal[kMaxDirs];
+    __shared__ double sg[kMaxDirs], sal[kMaxDirs];
+    __shared__ double st[kSmallThreads];
+    __shared__ double tr;
+    __shared__ int bad, ok;
     const int w = c->w_cur;
     const int it = c->it;
     const int ne = w * w + w;
-    const int np = gram_ctas(int64_t(c->lay.nc) * 9, gx);
+    const int np = gram_parts(c->lay.nc * 9, gx);
     const double* part = partial + int64_t(p) * gx * kGramMax;
-    // Sum of the CTA partials of every entry.  The partials sit in L2, written by the Gram CTAs, so
-    // the sum is bound by load latency: G lanes share an entry (G a power of two, as many as the
-    // block allows, at most a warp); lane g of the group takes the partials b = g, g + G, ... into
-    // eight interleaved sums (eight loads in flight), which are added in a fixed tree, and the
-    // group's sums meet in a fixed shuffle tree.  The order depends on (w, np) alone.
+    // Sum of the Gram CTAs' partials of this CTA's entries.  They sit in L2, so the sum is bound by load
+    // latency: G threads share an entry, group g takes the partials b = g, g + G, ... six loads in
+    // flight, and the groups' sums meet in shared memory.  The order depends on (w, np) alone.
     {
-        int G = 1;
-        while (G < 32 && 2 * G * ne <= int(blockDim.x)) G *= 2;
-        const int per_round = int(blockDim.x) / G;
-        for (int e0 = 0; e0 < ne; e0 += per_round) {
-            const int e = e0 + int(threadIdx.x) / G, g = int(threadIdx.x) % G;
-            // warps holding no entry of this pass skip the arithmetic (and their shuffles) whole
-            if (e0 + int(threadIdx.x & ~31u) / G >= ne) continue;
-            ExactSum<T> acc[8];
-            if (e < ne) {
-                int b = g;
-                for (; b + 7 * G < np; b += 8 * G)
+        const int eb = (ne + kSmallCtas - 1) / kSmallCtas;   // entries of a CTA
+        const int G = min(kSmallThreads / eb, kSmallGroups);
+        const int g = t / eb, el = t - eb * g, e = rank * eb + el;
+        if (g < G) {
+            ExactSum<T> s;
+            if (e < ne)
+                for (int b0 = g; b0 < np; b0 += 6 * G) {
+                    double v[6];
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) load_partial(acc[k], part + int64_t(b + k * G) * kGramMax + e);
+                    for (int u = 0; u < 6; ++u) v[u] = b0 + u * G < np ? part[int64_t(b0 + u * G) * kGramMax + e] : 0.0;
 #pragma unroll
-                for (int k = 0; k < 7; ++k)
-                    if (b + k * G < np) load_partial(acc[k], part + int64_t(b + k * G) * kGramMax + e);
-            }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) combine(acc[k], acc[k + 4]);
-            combine(acc[0], acc[2]);
-            combine(acc[1], acc[3]);
-            combine(acc[0], acc[1]);
-            for (int o = G / 2; o > 0; o >>= 1) combine_shfl(acc[0], o);
-            if (e < ne && g == 0) {
-                const double s = acc[0].value();
-                if (e < w * w) sA[e / w][e % w] = s;
-                else sg[e - w * w] = s;
-            }
+                    for (int u = 0; u < 6; ++u)
+                        if (b0 + u * G < np) add_slot(s, v[u]);
+                }
+            store_partial(&st[t], s);
         }
-    }
-    __syncthreads();
-    // symmetrise
-    double sym = 0.0;
-    const int i = threadIdx.x / kMaxDirs, j = threadIdx.x % kMaxDirs;
-    if (threadIdx.x < kMaxDirs * kMaxDirs && i < w && j < w) sym = 0.5 * (sA[i][j] + sA[j][i]);
-    __syncthreads();
-    if (threadIdx.x < kMaxDirs * kMaxDirs && i < w && j < w) sA[i][j] = sym;
-    __syncthreads();
-    if (w == 1) {
-        if (threadIdx.x == 0) sX[0][0] = sA[0][0] > 0.0 ? 1.0 / sA[0][0] : 0.0;
+        if (t == 0) bad = 0;
         __syncthreads();
-    } else if (!inverse_certified(sA, sX, w)) {
-        pinv_sym_jacobi(sA, sV, sX, w);
-        if (threadIdx.x == 0) c->pinv_steps += 1;
-    }
-    if (threadIdx.x < kMaxDirs * kMaxDirs) {
-        dpinv[(int64_t(p) * mi1 + it) * kMaxDirs * kMaxDirs + threadIdx.x] = (i < w && j < w) ? sX[i][j] : 0.0;
-    }
-    // alpha = Delta^+ gamma and gamma^T alpha: thread (a, b) = 16 a + b forms one product, the
-    // 16 lanes of row a add theirs in a fixed shuffle tree (short float64 chains)
-    if (threadIdx.x < kMaxDirs * kMaxDirs) {
-        double s = (i < w && j < w) ? sX[i][j] * sg[j] : 0.0;
-#pragma unroll
-        for (int o = kMaxDirs / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (j == 0 && i < w) {
-            sal[i] = s;
-            c->alpha_v[i] = s;
+        cluster_wait();
+        if (t < eb && e < ne) {   // here g = 0 and el = t
+            ExactSum<T> a, b;
+#pragma unroll 4
+            for (int k = 0; k + 1 < G; k += 2) {
+                load_partial(a, &st[k * eb + t]);
+                load_partial(b, &st[(k + 1) * eb + t]);
+            }
+            if (G & 1) load_partial(a, &st[(G - 1) * eb + t]);
+            combine(a, b);
+            store_remote(e < w * w ? &sA[e / w][e % w] : &sg[e - w * w], 0, a.value());
         }
+        cluster_arrive();
+        cluster_wait();
+        if (rank != 0) return;
+    }
+    double* Dp = dpinv + (int64_t(p) * mi1 + it) * kMaxDirs * kMaxDirs;
+    if (w == 1) {
+        if (t < kMaxDirs * kMaxDirs && t > 0) Dp[t] = 0.0;
+        if (t == 0) {
+            const double x = sA[0][0] > 0.0 ? 1.0 / sA[0][0] : 0.0, al = x * sg[0], ga = sg[0] * al;
+            Dp[0] = x;
+            c->alpha_v[0] = al;
+            c->ga = ga;
+            if (!(ga == ga)) { c->done = 1; c->status = BA_ERR_BREAKDOWN; }
+        }
+        return;
+    }
+    if (t < kInvThreads) {
+        inverse_sweeps(sA, sX, w, &bad);
+    } else if (wid == kInvThreads / 32) {
+        const double d = warp_sum(lane < w ? sA[lane][lane] : 0.0);
+        if (lane == 0) tr = d;
     }
     __syncthreads();
-    if (threadIdx.x < 32) {
-        double s = int(threadIdx.x) < w ? sg[threadIdx.x] * sal[threadIdx.x] : 0.0;
-        s = warp_sum(s);
-        if (threadIdx.x == 0) {
-            c->ga = s;
-            if (!(s == s)) { c->done = 1; c->status = BA_ERR_BREAKDOWN; }
+    // alpha = Delta^+ gamma (warp 0: two lanes per row) and gamma^T alpha, while warp 1 checks the
+    // certificate and the others store the inverse; once more after a pseudo-inverse
+    for (int pass = 0; pass < 2; ++pass) {
+        if (wid == 0) {
+            const int a = lane >> 1, b0 = (lane & 1) * (kMaxDirs / 2);
+            double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+            for (int b = 0; b < kMaxDirs / 2; b += 2) {
+                if (a < w && b0 + b < w) s0 += sX[a][b0 + b] * sg[b0 + b];
+                if (a < w && b0 + b + 1 < w) s1 += sX[a][b0 + b + 1] * sg[b0 + b + 1];
+            }
+            double s = s0 + s1;
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            if (a < w && !(lane & 1)) {
+                sal[a] = s;
+                c->alpha_v[a] = s;
+            }
+            double ga = a < w ? sg[a] * s : 0.0;
+#pragma unroll
+            for (int o = 2; o < 32; o <<= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
+            if (lane == 0) sal[0] = ga;
+        } else if (wid == 1 && pass == 0) {
+            const double trinv = warp_sum(lane < w ? sX[lane][lane] : 0.0);
+            // 1 / trace(A^{-1}) > 1e3 thr, i.e. 1e3 thr trace(A^{-1}) < 1 (false for a NaN)
+            const double thr = w * 2.220446049250313e-16 * tr;
+            if (lane == 0) ok = !bad && 1e3 * thr * trinv < 1.0;
+        } else if (wid >= 8 && wid < 16) {
+            const int e = t - 256, ei = e / kMaxDirs, ej = e % kMaxDirs;
+            Dp[e] = (ei < w && ej < w) ? sX[ei][ej] : 0.0;
         }
+        __syncthreads();
+        if (pass == 1 || ok) break;
+        pinv_sym_jacobi(sA, sV, sX, w);
+        if (t == 0) c->pinv_steps += 1;
+        __syncthreads();
+    }
+    if (t == 0) {
+        const double ga = sal[0];
+        c->ga = ga;
+        if (!(ga == ga)) { c->done = 1; c->status = BA_ERR_BREAKDOWN; }
     }
 }
 
-__device__ void mcg_decide(Ctl* c, const double* tot, double* hist, int* blk_off, int* blk_w, int mi1, int p, int nb);
-
-// x += P_i alpha; r -= Q_i alpha; z = D^{-1} r; totals of |r|^2 and r^T z, then (last CTA) the
-// decide step (grid: CTAs x problems; thread = one row, as in k_pcg_update).  The columns of the block
-// are requested together (up to 16 of P and of Q per row).
+// x += P_i alpha; r -= Q_i alpha; z = D^{-1} r; per CTA the sums of |r|^2 and r^T z (dpart), from which
+// k_mcg_phi's first CTA takes the decide step (grid: CTAs x problems; thread = one row, as in
+// k_pcg_update).  The columns of the block are requested together (up to 16 of P and of Q per row).
 template <typename T>
 __global__ void __launch_bounds__(kUpdThreads) k_mcg_update(const double* __restrict__ Dinv, const T* __restrict__ P,
                                                             const T* __restrict__ Q, T* __restrict__ x,
                                                             T* __restrict__ r, T* __restrict__ z,
-                                                            double* __restrict__ dpart, int* __restrict__ dcnt,
-                                                            double* __restrict__ hist, int* __restrict__ blk_off,
-                                                            int* __restrict__ blk_w, int mi1, Ctl* ctl) {
+                                                            double* __restrict__ dpart, const Ctl* __restrict__ ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const int p = blockIdx.y;
     const Ctl& c = ctl[p];
@@ -1703,9 +1819,9 @@ __global__ void __launch_bounds__(kUpdThreads) k_mcg_update(const double* __rest
     const int w = c.w_cur, off = c.off_cur;
     const T* Pp = P + c.lay.hoff + int64_t(off) * n;
     const T* Qp = Q + c.lay.hoff + int64_t(off) * n;
+    if (int64_t(blockIdx.x) * kUpdCams >= nc) return;   // no camera (a smaller problem of the batch)
     __shared__ T sal[kMaxDirs];
     __shared__ T sr[kUpdCams * 9];
-    __shared__ double tot[2];
     const int t = threadIdx.x, cl = t / 9, a = t - 9 * (t / 9);
     const int64_t jl = int64_t(blockIdx.x) * kUpdCams + cl;
     const bool act = t < kUpdCams * 9 && jl < nc;
@@ -1725,15 +1841,15 @@ __global__ void __launch_bounds__(kUpdThreads) k_mcg_update(const double* __rest
     ExactSum<T> v[2];
     T rv = T(0);
     if (act) {
-        T dx = T(0), dr = T(0);
+        T dx[2] = {T(0), T(0)}, dr[2] = {T(0), T(0)};
 #pragma unroll
         for (int b = 0; b < kMaxDirs; ++b)
-            if (b < w) {   // columns past w may hold anything (alpha there is 0)
-                dx += pv[b] * sal[b];
-                dr += qv[b] * sal[b];
+            if (b < w) {
+                dx[b & 1] += pv[b] * sal[b];
+                dr[b & 1] += qv[b] * sal[b];
             }
-        x[i] = xv + dx;
-        rv = r0 - dr;
+        x[i] = xv + (dx[0] + dx[1]);
+        rv = r0 - (dr[0] + dr[1]);
         r[i] = rv;
         v[0].add(rv, rv);
     }
@@ -1744,13 +1860,13 @@ __global__ void __launch_bounds__(kUpdThreads) k_mcg_update(const double* __rest
         z[i] = zs;
         v[1].add(rv, zs);
     }
-    if (grid_sum_finalize<T, 2>(v, dpart + int64_t(p) * gridDim.x * 2, dcnt + 4 * p + 1, tot) && threadIdx.x == 0)
-        mcg_decide(ctl + p, tot, hist, blk_off, blk_w, mi1, p, gridDim.y);
+    cta_publish<T, 2>(v, dpart + int64_t(p) * gridDim.x * 2);
 }
 
 // stop test, tau-test and the layout of the next block for problem p (one thread, after the
 // update's totals are in)
 __device__ void mcg_decide(Ctl* c, const double* tot, double* hist, int* blk_off, int* blk_w, int mi1, int p, int nb) {
+    if (c->done) return;   // the small solve found a NaN
     if (c->status == BA_ERR_TIMEOUT) { c->done = 1; return; }
     const double rr = tot[0], rz = tot[1];
     const int it = c->it + 1;
@@ -1798,7 +1914,6 @@ __device__ void mcg_decide(Ctl* c, const double* tot, double* hist, int* blk_off
     c->local_steps += local;
     c->w_new = w;
     c->new_off = c->cols;
-    c->hist_cols = c->cols;
     c->w_cur = w;
     c->off_cur = c->cols;
     blk_off[int64_t(p) * mi1 + it] = c->cols;
@@ -1812,7 +1927,8 @@ __device__ void mcg_decide(Ctl* c, const double* tot, double* hist, int* blk_off
 // row chunk of up to kPhiCols columns at once, 8 rows of each in flight (32 loads a lane), and reads z
 // once for all of them.  A column at a time with float64 shuffle trees ran at 2.1 TB/s (34 us on
 // 2000 columns of 9000 rows; now 21 us).  Fewer columns at once when there are not enough chunks for
-// the warps; a column's sum does not depend on it.
+// the warps; a column's sum does not depend on it.  The problem's first CTA runs the decide step
+// beside them.
 constexpr int kPhiCols = 4;
 template <typename T, int NC>
 __device__ __forceinline__ void phi_columns(const T* __restrict__ qc, int64_t n, const T* __restrict__ zp, int r0, int r1,
@@ -1844,23 +1960,38 @@ __device__ __forceinline__ void phi_columns(const T* __restrict__ qc, int64_t n,
 
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_mcg_phi(const T* __restrict__ Q, const T* __restrict__ z,
-                                                      double* __restrict__ phip, const Ctl* __restrict__ ctl) {
+                                                      double* __restrict__ phip, const double* __restrict__ dpart,
+                                                      int gu, double* __restrict__ hist_out, int* __restrict__ blk_off,
+                                                      int* __restrict__ blk_w, int mi1, Ctl* ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
-    const Ctl& c = ctl[blockIdx.y];
-    if (c.done) return;
+    const int p = blockIdx.y;
+    const Ctl& c = ctl[p];
+    if (!c.live) return;
     const int nc = c.lay.nc;
+    if (blockIdx.x == 0) {   // the decide step; nothing it writes is read by the other CTAs
+        __shared__ double tot[2];
+        const int wid = threadIdx.x >> 5;
+        if (wid < 2) {
+            const ExactSum<T> s = total_of<T, 2>(dpart + int64_t(p) * gu * 2, (nc + kUpdCams - 1) / kUpdCams, wid);
+            if ((threadIdx.x & 31) == 0) tot[wid] = s.value();
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) mcg_decide(ctl + p, tot, hist_out, blk_off, blk_w, mi1, p, gridDim.y);
+        return;
+    }
     const int64_t n = int64_t(nc) * 9;
     const int sz = c.sz, K = c.K, hist = c.hist_cols, chunks = c.n_eff * K;
     const int cz = (sz + K - 1) / K;
     const T* Qp = Q + c.lay.hoff;
     const T* zp = z + 9 * int64_t(c.lay.c0);
     double* ph = phip + c.lay.phoff;
-    const int64_t warps = gstride() >> 5;
+    const int64_t warps = int64_t(gridDim.x - 1) * (kThreads / 32);
     const int nb = 2 * int64_t(hist) * chunks >= kPhiCols * warps ? kPhiCols : 1;   // columns at once
-    const int64_t items = int64_t((hist + nb - 1) / nb) * chunks;
-    for (int64_t it = gtid() >> 5; it < items; it += warps) {
-        const int ch = int(it % chunks), c0 = int(it / chunks) * nb;
-        const int s = ch / K, k = ch - s * K;
+    const int64_t items = int64_t((hist + nb - 1) / nb) * chunks;   // below 2^31: the partials' buffer holds them
+    for (int64_t i64 = (gtid() - kThreads) >> 5; i64 < items; i64 += warps) {
+        const unsigned it = unsigned(i64), ch = it % unsigned(chunks);
+        const int c0 = int(it / unsigned(chunks)) * nb;
+        const int s = int(ch) / K, k = int(ch) - s * K;
         int j0 = s * sz + k * cz, j1 = j0 + cz;
         const int send = (s + 1) * sz < nc ? (s + 1) * sz : nc;
         if (j1 > send) j1 = send;
@@ -2340,14 +2471,14 @@ struct Solver {
     int mi1 = 0;              // per-problem stride of the per-step arrays (max_iters + 1)
     int gx = 1;               // grid width of the kernels over all rows of a problem (x += d)
     int gu = 1;               // grid width of the update kernels (kUpdCams cameras per CTA)
-    int gg = 1;               // Gram grid width
+    int gg = 1;               // Gram partials of the largest problem
     int gq = 1;               // grid width of the per-row kernels
     int gpq = 1;              // grid width of the reorthogonalisation (32-row blocks)
     int gphi = 1, gb = 1;     // Phi and beta grid widths
     int gcol = 1;             // grid width of the column pass of the symmetric product (a CTA per camera)
     std::vector<Layout> lay;  // of the current solve
     Buf P, Q, r, z, xw, PT, part_a, part_b, part_cam, dpinv, beta, phip, hist, blk_off, blk_w, ctl, outer, rt,
-        lay_d, dpart, dcnt, camdot, params, loops;
+        lay_d, dpart, dtot, camdot, params, loops;
     Ctl* h_ctl = nullptr;     // pinned, nb
     Outer* h_outer = nullptr; // pinned, nb
     Params* h_params = nullptr;   // pinned staging of the per-solve arguments
@@ -2633,7 +2764,7 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     w->gx = int(std::min<int64_t>(std::max(1, 4 * G / nb), (9 * int64_t(nc_max) + kThreads - 1) / kThreads));
     if ((int64_t(nc_max) + 27) / 28 > 65535) throw Error(BA_ERR_INVALID_ARG, "too many cameras in one problem");
     w->gu = (nc_max + kUpdCams - 1) / kUpdCams;
-    w->gg = int(std::min<int64_t>(G, (9 * int64_t(nc_max) + 127) / 128));
+    w->gg = int(std::min<int64_t>(G, (9 * int64_t(nc_max) + kGramRows - 1) / kGramRows));
     w->gq = std::max(1, G / nb);
     w->gpq = int(std::max<int64_t>(1, std::min<int64_t>((9 * int64_t(nc_max) + 31) / 32, 4 * G / nb)));
     w->gphi = std::max(1, 4 * G / nb);
@@ -2671,7 +2802,8 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     grow(w->outer, size_t(nb) * sizeof(Outer));
     grow(w->rt, size_t(n) * sizeof(double));
     grow(w->lay_d, size_t(nb) * sizeof(Layout));
-    grow(w->dpart, size_t(nb) * w->gu * 5 * sizeof(double));
+    grow(w->dpart, size_t(nb) * w->gu * 3 * sizeof(double));
+    grow(w->dtot, size_t(nb) * 2 * sizeof(double));
     grow(w->camdot, size_t(s.n_c) * 2 * sizeof(double));
     grow(w->params, sizeof(Params));
     grow(w->loops, sizeof(Loops));
@@ -2681,10 +2813,6 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
         w->h_hist_n = 0;
         BA_CUDA_TRY(cudaMallocHost(&w->h_hist, sizeof(double) * size_t(nb) * w->mi1));
         w->h_hist_n = size_t(nb) * w->mi1;
-    }
-    if (w->dcnt.bytes < size_t(nb) * 4 * sizeof(int)) {
-        grow(w->dcnt, size_t(nb) * 4 * sizeof(int));
-        BA_CUDA_TRY(cudaMemset(w->dcnt.p, 0, w->dcnt.bytes));
     }
     BA_CUDA_TRY(cudaMemcpy(w->lay_d.p, lay.data(), sizeof(Layout) * nb, cudaMemcpyHostToDevice));
     w->lay = lay;
@@ -2707,7 +2835,7 @@ void solver_destroy(Solver* w) {
     if (!w) return;
     Buf* bufs[] = {&w->P, &w->Q, &w->r, &w->z, &w->xw, &w->PT, &w->part_a, &w->part_b, &w->part_cam, &w->dpinv,
                    &w->beta, &w->phip, &w->hist, &w->blk_off, &w->blk_w, &w->ctl, &w->outer, &w->rt,
-                   &w->lay_d, &w->dpart, &w->dcnt, &w->camdot, &w->params, &w->loops};
+                   &w->lay_d, &w->dpart, &w->dtot, &w->camdot, &w->params, &w->loops};
     for (Buf* b : bufs) free_buf(*b);
     for (SolveExec* e : w->execs) {
         cudaGraphExecDestroy(e->exec);
@@ -2810,22 +2938,24 @@ static int enqueue_iteration(Solver* w, const Structure& s, const T* S, const T*
     T* r = ptr<T>(w->r);
     T* z = ptr<T>(w->z);
     Ctl* ctl = ptr<Ctl>(w->ctl);
-    int* dcnt = ptr<int>(w->dcnt);
     const int Gt = num_sms();   // tile-streaming products: one CTA per SM
     if (!mcg) {
         const int np = enqueue_product<T, 1>(w, s, S, Su, P, kSelLive, Q, r, st);
         launch_chained(k_pcg_update<T>, dim3(w->gu, nb), dim3(kUpdThreads), 0, st, Dinv, P, Q, x, r, z,
-                       ptr<double>(w->camdot), ptr<double>(w->dpart), dcnt, ptr<double>(w->hist), ctl);
-        launch_chained(k_pcg_dir<T>, dim3(w->gq, nb), dim3(kThreads), 0, st, z, P, ctl);
+                       ptr<double>(w->camdot), ptr<double>(w->dpart), ptr<double>(w->dtot), ctl);
+        launch_chained(k_pcg_dir<T>, dim3(w->gq, nb), dim3(kThreads), 0, st, z, P, ptr<double>(w->dpart), w->gu,
+                       ptr<double>(w->dtot), ptr<double>(w->hist), ctl);
         return np + 2;
     } else {
-        launch_chained(k_mcg_gram<T>, dim3(w->gg, nb), dim3(kThreads), 0, st, P, Q, r, ptr<double>(w->part_a), ctl);
-        launch_chained(k_mcg_small<T>, dim3(nb), dim3(kSmallThreads), 0, st, ctl, ptr<double>(w->part_a), w->gg,
+        launch_chained(k_mcg_gram<T>, dim3(std::min(w->gg, std::max(1, 2 * num_sms() / nb)), nb), dim3(kGramThreads), 0,
+                       st, P, Q, r, ptr<double>(w->part_a), w->gg, ctl);
+        launch_chained(k_mcg_small<T>, dim3(nb * kSmallCtas), dim3(kSmallThreads), 0, st, ctl, ptr<double>(w->part_a), w->gg,
                        ptr<double>(w->dpinv), w->mi1);
         launch_chained(k_mcg_update<T>, dim3(w->gu, nb), dim3(kUpdThreads), 0, st, Dinv, P, Q, x, r, z,
-                       ptr<double>(w->dpart) + 3 * size_t(nb) * w->gu, dcnt, ptr<double>(w->hist),
-                       ptr<int>(w->blk_off), ptr<int>(w->blk_w), w->mi1, ctl);
-        launch_chained(k_mcg_phi<T>, dim3(w->gphi, nb), dim3(kThreads), 0, st, Q, z, ptr<double>(w->phip), ctl);
+                       ptr<double>(w->dpart), ctl);
+        launch_chained(k_mcg_phi<T>, dim3(w->gphi + 1, nb), dim3(kThreads), 0, st, Q, z, ptr<double>(w->phip),
+                       ptr<double>(w->dpart), w->gu, ptr<double>(w->hist), ptr<int>(w->blk_off),
+                       ptr<int>(w->blk_w), w->mi1, ctl);
         T* betat = ptr<T>(w->beta);
         launch_chained(k_mcg_beta<T>, dim3(w->gb, nb), dim3(kThreads), 0, st, ptr<double>(w->phip),
                        ptr<double>(w->dpinv), ptr<int>(w->blk_off), ptr<int>(w->blk_w), betat, ctl, w->mi1);
