@@ -10,7 +10,7 @@
 //                   to (j, k) and transposed to (k, j); float64: a warp per upper block, three
 //                   entries per lane (_rows); float32: three blocks per warp, a 3x3 sub-block per
 //                   lane (_sub)
-//   k_block_jacobi  one thread per camera: D_j^{-1} = (S_jj)^{-1} through Cholesky
+//   k_block_jacobi  one warp per camera: D_j^{-1} = (S_jj)^{-1} by symmetric Gauss-Jordan sweeps
 // Mixed precision builds no float64 U, G or S_jj.  r, J_p, J_l (for b~ and the true residual
 // S x = sum_o J_p^T (J_p x - J_l V^-1 sum J_l^T J_p x) + lambda D_p x) are formed and used in
 // double-float arithmetic on the float32 pipe (df64.cuh; the *_df kernels), and the float32 system
@@ -297,20 +297,22 @@ __global__ void k_landmarks(int32_t n_l, const int64_t* __restrict__ pt_ptr, con
                             int* status) {
     for (int64_t t = gtid(); t < n_l; t += gstride()) {
         const int64_t l = order[t];
+        // chained multiply-adds: a sum of two products added to the accumulator costs an addition more,
+        // a third of this kernel's float64 operations (their pipe bounds every float64 kernel here)
         double v00 = 0, v01 = 0, v02 = 0, v11 = 0, v12 = 0, v22 = 0, b0 = 0, b1 = 0, b2 = 0;
         for (int64_t o = pt_ptr[l]; o < pt_ptr[l + 1]; ++o) {
             const double* j = Jl + 6 * o;
             double a0 = j[0], a1 = j[1], a2 = j[2], c0 = j[3], c1 = j[4], c2 = j[5];
             double r0 = r[2 * o], r1 = r[2 * o + 1];
-            v00 += a0 * a0 + c0 * c0;
-            v01 += a0 * a1 + c0 * c1;
-            v02 += a0 * a2 + c0 * c2;
-            v11 += a1 * a1 + c1 * c1;
-            v12 += a1 * a2 + c1 * c2;
-            v22 += a2 * a2 + c2 * c2;
-            b0 += a0 * r0 + c0 * r1;
-            b1 += a1 * r0 + c1 * r1;
-            b2 += a2 * r0 + c2 * r1;
+            v00 = fma(c0, c0, fma(a0, a0, v00));
+            v01 = fma(c0, c1, fma(a0, a1, v01));
+            v02 = fma(c0, c2, fma(a0, a2, v02));
+            v11 = fma(c1, c1, fma(a1, a1, v11));
+            v12 = fma(c1, c2, fma(a1, a2, v12));
+            v22 = fma(c2, c2, fma(a2, a2, v22));
+            b0 = fma(c0, r1, fma(a0, r0, b0));
+            b1 = fma(c1, r1, fma(a1, r0, b1));
+            b2 = fma(c2, r1, fma(a2, r0, b2));
         }
         v00 = damp(v00, damping, lambda);
         v11 = damp(v11, damping, lambda);
@@ -384,6 +386,32 @@ __device__ __forceinline__ double warp_sum(double v) {
 
 constexpr int kCamThreads = 128;
 
+// Sums of N <= 64 values over the warp by recursive halving: in each step a lane keeps one half of the
+// values it still holds and hands the other half over, so the 64 sums cost 62 additions per lane instead
+// of the 320 of 64 shuffle trees (with these and chained multiply-adds k_cameras takes 121 us instead of
+// 290 us on 601 cameras, k_schur_diag 102 us instead of 234 us).  Lane l ends with the sums
+// of values 2 l and 2 l + 1, written to out (zero past N).
+template <int N>
+__device__ __forceinline__ void warp_sums(double (&v)[N], double* out) {
+    const int lane = threadIdx.x & 31;
+    double h[32];
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+        const double a = k < N ? v[k < N ? k : 0] : 0.0, b = k + 32 < N ? v[k + 32 < N ? k + 32 : 0] : 0.0;
+        const bool up = lane & 16;
+        h[k] = (up ? b : a) + __shfl_xor_sync(0xffffffffu, up ? a : b, 16);
+    }
+#pragma unroll
+    for (int m = 16; m >= 2; m >>= 1) {
+        const bool up = lane & (m >> 1);
+#pragma unroll
+        for (int k = 0; k < m; ++k)
+            h[k] = (up ? h[k + m] : h[k]) + __shfl_xor_sync(0xffffffffu, up ? h[k] : h[k + m], m >> 1);
+    }
+    out[2 * lane] = h[0];
+    out[2 * lane + 1] = h[1];
+}
+
 // U_lambda, b_p and b~ of one camera per CTA.
 __global__ void __launch_bounds__(kCamThreads) k_cameras(
     int32_t n_c, const int64_t* __restrict__ cam_ptr, const int32_t* __restrict__ cam_obs,
@@ -394,11 +422,9 @@ __global__ void __launch_bounds__(kCamThreads) k_cameras(
     __shared__ double fin[64];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int j = blockIdx.x; j < n_c; j += gridDim.x) {
-        double u[45], b[9];
+        double u[54];
 #pragma unroll
-        for (int k = 0; k < 45; ++k) u[k] = 0.0;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) b[k] = 0.0;
+        for (int k = 0; k < 54; ++k) u[k] = 0.0;
         const int64_t beg = cam_ptr[j], end = cam_ptr[j + 1];
         for (int64_t q = beg + threadIdx.x; q < end; q += blockDim.x) {
             const int64_t o = cam_obs[q];
@@ -413,16 +439,12 @@ __global__ void __launch_bounds__(kCamThreads) k_cameras(
 #pragma unroll
             for (int a = 0; a < 9; ++a) {
 #pragma unroll
-                for (int bb = a; bb < 9; ++bb) u[t++] += c0[a] * c0[bb] + c1[a] * c1[bb];
-                b[a] += c0[a] * r0 + c1[a] * r1;
+                for (int bb = a; bb < 9; ++bb, ++t) u[t] = fma(c1[a], c1[bb], fma(c0[a], c0[bb], u[t]));
+                u[45 + a] = fma(c1[a], r1, fma(c0[a], r0, u[45 + a]));
             }
         }
-        // reduce the 54 sums
-#pragma unroll
-        for (int k = 0; k < 54; ++k) {
-            double v = warp_sum(k < 45 ? u[k] : b[k - 45]);
-            if (lane == 0) red[wid][k] = v;
-        }
+        // reduce the 54 sums (U's upper triangle, then b_p)
+        warp_sums<54>(u, red[wid]);
         __syncthreads();
         if (threadIdx.x < 54) {
             double v = 0;
@@ -454,7 +476,7 @@ __global__ void __launch_bounds__(kCamThreads) k_cameras(
             double e0 = el[0], e1 = el[1], e2 = el[2];
             const double* g = G + 27 * o;
 #pragma unroll
-            for (int a = 0; a < 9; ++a) t9[a] += g[3 * a] * e0 + g[3 * a + 1] * e1 + g[3 * a + 2] * e2;
+            for (int a = 0; a < 9; ++a) t9[a] = fma(g[3 * a + 2], e2, fma(g[3 * a + 1], e1, fma(g[3 * a], e0, t9[a])));
         }
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
@@ -479,9 +501,9 @@ __global__ void __launch_bounds__(kCamThreads) k_schur_diag(int32_t n_c, const i
                                                            const int32_t* __restrict__ cam_obs,
                                                            const double* __restrict__ G, const double* __restrict__ U,
                                                            double* __restrict__ Sd) {
-    __shared__ double red[kCamThreads / 32][48];
+    __shared__ double red[kCamThreads / 32][64];
     __shared__ double fin[48];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int wid = threadIdx.x >> 5;
     for (int j = blockIdx.x; j < n_c; j += gridDim.x) {
         double acc[45];
 #pragma unroll
@@ -495,14 +517,10 @@ __global__ void __launch_bounds__(kCamThreads) k_schur_diag(int32_t n_c, const i
 #pragma unroll
             for (int a = 0; a < 9; ++a)
 #pragma unroll
-                for (int bb = a; bb < 9; ++bb)
-                    acc[t++] += gv[3 * a] * gv[3 * bb] + gv[3 * a + 1] * gv[3 * bb + 1] + gv[3 * a + 2] * gv[3 * bb + 2];
+                for (int bb = a; bb < 9; ++bb, ++t)
+                    acc[t] = fma(gv[3 * a + 2], gv[3 * bb + 2], fma(gv[3 * a + 1], gv[3 * bb + 1], fma(gv[3 * a], gv[3 * bb], acc[t])));
         }
-#pragma unroll
-        for (int k = 0; k < 45; ++k) {
-            double v = warp_sum(acc[k]);
-            if (lane == 0) red[wid][k] = v;
-        }
+        warp_sums<45>(acc, red[wid]);
         __syncthreads();
         if (threadIdx.x < 45) {
             double v = 0;
@@ -527,14 +545,18 @@ __global__ void __launch_bounds__(kCamThreads) k_schur_diag(int32_t n_c, const i
 // lanes 0..26 load the two 27-value G blocks of every pair of the chunk (one coalesced load per
 // block, all of the chunk's loads in flight together), stage them in shared memory, and every
 // lane then accumulates its entries over the chunk's pairs in order (lane p fetches the indices of
-// pair p; 16-pair chunks measured no faster).
+// pair p; 16-pair chunks measured no faster).  Bound by the float64 pipe, so an entry's term is three
+// chained multiply-adds (a sum of three products added to the entry cost a fourth operation), and the CTAs
+// are two warps, so that a problem with few blocks uses every SM (16 cameras: 120 blocks ran on 15 SMs).
+// 601 cameras: 764 us before, 507 us now; 16 cameras: 73 us, 43 us now.
+constexpr int kOffRowsThreads = 64;
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_schur_off_rows(
+__global__ void __launch_bounds__(kOffRowsThreads, 12) k_schur_off_rows(
     int64_t n_up, const int64_t* __restrict__ up_dst, const int64_t* __restrict__ up_mdst,
     const int64_t* __restrict__ pair_ptr, const int2* __restrict__ pairs, const T* __restrict__ G,
     T* __restrict__ S) {
     constexpr int kChunk = 8;
-    __shared__ T sg[kThreads / 32][kChunk][2][28];
+    __shared__ T sg[kOffRowsThreads / 32][kChunk][2][28];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t nw = gstride() >> 5;
     const int e0 = lane, e1 = lane + 32, e2 = lane + 64;
@@ -572,9 +594,9 @@ __global__ void __launch_bounds__(kThreads) k_schur_off_rows(
             for (int p = 0; p < np; ++p) {
                 const T* x = sg[wid][p][0];
                 const T* y = sg[wid][p][1];
-                s0 += x[3 * a0] * y[3 * b0] + x[3 * a0 + 1] * y[3 * b0 + 1] + x[3 * a0 + 2] * y[3 * b0 + 2];
-                s1 += x[3 * a1] * y[3 * b1] + x[3 * a1 + 1] * y[3 * b1 + 1] + x[3 * a1 + 2] * y[3 * b1 + 2];
-                s2 += x[3 * a2] * y[3 * b2] + x[3 * a2 + 1] * y[3 * b2 + 1] + x[3 * a2 + 2] * y[3 * b2 + 2];
+                s0 = fma(x[3 * a0 + 2], y[3 * b0 + 2], fma(x[3 * a0 + 1], y[3 * b0 + 1], fma(x[3 * a0], y[3 * b0], s0)));
+                s1 = fma(x[3 * a1 + 2], y[3 * b1 + 2], fma(x[3 * a1 + 1], y[3 * b1 + 1], fma(x[3 * a1], y[3 * b1], s1)));
+                s2 = fma(x[3 * a2 + 2], y[3 * b2 + 2], fma(x[3 * a2 + 1], y[3 * b2 + 1], fma(x[3 * a2], y[3 * b2], s2)));
             }
         }
         T* Sj = S + up_dst[u];
@@ -1266,67 +1288,83 @@ __global__ void k_df_to_double(double* __restrict__ buf, int64_t n) {
     }
 }
 
-// D_j^{-1} = (S_jj)^{-1} = L^{-T} L^{-1} from the Cholesky factor of the diagonal block.
+// D_j^{-1} = (S_jj)^{-1} by symmetric Gauss-Jordan sweeps on the diagonal (a pivot that is not positive
+// marks a block that is not positive definite: the pivots are those of the Cholesky factorisation).
 // With lam != nullptr the block is first scaled by its diagonal, B^ = s B s with s_a = B_aa^{-1/2};
 // Dinv then receives (B^)^{-1} in double-float (hi, lo in the 8 bytes of a float64), lam the scale
 // factors and lam32 their float32 roundings.
-__global__ void k_block_jacobi(int32_t n_c, const double* __restrict__ Sd, double* __restrict__ Dinv,
-                               double* __restrict__ lam, float* __restrict__ lam32, int* status) {
-    for (int64_t j = gtid(); j < n_c; j += gstride()) {
-        double L[81];
-        for (int e = 0; e < 81; ++e) L[e] = Sd[81 * j + e];
-        if (lam) {
-            double sc[9];
-            for (int a = 0; a < 9; ++a) {
-                sc[a] = L[9 * a + a] > 0.0 ? 1.0 / sqrt(L[9 * a + a]) : 1.0;
-                lam[9 * j + a] = sc[a];
-                lam32[9 * j + a] = float(sc[a]);
-            }
-            for (int a = 0; a < 9; ++a)
-                for (int b = 0; b < 9; ++b) L[9 * a + b] *= sc[a] * sc[b];
+// A warp per camera: lane l owns the entries l and l + 32 of the 45 of the lower triangle, which meet in
+// shared memory.  A sweep's chain is the pivot's reciprocal (four dependent float64 operations of about
+// 150 cycles) and one multiply-add, the entries' products formed meanwhile; a thread per camera took 34 us
+// for its Cholesky factor, triangular inverse and product, whatever the camera count (now 8 us).
+constexpr int kBjThreads = 64;
+__global__ void __launch_bounds__(kBjThreads) k_block_jacobi(int32_t n_c, const double* __restrict__ Sd,
+                                                            double* __restrict__ Dinv, double* __restrict__ lam,
+                                                            float* __restrict__ lam32, int* status) {
+    __shared__ double sx[kBjThreads / 32][9][9];
+    __shared__ double ssc[kBjThreads / 32][9];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    double(*X)[9] = sx[wid];
+    double* sc = ssc[wid];
+    int ei[2], ej[2];   // this lane's entries (row, column), row >= column
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        int q = lane + 32 * u, i = 0;
+        while (q > i) q -= ++i;
+        ei[u] = i;
+        ej[u] = q;
+    }
+    for (int64_t j = gtid() >> 5; j < n_c; j += gstride() >> 5) {
+        const double* B = Sd + 81 * j;
+        if (lam && lane < 9) {
+            const double d = B[10 * lane];
+            const double v = d > 0.0 ? 1.0 / sqrt(d) : 1.0;
+            sc[lane] = v;
+            lam[9 * j + lane] = v;
+            lam32[9 * j + lane] = float(v);
         }
-        // Cholesky with reciprocal square roots: L[c][c] keeps 1 / l_cc (the exact float64 divisions
-        // and square roots are long dependent chains on this GPU's narrow float64 pipe)
+        __syncwarp();
+        double x[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            x[u] = 0.0;
+            if (lane + 32 * u < 45) {
+                x[u] = B[9 * ei[u] + ej[u]];
+                if (lam) x[u] *= sc[ei[u]] * sc[ej[u]];
+                X[ei[u]][ej[u]] = X[ej[u]][ei[u]] = x[u];
+            }
+        }
         bool ok = true;
-        for (int c = 0; c < 9; ++c) {
-            double d = L[9 * c + c];
-            for (int k = 0; k < c; ++k) d -= L[9 * c + k] * L[9 * c + k];
-            if (!(d > 0.0)) { ok = false; d = 1.0; }
-            const double ic = rsqrt_fast(d);
-            L[9 * c + c] = ic;
-            for (int a = c + 1; a < 9; ++a) {
-                double v = L[9 * a + c];
-                for (int k = 0; k < c; ++k) v -= L[9 * a + k] * L[9 * c + k];
-                L[9 * a + c] = v * ic;
+        for (int k = 0; k < 9; ++k) {
+            __syncwarp();   // X holds the block after k sweeps
+            const double p = X[k][k];
+            double a[2], b[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                // the new entry is b - a / p in every position: x_ij - x_ik x_kj / p off the pivot's
+                // row and column, x_kj / p and x_ik / p on them, -1 / p on the pivot
+                const bool in = lane + 32 * u < 45, on = ei[u] == k || ej[u] == k;
+                a[u] = in ? (on ? (ei[u] == ej[u] ? 1.0 : -x[u]) : X[ei[u]][k] * X[k][ej[u]]) : 0.0;
+                b[u] = on ? 0.0 : x[u];
             }
-        }
-        if (!ok) atomicExch(status, BA_ERR_SINGULAR);
-        // Li = L^{-1} (lower), column by column
-        double Li[81];
-        for (int k = 0; k < 81; ++k) Li[k] = 0.0;
-        for (int c = 0; c < 9; ++c) {
-            Li[9 * c + c] = L[9 * c + c];
-            for (int a = c + 1; a < 9; ++a) {
-                double v = 0.0;
-                for (int k = c; k < a; ++k) v -= L[9 * a + k] * Li[9 * k + c];
-                Li[9 * a + c] = v * L[9 * a + a];
-            }
-        }
-        double* D = Dinv + 81 * j;
-        for (int a = 0; a < 9; ++a) {
-            for (int b = a; b < 9; ++b) {
-                double v = 0.0;
-                for (int k = b; k < 9; ++k) v += Li[9 * k + a] * Li[9 * k + b];
-                if (lam) {
-                    const df64 d = df_from(v);
-                    df_st(reinterpret_cast<float2*>(D) + 9 * a + b, d);
-                    df_st(reinterpret_cast<float2*>(D) + 9 * b + a, d);
-                } else {
-                    D[9 * a + b] = v;
-                    D[9 * b + a] = v;
+            ok = ok && p > 0.0;
+            const double r = rcp_fast(p > 0.0 ? p : 1.0);
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+                if (lane + 32 * u < 45) {
+                    x[u] = fma(-a[u], r, b[u]);
+                    X[ei[u]][ej[u]] = X[ej[u]][ei[u]] = x[u];
                 }
-            }
         }
+        if (!ok && lane == 0) atomicExch(status, BA_ERR_SINGULAR);
+        __syncwarp();
+        for (int e = lane; e < 81; e += 32) {   // the sweeps leave the negative of the inverse
+            const double v = -X[e / 9][e % 9];
+            if (lam) df_st(reinterpret_cast<float2*>(Dinv) + 81 * j + e, df_from(v));
+            else Dinv[81 * j + e] = v;
+        }
+        __syncwarp();
     }
 }
 
@@ -1516,9 +1554,15 @@ void launch_schur_diag32(const Structure& s, System& y, cudaStream_t st) {
                                                          y.Sd, y.G32);
 }
 
+// a warp per block; past 128 CTAs per SM a stride loop
+static int off_rows_grid(int64_t n_up) {
+    const int64_t g = (n_up * 32 + kOffRowsThreads - 1) / kOffRowsThreads;
+    return int(g < num_sms() * 128 ? g : num_sms() * 128);
+}
+
 void launch_schur(const Structure& s, System& y, cudaStream_t st) {
     if (s.n_up > 0)
-        k_schur_off_rows<double><<<grid_for(s.n_up * 32, kThreads), kThreads, 0, st>>>(
+        k_schur_off_rows<double><<<off_rows_grid(s.n_up), kOffRowsThreads, 0, st>>>(
             s.n_up, s.up_dst, s.up_mdst, s.up_pair_ptr, s.pairs, y.G, y.S);
     k_put_diag<double><<<grid_for(int64_t(s.n_c) * 81, kThreads), kThreads, 0, st>>>(
         s.n_c, s.row_ptr, s.tile_ptr, s.diag_pos, y.Sd, nullptr, y.S, nullptr, nullptr);
@@ -1562,12 +1606,12 @@ void launch_cam_prep(const Structure& s, System& y, cudaStream_t st) {
 // Float64: D^{-1}.  Mixed precision: Lam and the inverse blocks of the scaled system only (its solves
 // use no other; launch_block_jacobi_plain forms D^{-1} when it is asked for).
 void launch_block_jacobi(const Structure& s, System& y, cudaStream_t st) {
-    if (y.S32) k_block_jacobi<<<grid_for(s.n_c, 64), 64, 0, st>>>(s.n_c, y.Sd, y.Dhat, y.lam, y.lam32, y.status);
+    if (y.S32) k_block_jacobi<<<grid_for(int64_t(s.n_c) * 32, kBjThreads), kBjThreads, 0, st>>>(s.n_c, y.Sd, y.Dhat, y.lam, y.lam32, y.status);
     else launch_block_jacobi_plain(s, y, st);
 }
 
 void launch_block_jacobi_plain(const Structure& s, System& y, cudaStream_t st) {
-    k_block_jacobi<<<grid_for(s.n_c, 64), 64, 0, st>>>(s.n_c, y.Sd, y.Dinv, nullptr, nullptr, y.status);
+    k_block_jacobi<<<grid_for(int64_t(s.n_c) * 32, kBjThreads), kBjThreads, 0, st>>>(s.n_c, y.Sd, y.Dinv, nullptr, nullptr, y.status);
 }
 
 
