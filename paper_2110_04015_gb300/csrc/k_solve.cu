@@ -2121,8 +2121,11 @@ struct PqShape;
 template <> struct PqShape<float> { static constexpr int kSlices = 16, kTile = 256; };
 template <> struct PqShape<double> { static constexpr int kSlices = 8, kTile = 128; };
 
-template <typename T>
-__global__ void __launch_bounds__(PqShape<T>::kSlices * 32, 2) k_mcg_pq(T* __restrict__ P, T* __restrict__ Q,
+// RL rows per lane: a column's 16 betas are read from shared memory once for 32 RL rows.  With one row
+// that read (16 words a lane for 16 multiply-adds) slows the kernel once every SM has work (17.7 us on average
+// over a 1000-camera solve, 15.5 us with two rows); with fewer rows than that, more CTAs count for more.
+template <typename T, int RL>
+__global__ void __launch_bounds__(PqShape<T>::kSlices * 32, RL == 1 ? 2 : 1) k_mcg_pq(T* __restrict__ P, T* __restrict__ Q,
                                                                      const T* __restrict__ z, const T* __restrict__ beta,
                                                                      T* __restrict__ PT, const Ctl* __restrict__ ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
@@ -2143,13 +2146,14 @@ __global__ void __launch_bounds__(PqShape<T>::kSlices * 32, 2) k_mcg_pq(T* __res
     T* Pp = P + c.lay.hoff;
     T* Qp = Q + c.lay.hoff;
     const T* Bp = beta + c.lay.boff * kMaxDirs;
-    for (int64_t base = int64_t(blockIdx.x) * 32; base < n; base += int64_t(gridDim.x) * 32) {
-        const int64_t row = base + lane;
-        const bool act = row < n;
-        T ap[kMaxDirs], aq[kUpdQ ? kMaxDirs : 1];
+    static_assert(!kUpdQ || RL == 1, "two rows per lane in the float32 sweeps only");
+    for (int64_t base = int64_t(blockIdx.x) * (32 * RL); base < n; base += int64_t(gridDim.x) * (32 * RL)) {
+        const int64_t row = base + lane;   // and row + 32
+        T ap[RL][kMaxDirs], aq[kUpdQ ? kMaxDirs : 1];
 #pragma unroll
         for (int s = 0; s < kMaxDirs; ++s) {
-            ap[s] = T(0);
+#pragma unroll
+            for (int h = 0; h < RL; ++h) ap[h][s] = T(0);
             if constexpr (kUpdQ) aq[s] = T(0);
         }
         // beta tile t + 1 is copied while tile t is used (rows of 16 values; past w they may hold
@@ -2172,20 +2176,22 @@ __global__ void __launch_bounds__(PqShape<T>::kSlices * 32, 2) k_mcg_pq(T* __res
             const T* pc = Pp + int64_t(c0) * n + row;
             const T* qc = Qp + int64_t(c0) * n + row;
             for (int cl = k; cl < tc; cl += NS * U) {
-                T pv[U], qv[U];
+                T pv[RL][U], qv[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const int cu = cl + u * NS;
-                    const bool in = act && cu < tc;
-                    pv[u] = in ? pc[int64_t(cu) * n] : T(0);
-                    if constexpr (kUpdQ) qv[u] = in ? qc[int64_t(cu) * n] : T(0);
+#pragma unroll
+                    for (int h = 0; h < RL; ++h)
+                        pv[h][u] = row + 32 * h < n && cu < tc ? pc[int64_t(cu) * n + 32 * h] : T(0);
+                    if constexpr (kUpdQ) qv[u] = row < n && cu < tc ? qc[int64_t(cu) * n] : T(0);
                 }
                 if (w == 1) {
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
                         const int cu = cl + u * NS;
                         const T b0 = cu < tc ? sB[cu][0] : T(0);
-                        ap[0] += pv[u] * b0;
+#pragma unroll
+                        for (int h = 0; h < RL; ++h) ap[h][0] += pv[h][u] * b0;
                         if constexpr (kUpdQ) aq[0] += qv[u] * b0;
                     }
                 } else {
@@ -2196,15 +2202,19 @@ __global__ void __launch_bounds__(PqShape<T>::kSlices * 32, 2) k_mcg_pq(T* __res
 #pragma unroll
                         for (int s = 0; s < kMaxDirs; s += 2) {
                             if constexpr (kUpdQ) {
-                                ap[s] += pv[u] * sB[cu][s];
-                                ap[s + 1] += pv[u] * sB[cu][s + 1];
+                                ap[0][s] += pv[0][u] * sB[cu][s];
+                                ap[0][s + 1] += pv[0][u] * sB[cu][s + 1];
                                 aq[s] += qv[u] * sB[cu][s];
                                 aq[s + 1] += qv[u] * sB[cu][s + 1];
                             } else {   // packed: each half rounds like a scalar fused multiply-add
                                 const float2 b2 = *reinterpret_cast<const float2*>(&sB[cu][s]);
-                                const float2 v = __ffma2_rn(make_float2(pv[u], pv[u]), b2, make_float2(ap[s], ap[s + 1]));
-                                ap[s] = v.x;
-                                ap[s + 1] = v.y;
+#pragma unroll
+                                for (int h = 0; h < RL; ++h) {
+                                    const float2 v = __ffma2_rn(make_float2(pv[h][u], pv[h][u]), b2,
+                                                                make_float2(ap[h][s], ap[h][s + 1]));
+                                    ap[h][s] = v.x;
+                                    ap[h][s + 1] = v.y;
+                                }
                             }
                         }
                     }
@@ -2213,8 +2223,6 @@ __global__ void __launch_bounds__(PqShape<T>::kSlices * 32, 2) k_mcg_pq(T* __res
             __syncthreads();
         }
         // column s of the new block is added by warp s mod NS, over the slices in order
-        const int sub = act ? int(row / 9) / sz : 0;
-        const T zr = act ? z[r0g + row] : T(0);
         auto slices = [&](const T* acc, auto&& put) {
             __syncthreads();
 #pragma unroll
@@ -2228,26 +2236,30 @@ __global__ void __launch_bounds__(PqShape<T>::kSlices * 32, 2) k_mcg_pq(T* __res
                 put(s, sum);
             }
         };
-        if constexpr (kUpdQ) {
-            slices(ap, [&](int s, T sum) {
-                if (act && s < w) Pp[int64_t(off + s) * n + row] = (s == (local ? sub : 0) ? zr : T(0)) - sum;
-            });
-            slices(aq, [&](int s, T sum) {
-                if (act && s < w) Qp[int64_t(off + s) * n + row] -= sum;
-            });
-        } else {
+#pragma unroll
+        for (int h = 0; h < RL; ++h) {
+            const int64_t rh = row + 32 * h;
+            const bool act = rh < n;
+            const int sub = act ? int(rh / 9) / sz : 0;
+            const T zr = act ? z[r0g + rh] : T(0);
             T pn = T(0);
-            slices(ap, [&](int s, T sum) {   // NS = kMaxDirs: one column per warp
+            slices(ap[h], [&](int s, T sum) {
                 pn = s < w ? (s == (local ? sub : 0) ? zr : T(0)) - sum : T(0);
-                if (act && s < w) Pp[int64_t(off + s) * n + row] = pn;
+                if (act && s < w) Pp[int64_t(off + s) * n + rh] = pn;
             });
-            // row-major copy of the new block for the multi-column product (zero past w)
-            static_assert(kUpdQ || NS == kMaxDirs, "one column per warp");
-            __syncthreads();
-            red[0][lane][k] = pn;
-            __syncthreads();
-            const int rr = threadIdx.x / kMaxDirs, ss = threadIdx.x % kMaxDirs;
-            if (base + rr < n) PT[(r0g + base) * kMaxDirs + threadIdx.x] = red[0][rr][ss];
+            if constexpr (kUpdQ) {
+                slices(aq, [&](int s, T sum) {
+                    if (act && s < w) Qp[int64_t(off + s) * n + rh] -= sum;
+                });
+            } else {
+                // row-major copy of the new block for the multi-column product (zero past w)
+                static_assert(kUpdQ || NS == kMaxDirs, "one column per warp");
+                __syncthreads();
+                red[0][lane][k] = pn;
+                __syncthreads();
+                const int rr = threadIdx.x / kMaxDirs, ss = threadIdx.x % kMaxDirs;
+                if (base + 32 * h + rr < n) PT[(r0g + base + 32 * h) * kMaxDirs + threadIdx.x] = red[0][rr][ss];
+            }
         }
         __syncthreads();
     }
@@ -2967,13 +2979,14 @@ static int enqueue_iteration(Solver* w, const Structure& s, const T* S, const T*
             if (w->use_l)
                 launch_spmv<T, 0, false, false>(w->spmv_cfg, st, s.row_ptr, s.tile_ptr, s.col, S, z, w->items_l,
                                                 kSelLocal, Q, nullptr, nullptr, ctl, nullptr);
-            launch_chained(k_mcg_pq<T>, dim3(w->gpq, nb), dim3(PqShape<T>::kSlices * 32), 0, st, P, Q, z, betat, (T*)nullptr,
-                           ctl);
+            launch_chained(k_mcg_pq<T, 1>, dim3(w->gpq, nb), dim3(PqShape<T>::kSlices * 32), 0, st, P, Q, z, betat,
+                           (T*)nullptr, ctl);
             return w->use_l ? 8 : 7;
         } else {
             // Algorithm 2: Q_{i+1} = S P_{i+1}
-            launch_chained(k_mcg_pq<T>, dim3(w->gpq, nb), dim3(PqShape<T>::kSlices * 32), 0, st, P, Q, z, betat, ptr<T>(w->PT),
-                           ctl);
+            // two rows per lane once they still give nearly every SM a CTA (a row's sum is the same either way)
+            auto pq = w->n >= int64_t(48) * Gt ? k_mcg_pq<T, 2> : k_mcg_pq<T, 1>;
+            launch_chained(pq, dim3(w->gpq, nb), dim3(PqShape<T>::kSlices * 32), 0, st, P, Q, z, betat, ptr<T>(w->PT), ctl);
             const int np = enqueue_product<T, 2>(w, s, S, Su, P, kSelW1, Q, nullptr, st);
             launch_chained(k_spmm<T>, dim3(Gt), dim3(SpmmCfg::kWarps * 32), spmm_smem<T>(), st, s.row_ptr, s.tile_ptr,
                            s.col, S, ptr<T>(w->PT), w->items_g, static_cast<T*>(w->mm_part), Q, ctl);
