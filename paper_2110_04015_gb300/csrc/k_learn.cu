@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "ba_internal.cuh"
+#include "df64.cuh"
 
 namespace ba {
 
@@ -90,6 +91,12 @@ Offsets offsets() {
     return o;
 }
 
+// a b as a double-float (exact barring underflow)
+__device__ __forceinline__ df64 product(float a, float b) {
+    const float p = __fmul_rn(a, b);
+    return df64(p, __fmaf_rn(a, b, -p));
+}
+
 // ---- graph -----------------------------------------------------------------------------------
 
 // c of every stored block (CSR order; 0 on the diagonal) and d_j, one warp per block-row.
@@ -122,10 +129,17 @@ __global__ void k_gnn_edges(int32_t n_c, const int64_t* __restrict__ row_ptr, co
                             sum += v * v;
                         }
                 } else {
-                    for (int e = 0; e < 81; ++e) {
-                        const double v = S32[s_at(tile_ptr, j, q, e)];
-                        sum += v * v;
+                    // the squares are exact in double-float and so is their sum to 2^-47, without the
+                    // 162 float64 operations and conversions of a float64 sum (28 us -> 11 us for 240 cameras)
+                    const float* blk = S32 + s_at(tile_ptr, j, q, 0);
+                    df64 a0(0.f), a1(0.f), a2(0.f);
+#pragma unroll 3
+                    for (int e = 0; e < 81; e += 3) {
+                        a0 += product(blk[e], blk[e]);
+                        a1 += product(blk[e + 1], blk[e + 1]);
+                        a2 += product(blk[e + 2], blk[e + 2]);
                     }
+                    sum = df_to(a0 + a1 + a2);
                 }
             }
             const float cq = float(sqrt(sum));
@@ -155,27 +169,77 @@ __global__ void k_gnn_features(int32_t n_c, const double* __restrict__ aux, cons
 }
 
 // standardise the centre (per axis: mean removed, divided by the axis' root mean square) and
-// log(1 + d) (mean removed, divided by its standard deviation); one CTA
-__global__ void k_gnn_standardize(int32_t n_c, float* __restrict__ X) {
-    const int cols[4] = {0, 1, 2, 6};
-    for (int ci = 0; ci < 4; ++ci) {
-        const int f = cols[ci];
-        double s = 0.0;
-        for (int64_t j = threadIdx.x; j < n_c; j += blockDim.x) s += X[kF * j + f];
-        const double mean = cta_sum(s) / n_c;
-        double q = 0.0;
-        for (int64_t j = threadIdx.x; j < n_c; j += blockDim.x) {
-            const double v = X[kF * j + f] - mean;
-            q += v * v;
-        }
-        const double rms = sqrt(cta_sum(q) / n_c);
-        const double inv = rms > 0.0 ? 1.0 / rms : 1.0;
-        for (int64_t j = threadIdx.x; j < n_c; j += blockDim.x) X[kF * j + f] = float((X[kF * j + f] - mean) * inv);
+// log(1 + d) (mean removed, divided by its standard deviation); one CTA, a quarter of its threads per
+// column (the columns in turn took 18 us)
+constexpr int kStdThreads = 1024;
+__global__ void __launch_bounds__(kStdThreads) k_gnn_standardize(int32_t n_c, float* __restrict__ X) {
+    constexpr int NT = kStdThreads / 4;
+    __shared__ float2 red[kStdThreads / 32];
+    __shared__ float2 stat[4];
+    const int grp = threadIdx.x / NT, t = threadIdx.x % NT, f = grp < 3 ? grp : 6;
+    // f(the sum of v over the threads of this quarter), computed once per quarter: a float64 division by
+    // every thread would queue on the float64 pipe
+    auto quarter = [&](df64 v, auto&& fn) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += df_shfl_xor(v, o);
+        if ((threadIdx.x & 31) == 0) df_st(&red[threadIdx.x >> 5], v);
         __syncthreads();
+        if (t == 0) {
+            df64 s(0.f);
+#pragma unroll
+            for (int w = 0; w < NT / 32; ++w) s += df_ld(&red[grp * (NT / 32) + w]);
+            df_st(&stat[grp], df_from(fn(df_to(s))));
+        }
+        __syncthreads();
+        return df_ld(&stat[grp]);
+    };
+    df64 s(0.f);
+    for (int64_t j = t; j < n_c; j += NT) s += df64(X[kF * j + f]);
+    const df64 mean = quarter(s, [&](double v) { return v / n_c; });
+    df64 q(0.f);
+    for (int64_t j = t; j < n_c; j += NT) {
+        const df64 v = df64(X[kF * j + f]) - mean;
+        q += v * v;
+    }
+    const df64 inv = quarter(q, [&](double v) { return v > 0.0 ? 1.0 / sqrt(v / n_c) : 1.0; });
+    for (int64_t j = t; j < n_c; j += NT) {
+        const df64 v = (df64(X[kF * j + f]) - mean) * inv;
+        X[kF * j + f] = __fadd_rn(v.hi, v.lo);
     }
 }
 
 // ---- forward -----------------------------------------------------------------------------------
+
+// sum_k c_jk H_k over block-row j, lane l taking features l and l + 32 (one warp; fi <= 64).  The lanes
+// fetch 32 columns and weights at once and hand them round, so eight rows of H are in flight.
+__device__ __forceinline__ void row_combination(const int32_t* __restrict__ col, const float* __restrict__ c,
+                                                const float* __restrict__ H, int fi, int64_t q0, int64_t q1, float& a0,
+                                                float& a1) {
+    const int lane = threadIdx.x & 31;
+    a0 = a1 = 0.f;
+    for (int64_t base = q0; base < q1; base += 32) {
+        const int n = q1 - base < 32 ? int(q1 - base) : 32;
+        const int kl = lane < n ? col[base + lane] : 0;
+        const float wl = lane < n ? c[base + lane] : 0.f;
+        for (int q = 0; q < n; q += 8) {
+            float h0[8], h1[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {   // past n: row 0 with weight zero, not added
+                const float* hk = H + int64_t(__shfl_sync(0xffffffffu, kl, (q + u) & 31)) * fi;
+                h0[u] = lane < fi ? hk[lane] : 0.f;
+                h1[u] = lane + 32 < fi ? hk[lane + 32] : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float w = __shfl_sync(0xffffffffu, wl, (q + u) & 31);
+                if (q + u < n) {
+                    a0 += w * h0[u];
+                    a1 += w * h1[u];
+                }
+            }
+        }
+    }
+}
 
 // AH_j = (sum_k c_jk H_k) / d_j, one warp per row, lanes over the fi <= 64 features
 __global__ void k_gnn_aggregate(int32_t n_c, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
@@ -183,13 +247,8 @@ __global__ void k_gnn_aggregate(int32_t n_c, const int64_t* __restrict__ row_ptr
                                 int fi, float* __restrict__ AH, int bf16) {
     const int lane = threadIdx.x & 31;
     for (int64_t j = gtid() >> 5; j < n_c; j += gstride() >> 5) {
-        float a0 = 0.f, a1 = 0.f;
-        for (int64_t q = row_ptr[j]; q < row_ptr[j + 1]; ++q) {
-            const float w = c[q];
-            const float* hk = H + int64_t(col[q]) * fi;
-            if (lane < fi) a0 += w * hk[lane];
-            if (lane + 32 < fi) a1 += w * hk[lane + 32];
-        }
+        float a0, a1;
+        row_combination(col, c, H, fi, row_ptr[j], row_ptr[j + 1], a0, a1);
         const float inv = d[j] > 0.f ? 1.f / d[j] : 0.f;
         if (lane < fi) AH[j * fi + lane] = bf16 ? round_bf16(a0 * inv) : a0 * inv;
         if (lane + 32 < fi) AH[j * fi + lane + 32] = bf16 ? round_bf16(a1 * inv) : a1 * inv;
@@ -206,7 +265,9 @@ __global__ void k_gnn_dense(int32_t n_c, int fi, const float* __restrict__ H, co
         float z = b[o];
         const float* h = H + j * fi;
         const float* ah = AH + j * fi;
+#pragma unroll 16
         for (int i = 0; i < fi; ++i) z += h[i] * Ws[i * kH + o];
+#pragma unroll 16
         for (int i = 0; i < fi; ++i) z += ah[i] * Wn[i * kH + o];
         Z[idx] = z;
         const float r = z > 0.f ? z : 0.f;
@@ -237,7 +298,9 @@ __global__ void k_gnn_center(int32_t n_c, const float* __restrict__ s, const flo
     }
     const double sd = cta_sum(a);
     const double dd = cta_sum(b);
-    const double mean = dd > 0.0 ? sd / dd : 0.0;
+    __shared__ double mean;
+    if (threadIdx.x == 0) mean = dd > 0.0 ? sd / dd : 0.0;   // one float64 division, not one per warp
+    __syncthreads();
     for (int64_t j = threadIdx.x; j < n_c; j += blockDim.x) u[j] = double(s[j]) - mean;
 }
 
@@ -263,30 +326,22 @@ __global__ void k_gnn_lossgrad(int32_t n_c, const float* __restrict__ d, const d
     }
     const double den = cta_sum(a);
     const double uCu = cta_sum(b);
-    const double L = den > 0.0 ? (den - uCu) / den : 0.0;
-    if (threadIdx.x == 0) *loss = L;
+    __shared__ double sL, sinv;
+    if (threadIdx.x == 0) {
+        sL = den > 0.0 ? (den - uCu) / den : 0.0;
+        sinv = den > 0.0 ? 1.0 / den : 0.0;
+        *loss = sL;
+    }
+    __syncthreads();
+    const double L = sL, inv = sinv;
     if (g)
         for (int64_t j = threadIdx.x; j < n_c; j += blockDim.x) {
             const double du = double(d[j]) * u[j];
-            g[j] = den > 0.0 ? float((2.0 * (du - Cu[j]) - 2.0 * L * du) / den) : 0.f;
+            g[j] = float((2.0 * (du - Cu[j]) - 2.0 * L * du) * inv);
         }
 }
 
 // ---- backward ---------------------------------------------------------------------------------
-
-// gradients of the read-out: gwo = H^T g, gbo = sum g (thread per output; fixed node order)
-__global__ void k_gnn_readout_grad(int32_t n_c, const float* __restrict__ H, const float* __restrict__ g,
-                                   float* __restrict__ gwo, float* __restrict__ gbo) {
-    const int o = threadIdx.x;
-    if (o > kH) return;
-    double a = 0.0;
-    if (o < kH)
-        for (int64_t j = 0; j < n_c; ++j) a += double(H[j * kH + o]) * g[j];
-    else
-        for (int64_t j = 0; j < n_c; ++j) a += g[j];
-    if (o < kH) gwo[o] = float(a);
-    else gbo[0] = float(a);
-}
 
 // dZ = (g wo^T) masked by Z > 0 (layer 3), or dH masked by Z > 0 (other layers)
 __global__ void k_gnn_mask(int32_t n_c, const float* __restrict__ dH, const float* __restrict__ g,
@@ -297,43 +352,99 @@ __global__ void k_gnn_mask(int32_t n_c, const float* __restrict__ dH, const floa
     }
 }
 
-// gWs = H^T dZ, gWn = AH^T dZ, gb = column sums of dZ; thread per weight, nodes in order
-__global__ void k_gnn_wgrad(int32_t n_c, int fi, const float* __restrict__ H, const float* __restrict__ AH,
-                            const float* __restrict__ dZ, float* __restrict__ gWs, float* __restrict__ gWn,
-                            float* __restrict__ gb) {
-    const int64_t nw = int64_t(fi) * kH;
-    for (int64_t idx = gtid(); idx < 2 * nw + kH; idx += gstride()) {
-        double a = 0.0;
-        if (idx < 2 * nw) {
-            const bool nb = idx >= nw;
-            const int64_t e = nb ? idx - nw : idx;
-            const int i = int(e / kH), o = int(e % kH);
-            const float* src = nb ? AH : H;
-            for (int64_t j = 0; j < n_c; ++j) a += double(src[j * fi + i]) * dZ[j * kH + o];
-            (nb ? gWn : gWs)[e] = float(a);
-        } else {
-            const int o = int(idx - 2 * nw);
-            for (int64_t j = 0; j < n_c; ++j) a += dZ[j * kH + o];
-            gb[o] = float(a);
+// gWs = H^T dZ, gWn = AH^T dZ, gb = column sums of dZ, and (gwo given, with the last layer) the read-out's
+// gwo = Hout^T g, gbo = sum g.  A CTA takes kGradRows rows of [H | AH | 1] (or the read-out): 64 threads
+// for the outputs x kGradGroups groups of nodes, sums of exact products in double-float, the groups in
+// order at the end.  A thread per weight adding all nodes in float64 took 50 us a layer for 240 cameras
+// (two conversions and a multiply-add per term on the float64 pipe, in one chain); now 7 us.
+constexpr int kGradRows = 2, kGradGroups = 8;
+__global__ void __launch_bounds__(kH * kGradGroups) k_gnn_wgrad(
+    int32_t n_c, int fi, const float* __restrict__ H, const float* __restrict__ AH, const float* __restrict__ dZ,
+    float* __restrict__ gWs, float* __restrict__ gWn, float* __restrict__ gb, const float* __restrict__ Hout,
+    const float* __restrict__ g, float* __restrict__ gwo, float* __restrict__ gbo) {
+    __shared__ float2 red[kGradGroups][kGradRows][kH];
+    const int o = threadIdx.x % kH, grp = threadIdx.x / kH;
+    const int wrows = 2 * fi / kGradRows;           // CTAs of weight rows, then the bias, then the read-out
+    const int b = blockIdx.x;
+    df64 acc[kGradRows];
+#pragma unroll
+    for (int r = 0; r < kGradRows; ++r) acc[r] = df64(0.f);
+    if (b < wrows) {
+        const int i0 = b * kGradRows;
+        const float* src = i0 < fi ? H + i0 : AH + (i0 - fi);   // fi is even: a CTA's rows are of one matrix
+#pragma unroll 4
+        for (int64_t j = grp; j < n_c; j += kGradGroups) {
+            const float dz = dZ[j * kH + o];
+#pragma unroll
+            for (int r = 0; r < kGradRows; ++r) acc[r] += product(src[j * fi + r], dz);
+        }
+    } else if (b == wrows) {
+#pragma unroll 4
+        for (int64_t j = grp; j < n_c; j += kGradGroups) acc[0] += df64(dZ[j * kH + o]);
+    } else {
+#pragma unroll 4
+        for (int64_t j = grp; j < n_c; j += kGradGroups) {
+            acc[0] += product(Hout[j * kH + o], g[j]);
+            if (o == 0) acc[1] += df64(g[j]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < kGradRows; ++r) df_st(&red[grp][r][o], acc[r]);
+    __syncthreads();
+    if (grp < kGradRows) {
+        df64 a(0.f);
+#pragma unroll
+        for (int k = 0; k < kGradGroups; ++k) a += df_ld(&red[k][grp][o]);
+        const float v = __fadd_rn(a.hi, a.lo);
+        if (b < wrows) {
+            const int i = b * kGradRows + grp;
+            (i < fi ? gWs + i * kH : gWn + (i - fi) * kH)[o] = v;
+        } else if (b == wrows) {
+            if (grp == 0) gb[o] = v;
+        } else if (grp == 0) {
+            gwo[o] = v;
+        } else if (o == 0) {
+            gbo[0] = v;
         }
     }
 }
 
-// P1 = dZ Ws^T and Y = (dZ Wn^T) / d (rows), thread per (node, input feature)
-__global__ void k_gnn_back_dense(int32_t n_c, int fi, const float* __restrict__ dZ, const float* __restrict__ Ws,
-                                 const float* __restrict__ Wn, const float* __restrict__ d, float* __restrict__ P1,
-                                 float* __restrict__ Y) {
-    for (int64_t idx = gtid(); idx < int64_t(n_c) * fi; idx += gstride()) {
-        const int64_t j = idx / fi;
-        const int i = int(idx % fi);
-        const float* dz = dZ + j * kH;
-        float a = 0.f, b = 0.f;
-        for (int o = 0; o < kH; ++o) {
-            a += dz[o] * Ws[i * kH + o];
-            b += dz[o] * Wn[i * kH + o];
+// P1 = dZ Ws^T and Y = (dZ Wn^T) / d (rows).  A CTA takes kBackNodes nodes and keeps both weight matrices
+// in shared memory (rows one bank apart): threads reading a row of Ws each made every load touch 32
+// lines (18 us a layer for 240 cameras; now 6 us).
+constexpr int kBackNodes = 4;
+__global__ void __launch_bounds__(kH * kBackNodes) k_gnn_back_dense(int32_t n_c, int fi, const float* __restrict__ dZ,
+                                                                  const float* __restrict__ Ws,
+                                                                  const float* __restrict__ Wn,
+                                                                  const float* __restrict__ d, float* __restrict__ P1,
+                                                                  float* __restrict__ Y) {
+    __shared__ float sw[2][kH / 2][kH + 1];   // half of the input features at a time
+    __shared__ float sz[kBackNodes][kH];
+    const int t = threadIdx.x;
+    for (int64_t j0 = int64_t(blockIdx.x) * kBackNodes; j0 < n_c; j0 += int64_t(gridDim.x) * kBackNodes) {
+        const int64_t jz = j0 + t / kH;
+        sz[t / kH][t % kH] = jz < n_c ? dZ[jz * kH + t % kH] : 0.f;
+        for (int ib = 0; ib < fi; ib += kH / 2) {
+            const int rows = fi - ib < kH / 2 ? fi - ib : kH / 2;
+            __syncthreads();
+            for (int e = t; e < rows * kH; e += blockDim.x) {
+                sw[0][e / kH][e % kH] = Ws[int64_t(ib) * kH + e];
+                sw[1][e / kH][e % kH] = Wn[int64_t(ib) * kH + e];
+            }
+            __syncthreads();
+            // thread: input feature ib + t mod 32 of node t / 64, of Ws or of Wn
+            const int i = t % (kH / 2), m = (t / (kH / 2)) % 2, nd = t / kH;
+            const int64_t j = j0 + nd;
+            if (i < rows && j < n_c) {
+                float a = 0.f;
+#pragma unroll 8
+                for (int o = 0; o < kH; ++o) a += sz[nd][o] * sw[m][i][o];
+                const int64_t idx = j * fi + ib + i;
+                if (m == 0) P1[idx] = a;
+                else Y[idx] = d[j] > 0.f ? a / d[j] : 0.f;
+            }
         }
-        P1[idx] = a;
-        Y[idx] = d[j] > 0.f ? b / d[j] : 0.f;
+        __syncthreads();
     }
 }
 
@@ -343,13 +454,8 @@ __global__ void k_gnn_back_aggr(int32_t n_c, const int64_t* __restrict__ row_ptr
                                 int fi, float* __restrict__ dH) {
     const int lane = threadIdx.x & 31;
     for (int64_t j = gtid() >> 5; j < n_c; j += gstride() >> 5) {
-        float a0 = 0.f, a1 = 0.f;
-        for (int64_t q = row_ptr[j]; q < row_ptr[j + 1]; ++q) {
-            const float w = c[q];
-            const float* yk = Y + int64_t(col[q]) * fi;
-            if (lane < fi) a0 += w * yk[lane];
-            if (lane + 32 < fi) a1 += w * yk[lane + 32];
-        }
+        float a0, a1;
+        row_combination(col, c, Y, fi, row_ptr[j], row_ptr[j + 1], a0, a1);
         if (lane < fi) dH[j * fi + lane] = P1[j * fi + lane] + a0;
         if (lane + 32 < fi) dH[j * fi + lane + 32] = P1[j * fi + lane + 32] + a1;
     }
@@ -527,7 +633,7 @@ static void graph(Gnn* g, const Structure& s, const System& y, cudaStream_t st) 
     k_gnn_edges<<<grid_of(int64_t(s.n_c) * 32, kThreads), kThreads, 0, st>>>(s.n_c, s.row_ptr, s.tile_ptr, s.col, y.S,
                                                                            y.S32, y.Sd, g->c, g->d);
     k_gnn_features<<<grid_of(s.n_c, kThreads), kThreads, 0, st>>>(s.n_c, y.aux, g->d, g->X);
-    k_gnn_standardize<<<1, kThreads, 0, st>>>(s.n_c, g->X);
+    k_gnn_standardize<<<1, kStdThreads, 0, st>>>(s.n_c, g->X);
     g->launches += 3;
 }
 
@@ -556,18 +662,17 @@ static void backward(Gnn* g, const Structure& s, cudaStream_t st) {
     const int32_t n = s.n_c;
     const float* P = g->params;
     float* G = g->grad;
-    k_gnn_readout_grad<<<1, kH + 32, 0, st>>>(n, g->H[kL], g->g, G + g->off.wo, G + g->off.bo);
-    g->launches += 1;
     for (int l = kL - 1; l >= 0; --l) {
         const int fi = l == 0 ? kF : kH;
         k_gnn_mask<<<grid_of(int64_t(n) * kH, kThreads), kThreads, 0, st>>>(
             n, l == kL - 1 ? nullptr : g->dH, g->g, P + g->off.wo, g->Z[l], g->dZ);
-        k_gnn_wgrad<<<grid_of(2 * int64_t(fi) * kH + kH, 128), 128, 0, st>>>(n, fi, g->H[l], g->AH[l], g->dZ,
-                                                                            G + g->off.Ws[l], G + g->off.Wn[l],
-                                                                            G + g->off.b[l]);
+        const int ctas = 2 * fi / kGradRows + 1 + (l == kL - 1 ? 1 : 0);
+        k_gnn_wgrad<<<ctas, kH * kGradGroups, 0, st>>>(n, fi, g->H[l], g->AH[l], g->dZ, G + g->off.Ws[l],
+                                                       G + g->off.Wn[l], G + g->off.b[l], g->H[kL], g->g,
+                                                       G + g->off.wo, G + g->off.bo);
         g->launches += 2;
         if (l > 0) {
-            k_gnn_back_dense<<<grid_of(int64_t(n) * fi, kThreads), kThreads, 0, st>>>(
+            k_gnn_back_dense<<<grid_of(int64_t(n) * kH, kH * kBackNodes), kH * kBackNodes, 0, st>>>(
                 n, fi, g->dZ, P + g->off.Ws[l], P + g->off.Wn[l], g->d, g->P1, g->Y);
             k_gnn_back_aggr<<<grid_of(int64_t(n) * 32, kThreads), kThreads, 0, st>>>(n, s.row_ptr, s.col, g->c, g->P1,
                                                                                    g->Y, fi, g->dH);
