@@ -40,6 +40,7 @@
 #include <vector>
 
 #include "ba_internal.cuh"
+#include "df64.cuh"
 
 namespace ba {
 
@@ -1655,6 +1656,80 @@ __device__ __forceinline__ void inverse_sweeps(double (*sA)[kMaxDirs + 1], doubl
     if (in) sX[i][j] = sX[j][i] = -x;   // the sweeps leave -A^{-1}
 }
 
+constexpr int kSmallThreads = 1024;
+// The small solve of a step, by a CTA of 512 threads or more (all of them call it; the CTA's writes
+// to m.A, m.g and m.bad = 0 come before a barrier): alpha = Delta^+ gamma into c->alpha_v, gamma^T alpha
+// into c->ga, Delta^+ into m.X and (not null) Dp.
+struct SmallSolve {
+    double A[kMaxDirs][kMaxDirs + 1], V[kMaxDirs][kMaxDirs + 1], X[kMaxDirs][kMaxDirs + 1];
+    double g[kMaxDirs], al[kMaxDirs];
+    double tr;
+    int bad, ok;
+};
+__device__ void solve_block(Ctl* c, SmallSolve& m, int w, double* Dp) {
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    if (w == 1) {
+        if (Dp && t < kMaxDirs * kMaxDirs && t > 0) Dp[t] = 0.0;
+        if (t == 0) {
+            const double x = m.A[0][0] > 0.0 ? 1.0 / m.A[0][0] : 0.0, al = x * m.g[0], ga = m.g[0] * al;
+            if (Dp) Dp[0] = x;
+            m.X[0][0] = x;
+            c->alpha_v[0] = al;
+            c->ga = ga;
+            if (!(ga == ga)) { c->done = 1; c->status = BA_ERR_BREAKDOWN; }
+        }
+        return;
+    }
+    if (t < kInvThreads) {
+        inverse_sweeps(m.A, m.X, w, &m.bad);
+    } else if (wid == kInvThreads / 32) {
+        const double d = warp_sum(lane < w ? m.A[lane][lane] : 0.0);
+        if (lane == 0) m.tr = d;
+    }
+    __syncthreads();
+    // alpha = Delta^+ gamma (warp 0: two lanes per row) and gamma^T alpha, while warp 1 checks the
+    // certificate and the others store the inverse; once more after a pseudo-inverse
+    for (int pass = 0; pass < 2; ++pass) {
+        if (wid == 0) {
+            const int a = lane >> 1, b0 = (lane & 1) * (kMaxDirs / 2);
+            double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+            for (int b = 0; b < kMaxDirs / 2; b += 2) {
+                if (a < w && b0 + b < w) s0 += m.X[a][b0 + b] * m.g[b0 + b];
+                if (a < w && b0 + b + 1 < w) s1 += m.X[a][b0 + b + 1] * m.g[b0 + b + 1];
+            }
+            double s = s0 + s1;
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            if (a < w && !(lane & 1)) {
+                m.al[a] = s;
+                c->alpha_v[a] = s;
+            }
+            double ga = a < w ? m.g[a] * s : 0.0;
+#pragma unroll
+            for (int o = 2; o < 32; o <<= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
+            if (lane == 0) m.al[0] = ga;
+        } else if (wid == 1 && pass == 0) {
+            const double trinv = warp_sum(lane < w ? m.X[lane][lane] : 0.0);
+            // 1 / trace(A^{-1}) > 1e3 thr, i.e. 1e3 thr trace(A^{-1}) < 1 (false for a NaN)
+            const double thr = w * 2.220446049250313e-16 * m.tr;
+            if (lane == 0) m.ok = !m.bad && 1e3 * thr * trinv < 1.0;
+        } else if (Dp && wid >= 8 && wid < 16) {
+            const int e = t - 256, ei = e / kMaxDirs, ej = e % kMaxDirs;
+            Dp[e] = (ei < w && ej < w) ? m.X[ei][ej] : 0.0;
+        }
+        __syncthreads();
+        if (pass == 1 || m.ok) break;
+        pinv_sym_jacobi(m.A, m.V, m.X, w);
+        if (t == 0) c->pinv_steps += 1;
+        __syncthreads();
+    }
+    if (t == 0) {
+        const double ga = m.al[0];
+        c->ga = ga;
+        if (!(ga == ga)) { c->done = 1; c->status = BA_ERR_BREAKDOWN; }
+    }
+}
+
 // Distributed shared memory of a cluster: the same variable of CTA `rank`, and the cluster's barrier.
 __device__ __forceinline__ void store_remote(double* var, int rank, double v) {
     uint32_t a;
@@ -1671,7 +1746,6 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 // positive (A positive definite) and 1 / trace(A^{-1}) <= lambda_min exceeds 1e3 times the threshold
 // w 2^-52 trace(A) >= w 2^-52 lambda_max: no eigenvalue is dropped, so A^+ = A^{-1}.  Otherwise the
 // eigen-decomposition runs.  1000 cameras, w = 16: 20.5 us in one CTA with the longer inverse, now 12.4 us.
-constexpr int kSmallThreads = 1024;
 constexpr int kSmallCtas = 8;
 constexpr int kSmallGroups = 32;   // groups of threads that share the partials of an entry
 template <typename T>
@@ -1681,7 +1755,7 @@ __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThrea
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const int p = blockIdx.x / kSmallCtas, rank = blockIdx.x % kSmallCtas;
     Ctl* c = ctl + p;
-    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const int t = threadIdx.x;
     const bool done = c->done != 0;
     if (rank == 0 && t == 0) {
         c->live = !done;
@@ -1691,11 +1765,8 @@ __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThrea
         cluster_wait();
         return;
     }
-    __shared__ double sA[kMaxDirs][kMaxDirs + 1], sV[kMaxDirs][kMaxDirs + 1], sX[kMaxDirs][kMaxDirs + 1];
-    __shared__ double sg[kMaxDirs], sal[kMaxDirs];
+    __shared__ SmallSolve sm;
     __shared__ double st[kSmallThreads];
-    __shared__ double tr;
-    __shared__ int bad, ok;
     const int w = c->w_cur;
     const int it = c->it;
     const int ne = w * w + w;
@@ -1721,7 +1792,7 @@ __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThrea
                 }
             store_partial(&st[t], s);
         }
-        if (t == 0) bad = 0;
+        if (t == 0) sm.bad = 0;
         __syncthreads();
         cluster_wait();
         if (t < eb && e < ne) {   // here g = 0 and el = t
@@ -1733,72 +1804,13 @@ __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThrea
             }
             if (G & 1) load_partial(a, &st[(G - 1) * eb + t]);
             combine(a, b);
-            store_remote(e < w * w ? &sA[e / w][e % w] : &sg[e - w * w], 0, a.value());
+            store_remote(e < w * w ? &sm.A[e / w][e % w] : &sm.g[e - w * w], 0, a.value());
         }
         cluster_arrive();
         cluster_wait();
         if (rank != 0) return;
     }
-    double* Dp = dpinv + (int64_t(p) * mi1 + it) * kMaxDirs * kMaxDirs;
-    if (w == 1) {
-        if (t < kMaxDirs * kMaxDirs && t > 0) Dp[t] = 0.0;
-        if (t == 0) {
-            const double x = sA[0][0] > 0.0 ? 1.0 / sA[0][0] : 0.0, al = x * sg[0], ga = sg[0] * al;
-            Dp[0] = x;
-            c->alpha_v[0] = al;
-            c->ga = ga;
-            if (!(ga == ga)) { c->done = 1; c->status = BA_ERR_BREAKDOWN; }
-        }
-        return;
-    }
-    if (t < kInvThreads) {
-        inverse_sweeps(sA, sX, w, &bad);
-    } else if (wid == kInvThreads / 32) {
-        const double d = warp_sum(lane < w ? sA[lane][lane] : 0.0);
-        if (lane == 0) tr = d;
-    }
-    __syncthreads();
-    // alpha = Delta^+ gamma (warp 0: two lanes per row) and gamma^T alpha, while warp 1 checks the
-    // certificate and the others store the inverse; once more after a pseudo-inverse
-    for (int pass = 0; pass < 2; ++pass) {
-        if (wid == 0) {
-            const int a = lane >> 1, b0 = (lane & 1) * (kMaxDirs / 2);
-            double s0 = 0.0, s1 = 0.0;
-#pragma unroll
-            for (int b = 0; b < kMaxDirs / 2; b += 2) {
-                if (a < w && b0 + b < w) s0 += sX[a][b0 + b] * sg[b0 + b];
-                if (a < w && b0 + b + 1 < w) s1 += sX[a][b0 + b + 1] * sg[b0 + b + 1];
-            }
-            double s = s0 + s1;
-            s += __shfl_xor_sync(0xffffffffu, s, 1);
-            if (a < w && !(lane & 1)) {
-                sal[a] = s;
-                c->alpha_v[a] = s;
-            }
-            double ga = a < w ? sg[a] * s : 0.0;
-#pragma unroll
-            for (int o = 2; o < 32; o <<= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
-            if (lane == 0) sal[0] = ga;
-        } else if (wid == 1 && pass == 0) {
-            const double trinv = warp_sum(lane < w ? sX[lane][lane] : 0.0);
-            // 1 / trace(A^{-1}) > 1e3 thr, i.e. 1e3 thr trace(A^{-1}) < 1 (false for a NaN)
-            const double thr = w * 2.220446049250313e-16 * tr;
-            if (lane == 0) ok = !bad && 1e3 * thr * trinv < 1.0;
-        } else if (wid >= 8 && wid < 16) {
-            const int e = t - 256, ei = e / kMaxDirs, ej = e % kMaxDirs;
-            Dp[e] = (ei < w && ej < w) ? sX[ei][ej] : 0.0;
-        }
-        __syncthreads();
-        if (pass == 1 || ok) break;
-        pinv_sym_jacobi(sA, sV, sX, w);
-        if (t == 0) c->pinv_steps += 1;
-        __syncthreads();
-    }
-    if (t == 0) {
-        const double ga = sal[0];
-        c->ga = ga;
-        if (!(ga == ga)) { c->done = 1; c->status = BA_ERR_BREAKDOWN; }
-    }
+    solve_block(c, sm, w, dpinv + (int64_t(p) * mi1 + it) * kMaxDirs * kMaxDirs);
 }
 
 // x += P_i alpha; r -= Q_i alpha; z = D^{-1} r; per CTA the sums of |r|^2 and r^T z (dpart), from which
@@ -2266,6 +2278,428 @@ __global__ void __launch_bounds__(PqShape<T>::kSlices * 32, RL == 1 ? 2 : 1) k_m
 }
 
 // ---------------------------------------------------------------------------------------
+// A float32 sweep of a problem of at most kOneCams cameras in one CTA.
+//
+// Such a problem has no work for a chip: its iterations were 4 (PCG) or 9 (MCG) launches of 2.5 to 6 us
+// each.  Here a CTA runs the whole sweep between barriers, with S, the vectors and the current block in
+// shared memory.  The history stays in the problem's global arrays, which this kernel alone uses for it, in
+// tiles of 64 columns stored row by row (hist_at), so that threads on neighbouring columns read
+// neighbouring words.  It does what the kernels above do, step by step: exact-product sums in float
+// pairs, the float64 small solve, the same decide steps.  13 cameras, MCG: 25 -> 9 us per iteration.
+//
+// The rule: float32 sweeps of problems with nc <= kOneCams (S takes 324 nc^2 bytes: 130 KB of shared memory
+// at 20 cameras), whatever else is in the batch, so a problem's result does not depend on the others.
+// Larger problems run the kernels above; a handle whose tile waits give up at once (wait_polls = -1) does
+// too, since there is no tile wait here.
+constexpr int kOneCams = 20;
+constexpr int kOneRows = 9 * kOneCams;
+constexpr int kOneTile = 64;
+constexpr int kOneThreads = 512;   // solve_block uses as many; more would leave 64 registers a thread
+
+struct OneSmem {
+    Ctl c;
+    SmallSolve s;
+    // the current block and its image (one_at), zero past its width up to a multiple of four
+    __align__(16) float PT[kOneRows * kMaxDirs + 4 * kOneCams], QT[kOneRows * kMaxDirs + 4 * kOneCams];
+    float x[kOneRows], r[kOneRows], z[kOneRows];
+    double st[kOneThreads];
+    double tot[4];
+    float scal[2], al[kMaxDirs];
+};
+
+// Element (row i, column 0) of PT and QT: rows of 16, a camera's nine rows 20 banks after the last one's, so
+// that the 16-byte reads of four consecutive cameras fall on different banks.
+__device__ __forceinline__ int one_at(int i) { return kMaxDirs * i + 4 * (i / 9); }
+
+// element (row i, column c) of a history of n rows
+__device__ __forceinline__ int64_t hist_at(int n, int i, int c) {
+    return (int64_t(c / kOneTile) * n + i) * kOneTile + c % kOneTile;
+}
+
+// QT = S PT for the first w columns (S dense in shared memory, block (j, k) at 81 (nc j + k)).  Thread =
+// (three rows of a camera, quarter of the column cameras, group of NCOL = 4 columns, or the one column of
+// a global step); the quarters meet in shuffles.  Bound by shared-memory reads: a row of PT serves three
+// rows of S (one row per thread took 6.3k cycles for one column of 13 cameras, 12.3k for seven).
+template <int NCOL>
+__device__ __forceinline__ void one_product(const float* S, OneSmem& m, int nc, int w) {
+    const int tr = 3 * nc, total = 4 * tr * ((w + NCOL - 1) / NCOL), lane = threadIdx.x & 31;
+    for (int u = threadIdx.x; u - lane < total; u += kOneThreads) {   // whole warps, for the shuffles
+        const bool in = u < total;
+        const int quarter = u & 3, rg = u >> 2, g = rg / tr, trio = rg - tr * g;
+        const int j = trio / 3, a0 = 3 * (trio - 3 * j);
+        float acc[3][NCOL];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int cc = 0; cc < NCOL; ++cc) acc[a][cc] = 0.f;
+        for (int k = in ? quarter : nc; k < nc; k += 4) {
+            const float* b = S + (nc * j + k) * 81 + 9 * a0;
+            const float* pk = m.PT + one_at(9 * k) + NCOL * g;
+#pragma unroll
+            for (int e = 0; e < 9; ++e) {
+                float pv[NCOL];
+                if constexpr (NCOL == 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(pk + kMaxDirs * e);
+                    pv[0] = v.x, pv[1] = v.y, pv[2] = v.z, pv[3] = v.w;
+                } else {
+                    pv[0] = pk[kMaxDirs * e];
+                }
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+#pragma unroll
+                    for (int cc = 0; cc < NCOL; ++cc) acc[a][cc] = fmaf(b[9 * a + e], pv[cc], acc[a][cc]);
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int cc = 0; cc < NCOL; ++cc) {
+                acc[a][cc] += __shfl_xor_sync(0xffffffffu, acc[a][cc], 1);
+                acc[a][cc] += __shfl_xor_sync(0xffffffffu, acc[a][cc], 2);
+            }
+        if (in && quarter == 0) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int cc = 0; cc < NCOL; ++cc)
+                    m.QT[one_at(9 * j + a0 + a) + NCOL * g + cc] = NCOL * g + cc < w ? acc[a][cc] : 0.f;
+        }
+    }
+}
+
+// Sums of NV values over the rows (threads 0 .. kOneRows - 1 hold them, zeros past the problem), the
+// same in every thread.  Contains a barrier before and after the sums are read.
+template <int NV>
+__device__ __forceinline__ void one_sums(ExactSum<float> (&v)[NV], double* st) {
+    constexpr int NWR = (kOneRows + 31) / 32;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (wid < NWR) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            v[k] = warp_total(v[k]);
+            if (lane == 0) store_partial(&st[NV * wid + k], v[k]);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        ExactSum<float> a, b;
+        static_assert(NWR % 2 == 0, "pairs of warps");
+#pragma unroll
+        for (int q = 0; q < NWR; q += 2) {
+            load_partial(a, &st[NV * q + k]);
+            load_partial(b, &st[NV * (q + 1) + k]);
+        }
+        combine(a, b);
+        v[k] = a;
+    }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(kOneThreads, 1)
+    k_one_cta(int mcg, const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ tile_ptr,
+              const int32_t* __restrict__ col, const float* __restrict__ Sg, const double* __restrict__ Dinv,
+              float* __restrict__ xg, const float* __restrict__ rg, const float* __restrict__ zg, float* P, float* Q,
+              double* phip, double* dpinv, float* beta, int* __restrict__ colblk, double* __restrict__ hist,
+              int* blk_off, int* blk_w, int mi1, Ctl* ctl) {
+    const int p = blockIdx.x, t = threadIdx.x;
+    if (ctl[p].lay.nc > kOneCams || ctl[p].done) return;
+    extern __shared__ __align__(16) unsigned char smem_one[];
+    OneSmem& m = *reinterpret_cast<OneSmem*>(smem_one);
+    float* S = reinterpret_cast<float*>(smem_one + (sizeof(OneSmem) + 15) / 16 * 16);
+    const Layout L = ctl[p].lay;
+    const int nc = L.nc, n = 9 * nc, c0 = L.c0;
+    if (t == 0) m.c = ctl[p];
+    for (int u = t; u < nc * nc * 81; u += kOneThreads) S[u] = 0.f;
+    for (int u = t; u < kOneRows * kMaxDirs + 4 * kOneCams; u += kOneThreads) m.PT[u] = m.QT[u] = 0.f;
+    __syncthreads();
+    for (int j = 0; j < nc; ++j) {
+        const int64_t rj = row_ptr[c0 + j], base = tile_ptr[c0 + j] * kTile;
+        const int nj = int(row_ptr[c0 + j + 1] - rj);
+        for (int u = t; u < 81 * nj; u += kOneThreads) {
+            const int q = u / 81, e = u - 81 * q;
+            S[(nc * j + (col[rj + q] - c0)) * 81 + e] = Sg[(base + q) * 81 + e];
+        }
+    }
+    const bool act = t < n;
+    const int cam = t / 9, own_at = one_at(t);   // this thread's row of PT and QT
+    DinvRow<float> D;
+    D.load(Dinv + 9 * (9 * int64_t(c0) + t), act);
+    if (act) {
+        m.x[t] = 0.f;
+        m.r[t] = rg[9 * c0 + t];
+        m.PT[own_at] = m.z[t] = zg[9 * c0 + t];
+    }
+    float* Pp = P + L.hoff;
+    float* Qp = Q + L.hoff;
+    __syncthreads();
+    if (!mcg) {
+        // Algorithm 1: the direction p is column 0 of PT, q = S p column 0 of QT
+        while (true) {
+            one_product<1>(S, m, nc, 1);
+            __syncthreads();
+            ExactSum<float> d[2];
+            if (act) {
+                d[0].add(m.QT[own_at], m.PT[own_at]);
+                d[1].add(m.PT[own_at], m.r[t]);
+            }
+            one_sums<2>(d, m.st);
+            const float alpha = __fdiv_rn(__fadd_rn(d[1].hi, d[1].lo), __fadd_rn(d[0].hi, d[0].lo));
+            ExactSum<float> v[3];
+            float rv = 0.f, qv = 0.f;
+            if (act) {
+                qv = m.QT[own_at];
+                m.x[t] += alpha * m.PT[own_at];
+                rv = m.r[t] - alpha * qv;
+                m.r[t] = rv;
+                v[0].add(rv, rv);
+            }
+            __syncthreads();
+            float zs = 0.f;
+            if (act) {
+                zs = D.dot(m.r + 9 * cam);
+                v[1].add(qv, zs);
+                v[2].add(rv, zs);
+            }
+            one_sums<3>(v, m.st);
+            if (t == 0) m.scal[0] = float(v[1].value() * fast_rcp<2>(d[0].value()));
+            if (t == 32) {   // the stop test beside it
+                m.tot[0] = v[0].value();
+                m.tot[1] = v[1].value();
+                m.tot[2] = v[2].value();
+                pcg_decide(&m.c, d[0].value(), d[1].value(), m.tot, hist, p, gridDim.x);
+            }
+            __syncthreads();
+            if (m.c.done) break;
+            if (act) m.PT[own_at] = zs - m.scal[0] * m.PT[own_at];
+            __syncthreads();
+        }
+    } else {
+        const int n_eff = L.n_eff, sz = L.sz;
+        double* ph = phip + L.phoff;
+        float2* dp = reinterpret_cast<float2*>(dpinv) + int64_t(p) * mi1 * kMaxDirs * kMaxDirs;
+        float* bt = beta + L.boff * kMaxDirs;
+        int* cb = colblk + L.boff;
+        const int* bo = blk_off + int64_t(p) * mi1;
+        const int* bw = blk_w + int64_t(p) * mi1;
+        one_product<1>(S, m, nc, 1);   // Q_0 = S P_0
+        if (t == 0) cb[0] = 0;
+        __syncthreads();
+        if (act) {
+            Pp[hist_at(n, t, 0)] = m.PT[own_at];
+            Qp[hist_at(n, t, 0)] = m.QT[own_at];
+        }
+        while (true) {
+            const int w = m.c.w_cur, it = m.c.it, ne = w * w + w;
+            // Gram: groups of ne threads over the rows
+            {
+                const int G = min(kOneThreads / ne, 16), g = t / ne, e = t - ne * g;
+                if (t == 0) m.s.bad = 0;
+                if (g < G) {
+                    const int a = e < w * w ? e / w : e - w * w, b = e - w * a;
+                    ExactSum<float> s0, s1;
+                    for (int i = g; i < n; i += 2 * G) {
+                        const int i1 = i + G, o0 = one_at(i), o1 = one_at(i1);
+                        if (e < w * w) s0.add(m.QT[o0 + a], m.PT[o0 + b]);
+                        else s0.add(m.PT[o0 + a], m.r[i]);
+                        if (i1 < n) {
+                            if (e < w * w) s1.add(m.QT[o1 + a], m.PT[o1 + b]);
+                            else s1.add(m.PT[o1 + a], m.r[i1]);
+                        }
+                    }
+                    combine(s0, s1);
+                    store_partial(&m.st[t], s0);
+                }
+                __syncthreads();
+                if (t < ne) {
+                    ExactSum<float> s0, s1;
+                    for (int k = 0; k < G; k += 2) {
+                        load_partial(s0, &m.st[k * ne + t]);
+                        if (k + 1 < G) load_partial(s1, &m.st[(k + 1) * ne + t]);
+                    }
+                    combine(s0, s1);
+                    const double v = s0.value();
+                    if (t < w * w) m.s.A[t / w][t % w] = v;
+                    else m.s.g[t - w * w] = v;
+                }
+                __syncthreads();
+            }
+            solve_block(&m.c, m.s, w, nullptr);
+            __syncthreads();
+            if (t < kMaxDirs * kMaxDirs) {   // Delta^+ in double-float for the reorthogonalisation
+                const int a = t / kMaxDirs, b = t % kMaxDirs;
+                if (a < w && b < w) {
+                    const double v = m.s.X[a][b];
+                    const float h = __double2float_rn(v);
+                    dp[int64_t(it) * kMaxDirs * kMaxDirs + t] = make_float2(h, __double2float_rn(v - double(h)));
+                }
+            } else if (t < kMaxDirs * kMaxDirs + kMaxDirs) {
+                const int b = t - kMaxDirs * kMaxDirs;
+                m.al[b] = b < w ? float(m.c.alpha_v[b]) : 0.f;
+            }
+            __syncthreads();
+            // update
+            ExactSum<float> v[2];
+            if (act) {
+                float dx = 0.f, dr = 0.f;
+                for (int b = 0; b < w; ++b) {
+                    dx += m.PT[own_at + b] * m.al[b];
+                    dr += m.QT[own_at + b] * m.al[b];
+                }
+                m.x[t] += dx;
+                const float rv = m.r[t] - dr;
+                m.r[t] = rv;
+                v[0].add(rv, rv);
+            }
+            __syncthreads();
+            float zs = 0.f;
+            if (act) {
+                zs = D.dot(m.r + 9 * cam);
+                m.z[t] = zs;
+                v[1].add(m.r[t], zs);
+            }
+            one_sums<2>(v, m.st);
+            if (t == 0) {
+                m.tot[0] = v[0].value();
+                m.tot[1] = v[1].value();
+                m.c.hist_cols = m.c.cols;
+                mcg_decide(&m.c, m.tot, hist, blk_off, blk_w, mi1, p, gridDim.x);
+            }
+            __syncthreads();
+            if (m.c.done) break;
+            const int hc = m.c.hist_cols, wn = m.c.w_new, off = m.c.new_off;
+            const bool local = m.c.local != 0;
+            // Phi: column c of the history against z over subset s, slot s hc + c
+            for (int u = t; u < hc * n_eff; u += kOneThreads) {
+                const int s = u / hc, c = u - hc * s;
+                const int i0 = 9 * s * sz, i1 = min(9 * (s + 1) * sz, n);
+                const float* q = Qp + hist_at(n, 0, c);
+                ExactSum<float> a0, a1, a2;
+                for (int i = i0; i < i1; i += 9) {   // a camera's rows
+                    float qv[9];
+#pragma unroll
+                    for (int e = 0; e < 9; ++e) qv[e] = q[(i + e) * kOneTile];
+#pragma unroll
+                    for (int e = 0; e < 9; e += 3) {
+                        a0.add(qv[e], m.z[i + e]);
+                        a1.add(qv[e + 1], m.z[i + e + 1]);
+                        a2.add(qv[e + 2], m.z[i + e + 2]);
+                    }
+                }
+                combine(a0, a1);
+                combine(a0, a2);
+                store_partial(ph + u, a0);
+            }
+            __syncthreads();
+            if (!local) {   // a global step: over every subset, into the first one's slots
+                for (int c = t; c < hc; c += kOneThreads) {
+                    double v[kMaxDirs];
+#pragma unroll
+                    for (int s = 0; s < kMaxDirs; ++s) v[s] = s < n_eff ? ph[s * hc + c] : 0.0;
+                    ExactSum<float> a;
+#pragma unroll
+                    for (int s = 0; s < kMaxDirs; ++s)
+                        if (s < n_eff) add_slot(a, v[s]);
+                    store_partial(ph + c, a);
+                }
+                __syncthreads();
+            }
+            // beta = Delta_j^+ Phi_j, entry (column c, new column s), products in double-float
+            for (int u = t; u < hc * wn; u += kOneThreads) {
+                const int s = u / hc, c = u - hc * s, jb = cb[c], o = bo[jb], wj = bw[jb];
+                const float2* Dr = dp + (int64_t(jb) * kMaxDirs + (c - o)) * kMaxDirs;
+                const double* phs = ph + s * hc + o;
+                df64 acc(0.f);
+                for (int b0 = 0; b0 < wj; b0 += 8) {   // eight terms' loads in flight
+                    double v[8];
+                    float2 dv[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        v[e] = b0 + e < wj ? phs[b0 + e] : 0.0;
+                        dv[e] = b0 + e < wj ? Dr[b0 + e] : make_float2(0.f, 0.f);
+                    }
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        if (b0 + e < wj) {
+                            ExactSum<float> f;
+                            add_slot(f, v[e]);
+                            acc += df64(dv[e].x, dv[e].y) * df_fast_two_sum(f.hi, f.lo);
+                        }
+                }
+                bt[int64_t(c) * kMaxDirs + s] = __fadd_rn(acc.hi, acc.lo);
+            }
+            __syncthreads();
+            // P_new = Z - P_hist beta: thread = (three rows, four new columns, an eighth of every 32 columns)
+            {
+                const int tr = 3 * nc, total = 8 * tr * ((wn + 3) / 4);
+                for (int u = t; u - (t & 31) < total; u += kOneThreads) {   // whole warps, for the shuffles
+                    const bool in = u < total;
+                    const int part = u & 7, rg2 = u >> 3, g = rg2 / tr, i0 = 3 * (rg2 - tr * g);
+                    float acc[3][4];
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+#pragma unroll
+                        for (int cc = 0; cc < 4; ++cc) acc[a][cc] = 0.f;
+#pragma unroll 2
+                    for (int c = in ? 4 * part : hc; c < hc; c += 32) {
+                        // all seven loads in flight; P past hc is not used, beta past wn reaches sums that
+                        // are not used
+                        float4 pl[3], bl[4];
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) pl[a] = *reinterpret_cast<const float4*>(Pp + hist_at(n, i0 + a, c));
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            bl[e] = *reinterpret_cast<const float4*>(bt + int64_t(min(c + e, hc - 1)) * kMaxDirs + 4 * g);
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+                            const float pe[4] = {pl[a].x, c + 1 < hc ? pl[a].y : 0.f, c + 2 < hc ? pl[a].z : 0.f,
+                                                 c + 3 < hc ? pl[a].w : 0.f};
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                acc[a][0] = fmaf(pe[e], bl[e].x, acc[a][0]);
+                                acc[a][1] = fmaf(pe[e], bl[e].y, acc[a][1]);
+                                acc[a][2] = fmaf(pe[e], bl[e].z, acc[a][2]);
+                                acc[a][3] = fmaf(pe[e], bl[e].w, acc[a][3]);
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+#pragma unroll
+                        for (int cc = 0; cc < 4; ++cc)
+#pragma unroll
+                            for (int o = 1; o < 8; o <<= 1) acc[a][cc] += __shfl_xor_sync(0xffffffffu, acc[a][cc], o);
+                    if (in && part < 3) {   // three lanes store a row each
+                        const int i = i0 + part, own = local ? (i / 9) / sz : 0;
+#pragma unroll
+                        for (int cc = 0; cc < 4; ++cc) {
+                            const int s = 4 * g + cc;
+                            const float v = part == 0 ? acc[0][cc] : (part == 1 ? acc[1][cc] : acc[2][cc]);
+                            m.PT[one_at(i) + s] = s < wn ? (s == own ? m.z[i] : 0.f) - v : 0.f;
+                        }
+                    }
+                }
+            }
+            for (int u = t; u < wn; u += kOneThreads) cb[off + u] = it + 1;
+            __syncthreads();
+            if (wn == 1) one_product<1>(S, m, nc, 1);
+            else one_product<4>(S, m, nc, wn);
+            __syncthreads();
+            for (int u = t; u < n * wn; u += kOneThreads) {
+                const int i = u / wn, s = u - wn * i;
+                const int64_t o = hist_at(n, i, off + s);
+                Pp[o] = m.PT[one_at(i) + s];
+                Qp[o] = m.QT[one_at(i) + s];
+            }
+            __syncthreads();
+        }
+    }
+    if (act) xg[9 * c0 + t] = m.x[t];
+    if (t == 0) ctl[p] = m.c;
+}
+constexpr size_t one_smem(int nc) { return (sizeof(OneSmem) + 15) / 16 * 16 + sizeof(float) * 81 * size_t(nc) * nc; }
+
+// ---------------------------------------------------------------------------------------
 // true residual t = -b~ - S x in float64; partial[2 j], partial[2 j + 1] = camera j's sums of
 // t^2 and b~^2 (one warp per camera, all problems)
 
@@ -2448,12 +2882,13 @@ __global__ void k_refine_after(const Ctl* __restrict__ ctl, Outer* outer, const 
 // loop body, work lists, wait bound and every buffer address (a reallocation bumps `allocs`).
 struct GraphKey {
     int mcg = -1, fp32 = -1, chunk = 0, mi1 = 0, use_l = -1, epoch = -1, polls = -1, nb = -1, host = -1, cfg = -1;
+    int one = -1;                     // cameras of the largest problem that one CTA solves
     uint64_t allocs = ~uint64_t(0);   // buffer generation (any reallocation invalidates the graph)
     const void* ptrs[4] = {};
     bool operator==(const GraphKey& o) const {
         if (mcg != o.mcg || fp32 != o.fp32 || chunk != o.chunk || mi1 != o.mi1 || use_l != o.use_l ||
             epoch != o.epoch || polls != o.polls || nb != o.nb || host != o.host || cfg != o.cfg ||
-            allocs != o.allocs)
+            one != o.one || allocs != o.allocs)
             return false;
         for (int i = 0; i < 4; ++i) if (ptrs[i] != o.ptrs[i]) return false;
         return true;
@@ -2487,9 +2922,10 @@ struct Solver {
     int gq = 1;               // grid width of the per-row kernels
     int gpq = 1;              // grid width of the reorthogonalisation (32-row blocks)
     int gphi = 1, gb = 1;     // Phi and beta grid widths
+    int one_cams = 0;         // cameras of the largest problem that k_one_cta solves (0: none)
     int gcol = 1;             // grid width of the column pass of the symmetric product (a CTA per camera)
     std::vector<Layout> lay;  // of the current solve
-    Buf P, Q, r, z, xw, PT, part_a, part_b, part_cam, dpinv, beta, phip, hist, blk_off, blk_w, ctl, outer, rt,
+    Buf P, Q, r, z, xw, PT, part_a, part_b, part_cam, dpinv, beta, colblk, phip, hist, blk_off, blk_w, ctl, outer, rt,
         lay_d, dpart, dtot, camdot, params, loops;
     Ctl* h_ctl = nullptr;     // pinned, nb
     Outer* h_outer = nullptr; // pinned, nb
@@ -2690,6 +3126,7 @@ static void set_smem_attrs() {
     set_spmv_attrs<1>();
     set_spmv_attrs<2>();
     BA_CUDA_TRY(cudaFuncSetAttribute(k_spmm<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(spmm_smem<float>())));
+    BA_CUDA_TRY(cudaFuncSetAttribute(k_one_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, int(one_smem(kOneCams))));
     done = true;
 }
 
@@ -2763,7 +3200,9 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
         L.hoff = hoff;
         L.phoff = phoff;
         L.boff = boff;
-        hoff += cap * 9 * int64_t(L.nc);
+        // (a problem that one CTA solves keeps its history in whole tiles of columns; 16-byte aligned)
+        const int64_t cols = fp32 && L.nc <= kOneCams ? (cap + kOneTile - 1) / kOneTile * kOneTile : cap;
+        hoff += (cols * 9 * int64_t(L.nc) + 3) / 4 * 4;
         phoff += cap * L.n_eff * L.K;
         boff += cap;
     }
@@ -2807,6 +3246,11 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     grow(w->dpinv, size_t(nb) * w->mi1 * kMaxDirs * kMaxDirs * sizeof(double));
     grow(w->beta, size_t(boff) * kMaxDirs * sizeof(double));
     grow(w->phip, size_t(phoff) * sizeof(double));
+    w->one_cams = 0;   // float32: the largest problem that one CTA solves
+    if (fp32 && a.wait_polls > 0)
+        for (const Layout& L : lay)
+            if (L.nc <= kOneCams) w->one_cams = std::max(w->one_cams, L.nc);
+    if (w->one_cams > 0) grow(w->colblk, size_t(boff) * sizeof(int));
     grow(w->hist, size_t(nb) * w->mi1 * sizeof(double));
     grow(w->blk_off, size_t(nb) * w->mi1 * sizeof(int));
     grow(w->blk_w, size_t(nb) * w->mi1 * sizeof(int));
@@ -2846,7 +3290,7 @@ Solver* solver_create() { return new Solver(); }
 void solver_destroy(Solver* w) {
     if (!w) return;
     Buf* bufs[] = {&w->P, &w->Q, &w->r, &w->z, &w->xw, &w->PT, &w->part_a, &w->part_b, &w->part_cam, &w->dpinv,
-                   &w->beta, &w->phip, &w->hist, &w->blk_off, &w->blk_w, &w->ctl, &w->outer, &w->rt,
+                   &w->beta, &w->colblk, &w->phip, &w->hist, &w->blk_off, &w->blk_w, &w->ctl, &w->outer, &w->rt,
                    &w->lay_d, &w->dpart, &w->dtot, &w->camdot, &w->params, &w->loops};
     for (Buf* b : bufs) free_buf(*b);
     for (SolveExec* e : w->execs) {
@@ -3011,6 +3455,16 @@ static int krylov_init(Solver* w, const Structure& s, const T* S, const T* Su, c
     return 2 + (q0 ? enqueue_product<T, 0>(w, s, S, Su, ptr<T>(w->P), kSelLive, ptr<T>(w->Q), nullptr, st) : 0);
 }
 
+// The sweeps of the problems that one CTA solves, right after krylov_init; returns the launches.
+static int enqueue_one_cta(Solver* w, const Structure& s, const System& y, bool mcg, cudaStream_t st) {
+    if (w->one_cams == 0) return 0;
+    k_one_cta<<<w->nb, kOneThreads, one_smem(w->one_cams), st>>>(
+        mcg, s.row_ptr, s.tile_ptr, s.col, y.S32, y.Dhat, ptr<float>(w->xw), ptr<float>(w->r), ptr<float>(w->z),
+        ptr<float>(w->P), ptr<float>(w->Q), ptr<double>(w->phip), ptr<double>(w->dpinv), ptr<float>(w->beta),
+        ptr<int>(w->colblk), ptr<double>(w->hist), ptr<int>(w->blk_off), ptr<int>(w->blk_w), w->mi1, ptr<Ctl>(w->ctl));
+    return 1;
+}
+
 // true residual t = -b~ - S x into out (may be null) and, per problem, its norms into ctl (true_rr,
 // bb): explicit tiled S in float64 precision, the implicit operator (double-float arithmetic) in mixed precision.
 static int true_residual(Solver* w, const Structure& s, const System& y, const double* x, double* out,
@@ -3062,11 +3516,12 @@ static cudaGraphConditionalHandle capture_handle(cudaStream_t cs) {
 // chunk iterations; loop condition } on the body stream cb.
 // Sets *pre (launches before the loop) and *per_pass (launches per pass of the loop).
 template <typename T>
-static void capture_krylov(Solver* w, const Structure& s, const T* S, const T* Su, const double* Dinv,
+static void capture_krylov(Solver* w, const Structure& s, const System& y, const T* S, const T* Su, const double* Dinv,
                            const double* rhs, double sign, const double* scale, T* x, const Outer* outer, bool mcg,
                            int chunk, cudaStream_t cs, cudaStream_t cb, int* pre, int* per_pass) {
     const cudaGraphConditionalHandle h = capture_handle(cs);
     *pre = krylov_init<T>(w, s, S, Su, Dinv, rhs, sign, scale, x, outer, cs, mcg) + 1;
+    if (sizeof(T) == 4) *pre += enqueue_one_cta(w, s, y, mcg, cs);
     k_loop_cond<<<1, kThreads, 0, cs>>>(h, 1, ptr<Ctl>(w->ctl), w->nb, ptr<Loops>(w->loops), 1, chunk,
                                         ptr<Params>(w->params));
     cudaGraph_t body = capture_while(cs, h);
@@ -3096,7 +3551,7 @@ static cudaGraphExec_t build_solve_graph(Solver* w, const Structure& s, const Sy
     BA_CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     try {
         if (!fp32) {
-            capture_krylov<double>(w, s, y.S, nullptr, y.Dinv, y.bt, -1.0, nullptr, x, nullptr, mcg, a.chunk, cs,
+            capture_krylov<double>(w, s, y, y.S, nullptr, y.Dinv, y.bt, -1.0, nullptr, x, nullptr, mcg, a.chunk, cs,
                                    w->cap2, &gc.pre, &gc.body);
             gc.post = true_residual(w, s, y, x, nullptr, cs);
         } else {
@@ -3110,7 +3565,7 @@ static cudaGraphExec_t build_solve_graph(Solver* w, const Structure& s, const Sy
             cudaStream_t c2 = w->cap2;
             BA_CUDA_TRY(cudaStreamBeginCaptureToGraph(c2, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
             int kpre = 0;
-            capture_krylov<float>(w, s, y.S32, y.S32u, y.Dhat, ptr<double>(w->rt), 1.0, y.lam, ptr<float>(w->xw),
+            capture_krylov<float>(w, s, y, y.S32, y.S32u, y.Dhat, ptr<double>(w->rt), 1.0, y.lam, ptr<float>(w->xw),
                                   ptr<Outer>(w->outer), mcg, a.chunk, c2, w->cap3, &kpre, &gc.body);
             k_accumulate<<<dim3(w->gx, nb), kThreads, 0, c2>>>(ptr<Layout>(w->lay_d), ptr<Outer>(w->outer),
                                                                ptr<float>(w->xw), y.lam, x, y.xd);
@@ -3212,6 +3667,7 @@ static void run_host_loops(Solver* w, const Structure& s, const System& y, const
             if (!any) break;
             launches += krylov_init<float>(w, s, y.S32, y.S32u, y.Dhat, ptr<double>(w->rt), 1.0, y.lam,
                                            ptr<float>(w->xw), ptr<Outer>(w->outer), st, a.mcg != 0);
+            launches += enqueue_one_cta(w, s, y, a.mcg != 0, st);
             k_loop_cond<<<1, kThreads, 0, st>>>(none, 0, ptr<Ctl>(w->ctl), nb, lp, 1, a.chunk, prm);
             launches += 1 + host_krylov_loop(w, chunk_exec, gc, a, st, waits);
             k_accumulate<<<dim3(w->gx, nb), kThreads, 0, st>>>(ptr<Layout>(w->lay_d), ptr<Outer>(w->outer),
@@ -3242,6 +3698,7 @@ static cudaGraphExec_t solve_graph(Solver* w, const Structure& s, const System& 
     key.nb = w->nb;
     key.host = a.host_loop;
     key.cfg = a.spmv_cfg;
+    key.one = w->one_cams;
     key.allocs = g_allocs.load();
     const void* ptrs[4] = {x, fp32 ? (const void*)y.S32 : (const void*)y.S, w->items_g.items, w->items_l.items};
     for (int i = 0; i < 4; ++i) key.ptrs[i] = ptrs[i];
