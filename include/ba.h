@@ -87,8 +87,8 @@ typedef struct ba_options {
     int32_t max_refine;        /* MIXED: maximum outer refinement sweeps (default 64) */
     int32_t item_blocks;       /* stored 9x9 blocks of S per work item of the block-sparse products
                                   (longer rows are split): 0 (default) = 512, or 256 below 1200
-                                  (float64: 800) cameras; else a multiple of 32 in [32, 4096];
-                                  ba_autotune sets it */
+                                  cameras (float64: 256 below 800, 128 below 450, 64 below 200);
+                                  else a multiple of 32 in [32, 4096]; ba_autotune sets it */
     int32_t wait_polls;        /* bounded device waits: polls of a tile copy's barrier before the
                                   solve gives up with BA_ERR_TIMEOUT (the kernel then waits for its
                                   own copies still in flight, with the default bound, and returns).

@@ -2974,15 +2974,21 @@ static T* ptr(const Buf& b) {
     return static_cast<T*>(b.p);
 }
 
-// Default blocks per work item: 16 tiles, and 8 for problems whose rows are too few to keep every warp
+// Default blocks per work item: 16 tiles, and fewer for problems whose rows are too few to keep every warp
 // busy with 16 (the longest item then sets the time).  Rows up to that length are one item; longer
 // rows are split, and the row's pieces combined by the last one to finish.  The rule depends on the
 // problem's own camera count alone, so its products sum in the same order alone and in any batch.
 // Measured on GB300, product at 512 / 256 blocks: float32 601 cameras 33.8 / 26.0 us (the solves 16 %
 // faster), 1000 cameras 43.4 / 41.9 us, 1936 cameras 118.1 / 119.1 us (MCG 2.5 % slower); float64 601
-// cameras 82.0 / 71.1 us, 1000 cameras 166 / 174 us.  64 and 128 blocks suit single problems of
-// 150 .. 300 cameras (up to 25 % of a product) and cost a batch of such problems as much.
-static int default_item_blocks(int n_cams, bool fp32) { return n_cams < (fp32 ? 1200 : 800) ? 256 : 512; }
+// cameras 82.0 / 71.1 us, 1000 cameras 166 / 174 us.  Float64 below that, at 256 / 128 / 64 blocks: 300
+// cameras 46.8 / 33.3 / 41.3 us, 150 cameras 30.9 / 28.7 / 20.9 us (a float64 tile takes about 3 us, so a
+// row in one warp is a long chain); a float64 batch of 48 problems of 100 to 400 cameras pays for it
+// (530 / 580 / 697 us).  Float32 keeps 256 there: 128 gains 14 % of a PCG solve at 300 cameras and
+// nothing at 150, and costs a batch 5 %.
+static int default_item_blocks(int n_cams, bool fp32) {
+    if (fp32) return n_cams < 1200 ? 256 : 512;
+    return n_cams < 200 ? 64 : (n_cams < 450 ? 128 : (n_cams < 800 ? 256 : 512));
+}
 
 // Items of the block-sparse product, problem by problem: each (row, segment) split into chunks of
 // at most cb blocks (cb = forced_cb, else default_item_blocks).
