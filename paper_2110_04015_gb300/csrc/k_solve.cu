@@ -1319,14 +1319,14 @@ __global__ void __launch_bounds__(kUpdThreads) k_pcg_update(const double* __rest
     }
 }
 
-// stop test for problem p (one thread); hist is iteration-major (it x nb)
+// stop test for problem p (one thread); hist is iteration-major (it x nb), null: not written
 __device__ void pcg_decide(Ctl* c, double D, double g, const double* tot, double* hist, int p, int nb) {
     if (c->status == BA_ERR_TIMEOUT) { c->done = 1; return; }
     const double rr = tot[0];
     const int it = c->it + 1;
     c->it = it;
     c->rr = rr;
-    hist[int64_t(c->hist_off + it - 1) * nb + p] = rr * c->rr0_inv * c->hist_scale;   // squared relative residual
+    if (hist) hist[int64_t(c->hist_off + it - 1) * nb + p] = rr * c->rr0_inv * c->hist_scale;   // squared relative residual
     if (!(D > 0.0) || !(rr == rr) || isinf(rr)) {
         c->done = 1;
         c->status = BA_ERR_BREAKDOWN;
@@ -2700,6 +2700,143 @@ __global__ void __launch_bounds__(kOneThreads, 1)
 constexpr size_t one_smem(int nc) { return (sizeof(OneSmem) + 15) / 16 * 16 + sizeof(float) * 81 * size_t(nc) * nc; }
 
 // ---------------------------------------------------------------------------------------
+// A float64 PCG solve of a problem of at most kCluCams cameras in one cluster of 8 CTAs.
+//
+// As for k_one_cta, an iteration of three launches had almost no work in it (16 cameras: 15 us).  In float64
+// one SM would still need 6 us for the product of 16 cameras (its pipe does 1.7 lanes a clock), so the
+// cameras go round a cluster's CTAs (camera j to CTA j mod 8), each with its rows of S in shared memory; the
+// rows' vectors live in the registers of its first warp, and the CTAs exchange the sums and the direction
+// through distributed shared memory, three cluster barriers per iteration (16 cameras: 6 us).  The rule is
+// the camera count alone, as for k_one_cta, and so is the exception (wait_polls = -1).
+constexpr int kCluCams = 24;
+constexpr int kCluThreads = 256;
+constexpr int kCluOwn = kCluCams / kSmallCtas;   // cameras of a CTA, 27 rows: one warp
+static_assert(9 * kCluOwn <= 32 && kCluCams % kSmallCtas == 0, "a CTA's rows in one warp");
+
+__global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kCluThreads)
+    k_pcg_cluster(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ tile_ptr,
+                  const int32_t* __restrict__ col, const double* __restrict__ Sg, const double* __restrict__ Dinv,
+                  double* __restrict__ xg, const double* __restrict__ rg, const double* __restrict__ zg,
+                  double* __restrict__ hist, Ctl* ctl) {
+    cluster_arrive();   // waited for before the first store to another CTA: every CTA has started by then
+    const int p = blockIdx.x / kSmallCtas, rank = blockIdx.x % kSmallCtas;
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    if (ctl[p].lay.nc > kCluCams || ctl[p].done) {   // the same in every CTA: the first one writes ctl after barriers
+        cluster_wait();
+        return;
+    }
+    extern __shared__ double S[];   // own camera m, column camera k: block at 81 (nc m + k)
+    __shared__ Ctl sc;
+    __shared__ double sp[9 * kCluCams], sq[9 * kCluOwn], dots[kSmallCtas][2], sums[kSmallCtas][3], tot[3];
+    __shared__ int stop;
+    const Layout L = ctl[p].lay;
+    const int nc = L.nc, c0 = L.c0, own = rank < nc ? (nc - rank + kSmallCtas - 1) / kSmallCtas : 0;
+    if (t == 0) sc = ctl[p];
+    for (int u = t; u < own * nc * 81; u += kCluThreads) S[u] = 0.0;
+    for (int u = t; u < 9 * nc; u += kCluThreads) sp[u] = zg[9 * c0 + u];
+    __syncthreads();
+    for (int m = 0; m < own; ++m) {
+        const int j = c0 + rank + kSmallCtas * m;
+        const int64_t rj = row_ptr[j], base = tile_ptr[j] * kTile;
+        const int nj = int(row_ptr[j + 1] - rj);
+        for (int u = t; u < 81 * nj; u += kCluThreads) {
+            const int q = u / 81, e = u - 81 * q;
+            S[(nc * m + (col[rj + q] - c0)) * 81 + e] = Sg[(base + q) * 81 + e];
+        }
+    }
+    // the first warp's lanes hold the CTA's rows
+    const int m = lane / 9, a = lane - 9 * m, j = rank + kSmallCtas * m;
+    const bool act = wid == 0 && m < own;
+    const int64_t gi = 9 * int64_t(c0 + j) + a;
+    DinvRow<double> D;
+    D.load(Dinv + 9 * gi, act);
+    double x = 0.0, r = act ? rg[gi] : 0.0, pv = act ? zg[gi] : 0.0;
+    // the product's threads: row ru of the CTA, column cameras part, part + 8, ...
+    const int ru = t >> 3, part = t & 7;
+    const bool in = ru < 9 * own;
+    const double* Srow = S + (nc * (in ? ru / 9 : 0)) * 81 + 9 * (ru % 9);
+    __syncthreads();
+    cluster_wait();
+    while (true) {
+        double s3[3] = {0.0, 0.0, 0.0};
+        if (in)
+            for (int k = part; k < nc; k += 8)
+#pragma unroll
+                for (int b = 0; b < 9; ++b) s3[b % 3] += Srow[81 * k + b] * sp[9 * k + b];
+        double s = (s3[0] + s3[1]) + s3[2];
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (in && part == 0) sq[ru] = s;
+        __syncthreads();
+        double q = 0.0, rD = 0.0, Delta = 0.0, gamma = 0.0, zs = 0.0;
+        if (wid == 0) {
+            q = act ? sq[lane] : 0.0;
+            const double d = warp_sum(q * pv), g = warp_sum(pv * r);
+            if (lane < kSmallCtas) {
+                store_remote(&dots[rank][0], lane, d);
+                store_remote(&dots[rank][1], lane, g);
+            }
+        }
+        cluster_arrive();
+        cluster_wait();
+        if (wid == 0) {
+            Delta = lane < kSmallCtas ? dots[lane][0] : 0.0;
+            gamma = lane < kSmallCtas ? dots[lane][1] : 0.0;
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) {
+                Delta += __shfl_xor_sync(0xffffffffu, Delta, o);
+                gamma += __shfl_xor_sync(0xffffffffu, gamma, o);
+            }
+            Delta = __shfl_sync(0xffffffffu, Delta, 0);
+            gamma = __shfl_sync(0xffffffffu, gamma, 0);
+            rD = fast_rcp<2>(Delta);
+            const double alpha = gamma * rD;
+            x += alpha * pv;
+            r -= alpha * q;
+            double rb[9];
+#pragma unroll
+            for (int b = 0; b < 9; ++b) rb[b] = __shfl_sync(0xffffffffu, r, (9 * m + b) & 31);
+            zs = act ? D.dot(rb) : 0.0;
+            const double v0 = warp_sum(r * r), v1 = warp_sum(q * zs), v2 = warp_sum(r * zs);
+            if (lane < kSmallCtas) {
+                store_remote(&sums[rank][0], lane, v0);
+                store_remote(&sums[rank][1], lane, v1);
+                store_remote(&sums[rank][2], lane, v2);
+            }
+        }
+        cluster_arrive();
+        cluster_wait();
+        if (wid == 0) {
+            double v[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) v[k] = lane < kSmallCtas ? sums[lane][k] : 0.0;
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+            const double beta = __shfl_sync(0xffffffffu, v[1], 0) * rD;
+            pv = zs - beta * pv;
+            if (act)
+#pragma unroll
+                for (int dst = 0; dst < kSmallCtas; ++dst) store_remote(&sp[9 * j + a], dst, pv);
+            if (lane == 0) {   // every CTA takes the same decision; the first one records it
+#pragma unroll
+                for (int k = 0; k < 3; ++k) tot[k] = v[k];
+                pcg_decide(&sc, Delta, gamma, tot, rank == 0 ? hist : nullptr, p, int(gridDim.x) / kSmallCtas);
+                stop = sc.done;
+            }
+            __syncwarp();
+        }
+        cluster_arrive();
+        cluster_wait();
+        if (stop) break;
+    }
+    if (act) xg[gi] = x;
+    if (rank == 0 && t == 0) ctl[p] = sc;
+}
+constexpr size_t clu_smem(int nc) { return sizeof(double) * 81 * size_t(nc) * ((nc + kSmallCtas - 1) / kSmallCtas); }
+
+// ---------------------------------------------------------------------------------------
 // true residual t = -b~ - S x in float64; partial[2 j], partial[2 j + 1] = camera j's sums of
 // t^2 and b~^2 (one warp per camera, all problems)
 
@@ -2882,7 +3019,7 @@ __global__ void k_refine_after(const Ctl* __restrict__ ctl, Outer* outer, const 
 // loop body, work lists, wait bound and every buffer address (a reallocation bumps `allocs`).
 struct GraphKey {
     int mcg = -1, fp32 = -1, chunk = 0, mi1 = 0, use_l = -1, epoch = -1, polls = -1, nb = -1, host = -1, cfg = -1;
-    int one = -1;                     // cameras of the largest problem that one CTA solves
+    int one = -1;                     // cameras of the largest problem that one CTA or cluster solves
     uint64_t allocs = ~uint64_t(0);   // buffer generation (any reallocation invalidates the graph)
     const void* ptrs[4] = {};
     bool operator==(const GraphKey& o) const {
@@ -2922,7 +3059,7 @@ struct Solver {
     int gq = 1;               // grid width of the per-row kernels
     int gpq = 1;              // grid width of the reorthogonalisation (32-row blocks)
     int gphi = 1, gb = 1;     // Phi and beta grid widths
-    int one_cams = 0;         // cameras of the largest problem that k_one_cta solves (0: none)
+    int one_cams = 0;         // cameras of the largest problem that k_one_cta or k_pcg_cluster solves (0: none)
     int gcol = 1;             // grid width of the column pass of the symmetric product (a CTA per camera)
     std::vector<Layout> lay;  // of the current solve
     Buf P, Q, r, z, xw, PT, part_a, part_b, part_cam, dpinv, beta, colblk, phip, hist, blk_off, blk_w, ctl, outer, rt,
@@ -3133,6 +3270,7 @@ static void set_smem_attrs() {
     set_spmv_attrs<2>();
     BA_CUDA_TRY(cudaFuncSetAttribute(k_spmm<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(spmm_smem<float>())));
     BA_CUDA_TRY(cudaFuncSetAttribute(k_one_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, int(one_smem(kOneCams))));
+    BA_CUDA_TRY(cudaFuncSetAttribute(k_pcg_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, int(clu_smem(kCluCams))));
     done = true;
 }
 
@@ -3252,11 +3390,13 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     grow(w->dpinv, size_t(nb) * w->mi1 * kMaxDirs * kMaxDirs * sizeof(double));
     grow(w->beta, size_t(boff) * kMaxDirs * sizeof(double));
     grow(w->phip, size_t(phoff) * sizeof(double));
-    w->one_cams = 0;   // float32: the largest problem that one CTA solves
-    if (fp32 && a.wait_polls > 0)
+    // the largest problem that k_one_cta (float32) or k_pcg_cluster (float64 PCG) solves
+    w->one_cams = 0;
+    const int small = fp32 ? kOneCams : (a.mcg ? 0 : kCluCams);
+    if (a.wait_polls > 0)
         for (const Layout& L : lay)
-            if (L.nc <= kOneCams) w->one_cams = std::max(w->one_cams, L.nc);
-    if (w->one_cams > 0) grow(w->colblk, size_t(boff) * sizeof(int));
+            if (L.nc <= small) w->one_cams = std::max(w->one_cams, L.nc);
+    if (fp32 && w->one_cams > 0) grow(w->colblk, size_t(boff) * sizeof(int));
     grow(w->hist, size_t(nb) * w->mi1 * sizeof(double));
     grow(w->blk_off, size_t(nb) * w->mi1 * sizeof(int));
     grow(w->blk_w, size_t(nb) * w->mi1 * sizeof(int));
@@ -3461,9 +3601,16 @@ static int krylov_init(Solver* w, const Structure& s, const T* S, const T* Su, c
     return 2 + (q0 ? enqueue_product<T, 0>(w, s, S, Su, ptr<T>(w->P), kSelLive, ptr<T>(w->Q), nullptr, st) : 0);
 }
 
-// The sweeps of the problems that one CTA solves, right after krylov_init; returns the launches.
-static int enqueue_one_cta(Solver* w, const Structure& s, const System& y, bool mcg, cudaStream_t st) {
+// The solves of the problems that one CTA or one cluster solves, right after krylov_init (x: the float64
+// solution); returns the launches.
+static int enqueue_small(Solver* w, const Structure& s, const System& y, bool mcg, double* x, cudaStream_t st) {
     if (w->one_cams == 0) return 0;
+    if (y.S) {
+        k_pcg_cluster<<<w->nb * kSmallCtas, kCluThreads, clu_smem(w->one_cams), st>>>(
+            s.row_ptr, s.tile_ptr, s.col, y.S, y.Dinv, x, ptr<double>(w->r), ptr<double>(w->z), ptr<double>(w->hist),
+            ptr<Ctl>(w->ctl));
+        return 1;
+    }
     k_one_cta<<<w->nb, kOneThreads, one_smem(w->one_cams), st>>>(
         mcg, s.row_ptr, s.tile_ptr, s.col, y.S32, y.Dhat, ptr<float>(w->xw), ptr<float>(w->r), ptr<float>(w->z),
         ptr<float>(w->P), ptr<float>(w->Q), ptr<double>(w->phip), ptr<double>(w->dpinv), ptr<float>(w->beta),
@@ -3527,7 +3674,7 @@ static void capture_krylov(Solver* w, const Structure& s, const System& y, const
                            int chunk, cudaStream_t cs, cudaStream_t cb, int* pre, int* per_pass) {
     const cudaGraphConditionalHandle h = capture_handle(cs);
     *pre = krylov_init<T>(w, s, S, Su, Dinv, rhs, sign, scale, x, outer, cs, mcg) + 1;
-    if (sizeof(T) == 4) *pre += enqueue_one_cta(w, s, y, mcg, cs);
+    *pre += enqueue_small(w, s, y, mcg, sizeof(T) == 8 ? reinterpret_cast<double*>(x) : nullptr, cs);
     k_loop_cond<<<1, kThreads, 0, cs>>>(h, 1, ptr<Ctl>(w->ctl), w->nb, ptr<Loops>(w->loops), 1, chunk,
                                         ptr<Params>(w->params));
     cudaGraph_t body = capture_while(cs, h);
@@ -3656,6 +3803,7 @@ static void run_host_loops(Solver* w, const Structure& s, const System& y, const
     int64_t launches = 0;
     if (!fp32) {
         launches += krylov_init<double>(w, s, y.S, nullptr, y.Dinv, y.bt, -1.0, nullptr, x, nullptr, st, a.mcg != 0);
+        launches += enqueue_small(w, s, y, a.mcg != 0, x, st);
         k_loop_cond<<<1, kThreads, 0, st>>>(none, 0, ptr<Ctl>(w->ctl), nb, lp, 1, a.chunk, prm);
         launches += 1 + host_krylov_loop(w, chunk_exec, gc, a, st, waits);
         launches += true_residual(w, s, y, x, nullptr, st);
@@ -3673,7 +3821,7 @@ static void run_host_loops(Solver* w, const Structure& s, const System& y, const
             if (!any) break;
             launches += krylov_init<float>(w, s, y.S32, y.S32u, y.Dhat, ptr<double>(w->rt), 1.0, y.lam,
                                            ptr<float>(w->xw), ptr<Outer>(w->outer), st, a.mcg != 0);
-            launches += enqueue_one_cta(w, s, y, a.mcg != 0, st);
+            launches += enqueue_small(w, s, y, a.mcg != 0, nullptr, st);
             k_loop_cond<<<1, kThreads, 0, st>>>(none, 0, ptr<Ctl>(w->ctl), nb, lp, 1, a.chunk, prm);
             launches += 1 + host_krylov_loop(w, chunk_exec, gc, a, st, waits);
             k_accumulate<<<dim3(w->gx, nb), kThreads, 0, st>>>(ptr<Layout>(w->lay_d), ptr<Outer>(w->outer),

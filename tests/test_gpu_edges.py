@@ -1,13 +1,14 @@
 """The solver's kernels at the sizes where their partitions end: camera counts around the update
 kernels' 14 cameras per CTA and the Gram kernel's 64 rows, direction widths 1 to 16, histories past the
 reorthogonalisation's tiles, and residuals far from one (the float32 sweeps solve for the residual
-divided by a power of two)."""
+divided by a power of two), and the camera counts up to which one CTA (float32 sweeps, 20) or one
+cluster (float64 PCG, 24) solves a problem."""
 import numpy as np
 import pytest
 
 from oracle import lm as olm
 from oracle import solvers as osol
-from paper_2110_04015_gb300 import binding
+from paper_2110_04015_gb300 import binding, problem
 from paper_2110_04015_gb300 import synthetic as sy
 from tests._gpu import energy_err
 
@@ -31,7 +32,7 @@ def _solve(p, args, tol):
 # recursive residual stops, and the true one stays within 1.5 of it), together with the energy norm of
 # the error against the dense solution, at the bound that the other tests hold solves to 1e-6 to.
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
-@pytest.mark.parametrize("n_cams", [2, 3, 7, 8, 14, 15, 28, 43, 57])
+@pytest.mark.parametrize("n_cams", [2, 3, 7, 8, 14, 15, 20, 21, 24, 25, 28, 43, 57])
 def test_camera_counts_around_the_partitions(n_cams, precision):
     sc, m, lin = _system(n_cams, 45 * n_cams + 7)
     ref = osol.dense_solve(lin.S, lin.btilde)
@@ -54,3 +55,22 @@ def test_sweeps_on_small_residuals_converge(rel):
         for args in SOLVES[:3]:
             st = _solve(p, args, 1e-12)
             assert st["status"] == 0 and st["true_rel_residual"] <= 1e-12, (args, st)
+
+
+# Problems on both sides of those counts in one batch: each gives the bits of its solo solve.
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_small_problems_in_a_batch_give_their_solo_bits(precision):
+    scenes = [sy.tiny(n, n_cams=n, n_pts=50 * n) for n in (13, 30, 20, 24, 60, 21, 7)]
+    solo = []
+    for sc in scenes:
+        with problem.from_scene(sc, precision=precision) as p:
+            p.ba_build_normal(1e-4)
+            solo.append([(_solve(p, a, 1e-9), p.ba_get_delta().copy())[1] for a in SOLVES])
+    off = np.cumsum([0] + [sc.n_cams for sc in scenes])
+    with problem.from_scenes(scenes, precision=precision) as b:
+        b.ba_build_normal(1e-4)
+        for k, a in enumerate(SOLVES):
+            assert _solve(b, a, 1e-9)["status"] == 0
+            x = b.ba_get_delta()
+            for q in range(len(scenes)):
+                assert np.array_equal(x[off[q]:off[q + 1]], solo[q][k]), (a, scenes[q].n_cams)
