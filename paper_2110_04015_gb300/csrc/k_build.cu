@@ -1242,14 +1242,15 @@ __global__ void __launch_bounds__(kCamThreads) k_jres_cam_df(
 }
 
 // Back-substitution in double-float: dx_l = -V_l^{-1} (b_l + sum_o J_l^T J_p dx_p,cam(o)) (Eq. 15 with
-// the sign that follows from Eq. 6); dxpd: dx_p split into double-float per camera.
-__global__ void k_back_sub_df(int32_t n_l, const int64_t* __restrict__ pt_ptr, const int32_t* __restrict__ order,
+// the sign that follows from Eq. 6); dxpd: dx_p split into double-float per camera.  Landmarks in index
+// order: neighbouring lanes then read neighbouring observations' rows (1000 banded cameras 83 us by track
+// length, 62 us; 1000 dense cameras 161 us, 155 us).
+__global__ void k_back_sub_df(int32_t n_l, const int64_t* __restrict__ pt_ptr,
                               const int32_t* __restrict__ oc, const float2* __restrict__ Jc,
                               const float2* __restrict__ Jl, const float2* __restrict__ Lall,
                               const float2* __restrict__ bl, const float2* __restrict__ dxpd,
                               double* __restrict__ dxl) {
-    for (int64_t t = gtid(); t < n_l; t += gstride()) {
-        const int64_t l = order[t];
+    for (int64_t l = gtid(); l < n_l; l += gstride()) {
         df64 s0 = ldd(bl + 3 * l), s1 = ldd(bl + 3 * l + 1), s2 = ldd(bl + 3 * l + 2);
         for (int64_t o = pt_ptr[l]; o < pt_ptr[l + 1]; ++o) {
             const float2* xc = dxpd + 9 * int64_t(oc[o]);
@@ -1372,13 +1373,13 @@ __global__ void k_to_float(const double* __restrict__ in, float* __restrict__ ou
     for (int64_t i = gtid(); i < n; i += gstride()) out[i] = static_cast<float>(in[i]);
 }
 
-// dx_l = -L^{-T} (e_l + sum_o G_o^T dx_p,cam(o))
-__global__ void k_back_substitute(int32_t n_l, const int64_t* __restrict__ pt_ptr, const int32_t* __restrict__ order,
+// dx_l = -L^{-T} (e_l + sum_o G_o^T dx_p,cam(o)).  Landmarks in index order, as in k_back_sub_df (601 cameras:
+// 160 us by track length, 101 us)
+__global__ void k_back_substitute(int32_t n_l, const int64_t* __restrict__ pt_ptr,
                                   const int32_t* __restrict__ oc, const double* __restrict__ G,
                                   const double* __restrict__ Lall, const double* __restrict__ e,
                                   const double* __restrict__ dxp, double* __restrict__ dxl) {
-    for (int64_t t = gtid(); t < n_l; t += gstride()) {
-        const int64_t l = order[t];
+    for (int64_t l = gtid(); l < n_l; l += gstride()) {
         double a0 = e[3 * l], a1 = e[3 * l + 1], a2 = e[3 * l + 2];
         for (int64_t o = pt_ptr[l]; o < pt_ptr[l + 1]; ++o) {
             const double* g = G + 27 * o;
@@ -1621,13 +1622,13 @@ void launch_to_float(const double* in, float* out, int64_t n, cudaStream_t st) {
 
 void launch_back_substitute(const Structure& s, const System& y, const double* dxp, double* dxl, cudaStream_t st) {
     if (y.G)
-        k_back_substitute<<<grid_for(s.n_l, kThreads), kThreads, 0, st>>>(s.n_l, s.pt_ptr, s.lm_order, s.obs_cam, y.G,
+        k_back_substitute<<<grid_for(s.n_l, kThreads), kThreads, 0, st>>>(s.n_l, s.pt_ptr, s.obs_cam, y.G,
                                                                            y.L, y.e, dxp, dxl);
     else {
         // mixed precision: dx_p split into double-float (the true residual's buffer, idle here)
         k_split_df<<<grid_for(int64_t(s.n_c) * 9, kThreads), kThreads, 0, st>>>(dxp, y.xd, int64_t(s.n_c) * 9);
         k_back_sub_df<<<grid_for(s.n_l, kThreads), kThreads, 0, st>>>(
-            s.n_l, s.pt_ptr, s.lm_order, s.obs_cam, reinterpret_cast<const float2*>(y.Jc),
+            s.n_l, s.pt_ptr, s.obs_cam, reinterpret_cast<const float2*>(y.Jc),
             reinterpret_cast<const float2*>(y.Jl), reinterpret_cast<const float2*>(y.L),
             reinterpret_cast<const float2*>(y.bl), y.xd, dxl);
     }
