@@ -56,7 +56,7 @@ constexpr int kUpdCams = 14;
 constexpr int kUpdThreads = 128;
 
 // Where one problem of the batch lives (fixed for a solve).
-struct Layout {
+struct Layout {           // no padding (compared as bytes)
     int c0, nc;          // first camera, number of cameras
     int64_t hoff;        // first element of its direction history (cap columns of 9 nc rows)
     int64_t phoff;       // first Phi partial
@@ -3074,6 +3074,7 @@ struct Solver {
     int64_t launches = 0;     // kernel executions issued by the current solve
     cudaStream_t cap_stream = nullptr, cap2 = nullptr, cap3 = nullptr;   // capture streams (nested loops)
     std::vector<SolveExec*> execs;   // instantiated solve graphs
+    cudaEvent_t ev0 = nullptr, ev1 = nullptr;   // around a solve
     // work lists of the block-sparse products: whole rows, rows split by pose subset, and whole rows of
     // the upper triangle (the symmetric one-column products of mixed precision)
     ItemList items_g, items_l, items_u;
@@ -3403,6 +3404,7 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     grow(w->ctl, size_t(nb) * sizeof(Ctl));
     grow(w->outer, size_t(nb) * sizeof(Outer));
     grow(w->rt, size_t(n) * sizeof(double));
+    const void* lay_p = w->lay_d.p;
     grow(w->lay_d, size_t(nb) * sizeof(Layout));
     grow(w->dpart, size_t(nb) * w->gu * 3 * sizeof(double));
     grow(w->dtot, size_t(nb) * 2 * sizeof(double));
@@ -3416,8 +3418,14 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
         BA_CUDA_TRY(cudaMallocHost(&w->h_hist, sizeof(double) * size_t(nb) * w->mi1));
         w->h_hist_n = size_t(nb) * w->mi1;
     }
-    BA_CUDA_TRY(cudaMemcpy(w->lay_d.p, lay.data(), sizeof(Layout) * nb, cudaMemcpyHostToDevice));
-    w->lay = lay;
+    // the layouts change with the solver and its options, not from solve to solve: the upload (a host wait of
+    // about 10 us) is skipped when the device holds them already
+    if (lay_p != w->lay_d.p || w->lay.size() != lay.size() ||
+        std::memcmp(w->lay.data(), lay.data(), sizeof(Layout) * lay.size()) != 0) {
+        w->lay.clear();
+        BA_CUDA_TRY(cudaMemcpy(w->lay_d.p, lay.data(), sizeof(Layout) * nb, cudaMemcpyHostToDevice));
+        w->lay = lay;
+    }
     w->spmv_cfg = a.spmv_cfg >= 0 && a.spmv_cfg < kSpmvShapes ? a.spmv_cfg : 0;
     ensure_items(w, s, a.mcg ? n_dirs : 1, a.item_blocks, fp32, w->spmv_cfg);
     w->items_g.polls = a.wait_polls;
@@ -3453,6 +3461,8 @@ void solver_destroy(Solver* w) {
     if (w->h_params) cudaFreeHost(w->h_params);
     if (w->h_loops) cudaFreeHost(w->h_loops);
     if (w->h_hist) cudaFreeHost(w->h_hist);
+    if (w->ev0) cudaEventDestroy(w->ev0);
+    if (w->ev1) cudaEventDestroy(w->ev1);
     if (w->cap_stream) cudaStreamDestroy(w->cap_stream);
     if (w->cap2) cudaStreamDestroy(w->cap2);
     if (w->cap3) cudaStreamDestroy(w->cap3);
@@ -3901,9 +3911,10 @@ void solver_run(Solver* w, const Structure& s, const System& y, const SolveArgs&
     GraphCounts gc;
     cudaGraphExec_t exec = solve_graph(w, s, y, a, x, gc);
 
-    cudaEvent_t e0, e1;
-    BA_CUDA_TRY(cudaEventCreate(&e0));
-    BA_CUDA_TRY(cudaEventCreate(&e1));
+    // the solver's events, made once (on the device of the handle)
+    if (!w->ev0) BA_CUDA_TRY(cudaEventCreate(&w->ev0));
+    if (!w->ev1) BA_CUDA_TRY(cudaEventCreate(&w->ev1));
+    const cudaEvent_t e0 = w->ev0, e1 = w->ev1;
     BA_CUDA_TRY(cudaEventRecord(e0, st));
     // the solve: its arguments in, one graph launch, the results out, one wait
     Params* hp = w->h_params;
@@ -3929,8 +3940,6 @@ void solver_run(Solver* w, const Structure& s, const System& y, const SolveArgs&
     BA_CUDA_TRY(cudaGetLastError());
     float ms = 0.f;
     cudaEventElapsedTime(&ms, e0, e1);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
 
     const Loops lp = *w->h_loops;
     if (!a.host_loop) w->launches = gc.pre + int64_t(lp.outer) * gc.sweep + int64_t(lp.inner) * gc.body + gc.post;
