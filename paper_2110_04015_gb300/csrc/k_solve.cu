@@ -844,9 +844,12 @@ __global__ void __launch_bounds__(kColWarps * 32, 12) k_spmv_col(const int64_t* 
 
 // Q[:, new_off + c] = S P[:, new_off + c] for the w > 1 columns of a new local block (Algorithm 2,
 // used by the float32 sweeps, where the Eq. 18 update cancels).  Tiles stream through
-// shared memory as in k_spmv; lane = 4 qi + g takes tile-local blocks qi, qi + 8, qi + 16, qi + 24
-// and columns 4g .. 4g + 3, so each 9x9 block multiplies up to 16 columns per read from shared
-// memory.  PT is the row-major copy (9 n_c x 16, all problems) of the new blocks.
+// shared memory as in k_spmv; CL lanes share a block (CL = 4, or 2 when no block is wider than 8
+// columns): lane = CL qi + g takes tile-local blocks qi, qi + 32 / CL, ... and columns
+// 4g .. 4g + 3, so each 9x9 block multiplies up to 4 CL columns per read from shared memory.  The kernel
+// is bound by what its lanes read from shared memory and L1 (81 words of S and 36 of P per 324
+// multiply-adds), so lanes left without columns cost as much as the others: N = 8 on 1000 dense cameras
+// took 94 us per local step with four lanes a block and takes 75 us with two (one lane for N = 4: 76 us).  PT is the row-major copy (9 n_c x 16, all problems) of the new blocks.
 // The multi-column product waits on L2 gathers of PT more than on its tiles, so it runs twice
 // the warps of k_spmv with one tile stage each (the other warps' copies and arithmetic cover a
 // warp's wait for its next tile); at most 128 registers a thread.
@@ -874,7 +877,7 @@ __device__ __forceinline__ void load_prow(const float* p, float2 (&v)[9][2]) {
     }
 }
 
-template <typename T>
+template <typename T, int CL>
 __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
     const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ tile_ptr, const int32_t* __restrict__ col,
     const T* __restrict__ S, const T* __restrict__ PT, ItemList L, T* __restrict__ part, T* __restrict__ Q,
@@ -886,7 +889,8 @@ __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
     extern __shared__ __align__(128) unsigned char smem_raw[];
     if (nothing_selected(ctl, L, sel)) return;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int qi = lane >> 2, g = lane & 3;
+    constexpr int NBK = 32 / CL;   // blocks per round
+    const int qi = lane / CL, g = lane % CL;
     T* tiles = reinterpret_cast<T*>(smem_raw) + size_t(wid) * NS * kTileElems;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem_raw + sizeof(T) * NW * NS * kTileElems) + wid * NS;
     T* red = reinterpret_cast<T*>(smem_raw + spmm_tiles_smem<T>()) + wid * (kMaxDirs * 9);
@@ -927,20 +931,20 @@ __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
         if (it.q1 > it.q0) {
             const int t0 = it.q0 >> 5, t1 = (it.q1 + 31) >> 5;
             const bool active = 4 * g < w;
-            // column cameras of this lane's blocks r * 8 + qi (r = 0..3) of tile t, -1 outside the
+            // column cameras of this lane's blocks r NBK + qi (r < CL) of tile t, -1 outside the
             // item; fetched one tile ahead.  The P rows of a block are gathered right before its
             // arithmetic: the other warps of the SM cover the wait
-            int kc[4], kn[4];
+            int kc[CL], kn[CL];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int q = t0 * 32 + r * 8 + qi;
+            for (int r = 0; r < CL; ++r) {
+                const int q = t0 * 32 + r * NBK + qi;
                 kc[r] = (active && q >= it.q0 && q < it.q1) ? col[rj + q] : -1;
             }
             float2 pv[9][2];
             for (int t = t0; t < t1; ++t) {
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const int q = (t + 1) * 32 + r * 8 + qi;
+                for (int r = 0; r < CL; ++r) {
+                    const int q = (t + 1) * 32 + r * NBK + qi;
                     kn[r] = (active && t + 1 < t1 && q < it.q1) ? col[rj + q] : -1;
                 }
                 const bool ok = mbar_wait(&bars[stage], (parity >> stage) & 1u, L.polls);
@@ -954,11 +958,11 @@ __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
                 const T* tile = tiles + stage * kTileElems;
                 if (active) {
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) {
+                    for (int r = 0; r < CL; ++r) {
                         if (kc[r] < 0) continue;
                         // rows 9k .. 9k + 8, columns 4g .. 4g + 3 of PT for this block
                         load_prow(PT + (int64_t(kc[r]) * 9) * kMaxDirs + 4 * g, pv);
-                        const T* blk = tile + (r * 8 + qi) * 81;
+                        const T* blk = tile + (r * NBK + qi) * 81;
 #pragma unroll
                         for (int a = 0; a < 9; ++a)
 #pragma unroll
@@ -971,7 +975,7 @@ __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
                     }
                 }
 #pragma unroll
-                for (int r = 0; r < 4; ++r) kc[r] = kn[r];
+                for (int r = 0; r < CL; ++r) kc[r] = kn[r];
                 __syncwarp();
                 if (f.item < f.end) {
                     fence_proxy_async();
@@ -984,7 +988,7 @@ __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
             }
             if (bad) break;
         }
-        // sum over the 8 lanes of each column group, then lanes 0..3 hold their columns
+        // sum over the NBK lanes of each column group, then lanes 0 .. CL - 1 hold their columns
         T accs[9][4];
 #pragma unroll
         for (int a = 0; a < 9; ++a) {
@@ -998,9 +1002,8 @@ __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
 #pragma unroll
             for (int cc = 0; cc < 4; ++cc) {
                 T v = accs[a][cc];
-                v += __shfl_xor_sync(0xffffffffu, v, 4);
-                v += __shfl_xor_sync(0xffffffffu, v, 8);
-                v += __shfl_xor_sync(0xffffffffu, v, 16);
+#pragma unroll
+                for (int o = CL; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
                 accs[a][cc] = v;
             }
         __syncwarp();
@@ -3019,13 +3022,14 @@ __global__ void k_refine_after(const Ctl* __restrict__ ctl, Outer* outer, const 
 // loop body, work lists, wait bound and every buffer address (a reallocation bumps `allocs`).
 struct GraphKey {
     int mcg = -1, fp32 = -1, chunk = 0, mi1 = 0, use_l = -1, epoch = -1, polls = -1, nb = -1, host = -1, cfg = -1;
+    int lanes = -1;                   // column lanes of k_spmm
     int one = -1;                     // cameras of the largest problem that one CTA or cluster solves
     uint64_t allocs = ~uint64_t(0);   // buffer generation (any reallocation invalidates the graph)
     const void* ptrs[4] = {};
     bool operator==(const GraphKey& o) const {
         if (mcg != o.mcg || fp32 != o.fp32 || chunk != o.chunk || mi1 != o.mi1 || use_l != o.use_l ||
             epoch != o.epoch || polls != o.polls || nb != o.nb || host != o.host || cfg != o.cfg ||
-            one != o.one || allocs != o.allocs)
+            lanes != o.lanes || one != o.one || allocs != o.allocs)
             return false;
         for (int i = 0; i < 4; ++i) if (ptrs[i] != o.ptrs[i]) return false;
         return true;
@@ -3081,6 +3085,7 @@ struct Solver {
     Buf tb;                    // transposed terms of the symmetric product (kTbHead + 1 values per upper block)
     int items_cb = -1;         // item chunk rule the lists were built with (0 = the default)
     int items_l_dirs = -1;
+    int col_lanes = 4;         // lanes that share a block in k_spmm: four columns each cover n_dirs
     bool use_l = false;        // the current MCG solve splits rows by pose subset (n_dirs > 1)
     int epoch = 0;             // incremented whenever a work list is rebuilt (captured graphs hold them)
     int spmv_cfg = 0;          // shape of the one-column products (SpmvShape)
@@ -3269,7 +3274,8 @@ static void set_smem_attrs() {
     set_spmv_attrs<0>();
     set_spmv_attrs<1>();
     set_spmv_attrs<2>();
-    BA_CUDA_TRY(cudaFuncSetAttribute(k_spmm<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(spmm_smem<float>())));
+    for (auto mm : {k_spmm<float, 2>, k_spmm<float, 4>})
+        BA_CUDA_TRY(cudaFuncSetAttribute(mm, cudaFuncAttributeMaxDynamicSharedMemorySize, int(spmm_smem<float>())));
     BA_CUDA_TRY(cudaFuncSetAttribute(k_one_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, int(one_smem(kOneCams))));
     BA_CUDA_TRY(cudaFuncSetAttribute(k_pcg_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, int(clu_smem(kCluCams))));
     done = true;
@@ -3311,6 +3317,7 @@ static void ensure_items(Solver* w, const Structure& s, int n_dirs, int forced_c
         ++w->epoch;
     }
     w->use_l = n_dirs > 1;
+    w->col_lanes = n_dirs <= 8 ? 2 : 4;
     set_smem_attrs();
 }
 
@@ -3588,7 +3595,8 @@ static int enqueue_iteration(Solver* w, const Structure& s, const T* S, const T*
             auto pq = w->n >= int64_t(48) * Gt ? k_mcg_pq<T, 2> : k_mcg_pq<T, 1>;
             launch_chained(pq, dim3(w->gpq, nb), dim3(PqShape<T>::kSlices * 32), 0, st, P, Q, z, betat, ptr<T>(w->PT), ctl);
             const int np = enqueue_product<T, 2>(w, s, S, Su, P, kSelW1, Q, nullptr, st);
-            launch_chained(k_spmm<T>, dim3(Gt), dim3(SpmmCfg::kWarps * 32), spmm_smem<T>(), st, s.row_ptr, s.tile_ptr,
+            auto mm = w->col_lanes == 2 ? k_spmm<T, 2> : k_spmm<T, 4>;
+            launch_chained(mm, dim3(Gt), dim3(SpmmCfg::kWarps * 32), spmm_smem<T>(), st, s.row_ptr, s.tile_ptr,
                            s.col, S, ptr<T>(w->PT), w->items_g, static_cast<T*>(w->mm_part), Q, ctl);
             return 7 + np;
         }
@@ -3863,6 +3871,7 @@ static cudaGraphExec_t solve_graph(Solver* w, const Structure& s, const System& 
     key.host = a.host_loop;
     key.cfg = a.spmv_cfg;
     key.one = w->one_cams;
+    key.lanes = w->col_lanes;
     key.allocs = g_allocs.load();
     const void* ptrs[4] = {x, fp32 ? (const void*)y.S32 : (const void*)y.S, w->items_g.items, w->items_l.items};
     for (int i = 0; i < 4; ++i) key.ptrs[i] = ptrs[i];

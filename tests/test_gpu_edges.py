@@ -74,3 +74,16 @@ def test_small_problems_in_a_batch_give_their_solo_bits(precision):
             x = b.ba_get_delta()
             for q in range(len(scenes)):
                 assert np.array_equal(x[off[q]:off[q + 1]], solo[q][k]), (a, scenes[q].n_cams)
+
+
+# Direction counts on both sides of 8, up to which two lanes share a block in the multi-column product,
+# on problems that run it (more than 20 cameras), every step local.
+@pytest.mark.parametrize("dirs", [2, 4, 7, 8, 9, 16])
+def test_local_steps_of_every_width_class(dirs):
+    sc, m, lin = _system(45, 1500)
+    ref = osol.dense_solve(lin.S, lin.btilde)
+    with binding.Problem(sc.cams0, sc.pts0, sc.obs_cam, sc.obs_pt, m, precision="mixed") as p:
+        p.ba_build_normal(1e-4)
+        st = p.ba_solve_mcg(1e-11, 5000, dirs, 1e9)
+        assert st["status"] == 0 and st["local_steps"] > 0 and st["true_rel_residual"] <= 1e-11, st
+        assert energy_err(lin.S, p.ba_get_delta().ravel(), ref) < 1e-4
