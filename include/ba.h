@@ -78,7 +78,9 @@ typedef struct ba_options {
     int32_t precision;         /* ba_precision */
     int32_t chunk_iters;       /* Krylov iterations per pass of the solve graph's device-side loop
                                   between checks of the stop flags (default 8, 1..256); a solve is
-                                  one graph launch and the host waits once, at its end */
+                                  one graph launch and the host waits once, at its end (problems of
+                                  up to 20 cameras in MIXED, 24 in FP64 PCG, run a whole sweep in
+                                  one launch instead) */
     int32_t max_history;       /* MCG: maximum stored direction columns (default 0 = max_iters * n_dirs + 1);
                                   when it is full FP64 stops with OOM, while MIXED ends the float32
                                   sweep and the refinement starts another from the true residual */
@@ -93,7 +95,8 @@ typedef struct ba_options {
                                   solve gives up with BA_ERR_TIMEOUT (the kernel then waits for its
                                   own copies still in flight, with the default bound, and returns).
                                   0 (default) = 2^20; 1 .. 2^30; -1 = no poll at all, so every such
-                                  wait gives up at once (tests the timeout path) */
+                                  wait gives up at once (tests the timeout path; the smallest problems
+                                  then run the kernels that wait, like all others) */
     int32_t spmv_config;       /* warps x copy stages per CTA of the tile-streaming one-column product:
                                   0 (default) = float32 16 x 1, float64 8 x 1; 1 = 8 x 2 / 4 x 2;
                                   2 = 10 x 2 / 2 x 4; ba_autotune sets it */

@@ -69,8 +69,9 @@ struct Structure {
     float2* obs_xyd = nullptr;    // n_o x 2 (mixed precision): the measurements in double-float
     int64_t* pt_ptr = nullptr;    // n_l + 1
     int32_t* lm_order = nullptr;  // n_l: landmarks by decreasing track length (ties by index); the
-                                  // per-landmark kernels take them in this order so that the lanes of a
-                                  // warp loop over equally many observations
+                                  // kernels of the landmark factors take them in this order so that the
+                                  // lanes of a warp loop over equally many observations (the true
+                                  // residual and the back-substitution go in index order)
     int64_t* cam_ptr = nullptr;   // n_c + 1
     int32_t* cam_obs = nullptr;   // n_o: point-order slots grouped by camera
     // S pattern (full)

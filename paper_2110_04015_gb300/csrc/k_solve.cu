@@ -10,6 +10,8 @@
 // float64 iterative refinement of mixed precision is an outer WHILE node around it), so the host
 // launches the graph once and reads the results once; nothing inside a solve waits on the host.
 // A problem whose Ctl::done is set is skipped by every later launch while the others go on.
+// Problems of a few cameras run their whole sweep in one launch before that loop (k_one_cta,
+// k_pcg_cluster).
 //
 // Batches: problem b owns the cameras [c0, c0 + nc) of the handle (S is block-diagonal over the
 // problems, since no landmark is seen by two of them).  Per-problem kernels take the problem from
