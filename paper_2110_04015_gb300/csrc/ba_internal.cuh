@@ -180,7 +180,7 @@ void launch_schur(const Structure& s, System& y, cudaStream_t st);
 void launch_schur_mixed(const Structure& s, System& y, cudaStream_t st);
 // out = -b~ - S x with the implicit float64 operator (mixed precision, no explicit S)
 // S x = sum_o J_p^T (J_p x - J_l V^-1 sum J_l^T J_p x) + lambda D_p x;
-// partial[2 j], partial[2 j + 1] receive camera j's sums of out^2 and b~^2 (2 n_c values)
+// partial[3 j] .. partial[3 j + 2] receive camera j's sums of out^2, b~^2 and (Lam out)^2 (3 n_c values)
 int launch_implicit_residual(const Structure& s, const System& y, const double* x, double* out, double* partial,
                               cudaStream_t st);
 void launch_block_jacobi(const Structure& s, System& y, cudaStream_t st);

@@ -1198,12 +1198,12 @@ __global__ void k_jres_land_df(int32_t n_l, const int64_t* __restrict__ pt_ptr, 
 }
 
 // True residual, camera pass: out_j = -b~_j - (S x)_j with (S x)_j = sum_{o in j} J_p^T v_o (double-float)
-// + lambda D_p x_j (float64); camera j's |out_j|^2 and |b~_j|^2 into partial[2 j], partial[2 j + 1].
+// + lambda D_p x_j (float64); camera j's |out_j|^2, |b~_j|^2 and |Lam out_j|^2 into partial[3 j] ..
 __global__ void __launch_bounds__(kCamThreads) k_jres_cam_df(
     int32_t n_c, const int64_t* __restrict__ cam_ptr, const int32_t* __restrict__ cam_obs,
     const float2* __restrict__ Jc, const float2* __restrict__ uv, const double* __restrict__ dadd,
-    const double* __restrict__ x, const double* __restrict__ bt, double* __restrict__ out,
-    double* __restrict__ partial) {
+    const double* __restrict__ x, const double* __restrict__ bt, const double* __restrict__ lam,
+    double* __restrict__ out, double* __restrict__ partial) {
     __shared__ df64 red[kCamThreads / 32][9];
     for (int j = blockIdx.x; j < n_c; j += gridDim.x) {
         df64 acc[9];
@@ -1218,7 +1218,7 @@ __global__ void __launch_bounds__(kCamThreads) k_jres_cam_df(
             for (int a = 0; a < 9; ++a) acc[a] += jc[a] * u[0] + jc[9 + a] * u[1];
         }
         cta_sum_df<9>(acc, red);
-        double tt = 0.0, bb = 0.0;
+        double tt = 0.0, bb = 0.0, ss = 0.0;
         if (threadIdx.x < 9) {
             const int a = threadIdx.x;
             const int64_t i = 9 * int64_t(j) + a;
@@ -1226,15 +1226,19 @@ __global__ void __launch_bounds__(kCamThreads) k_jres_cam_df(
             const double b_ = bt[i];
             const double rv = -b_ - sx;
             if (out) out[i] = rv;
+            const double sv = lam[i] * rv;
             tt = rv * rv;
             bb = b_ * b_;
+            ss = sv * sv;
         }
         if (threadIdx.x < 32) {
             tt = warp_sum(tt);
             bb = warp_sum(bb);
+            ss = warp_sum(ss);
             if (threadIdx.x == 0) {
-                partial[2 * int64_t(j)] = tt;
-                partial[2 * int64_t(j) + 1] = bb;
+                partial[3 * int64_t(j)] = tt;
+                partial[3 * int64_t(j) + 1] = bb;
+                partial[3 * int64_t(j) + 2] = ss;
             }
         }
         __syncthreads();
@@ -1589,8 +1593,8 @@ int launch_implicit_residual(const Structure& s, const System& y, const double* 
         reinterpret_cast<float2*>(y.uv));
     k_jres_cam_df<<<cam_grid(s), kCamThreads, 0, st>>>(s.n_c, s.cam_ptr, s.cam_obs,
                                                        reinterpret_cast<const float2*>(y.Jc),
-                                                       reinterpret_cast<const float2*>(y.uv), y.dadd, x, y.bt, out,
-                                                       partial);
+                                                       reinterpret_cast<const float2*>(y.uv), y.dadd, x, y.bt, y.lam,
+                                                       out, partial);
     return 3;
 }
 

@@ -90,6 +90,7 @@ struct Ctl {
                        // first CTA runs the decide step, which may set done meanwhile)
     double alpha_v[kMaxDirs];
     double true_rr, bb;                 // true residual and |rhs|^2
+    double scaled_rr;  // mixed precision: |Lam (true residual)|^2
     double stag;       // float32 sweeps: stop when t_i (energy decrease / r^T D^-1 r) falls below this
     int direct_q;      // 1: Q_{i+1} = S P_{i+1} (Algorithm 2); 0: the Q update of Eq. 18
     int pinv_steps;    // steps whose Delta_i took the eigen-decomposition pseudo-inverse
@@ -116,8 +117,9 @@ struct Outer {
     double bb;         // |b~|^2
     double tr;         // |-b~ - S x|^2 of the current x
     double tr_prev;    // the same before the last sweep (scales that sweep's residual history)
+    double sr;         // |Lam (-b~ - S x)|^2 of the current x: the residual of the sweeps' scaled system
     double tol_in;     // relative tolerance of the next inner sweep
-    double unit;       // power of two near |-b~ - S x|: the sweep solves for the residual divided by it
+    double unit;       // power of two near sqrt(sr): the sweep solves for Lam (-b~ - S x) divided by it
     int status;
     int active;        // still refining
     int swept;         // takes part in the sweep being run
@@ -1057,9 +1059,10 @@ __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
 // ---------------------------------------------------------------------------------------
 // initialisation shared by both algorithms: x = 0, r = sign * rhs, z = D^{-1} r, P_0 = z
 // (grid: update CTAs x problems; thread = row, as in the update kernels; partial: one slot per CTA).
-// outer (mixed precision, may be null): r is divided by the sweep's unit, a power of two, so that the
-// float32 sums of a sweep start near one whatever the residual's size (their error terms would
-// otherwise leave the float32 range on late sweeps).
+// outer (mixed precision, may be null): r is divided by the sweep's unit, a power of two near |r|, so that
+// a sweep starts with |r| in [1, 2) whatever the residual's size and the units of the cameras and
+// landmarks (the error terms of its float32 sums, and Delta^+ in double-float, would otherwise leave the
+// float32 range on late sweeps, or on the first one of a scene with coordinates of 1e-9).
 
 template <typename T>
 __global__ void __launch_bounds__(kUpdThreads) k_init_vec(const Layout* __restrict__ lay, const double* __restrict__ rhs,
@@ -2889,16 +2892,13 @@ __global__ void k_true_residual(int32_t n_c, const int64_t* __restrict__ row_ptr
     }
 }
 
-// per problem: ctl.true_rr and ctl.bb from the per-camera partials (camera order)
-__global__ void k_true_reduce(Ctl* ctl, const double* __restrict__ partial) {
+// per problem: ctl.true_rr, ctl.bb and (ns = 3) ctl.scaled_rr from the ns per-camera partials (camera
+// order); a warp per sum
+__global__ void k_true_reduce(Ctl* ctl, const double* __restrict__ partial, int ns) {
     Ctl* c = ctl + blockIdx.x;
-    const double* pp = partial + 2 * int64_t(c->lay.c0);
-    const double a = sum_partials(pp, c->lay.nc, 2, 0);
-    const double b = sum_partials(pp, c->lay.nc, 2, 1);
-    if (threadIdx.x == 0) {
-        c->true_rr = a;
-        c->bb = b;
-    }
+    const int k = threadIdx.x >> 5;
+    const double v = sum_partials(partial + ns * int64_t(c->lay.c0), c->lay.nc, ns, k);
+    if ((threadIdx.x & 31) == 0) (k == 0 ? c->true_rr : k == 1 ? c->bb : c->scaled_rr) = v;
 }
 
 // mixed precision: x += unit Lam d, a float32 sweep's correction mapped back from the scaled system,
@@ -2927,21 +2927,27 @@ __global__ void k_start_refine(int64_t n, const double* __restrict__ bt, double*
     }
 }
 
-// One CTA per problem: |b~|^2 (fixed order) and the refinement state at x = 0.
-__global__ void k_outer_init(const Layout* __restrict__ lay, const double* __restrict__ bt, Outer* outer) {
+// One CTA per problem: |b~|^2 and |Lam b~|^2 (fixed order) and the refinement state at x = 0.
+__global__ void k_outer_init(const Layout* __restrict__ lay, const double* __restrict__ bt,
+                             const double* __restrict__ lam, Outer* outer) {
     const Layout L = lay[blockIdx.x];
     const int64_t n = int64_t(L.nc) * 9;
     const double* b = bt + 9 * int64_t(L.c0);
-    double v[1] = {0.0};
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) v[0] += b[i] * b[i];
-    __shared__ double s[1];
-    cta_sum_write<1>(v, s);
+    double v[2] = {0.0, 0.0};
+    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+        const double sb = lam[9 * int64_t(L.c0) + i] * b[i];
+        v[0] += b[i] * b[i];
+        v[1] += sb * sb;
+    }
+    __shared__ double s[2];
+    cta_sum_write<2>(v, s);
     if (threadIdx.x == 0) {
         Outer o;
         memset(&o, 0, sizeof(o));
         o.bb = s[0];
         o.tr = s[0];
         o.tr_prev = s[0];
+        o.sr = s[1];
         o.unit = 1.0;
         o.status = s[0] == 0.0 ? BA_OK : BA_ERR_NOT_CONVERGED;
         o.active = s[0] == 0.0 ? 0 : 1;
@@ -2972,7 +2978,7 @@ __global__ void k_refine_plan(Outer* outer, int nb, const Params* __restrict__ p
         double t = need > 0.1 * inner_tol ? fmax(0.3 * need, 0.1 * inner_tol) : inner_tol;
         if (t >= 1.0) t = 0.5;
         o->tol_in = t;
-        o->unit = ldexp(1.0, max(-900, min(900, ilogb(sqrt(o->tr)))));
+        o->unit = o->sr > 0.0 ? ldexp(1.0, max(-900, min(900, ilogb(sqrt(o->sr))))) : 1.0;
         o->max_in = prm->max_iters - o->iters;
         o->swept = 1;
         mine = 1;
@@ -2999,6 +3005,7 @@ __global__ void k_refine_after(const Ctl* __restrict__ ctl, Outer* outer, const 
     o->cols = mcg ? c.cols : 1;
     o->tr_prev = o->tr;
     o->tr = c.true_rr;
+    o->sr = c.scaled_rr;
     if (c.status == BA_ERR_BREAKDOWN || c.status == BA_ERR_OOM || c.status == BA_ERR_TIMEOUT) {
         o->status = c.status;
         o->active = 0;
@@ -3396,7 +3403,7 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     grow(w->PT, size_t(n) * kMaxDirs * elt);
     grow(w->part_a, size_t(nb) * w->gg * kGramMax * sizeof(double));
     grow(w->part_b, size_t(nb) * w->gu * sizeof(double));
-    grow(w->part_cam, size_t(s.n_c) * 2 * sizeof(double));
+    grow(w->part_cam, size_t(s.n_c) * 3 * sizeof(double));
     grow(w->dpinv, size_t(nb) * w->mi1 * kMaxDirs * kMaxDirs * sizeof(double));
     grow(w->beta, size_t(boff) * kMaxDirs * sizeof(double));
     grow(w->phip, size_t(phoff) * sizeof(double));
@@ -3642,15 +3649,16 @@ static int enqueue_small(Solver* w, const Structure& s, const System& y, bool mc
 // bb): explicit tiled S in float64 precision, the implicit operator (double-float arithmetic) in mixed precision.
 static int true_residual(Solver* w, const Structure& s, const System& y, const double* x, double* out,
                          cudaStream_t st) {
-    int n = 0;
+    int n = 0, sums = 2;
     if (y.S) {
         k_true_residual<<<grid_for_host(int64_t(s.n_c) * 32), kThreads, 0, st>>>(
             s.n_c, s.row_ptr, s.tile_ptr, s.col, y.S, x, y.bt, out, ptr<double>(w->part_cam));
         n = 1;
     } else {
         n = launch_implicit_residual(s, y, x, out, ptr<double>(w->part_cam), st);
+        sums = 3;
     }
-    k_true_reduce<<<w->nb, 32, 0, st>>>(ptr<Ctl>(w->ctl), ptr<double>(w->part_cam));
+    k_true_reduce<<<w->nb, 32 * sums, 0, st>>>(ptr<Ctl>(w->ctl), ptr<double>(w->part_cam), sums);
     return n + 1;
 }
 
@@ -3729,7 +3737,7 @@ static cudaGraphExec_t build_solve_graph(Solver* w, const Structure& s, const Sy
             gc.post = true_residual(w, s, y, x, nullptr, cs);
         } else {
             k_start_refine<<<grid_for_host(n), kThreads, 0, cs>>>(n, y.bt, x, ptr<double>(w->rt));
-            k_outer_init<<<nb, kThreads, 0, cs>>>(ptr<Layout>(w->lay_d), y.bt, ptr<Outer>(w->outer));
+            k_outer_init<<<nb, kThreads, 0, cs>>>(ptr<Layout>(w->lay_d), y.bt, y.lam, ptr<Outer>(w->outer));
             const cudaGraphConditionalHandle ho = capture_handle(cs);
             k_refine_plan<<<1, kThreads, 0, cs>>>(ptr<Outer>(w->outer), nb, ptr<Params>(w->params), ho, 1,
                                                   ptr<Loops>(w->loops), 0);
@@ -3829,7 +3837,7 @@ static void run_host_loops(Solver* w, const Structure& s, const System& y, const
         launches += true_residual(w, s, y, x, nullptr, st);
     } else {
         k_start_refine<<<grid_for_host(n), kThreads, 0, st>>>(n, y.bt, x, ptr<double>(w->rt));
-        k_outer_init<<<nb, kThreads, 0, st>>>(ptr<Layout>(w->lay_d), y.bt, ptr<Outer>(w->outer));
+        k_outer_init<<<nb, kThreads, 0, st>>>(ptr<Layout>(w->lay_d), y.bt, y.lam, ptr<Outer>(w->outer));
         k_refine_plan<<<1, kThreads, 0, st>>>(ptr<Outer>(w->outer), nb, prm, none, 0, lp, 0);
         launches += 3;
         for (int sweep = 0; sweep <= a.max_refine; ++sweep) {

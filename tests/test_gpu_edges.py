@@ -87,3 +87,32 @@ def test_local_steps_of_every_width_class(dirs):
         st = p.ba_solve_mcg(1e-11, 5000, dirs, 1e9)
         assert st["status"] == 0 and st["local_steps"] > 0 and st["true_rel_residual"] <= 1e-11, st
         assert energy_err(lin.S, p.ba_get_delta().ravel(), ref) < 1e-4
+
+
+# The same scene in other length units: translations and landmarks times s give the same residuals, and a
+# scaled system (Lam S Lam) that differs only through the damping's floor, while Lam and the unscaled
+# residual change by factors of s and 1 / s.  A float32 sweep must not depend on them: 16 cameras run in one
+# CTA, 45 in the kernels of an iteration.
+@pytest.mark.parametrize("n_cams", [16, 45])
+@pytest.mark.parametrize("s", [1e-12, 1e-9, 1e-6, 1e6])
+def test_length_units_do_not_leave_the_float32_range(n_cams, s):
+    sc, m, _ = _system(n_cams, 60 * n_cams)
+    cams = sc.cams0.copy()
+    cams[:, 3:6] *= s
+    with binding.Problem(cams, sc.pts0 * s, sc.obs_cam, sc.obs_pt, m, precision="mixed") as p:
+        p.ba_build_normal(1e-4)
+        for args in SOLVES:
+            st = _solve(p, args, 1e-10)
+            assert st["status"] == 0 and st["true_rel_residual"] <= 1e-10, (args, st)
+
+
+# Residuals far from one in the kernels of an iteration (problems of up to 20 cameras run in one CTA).  The
+# true residual in double-float is good to 2^-48 |S| |x|, at most about 1e3 |b~| 2^-48 = 4e-12 |b~| here.
+@pytest.mark.parametrize("rel", [1e-3, 1e-6, 1e-9])
+def test_sweeps_on_small_residuals_converge_above_one_cta(rel):
+    sc, m, _ = _system(45, 2700, sigma=0.0, rel_perturb=rel)
+    with binding.Problem(sc.cams0, sc.pts0, sc.obs_cam, sc.obs_pt, m, precision="mixed") as p:
+        p.ba_build_normal(1e-4)
+        for args in SOLVES[:3]:
+            st = _solve(p, args, 1e-11)
+            assert st["status"] == 0 and st["true_rel_residual"] <= 1e-11, (args, st)
