@@ -1165,6 +1165,17 @@ int ba_gnn_launch_count(const ba_gnn* g, int64_t* n) {
     return BA_OK;
 }
 
+// For the tests, not in ba.h: solver_interrupt_products on the handle's lists.
+int ba_test_interrupt_products(ba_problem* p) {
+    if (!p || !p->solver) return BA_ERR_INVALID_ARG;
+    try {
+        ba::solver_interrupt_products(p->solver, p->stream);
+    } catch (const Error& e) {
+        return fail(p, e);
+    }
+    return BA_OK;
+}
+
 int ba_get_launch_count(const ba_problem* p, int64_t* n) {
     if (!p || !n) return BA_ERR_INVALID_ARG;
     *n = p->launches;

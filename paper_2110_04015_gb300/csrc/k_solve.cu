@@ -3457,6 +3457,21 @@ static void free_buf(Buf& b) {
 
 Solver* solver_create() { return new Solver(); }
 
+// A warp whose tile wait gave up left its work item uncounted, so its group's arrival counter did not return to
+// zero and the next product would take the last chunk too early (or never): a solve that timed out clears
+// the counters of every list.
+static void clear_counters(Solver* w, cudaStream_t st) {
+    for (ItemList* l : {&w->items_g, &w->items_l, &w->items_u})
+        if (l->cnt) BA_CUDA_TRY(cudaMemsetAsync(l->cnt, 0, sizeof(int) * l->ngrp, st));
+}
+
+void solver_interrupt_products(Solver* w, cudaStream_t st) {
+    for (ItemList* l : {&w->items_g, &w->items_l, &w->items_u})
+        if (l->cnt) BA_CUDA_TRY(cudaMemsetAsync(l->cnt, 1, sizeof(int) * l->ngrp, st));   // no group's count
+    clear_counters(w, st);
+    BA_CUDA_TRY(cudaStreamSynchronize(st));
+}
+
 void solver_destroy(Solver* w) {
     if (!w) return;
     Buf* bufs[] = {&w->P, &w->Q, &w->r, &w->z, &w->xw, &w->PT, &w->part_a, &w->part_b, &w->part_cam, &w->dpinv,
@@ -3999,10 +4014,7 @@ void solver_run(Solver* w, const Structure& s, const System& y, const SolveArgs&
         for (size_t i = 0; i < h.size(); ++i) h[i] = std::sqrt(w->h_hist[i * nb + b]);
     }
     if (timed_out) {
-        // a warp whose tile wait gave up left its work item uncounted, so its group's arrival counter
-        // did not return to zero: clear the counters for the next product
-        if (w->items_g.cnt) BA_CUDA_TRY(cudaMemsetAsync(w->items_g.cnt, 0, sizeof(int) * w->items_g.ngrp, st));
-        if (w->items_l.cnt) BA_CUDA_TRY(cudaMemsetAsync(w->items_l.cnt, 0, sizeof(int) * w->items_l.ngrp, st));
+        clear_counters(w, st);
         BA_CUDA_TRY(cudaStreamSynchronize(st));
         ++host_waits;
     }

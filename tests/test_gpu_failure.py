@@ -72,3 +72,21 @@ def test_nan_parameter_is_reported_not_solved(precision, where):
         p.ba_build_normal(1e-4)
         st = p.ba_solve_pcg(1e-6, 1000)
         assert st["status"] == 0 and st["true_rel_residual"] <= 1.5e-6
+
+
+# A product that gives up leaves the arrival counters of its split rows off, and the next one on the handle
+# must not see that: ba_test_interrupt_products sets the counters of every work list and clears them as
+# a timed-out solve does.  Items of 32 blocks split every row of 150 cameras, also of the upper triangle.
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_counters_of_an_interrupted_product_are_cleared(precision):
+    sc = scene("dense-small")
+    with problem.from_scene(sc, precision=precision, item_blocks=32) as p:
+        p.ba_build_normal(1e-4)
+        solves = (lambda: p.ba_solve_pcg(1e-6, 1000), lambda: p.ba_solve_mcg(1e-6, 1000, 8, 3.0))
+        for solve in solves:
+            st = solve()
+            assert st["status"] == 0
+            x = p.ba_get_delta().copy()
+            assert binding.lib().ba_test_interrupt_products(p.h) == 0
+            assert solve()["status"] == 0
+            assert np.array_equal(p.ba_get_delta(), x)
