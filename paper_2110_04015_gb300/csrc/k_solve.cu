@@ -3033,12 +3033,13 @@ struct GraphKey {
     int mcg = -1, fp32 = -1, chunk = 0, mi1 = 0, use_l = -1, epoch = -1, polls = -1, nb = -1, host = -1, cfg = -1;
     int lanes = -1;                   // column lanes of k_spmm
     int one = -1;                     // cameras of the largest problem that one CTA or cluster solves
+    int all = -1;                     // one of them solves every problem
     uint64_t allocs = ~uint64_t(0);   // buffer generation (any reallocation invalidates the graph)
     const void* ptrs[4] = {};
     bool operator==(const GraphKey& o) const {
         if (mcg != o.mcg || fp32 != o.fp32 || chunk != o.chunk || mi1 != o.mi1 || use_l != o.use_l ||
             epoch != o.epoch || polls != o.polls || nb != o.nb || host != o.host || cfg != o.cfg ||
-            lanes != o.lanes || one != o.one || allocs != o.allocs)
+            lanes != o.lanes || one != o.one || all != o.all || allocs != o.allocs)
             return false;
         for (int i = 0; i < 4; ++i) if (ptrs[i] != o.ptrs[i]) return false;
         return true;
@@ -3073,6 +3074,7 @@ struct Solver {
     int gpq = 1;              // grid width of the reorthogonalisation (32-row blocks)
     int gphi = 1, gb = 1;     // Phi and beta grid widths
     int one_cams = 0;         // cameras of the largest problem that k_one_cta or k_pcg_cluster solves (0: none)
+    bool all_small = false;   // one of those two solves every problem
     int gcol = 1;             // grid width of the column pass of the symmetric product (a CTA per camera)
     std::vector<Layout> lay;  // of the current solve
     Buf P, Q, r, z, xw, PT, part_a, part_b, part_cam, dpinv, beta, colblk, phip, hist, blk_off, blk_w, ctl, outer, rt,
@@ -3409,10 +3411,12 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     grow(w->phip, size_t(phoff) * sizeof(double));
     // the largest problem that k_one_cta (float32) or k_pcg_cluster (float64 PCG) solves
     w->one_cams = 0;
+    w->all_small = true;
     const int small = fp32 ? kOneCams : (a.mcg ? 0 : kCluCams);
-    if (a.wait_polls > 0)
-        for (const Layout& L : lay)
-            if (L.nc <= small) w->one_cams = std::max(w->one_cams, L.nc);
+    for (const Layout& L : lay) {
+        if (L.nc <= small && a.wait_polls > 0) w->one_cams = std::max(w->one_cams, L.nc);
+        else w->all_small = false;
+    }
     if (fp32 && w->one_cams > 0) grow(w->colblk, size_t(boff) * sizeof(int));
     grow(w->hist, size_t(nb) * w->mi1 * sizeof(double));
     grow(w->blk_off, size_t(nb) * w->mi1 * sizeof(int));
@@ -3627,12 +3631,10 @@ static int enqueue_iteration(Solver* w, const Structure& s, const T* S, const T*
     }
 }
 
-// x = 0, r = sign * rhs, z = D^{-1} r, P_0 = z, the control blocks and (q0) Q_0 = S P_0; returns the
-// launches.  Algorithm 2 starts its iterations from Q_0; Algorithm 1 forms Q = S P first in every
-// iteration, so its solves pass q0 = false.
+// x = 0, r = sign * rhs, z = D^{-1} r, P_0 = z and the control blocks; returns the launches.
 template <typename T>
 static int krylov_init(Solver* w, const Structure& s, const T* S, const T* Su, const double* Dinv, const double* rhs,
-                       double sign, const double* scale, T* x, const Outer* outer, cudaStream_t st, bool q0 = true) {
+                       double sign, const double* scale, T* x, const Outer* outer, cudaStream_t st) {
     const int nb = w->nb;
     k_init_vec<T><<<dim3(w->gu, nb), kUpdThreads, 0, st>>>(ptr<Layout>(w->lay_d), rhs, sign, scale, Dinv, outer, x,
                                                             ptr<T>(w->r), ptr<T>(w->z), ptr<T>(w->P),
@@ -3640,11 +3642,11 @@ static int krylov_init(Solver* w, const Structure& s, const T* S, const T* Su, c
     k_init_ctl<T><<<nb, 32, 0, st>>>(ptr<Ctl>(w->ctl), ptr<Layout>(w->lay_d), ptr<double>(w->part_b), w->gu,
                                   ptr<Params>(w->params), sizeof(T) == 4 ? kStagnation : 0.0, sizeof(T) == 4 ? 1 : 0,
                                   outer, ptr<int>(w->blk_off), ptr<int>(w->blk_w), w->mi1);
-    return 2 + (q0 ? enqueue_product<T, 0>(w, s, S, Su, ptr<T>(w->P), kSelLive, ptr<T>(w->Q), nullptr, st) : 0);
+    return 2;
 }
 
-// The solves of the problems that one CTA or one cluster solves, right after krylov_init (x: the float64
-// solution); returns the launches.
+// The solves of the problems that one CTA or one cluster solves, right after krylov_init (x: the solution
+// of a float64 solve); returns the launches.
 static int enqueue_small(Solver* w, const Structure& s, const System& y, bool mcg, double* x, cudaStream_t st) {
     if (w->one_cams == 0) return 0;
     if (y.S) {
@@ -3658,6 +3660,20 @@ static int enqueue_small(Solver* w, const Structure& s, const System& y, bool mc
         ptr<float>(w->P), ptr<float>(w->Q), ptr<double>(w->phip), ptr<double>(w->dpinv), ptr<float>(w->beta),
         ptr<int>(w->colblk), ptr<double>(w->hist), ptr<int>(w->blk_off), ptr<int>(w->blk_w), w->mi1, ptr<Ctl>(w->ctl));
     return 1;
+}
+
+// The start of a sweep: krylov_init, the problems that are solved whole, and Q_0 = S P_0 of the others, from
+// which Algorithm 2 starts its iterations (Algorithm 1 forms Q = S P first in every one).  Problems that are
+// solved whole form their own Q_0 and are done by then: they take part in no tile-streaming product,
+// so no tile wait can end them.  Returns the launches.
+template <typename T>
+static int krylov_start(Solver* w, const Structure& s, const System& y, const T* S, const T* Su, const double* Dinv,
+                        const double* rhs, double sign, const double* scale, T* x, const Outer* outer, bool mcg,
+                        cudaStream_t st) {
+    int n = krylov_init<T>(w, s, S, Su, Dinv, rhs, sign, scale, x, outer, st);
+    n += enqueue_small(w, s, y, mcg, sizeof(T) == 8 ? reinterpret_cast<double*>(x) : nullptr, st);
+    if (mcg && !w->all_small) n += enqueue_product<T, 0>(w, s, S, Su, ptr<T>(w->P), kSelLive, ptr<T>(w->Q), nullptr, st);
+    return n;
 }
 
 // true residual t = -b~ - S x into out (may be null) and, per problem, its norms into ctl (true_rr,
@@ -3716,8 +3732,7 @@ static void capture_krylov(Solver* w, const Structure& s, const System& y, const
                            const double* rhs, double sign, const double* scale, T* x, const Outer* outer, bool mcg,
                            int chunk, cudaStream_t cs, cudaStream_t cb, int* pre, int* per_pass) {
     const cudaGraphConditionalHandle h = capture_handle(cs);
-    *pre = krylov_init<T>(w, s, S, Su, Dinv, rhs, sign, scale, x, outer, cs, mcg) + 1;
-    *pre += enqueue_small(w, s, y, mcg, sizeof(T) == 8 ? reinterpret_cast<double*>(x) : nullptr, cs);
+    *pre = krylov_start<T>(w, s, y, S, Su, Dinv, rhs, sign, scale, x, outer, mcg, cs) + 1;
     k_loop_cond<<<1, kThreads, 0, cs>>>(h, 1, ptr<Ctl>(w->ctl), w->nb, ptr<Loops>(w->loops), 1, chunk,
                                         ptr<Params>(w->params));
     cudaGraph_t body = capture_while(cs, h);
@@ -3845,8 +3860,7 @@ static void run_host_loops(Solver* w, const Structure& s, const System& y, const
     const cudaGraphConditionalHandle none = cudaGraphConditionalHandle();
     int64_t launches = 0;
     if (!fp32) {
-        launches += krylov_init<double>(w, s, y.S, nullptr, y.Dinv, y.bt, -1.0, nullptr, x, nullptr, st, a.mcg != 0);
-        launches += enqueue_small(w, s, y, a.mcg != 0, x, st);
+        launches += krylov_start<double>(w, s, y, y.S, nullptr, y.Dinv, y.bt, -1.0, nullptr, x, nullptr, a.mcg != 0, st);
         k_loop_cond<<<1, kThreads, 0, st>>>(none, 0, ptr<Ctl>(w->ctl), nb, lp, 1, a.chunk, prm);
         launches += 1 + host_krylov_loop(w, chunk_exec, gc, a, st, waits);
         launches += true_residual(w, s, y, x, nullptr, st);
@@ -3862,9 +3876,8 @@ static void run_host_loops(Solver* w, const Structure& s, const System& y, const
             bool any = false;
             for (int b = 0; b < nb && !any; ++b) any = w->h_outer[b].swept != 0;
             if (!any) break;
-            launches += krylov_init<float>(w, s, y.S32, y.S32u, y.Dhat, ptr<double>(w->rt), 1.0, y.lam,
-                                           ptr<float>(w->xw), ptr<Outer>(w->outer), st, a.mcg != 0);
-            launches += enqueue_small(w, s, y, a.mcg != 0, nullptr, st);
+            launches += krylov_start<float>(w, s, y, y.S32, y.S32u, y.Dhat, ptr<double>(w->rt), 1.0, y.lam,
+                                            ptr<float>(w->xw), ptr<Outer>(w->outer), a.mcg != 0, st);
             k_loop_cond<<<1, kThreads, 0, st>>>(none, 0, ptr<Ctl>(w->ctl), nb, lp, 1, a.chunk, prm);
             launches += 1 + host_krylov_loop(w, chunk_exec, gc, a, st, waits);
             k_accumulate<<<dim3(w->gx, nb), kThreads, 0, st>>>(ptr<Layout>(w->lay_d), ptr<Outer>(w->outer),
@@ -3896,6 +3909,7 @@ static cudaGraphExec_t solve_graph(Solver* w, const Structure& s, const System& 
     key.host = a.host_loop;
     key.cfg = a.spmv_cfg;
     key.one = w->one_cams;
+    key.all = w->all_small;
     key.lanes = w->col_lanes;
     key.allocs = g_allocs.load();
     const void* ptrs[4] = {x, fp32 ? (const void*)y.S32 : (const void*)y.S, w->items_g.items, w->items_l.items};

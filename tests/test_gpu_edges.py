@@ -116,3 +116,18 @@ def test_sweeps_on_small_residuals_converge_above_one_cta(rel):
         for args in SOLVES[:3]:
             st = _solve(p, args, 1e-11)
             assert st["status"] == 0 and st["true_rel_residual"] <= 1e-11, (args, st)
+
+
+# A problem that one CTA solves waits for no tile, so its solve launches no tile-streaming product: a sweep by MCG
+# is as many launches as one by PCG (its start, the one CTA, the loop test, the true residual and the next
+# sweep's plan), after the three launches that start the refinement.
+def test_one_cta_solves_launch_no_product():
+    sc, m, _ = _system(13, 777)
+    with binding.Problem(sc.cams0, sc.pts0, sc.obs_cam, sc.obs_pt, m, precision="mixed") as p:
+        p.ba_build_normal(1e-4)
+        per_sweep = []
+        for args in (None, (8, 3.0), (4, 1e9)):
+            before = p.ba_get_launch_count()
+            sweeps = _solve(p, args, 1e-6)["refinements"]
+            per_sweep.append((p.ba_get_launch_count() - before - 3) / sweeps)
+        assert per_sweep[0] == per_sweep[1] == per_sweep[2], per_sweep
