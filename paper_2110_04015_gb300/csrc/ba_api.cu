@@ -1165,6 +1165,17 @@ int ba_gnn_launch_count(const ba_gnn* g, int64_t* n) {
     return BA_OK;
 }
 
+// For the tests, not in ba.h: sums of the float32 sweeps over a and b (n values, host or device).
+int ba_test_phi_sum(const float* a, const float* b, int32_t n, int32_t chunk, double* out) {
+    if (!a || !b || !out || n < 1 || chunk < 1) return BA_ERR_INVALID_ARG;
+    try {
+        ba::test_phi_sum(a, b, n, chunk, out);
+    } catch (const Error& e) {
+        return e.code;
+    }
+    return BA_OK;
+}
+
 // For the tests, not in ba.h: solver_interrupt_products on the handle's lists.
 int ba_test_interrupt_products(ba_problem* p) {
     if (!p || !p->solver) return BA_ERR_INVALID_ARG;

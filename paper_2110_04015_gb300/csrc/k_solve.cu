@@ -210,6 +210,67 @@ __device__ __forceinline__ ExactSum<T> warp_total(ExactSum<T> s) {
     return s;
 }
 
+// A sum over lanes, warps and CTAs that stays within a float64 sum's error.  A float pair loses 2^-48 of the
+// partial sum at every addition, against 2^-53 in float64; a third term keeps what the low parts' additions
+// round off (two-sums again, on the float32 pipe), so the additions lose about 2^-72 and the total is rounded
+// once, by value().  float64: the sum itself.
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {   // fl(a + b), e = its exact error
+    const float t = __fadd_rn(a, b), bv = __fsub_rn(t, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, bv)), __fsub_rn(b, bv));
+    return t;
+}
+template <typename T>
+struct WideSum;
+template <>
+struct WideSum<double> {
+    using Slot = double;   // as stored between kernels
+    double s = 0.0;
+    __device__ __forceinline__ WideSum() {}
+    __device__ __forceinline__ WideSum(const ExactSum<double>& a) : s(a.s) {}
+    __device__ __forceinline__ void add(double v) { s += v; }
+    __device__ __forceinline__ void add(const WideSum& b) { s += b.s; }
+    __device__ __forceinline__ WideSum shfl_xor(int o) const {
+        WideSum b;
+        b.s = __shfl_xor_sync(0xffffffffu, s, o);
+        return b;
+    }
+    __device__ __forceinline__ Slot slot() const { return s; }
+    __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct WideSum<float> {
+    using Slot = float4;
+    float hi = 0.f, lo = 0.f, c = 0.f;
+    __device__ __forceinline__ WideSum() {}
+    __device__ __forceinline__ WideSum(const ExactSum<float>& a) : hi(a.hi), lo(a.lo) {}
+    __device__ __forceinline__ void add3(float h, float l, float k) {
+        float te, ue, ve;
+        hi = two_sum(hi, h, te);
+        lo = two_sum(lo, l, ue);
+        lo = two_sum(lo, te, ve);
+        c = __fadd_rn(__fadd_rn(c, k), __fadd_rn(ue, ve));
+    }
+    __device__ __forceinline__ void add(const Slot& v) { add3(v.x, v.y, v.z); }
+    __device__ __forceinline__ void add(const WideSum& b) { add3(b.hi, b.lo, b.c); }
+    __device__ __forceinline__ WideSum shfl_xor(int o) const {
+        WideSum b;
+        b.hi = __shfl_xor_sync(0xffffffffu, hi, o);
+        b.lo = __shfl_xor_sync(0xffffffffu, lo, o);
+        b.c = __shfl_xor_sync(0xffffffffu, c, o);
+        return b;
+    }
+    __device__ __forceinline__ Slot slot() const { return make_float4(hi, lo, c, 0.f); }
+    __device__ __forceinline__ double value() const { return double(hi) + (double(lo) + double(c)); }
+};
+template <typename T>
+using WideSlot = typename WideSum<T>::Slot;
+template <typename T>
+__device__ __forceinline__ WideSum<T> warp_total(WideSum<T> s) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s.add(s.shfl_xor(o));
+    return s;
+}
+
 // Value k of the kThreads / 32 warp sums in red (row stride nv), added as a fixed tree
 // ((w0 + w1) + (w2 + w3)) + ((w4 + w5) + (w6 + w7)): three dependent float64 additions.
 __device__ __forceinline__ double sum_warps(const double* red, int nv, int k) {
@@ -1942,7 +2003,9 @@ __device__ void mcg_decide(Ctl* c, const double* tot, double* hist, int* blk_off
 }
 
 // partial sums of Q[:, c]^T z over row chunks inside each subset:
-// phip[(c * n_eff + s) * K + k] for c < hist_cols, as store_partial slots (grid: CTAs x problems).
+// phip[(c * n_eff + s) * K + k] for c < hist_cols, as WideSum slots (grid: CTAs x problems).  Q^T z nearly
+// cancels against all but the last blocks, so the lanes' sums are added as wide ones: with float pairs throughout
+// beta's error against 64-bit sums reached 9e-8 of its column (6e-8 with float64 or wide sums over the lanes).
 // Reads the whole history once, so it is bound by memory (L2 while the history fits): a warp takes one
 // row chunk of up to kPhiCols columns at once, 8 rows of each in flight (32 loads a lane), and reads z
 // once for all of them.  A column at a time with float64 shuffle trees ran at 2.1 TB/s (34 us on
@@ -1952,7 +2015,7 @@ __device__ void mcg_decide(Ctl* c, const double* tot, double* hist, int* blk_off
 constexpr int kPhiCols = 4;
 template <typename T, int NC>
 __device__ __forceinline__ void phi_columns(const T* __restrict__ qc, int64_t n, const T* __restrict__ zp, int r0, int r1,
-                                            double* __restrict__ out, int64_t ostride) {
+                                            WideSlot<T>* __restrict__ out, int64_t ostride) {
     const int lane = threadIdx.x & 31;
     constexpr int U = 8;
     ExactSum<T> acc[NC];
@@ -1973,14 +2036,14 @@ __device__ __forceinline__ void phi_columns(const T* __restrict__ qc, int64_t n,
     }
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-        acc[c] = warp_total(acc[c]);
-        if (lane == 0) store_partial(out + c * ostride, acc[c]);
+        const WideSum<T> s = warp_total(WideSum<T>(acc[c]));
+        if (lane == 0) out[c * ostride] = s.slot();
     }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_mcg_phi(const T* __restrict__ Q, const T* __restrict__ z,
-                                                      double* __restrict__ phip, const double* __restrict__ dpart,
+                                                      WideSlot<T>* __restrict__ phip, const double* __restrict__ dpart,
                                                       int gu, double* __restrict__ hist_out, int* __restrict__ blk_off,
                                                       int* __restrict__ blk_w, int mi1, Ctl* ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
@@ -2004,7 +2067,7 @@ __global__ void __launch_bounds__(kThreads) k_mcg_phi(const T* __restrict__ Q, c
     const int cz = (sz + K - 1) / K;
     const T* Qp = Q + c.lay.hoff;
     const T* zp = z + 9 * int64_t(c.lay.c0);
-    double* ph = phip + c.lay.phoff;
+    WideSlot<T>* ph = phip + c.lay.phoff;
     const int64_t warps = int64_t(gridDim.x - 1) * (kThreads / 32);
     const int nb = 2 * int64_t(hist) * chunks >= kPhiCols * warps ? kPhiCols : 1;   // columns at once
     const int64_t items = int64_t((hist + nb - 1) / nb) * chunks;   // below 2^31: the partials' buffer holds them
@@ -2016,7 +2079,7 @@ __global__ void __launch_bounds__(kThreads) k_mcg_phi(const T* __restrict__ Q, c
         const int send = (s + 1) * sz < nc ? (s + 1) * sz : nc;
         if (j1 > send) j1 = send;
         const T* qc = Qp + int64_t(c0) * n;
-        double* out = ph + int64_t(c0) * chunks + ch;
+        WideSlot<T>* out = ph + int64_t(c0) * chunks + ch;
         const int m = hist - c0 < nb ? hist - c0 : nb;
         if (m == kPhiCols) phi_columns<T, kPhiCols>(qc, n, zp, 9 * j0, 9 * j1, out, chunks);
         else
@@ -2029,26 +2092,26 @@ __global__ void __launch_bounds__(kThreads) k_mcg_phi(const T* __restrict__ Q, c
 // (t = 0 .. nt - 1, whole warps): G of them share an entry, each adds every G-th partial into two
 // interleaved sums, and the group's sums meet in a fixed shuffle tree.
 template <typename T>
-__device__ __forceinline__ void phi_block(const double* ph, int off, int w, int ne, int m, int n_eff, int K, bool local,
+__device__ __forceinline__ void phi_block(const WideSlot<T>* ph, int off, int w, int ne, int m, int n_eff, int K, bool local,
                                           int t, int nt, double* sphi) {
     int G = 1;
     while (G < 32 && 2 * G * ne <= nt) G *= 2;
     const int e = t / G, g = t % G;
     if (t - (t & 31) >= ne * G) return;   // warps without an entry (their shuffles go whole)
-    ExactSum<T> a0, a1;
+    WideSum<T> a0, a1;
     if (e < ne) {
         const int a = e / w, s2 = e - w * (e / w);
         const int64_t cc = off + a;
-        const double* sp = local ? ph + (cc * n_eff + s2) * K : ph + cc * n_eff * K;
+        const WideSlot<T>* sp = local ? ph + (cc * n_eff + s2) * K : ph + cc * n_eff * K;
         int k = g;
         for (; k + G < m; k += 2 * G) {
-            load_partial(a0, sp + k);
-            load_partial(a1, sp + k + G);
+            a0.add(sp[k]);
+            a1.add(sp[k + G]);
         }
-        if (k < m) load_partial(a0, sp + k);
+        if (k < m) a0.add(sp[k]);
     }
-    combine(a0, a1);
-    for (int o = G / 2; o > 0; o >>= 1) combine_shfl(a0, o);
+    a0.add(a1);
+    for (int o = G / 2; o > 0; o >>= 1) a0.add(a0.shfl_xor(o));
     if (e < ne && g == 0) sphi[e] = a0.value();
 }
 
@@ -2070,7 +2133,7 @@ __device__ __forceinline__ double beta_entry(const double* Dp, const double* sph
 // thread per entry), smaller ones a warp each.  With a warp per 16 x 16 block the 128 float64
 // multiply-adds of a warp were a chain of 13 us (2000 columns); 4.8 us with the CTA.
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_mcg_beta(const double* __restrict__ phip, const double* __restrict__ dpinv,
+__global__ void __launch_bounds__(kThreads) k_mcg_beta(const WideSlot<T>* __restrict__ phip, const double* __restrict__ dpinv,
                                                        const int* __restrict__ blk_off, const int* __restrict__ blk_w,
                                                        T* __restrict__ beta, const Ctl* __restrict__ ctl, int mi1) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
@@ -2086,7 +2149,7 @@ __global__ void __launch_bounds__(kThreads) k_mcg_beta(const double* __restrict_
     const int n_eff = c.n_eff, K = c.K, w = c.w_new;
     const bool local = c.local != 0;
     const int m = local ? K : n_eff * K;   // partials per Phi entry
-    const double* ph = phip + c.lay.phoff;
+    const WideSlot<T>* ph = phip + c.lay.phoff;
     const int* bo = blk_off + int64_t(p) * mi1;
     const int* bw = blk_w + int64_t(p) * mi1;
     T* Bp = beta + c.lay.boff * kMaxDirs;
@@ -2100,9 +2163,9 @@ __global__ void __launch_bounds__(kThreads) k_mcg_beta(const double* __restrict_
                 if (e0 == 0 && part == ne) phi_block<T>(ph, off, w, ne, m, n_eff, K, local, lane, 32, swarp[wid]);
                 else if (lane < part) {
                     const int e = e0 + lane, a = e / w, s2 = e - w * (e / w);
-                    const double* sp = local ? ph + (int64_t(off + a) * n_eff + s2) * K : ph + int64_t(off + a) * n_eff * K;
-                    ExactSum<T> a0;
-                    for (int k = 0; k < m; ++k) load_partial(a0, sp + k);
+                    const WideSlot<T>* sp = local ? ph + (int64_t(off + a) * n_eff + s2) * K : ph + int64_t(off + a) * n_eff * K;
+                    WideSum<T> a0;
+                    for (int k = 0; k < m; ++k) a0.add(sp[k]);
                     swarp[wid][e] = a0.value();
                 }
             }
@@ -3408,7 +3471,7 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     grow(w->part_cam, size_t(s.n_c) * 3 * sizeof(double));
     grow(w->dpinv, size_t(nb) * w->mi1 * kMaxDirs * kMaxDirs * sizeof(double));
     grow(w->beta, size_t(boff) * kMaxDirs * sizeof(double));
-    grow(w->phip, size_t(phoff) * sizeof(double));
+    grow(w->phip, size_t(phoff) * (fp32 ? sizeof(WideSlot<float>) : sizeof(WideSlot<double>)));
     // the largest problem that k_one_cta (float32) or k_pcg_cluster (float64 PCG) solves
     w->one_cams = 0;
     w->all_small = true;
@@ -3600,11 +3663,11 @@ static int enqueue_iteration(Solver* w, const Structure& s, const T* S, const T*
                        ptr<double>(w->dpinv), w->mi1);
         launch_chained(k_mcg_update<T>, dim3(w->gu, nb), dim3(kUpdThreads), 0, st, Dinv, P, Q, x, r, z,
                        ptr<double>(w->dpart), ctl);
-        launch_chained(k_mcg_phi<T>, dim3(w->gphi + 1, nb), dim3(kThreads), 0, st, Q, z, ptr<double>(w->phip),
+        launch_chained(k_mcg_phi<T>, dim3(w->gphi + 1, nb), dim3(kThreads), 0, st, Q, z, ptr<WideSlot<T>>(w->phip),
                        ptr<double>(w->dpart), w->gu, ptr<double>(w->hist), ptr<int>(w->blk_off),
                        ptr<int>(w->blk_w), w->mi1, ctl);
         T* betat = ptr<T>(w->beta);
-        launch_chained(k_mcg_beta<T>, dim3(w->gb, nb), dim3(kThreads), 0, st, ptr<double>(w->phip),
+        launch_chained(k_mcg_beta<T>, dim3(w->gb, nb), dim3(kThreads), 0, st, ptr<WideSlot<T>>(w->phip),
                        ptr<double>(w->dpinv), ptr<int>(w->blk_off), ptr<int>(w->blk_w), betat, ctl, w->mi1);
         if constexpr (sizeof(T) == 8) {
             // Eq. 18: Q_{i+1} = S Z_{i+1} - sum_j Q_j beta_{i,j}; S Z over whole rows for the
@@ -4077,6 +4140,35 @@ void flush_l2(cudaStream_t st) {
         BA_CUDA_TRY(cudaMemset(buf, 0, bytes));
     }
     k_l2_read<<<num_sms() * 8, 256, 0, st>>>(static_cast<const uint4*>(buf), int64_t(bytes / 16), sink);
+}
+
+// a^T b as the float32 sweeps add it (for the tests): a chunk of `chunk` rows per warp as in k_mcg_phi, then the
+// chunks as in k_mcg_beta.
+__global__ void k_test_phi(const float* a, const float* b, int n, int chunk, WideSlot<float>* slots) {
+    const int r0 = blockIdx.x * chunk;
+    phi_columns<float, 1>(a, n, b, r0, min(r0 + chunk, n), slots + blockIdx.x, 1);
+}
+__global__ void k_test_phi_block(const WideSlot<float>* slots, int chunks, double* out) {
+    phi_block<float>(slots, 0, 1, 1, chunks, 1, chunks, true, threadIdx.x, 32, out);
+}
+
+void test_phi_sum(const float* a, const float* b, int n, int chunk, double* out) {
+    const int chunks = (n + chunk - 1) / chunk;
+    Buf ab, slots;
+    grow(ab, sizeof(float) * 2 * size_t(n) + sizeof(double));
+    grow(slots, sizeof(WideSlot<float>) * size_t(chunks) + sizeof(double));
+    float* da = ptr<float>(ab);
+    double* d = reinterpret_cast<double*>(ptr<WideSlot<float>>(slots) + chunks);
+    cudaError_t e = cudaMemcpy(da, a, sizeof(float) * n, cudaMemcpyDefault);
+    if (e == cudaSuccess) e = cudaMemcpy(da + n, b, sizeof(float) * n, cudaMemcpyDefault);
+    if (e == cudaSuccess) {
+        k_test_phi<<<chunks, 32>>>(da, da + n, n, chunk, ptr<WideSlot<float>>(slots));
+        k_test_phi_block<<<1, 32>>>(ptr<WideSlot<float>>(slots), chunks, d);
+        e = cudaMemcpy(out, d, sizeof(double), cudaMemcpyDefault);
+    }
+    free_buf(ab);
+    free_buf(slots);
+    BA_CUDA_TRY(e);
 }
 
 // The PCG product q = S p of every problem (k_spmv MODE 1, the kernel of Algorithm 1; in float32 the

@@ -1,0 +1,51 @@
+"""Sums over lanes, warps and CTAs of the float32 sweeps keep the accuracy of float64 sums.
+
+A lane's products are exact as float pairs; adding the lanes must not lose more than a float64 sum does.
+With one product per lane the total is rounded once: half an ulp of a float64 for the last rounding, twice that
+for the low terms' own, and additions that lose 2^-72 of the partial sums each (fewer than 2^8 in a row).
+"""
+import ctypes
+import math
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+from paper_2110_04015_gb300 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+def _cancelling(n, seed):
+    """float32 a, b whose products nearly cancel: sum |a b| is about 1e6 |a^T b|."""
+    rs = np.random.RandomState(seed)
+    a = rs.standard_normal(n).astype(np.float32)
+    b = rs.standard_normal(n).astype(np.float32)
+    h = n // 2
+    b[h:2 * h] = b[:h]
+    a[h:2 * h] = (-a[:h].astype(np.float64) * (1 + 1e-6 * rs.standard_normal(h))).astype(np.float32)
+    return a, b
+
+
+def _exact(a, b):
+    s = sum((Fraction(float(x)) * Fraction(float(y)) for x, y in zip(a, b)), Fraction(0))
+    t = math.fsum(np.abs(a.astype(np.float64) * b.astype(np.float64)))
+    return s, t
+
+
+def _ptr(v):
+    return ctypes.c_void_p(v.ctypes.data)
+
+
+def _within(got, a, b):
+    s, t = _exact(a, b)
+    return abs(Fraction(got) - s) <= Fraction(2) ** -52 * abs(s) + Fraction(2) ** -64 * Fraction(t)
+
+
+@pytest.mark.parametrize("n, chunk", [(9, 9), (32, 32), (126, 18), (1000, 27), (9000, 27), (4001, 32)])
+def test_phi_sums_are_as_accurate_as_float64(n, chunk):
+    for seed in range(4):
+        a, b = _cancelling(n, seed)
+        out = ctypes.c_double()
+        assert binding.lib().ba_test_phi_sum(_ptr(a), _ptr(b), n, chunk, ctypes.byref(out)) == 0
+        assert _within(out.value, a, b), (seed, out.value)
