@@ -219,6 +219,15 @@ __device__ __forceinline__ float two_sum(float a, float b, float& e) {   // fl(a
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, bv)), __fsub_rn(b, bv));
     return t;
 }
+// a float32 as float64, from its bits: a conversion instruction runs on the float64 pipe (about 150 cycles), this
+// on the integer pipe.  Subnormals (below 1e-38 of sums that start near one) become zero.
+__device__ __forceinline__ double widen(float f) {
+    const int b = __float_as_int(f), e = b & 0x7f800000;
+    if (e == 0x7f800000) return double(f);   // infinities and NaN
+    if (e == 0) return 0.0;
+    return __longlong_as_double(((static_cast<long long>(b & 0x7fffffff) + (896ll << 23)) << 29) |
+                                (static_cast<long long>(b & int(0x80000000)) << 32));
+}
 template <typename T>
 struct WideSum;
 template <>
@@ -227,6 +236,7 @@ struct WideSum<double> {
     double s = 0.0;
     __device__ __forceinline__ WideSum() {}
     __device__ __forceinline__ WideSum(const ExactSum<double>& a) : s(a.s) {}
+    __device__ __forceinline__ void set(double v) { s = v; }
     __device__ __forceinline__ void add(double v) { s += v; }
     __device__ __forceinline__ void add(const WideSum& b) { s += b.s; }
     __device__ __forceinline__ WideSum shfl_xor(int o) const {
@@ -250,6 +260,7 @@ struct WideSum<float> {
         lo = two_sum(lo, te, ve);
         c = __fadd_rn(__fadd_rn(c, k), __fadd_rn(ue, ve));
     }
+    __device__ __forceinline__ void set(const Slot& v) { hi = v.x, lo = v.y, c = v.z; }
     __device__ __forceinline__ void add(const Slot& v) { add3(v.x, v.y, v.z); }
     __device__ __forceinline__ void add(const WideSum& b) { add3(b.hi, b.lo, b.c); }
     __device__ __forceinline__ WideSum shfl_xor(int o) const {
@@ -260,10 +271,22 @@ struct WideSum<float> {
         return b;
     }
     __device__ __forceinline__ Slot slot() const { return make_float4(hi, lo, c, 0.f); }
-    __device__ __forceinline__ double value() const { return double(hi) + (double(lo) + double(c)); }
+    __device__ __forceinline__ double value() const { return widen(hi) + (widen(lo) + widen(c)); }
 };
 template <typename T>
 using WideSlot = typename WideSum<T>::Slot;
+// the sum in a slot of store_partial
+template <typename T>
+__device__ __forceinline__ WideSum<T> pair_of(double slot) {
+    WideSum<T> s;
+    if constexpr (sizeof(T) == 4) {
+        s.hi = __int_as_float(__double2loint(slot));
+        s.lo = __int_as_float(__double2hiint(slot));
+    } else {
+        s.s = slot;
+    }
+    return s;
+}
 template <typename T>
 __device__ __forceinline__ WideSum<T> warp_total(WideSum<T> s) {
 #pragma unroll
@@ -296,11 +319,11 @@ __device__ __forceinline__ void cta_sum_write(double (&v)[NV], double* out) {
     __syncthreads();
 }
 
-// Sum of the Gram-style partials slots[0 .. np) in a fixed order (one warp; every lane returns it).
+// Sum of the slots [0 .. np) in a fixed order (one warp; every lane returns it).
 template <typename T>
-__device__ __forceinline__ ExactSum<T> warp_sum_slots(const double* slots, int np) {
-    ExactSum<T> s;
-    for (int p = threadIdx.x & 31; p < np; p += 32) load_partial(s, slots + p);
+__device__ __forceinline__ WideSum<T> warp_sum_slots(const WideSlot<T>* slots, int np) {
+    WideSum<T> s;
+    for (int p = threadIdx.x & 31; p < np; p += 32) s.add(slots[p]);
     return warp_total(s);
 }
 
@@ -376,12 +399,13 @@ __device__ __forceinline__ bool nothing_selected(const Ctl* ctl, const ItemList&
     return !__any_sync(0xffffffffu, any);
 }
 
-// Sum the CTA's NV values (kUpdThreads threads) into partial[blockIdx.x * NV ..] (store_partial slots).
+// Sum the CTA's NV values (kUpdThreads threads) into partial[blockIdx.x * NV ..], as accurately as in float64
+// (a thread's value is one product, exact as a pair).
 // Warp k adds value k: 3 additions and one shuffle tree per value instead of a tree in every warp.
 // The next kernel adds the CTAs' partials (total_of): with the last CTA to arrive doing it here, its
 // fences, its counter and a second round of loads held an update for 3 us.
 template <typename T, int NV>
-__device__ __forceinline__ void cta_publish(const ExactSum<T> (&v)[NV], double* partial) {
+__device__ __forceinline__ void cta_publish(const ExactSum<T> (&v)[NV], WideSlot<T>* partial) {
     static_assert(NV <= kUpdThreads / 32, "one warp per value");
     __shared__ double st[NV][kUpdThreads];   // slots of store_partial
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -389,26 +413,39 @@ __device__ __forceinline__ void cta_publish(const ExactSum<T> (&v)[NV], double* 
     for (int k = 0; k < NV; ++k) store_partial(&st[k][threadIdx.x], v[k]);
     __syncthreads();
     if (wid < NV) {
-        ExactSum<T> s;
-#pragma unroll
-        for (int u = 0; u < kUpdThreads / 32; ++u) load_partial(s, &st[wid][lane + 32 * u]);
+        static_assert(kUpdThreads == 128, "four values a lane");
+        WideSum<T> s = pair_of<T>(st[wid][lane]);
+        s.add(pair_of<T>(st[wid][lane + 32]));
+        if constexpr (sizeof(T) == 4) {   // two chains: a wide addition is a dozen dependent operations
+            WideSum<T> s2 = pair_of<T>(st[wid][lane + 64]);
+            s2.add(pair_of<T>(st[wid][lane + 96]));
+            s.add(s2);
+        } else {
+            s.add(pair_of<T>(st[wid][lane + 64]));
+            s.add(pair_of<T>(st[wid][lane + 96]));
+        }
         s = warp_total(s);
-        if (lane == 0) store_partial(partial + int64_t(blockIdx.x) * NV + wid, s);
+        if (lane == 0) partial[int64_t(blockIdx.x) * NV + wid] = s.slot();
     }
 }
 
 // Total of value k over np CTA partials (one warp; every lane returns it): lane l adds partials
 // l, l + 32, ..., eight loads in flight, then the fixed shuffle tree.
 template <typename T, int NV>
-__device__ __forceinline__ ExactSum<T> total_of(const double* partial, int np, int k) {
-    ExactSum<T> s;
-    for (int b = threadIdx.x & 31; b < np; b += 8 * 32) {
-        double v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = b + 32 * u < np ? partial[int64_t(b + 32 * u) * NV + k] : 0.0;
+__device__ __forceinline__ WideSum<T> total_of(const WideSlot<T>* partial, int np, int k) {
+    WideSum<T> s;
+    const int lane = threadIdx.x & 31;
+    for (int b0 = 0; b0 < np; b0 += 8 * 32) {
+        WideSlot<T> v[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-            if (b + 32 * u < np) add_slot(s, v[u]);
+            v[u] = b0 + 32 * u + lane < np ? partial[int64_t(b0 + 32 * u + lane) * NV + k] : WideSlot<T>{};
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (b0 + 32 * u < np) {   // the same in every lane; past np the slots are zero
+                if (b0 == 0 && u == 0) s.set(v[u]);
+                else s.add(v[u]);
+            }
     }
     return warp_total(s);
 }
@@ -1130,10 +1167,9 @@ __global__ void __launch_bounds__(kUpdThreads) k_init_vec(const Layout* __restri
                                                           double sign, const double* __restrict__ scale,
                                                           const double* __restrict__ Dinv, const Outer* __restrict__ outer,
                                                           T* __restrict__ x, T* __restrict__ r, T* __restrict__ z,
-                                                          T* __restrict__ P, double* __restrict__ partial) {
+                                                          T* __restrict__ P, WideSlot<T>* __restrict__ partial) {
     const Layout L = lay[blockIdx.y];
     __shared__ T sr[kUpdCams * 9];
-    __shared__ double st[kUpdThreads];
     const int t = threadIdx.x, cl = t / 9, a = t - 9 * (t / 9);
     const int64_t jl = int64_t(blockIdx.x) * kUpdCams + cl;
     const bool act = t < kUpdCams * 9 && jl < L.nc;
@@ -1148,25 +1184,21 @@ __global__ void __launch_bounds__(kUpdThreads) k_init_vec(const Layout* __restri
         x[i] = T(0);
     }
     if (t < kUpdCams * 9) sr[t] = rv;
-    ExactSum<T> v;
-    v.add(rv, rv);
-    store_partial(&st[t], v);
+    ExactSum<T> v[1];
+    v[0].add(rv, rv);
     __syncthreads();
     if (act) {
         const T zs = D.dot(sr + 9 * cl);
         z[i] = zs;
         P[L.hoff + 9 * jl + a] = zs;
     }
-    if (t < 32) {
-        const ExactSum<T> s = warp_sum_slots<T>(st, kUpdThreads);
-        if (t == 0) store_partial(partial + int64_t(blockIdx.y) * gridDim.x + blockIdx.x, s);
-    }
+    cta_publish<T, 1>(v, partial + int64_t(blockIdx.y) * gridDim.x);
 }
 
 // One warp per problem.  outer (mixed precision, may be null) supplies the sweep's tolerance and
 // iteration budget and leaves the problems that are not refined any more done from the start.
 template <typename T>
-__global__ void k_init_ctl(Ctl* ctl, const Layout* __restrict__ lay, const double* __restrict__ partial, int np,
+__global__ void k_init_ctl(Ctl* ctl, const Layout* __restrict__ lay, const WideSlot<T>* __restrict__ partial, int np,
                            const Params* __restrict__ prm, double stag, int direct_q,
                            const Outer* __restrict__ outer, int* blk_off, int* blk_w, int mi1) {
     const int p = blockIdx.x;
@@ -1337,8 +1369,8 @@ __global__ void __launch_bounds__(kUpdThreads) k_pcg_update(const double* __rest
                                                             const T* __restrict__ Q, T* __restrict__ x,
                                                             T* __restrict__ r, T* __restrict__ z,
                                                             const double* __restrict__ camdot,
-                                                            double* __restrict__ dpart, double* __restrict__ dtot,
-                                                            Ctl* ctl) {
+                                                            WideSlot<T>* __restrict__ dpart,
+                                                            double* __restrict__ dtot, Ctl* ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const int p = blockIdx.y;
     const Ctl& c = ctl[p];
@@ -1416,7 +1448,7 @@ __device__ void pcg_decide(Ctl* c, double D, double g, const double* tot, double
 // another warp than beta (a problem that ends there gets one more direction, which nothing reads).
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_pcg_dir(const T* __restrict__ z, T* __restrict__ P,
-                                                      const double* __restrict__ dpart, int gu,
+                                                      const WideSlot<T>* __restrict__ dpart, int gu,
                                                       const double* __restrict__ dtot, double* __restrict__ hist,
                                                       Ctl* ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
@@ -1439,8 +1471,8 @@ __global__ void __launch_bounds__(kThreads) k_pcg_dir(const T* __restrict__ z, T
     load_partial(D, dtot + 2 * int64_t(p));
     load_partial(g, dtot + 2 * int64_t(p) + 1);
     const int wid = threadIdx.x >> 5;
-    if (wid < 3) {
-        const ExactSum<T> s = total_of<T, 3>(dpart + int64_t(p) * gu * 3, (nc + kUpdCams - 1) / kUpdCams, wid);
+    if (wid == 1 || (wid < 3 && blockIdx.x == 0)) {   // every CTA needs q^T z, the stop test the others
+        const WideSum<T> s = total_of<T, 3>(dpart + int64_t(p) * gu * 3, (nc + kUpdCams - 1) / kUpdCams, wid);
         if ((threadIdx.x & 31) == 0) tot[wid] = s.value();
         if (wid == 1 && (threadIdx.x & 31) == 0) sbeta = T(s.value() * fast_rcp<2>(D.value()));
     }
@@ -1889,7 +1921,8 @@ template <typename T>
 __global__ void __launch_bounds__(kUpdThreads) k_mcg_update(const double* __restrict__ Dinv, const T* __restrict__ P,
                                                             const T* __restrict__ Q, T* __restrict__ x,
                                                             T* __restrict__ r, T* __restrict__ z,
-                                                            double* __restrict__ dpart, const Ctl* __restrict__ ctl) {
+                                                            WideSlot<T>* __restrict__ dpart,
+                                                            const Ctl* __restrict__ ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const int p = blockIdx.y;
     const Ctl& c = ctl[p];
@@ -2043,8 +2076,8 @@ __device__ __forceinline__ void phi_columns(const T* __restrict__ qc, int64_t n,
 
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_mcg_phi(const T* __restrict__ Q, const T* __restrict__ z,
-                                                      WideSlot<T>* __restrict__ phip, const double* __restrict__ dpart,
-                                                      int gu, double* __restrict__ hist_out, int* __restrict__ blk_off,
+                                                      WideSlot<T>* __restrict__ phip,
+                                                      const WideSlot<T>* __restrict__ dpart, int gu, double* __restrict__ hist_out, int* __restrict__ blk_off,
                                                       int* __restrict__ blk_w, int mi1, Ctl* ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const int p = blockIdx.y;
@@ -2055,7 +2088,7 @@ __global__ void __launch_bounds__(kThreads) k_mcg_phi(const T* __restrict__ Q, c
         __shared__ double tot[2];
         const int wid = threadIdx.x >> 5;
         if (wid < 2) {
-            const ExactSum<T> s = total_of<T, 2>(dpart + int64_t(p) * gu * 2, (nc + kUpdCams - 1) / kUpdCams, wid);
+            const WideSum<T> s = total_of<T, 2>(dpart + int64_t(p) * gu * 2, (nc + kUpdCams - 1) / kUpdCams, wid);
             if ((threadIdx.x & 31) == 0) tot[wid] = s.value();
         }
         __syncthreads();
@@ -2373,7 +2406,7 @@ struct OneSmem {
     // the current block and its image (one_at), zero past its width up to a multiple of four
     __align__(16) float PT[kOneRows * kMaxDirs + 4 * kOneCams], QT[kOneRows * kMaxDirs + 4 * kOneCams];
     float x[kOneRows], r[kOneRows], z[kOneRows];
-    double st[kOneThreads];
+    __align__(16) double st[kOneThreads];
     double tot[4];
     float scal[2], al[kMaxDirs];
 };
@@ -2438,31 +2471,31 @@ __device__ __forceinline__ void one_product(const float* S, OneSmem& m, int nc, 
     }
 }
 
-// Sums of NV values over the rows (threads 0 .. kOneRows - 1 hold them, zeros past the problem), the
+// Sums of NV values over the rows (threads 0 .. kOneRows - 1 hold a product each, zeros past the problem), the
 // same in every thread.  Contains a barrier before and after the sums are read.
 template <int NV>
-__device__ __forceinline__ void one_sums(ExactSum<float> (&v)[NV], double* st) {
+__device__ __forceinline__ void one_sums(const ExactSum<float> (&v)[NV], WideSum<float> (&sum)[NV], float4* st) {
     constexpr int NWR = (kOneRows + 31) / 32;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (wid < NWR) {
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
-            v[k] = warp_total(v[k]);
-            if (lane == 0) store_partial(&st[NV * wid + k], v[k]);
+            const WideSum<float> s = warp_total(WideSum<float>(v[k]));
+            if (lane == 0) st[NV * wid + k] = s.slot();
         }
     }
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
-        ExactSum<float> a, b;
+        WideSum<float> a, b;
         static_assert(NWR % 2 == 0, "pairs of warps");
 #pragma unroll
         for (int q = 0; q < NWR; q += 2) {
-            load_partial(a, &st[NV * q + k]);
-            load_partial(b, &st[NV * (q + 1) + k]);
+            a.add(st[NV * q + k]);
+            b.add(st[NV * (q + 1) + k]);
         }
-        combine(a, b);
-        v[k] = a;
+        a.add(b);
+        sum[k] = a;
     }
     __syncthreads();
 }
@@ -2514,8 +2547,9 @@ __global__ void __launch_bounds__(kOneThreads, 1)
                 d[0].add(m.QT[own_at], m.PT[own_at]);
                 d[1].add(m.PT[own_at], m.r[t]);
             }
-            one_sums<2>(d, m.st);
-            const float alpha = __fdiv_rn(__fadd_rn(d[1].hi, d[1].lo), __fadd_rn(d[0].hi, d[0].lo));
+            WideSum<float> dg[2];
+            one_sums<2>(d, dg, reinterpret_cast<float4*>(m.st));
+            const float alpha = __fdiv_rn(__fadd_rn(dg[1].hi, dg[1].lo), __fadd_rn(dg[0].hi, dg[0].lo));
             ExactSum<float> v[3];
             float rv = 0.f, qv = 0.f;
             if (act) {
@@ -2532,13 +2566,14 @@ __global__ void __launch_bounds__(kOneThreads, 1)
                 v[1].add(qv, zs);
                 v[2].add(rv, zs);
             }
-            one_sums<3>(v, m.st);
-            if (t == 0) m.scal[0] = float(v[1].value() * fast_rcp<2>(d[0].value()));
+            WideSum<float> vs[3];
+            one_sums<3>(v, vs, reinterpret_cast<float4*>(m.st));
+            if (t == 0) m.scal[0] = float(vs[1].value() * fast_rcp<2>(dg[0].value()));
             if (t == 32) {   // the stop test beside it
-                m.tot[0] = v[0].value();
-                m.tot[1] = v[1].value();
-                m.tot[2] = v[2].value();
-                pcg_decide(&m.c, d[0].value(), d[1].value(), m.tot, hist, p, gridDim.x);
+                m.tot[0] = vs[0].value();
+                m.tot[1] = vs[1].value();
+                m.tot[2] = vs[2].value();
+                pcg_decide(&m.c, dg[0].value(), dg[1].value(), m.tot, hist, p, gridDim.x);
             }
             __syncthreads();
             if (m.c.done) break;
@@ -2629,10 +2664,11 @@ __global__ void __launch_bounds__(kOneThreads, 1)
                 m.z[t] = zs;
                 v[1].add(m.r[t], zs);
             }
-            one_sums<2>(v, m.st);
+            WideSum<float> vs[2];
+            one_sums<2>(v, vs, reinterpret_cast<float4*>(m.st));
             if (t == 0) {
-                m.tot[0] = v[0].value();
-                m.tot[1] = v[1].value();
+                m.tot[0] = vs[0].value();
+                m.tot[1] = vs[1].value();
                 m.c.hist_cols = m.c.cols;
                 mcg_decide(&m.c, m.tot, hist, blk_off, blk_w, mi1, p, gridDim.x);
             }
@@ -3467,11 +3503,12 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     grow(w->xw, size_t(n) * elt);
     grow(w->PT, size_t(n) * kMaxDirs * elt);
     grow(w->part_a, size_t(nb) * w->gg * kGramMax * sizeof(double));
-    grow(w->part_b, size_t(nb) * w->gu * sizeof(double));
+    const size_t wide = fp32 ? sizeof(WideSlot<float>) : sizeof(WideSlot<double>);
+    grow(w->part_b, size_t(nb) * w->gu * wide);
     grow(w->part_cam, size_t(s.n_c) * 3 * sizeof(double));
     grow(w->dpinv, size_t(nb) * w->mi1 * kMaxDirs * kMaxDirs * sizeof(double));
     grow(w->beta, size_t(boff) * kMaxDirs * sizeof(double));
-    grow(w->phip, size_t(phoff) * (fp32 ? sizeof(WideSlot<float>) : sizeof(WideSlot<double>)));
+    grow(w->phip, size_t(phoff) * wide);
     // the largest problem that k_one_cta (float32) or k_pcg_cluster (float64 PCG) solves
     w->one_cams = 0;
     w->all_small = true;
@@ -3489,7 +3526,7 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     grow(w->rt, size_t(n) * sizeof(double));
     const void* lay_p = w->lay_d.p;
     grow(w->lay_d, size_t(nb) * sizeof(Layout));
-    grow(w->dpart, size_t(nb) * w->gu * 3 * sizeof(double));
+    grow(w->dpart, size_t(nb) * w->gu * 3 * wide);
     grow(w->dtot, size_t(nb) * 2 * sizeof(double));
     grow(w->camdot, size_t(s.n_c) * 2 * sizeof(double));
     grow(w->params, sizeof(Params));
@@ -3652,8 +3689,8 @@ static int enqueue_iteration(Solver* w, const Structure& s, const T* S, const T*
     if (!mcg) {
         const int np = enqueue_product<T, 1>(w, s, S, Su, P, kSelLive, Q, r, st);
         launch_chained(k_pcg_update<T>, dim3(w->gu, nb), dim3(kUpdThreads), 0, st, Dinv, P, Q, x, r, z,
-                       ptr<double>(w->camdot), ptr<double>(w->dpart), ptr<double>(w->dtot), ctl);
-        launch_chained(k_pcg_dir<T>, dim3(w->gq, nb), dim3(kThreads), 0, st, z, P, ptr<double>(w->dpart), w->gu,
+                       ptr<double>(w->camdot), ptr<WideSlot<T>>(w->dpart), ptr<double>(w->dtot), ctl);
+        launch_chained(k_pcg_dir<T>, dim3(w->gq, nb), dim3(kThreads), 0, st, z, P, ptr<WideSlot<T>>(w->dpart), w->gu,
                        ptr<double>(w->dtot), ptr<double>(w->hist), ctl);
         return np + 2;
     } else {
@@ -3662,9 +3699,9 @@ static int enqueue_iteration(Solver* w, const Structure& s, const T* S, const T*
         launch_chained(k_mcg_small<T>, dim3(nb * kSmallCtas), dim3(kSmallThreads), 0, st, ctl, ptr<double>(w->part_a), w->gg,
                        ptr<double>(w->dpinv), w->mi1);
         launch_chained(k_mcg_update<T>, dim3(w->gu, nb), dim3(kUpdThreads), 0, st, Dinv, P, Q, x, r, z,
-                       ptr<double>(w->dpart), ctl);
+                       ptr<WideSlot<T>>(w->dpart), ctl);
         launch_chained(k_mcg_phi<T>, dim3(w->gphi + 1, nb), dim3(kThreads), 0, st, Q, z, ptr<WideSlot<T>>(w->phip),
-                       ptr<double>(w->dpart), w->gu, ptr<double>(w->hist), ptr<int>(w->blk_off),
+                       ptr<WideSlot<T>>(w->dpart), w->gu, ptr<double>(w->hist), ptr<int>(w->blk_off),
                        ptr<int>(w->blk_w), w->mi1, ctl);
         T* betat = ptr<T>(w->beta);
         launch_chained(k_mcg_beta<T>, dim3(w->gb, nb), dim3(kThreads), 0, st, ptr<WideSlot<T>>(w->phip),
@@ -3701,8 +3738,8 @@ static int krylov_init(Solver* w, const Structure& s, const T* S, const T* Su, c
     const int nb = w->nb;
     k_init_vec<T><<<dim3(w->gu, nb), kUpdThreads, 0, st>>>(ptr<Layout>(w->lay_d), rhs, sign, scale, Dinv, outer, x,
                                                             ptr<T>(w->r), ptr<T>(w->z), ptr<T>(w->P),
-                                                            ptr<double>(w->part_b));
-    k_init_ctl<T><<<nb, 32, 0, st>>>(ptr<Ctl>(w->ctl), ptr<Layout>(w->lay_d), ptr<double>(w->part_b), w->gu,
+                                                            ptr<WideSlot<T>>(w->part_b));
+    k_init_ctl<T><<<nb, 32, 0, st>>>(ptr<Ctl>(w->ctl), ptr<Layout>(w->lay_d), ptr<WideSlot<T>>(w->part_b), w->gu,
                                   ptr<Params>(w->params), sizeof(T) == 4 ? kStagnation : 0.0, sizeof(T) == 4 ? 1 : 0,
                                   outer, ptr<int>(w->blk_off), ptr<int>(w->blk_w), w->mi1);
     return 2;
@@ -4152,19 +4189,34 @@ __global__ void k_test_phi_block(const WideSlot<float>* slots, int chunks, doubl
     phi_block<float>(slots, 0, 1, 1, chunks, 1, chunks, true, threadIdx.x, 32, out);
 }
 
-void test_phi_sum(const float* a, const float* b, int n, int chunk, double* out) {
+// a^T b as k_pcg_update and k_pcg_dir add it: a product per thread, kUpdThreads a CTA
+__global__ void __launch_bounds__(kUpdThreads) k_test_update(const float* a, const float* b, int n, WideSlot<float>* slots) {
+    const int i = blockIdx.x * kUpdThreads + threadIdx.x;
+    ExactSum<float> v[1];
+    if (i < n) v[0].add(a[i], b[i]);
+    cta_publish<float, 1>(v, slots);
+}
+__global__ void k_test_update_total(const WideSlot<float>* slots, int np, double* out) {
+    const WideSum<float> s = total_of<float, 1>(slots, np, 0);
+    if (threadIdx.x == 0) *out = s.value();
+}
+
+void test_float_sums(const float* a, const float* b, int n, int chunk, double* out) {
     const int chunks = (n + chunk - 1) / chunk;
     Buf ab, slots;
     grow(ab, sizeof(float) * 2 * size_t(n) + sizeof(double));
-    grow(slots, sizeof(WideSlot<float>) * size_t(chunks) + sizeof(double));
+    const int ctas = (n + kUpdThreads - 1) / kUpdThreads, most = std::max(chunks, ctas);
+    grow(slots, sizeof(WideSlot<float>) * size_t(most) + 2 * sizeof(double));
     float* da = ptr<float>(ab);
-    double* d = reinterpret_cast<double*>(ptr<WideSlot<float>>(slots) + chunks);
+    double* d = reinterpret_cast<double*>(ptr<WideSlot<float>>(slots) + most);
     cudaError_t e = cudaMemcpy(da, a, sizeof(float) * n, cudaMemcpyDefault);
     if (e == cudaSuccess) e = cudaMemcpy(da + n, b, sizeof(float) * n, cudaMemcpyDefault);
     if (e == cudaSuccess) {
         k_test_phi<<<chunks, 32>>>(da, da + n, n, chunk, ptr<WideSlot<float>>(slots));
         k_test_phi_block<<<1, 32>>>(ptr<WideSlot<float>>(slots), chunks, d);
-        e = cudaMemcpy(out, d, sizeof(double), cudaMemcpyDefault);
+        k_test_update<<<ctas, kUpdThreads>>>(da, da + n, n, ptr<WideSlot<float>>(slots));
+        k_test_update_total<<<1, 32>>>(ptr<WideSlot<float>>(slots), ctas, d + 1);
+        e = cudaMemcpy(out, d, 2 * sizeof(double), cudaMemcpyDefault);
     }
     free_buf(ab);
     free_buf(slots);

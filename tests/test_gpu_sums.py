@@ -46,6 +46,16 @@ def _within(got, a, b):
 def test_phi_sums_are_as_accurate_as_float64(n, chunk):
     for seed in range(4):
         a, b = _cancelling(n, seed)
-        out = ctypes.c_double()
-        assert binding.lib().ba_test_phi_sum(_ptr(a), _ptr(b), n, chunk, ctypes.byref(out)) == 0
-        assert _within(out.value, a, b), (seed, out.value)
+        out = (ctypes.c_double * 2)()
+        assert binding.lib().ba_test_float_sums(_ptr(a), _ptr(b), n, chunk, out) == 0
+        assert _within(out[0], a, b), (seed, out[0])
+
+
+# |r|^2, r^T z and q^T z: a product per thread, so any n
+@pytest.mark.parametrize("n", [1, 126, 128, 129, 9000, 17424, 40000])
+def test_update_sums_are_as_accurate_as_float64(n):
+    for seed in range(3):
+        a, b = _cancelling(n, seed)
+        out = (ctypes.c_double * 2)()
+        assert binding.lib().ba_test_float_sums(_ptr(a), _ptr(b), n, 32, out) == 0
+        assert _within(out[1], a, b), (seed, out[1])
