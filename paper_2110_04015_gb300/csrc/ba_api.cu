@@ -1165,7 +1165,7 @@ int ba_gnn_launch_count(const ba_gnn* g, int64_t* n) {
     return BA_OK;
 }
 
-// For the tests, not in ba.h: the sums a^T b of the float32 sweeps (n values, host or device) into out[0..1].
+// For the tests, not in ba.h: the sums a^T b of the float32 sweeps (n values, host or device) into out[0..2].
 int ba_test_float_sums(const float* a, const float* b, int32_t n, int32_t chunk, double* out) {
     if (!a || !b || !out || n < 1 || chunk < 1) return BA_ERR_INVALID_ARG;
     try {

@@ -248,8 +248,8 @@ Solver* solver_create();
 // Leaves the products' arrival counters as an interrupted product may and clears them as a timed-out solve
 // does (for the tests: no input makes a tile wait run out in one warp and not in another).
 void solver_interrupt_products(Solver* w, cudaStream_t st);
-// a^T b of n float32 values by the sums of the reorthogonalisation, `chunk` rows a warp, and by those of the
-// update kernels, into out[0] and out[1] (for the tests).
+// a^T b of n float32 values by the sums of the reorthogonalisation, `chunk` rows a warp, by those of the
+// update kernels and (of whole cameras' 9 values) by the one-CTA sweep's, into out[0 .. 2] (for the tests).
 void test_float_sums(const float* a, const float* b, int n, int chunk, double* out);
 void solver_destroy(Solver* w);
 // Solve S x = -b~ into x (device, 9 n_c) for every problem of the batch; the history of recursive

@@ -260,6 +260,10 @@ struct WideSum<float> {
         lo = two_sum(lo, te, ve);
         c = __fadd_rn(__fadd_rn(c, k), __fadd_rn(ue, ve));
     }
+    __device__ __forceinline__ void mul_add(float a, float b) {
+        const float p = __fmul_rn(a, b);
+        add3(p, __fmaf_rn(a, b, -p), 0.f);
+    }
     __device__ __forceinline__ void set(const Slot& v) { hi = v.x, lo = v.y, c = v.z; }
     __device__ __forceinline__ void add(const Slot& v) { add3(v.x, v.y, v.z); }
     __device__ __forceinline__ void add(const WideSum& b) { add3(b.hi, b.lo, b.c); }
@@ -2388,8 +2392,9 @@ __global__ void __launch_bounds__(PqShape<T>::kSlices * 32, RL == 1 ? 2 : 1) k_m
 // each.  Here a CTA runs the whole sweep between barriers, with S, the vectors and the current block in
 // shared memory.  The history stays in the problem's global arrays, which this kernel alone uses for it, in
 // tiles of 64 columns stored row by row (hist_at), so that threads on neighbouring columns read
-// neighbouring words.  It does what the kernels above do, step by step: exact-product sums in float
-// pairs, the float64 small solve, the same decide steps.  13 cameras, MCG: 25 -> 9 us per iteration.
+// neighbouring words.  It does what the kernels above do, step by step: exact-product sums, the float64 small
+// solve and Delta^+ Phi, the same decide steps.
+// 13 cameras: PCG 7.5 us per iteration (launched kernels 14.5), MCG with 8 directions to 1e-9 18.8 us (35.2).
 //
 // The rule: float32 sweeps of problems with nc <= kOneCams (S takes 324 nc^2 bytes: 130 KB of shared memory
 // at 20 cameras), whatever else is in the batch, so a problem's result does not depend on the others.
@@ -2500,11 +2505,33 @@ __device__ __forceinline__ void one_sums(const ExactSum<float> (&v)[NV], WideSum
     __syncthreads();
 }
 
+// q^T z over the rows [i0, i1) of whole cameras (QS apart in q), by one thread: as accurate as float64.  (With
+// three chains of float pairs, Delta^+ in double-float and double-float products, beta's error against 64-bit
+// sums reached 1.1e-7 of its column; 6e-8, float32's rounding, with wide sums and a float64 product.)
+template <int QS>
+__device__ __forceinline__ double one_phi(const float* q, const float* z, int i0, int i1) {
+    WideSum<float> a0, a1, a2;
+    for (int i = i0; i < i1; i += 9) {   // a camera's rows
+        float qv[9];
+#pragma unroll
+        for (int e = 0; e < 9; ++e) qv[e] = q[(i + e) * QS];
+#pragma unroll
+        for (int e = 0; e < 9; e += 3) {
+            a0.mul_add(qv[e], z[i + e]);
+            a1.mul_add(qv[e + 1], z[i + e + 1]);
+            a2.mul_add(qv[e + 2], z[i + e + 2]);
+        }
+    }
+    a0.add(a1);
+    a0.add(a2);
+    return a0.value();
+}
+
 __global__ void __launch_bounds__(kOneThreads, 1)
     k_one_cta(int mcg, const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ tile_ptr,
               const int32_t* __restrict__ col, const float* __restrict__ Sg, const double* __restrict__ Dinv,
               float* __restrict__ xg, const float* __restrict__ rg, const float* __restrict__ zg, float* P, float* Q,
-              double* phip, double* dpinv, float* beta, int* __restrict__ colblk, double* __restrict__ hist,
+              WideSlot<float>* phip, double* dpinv, float* beta, int* __restrict__ colblk, double* __restrict__ hist,
               int* blk_off, int* blk_w, int mi1, Ctl* ctl) {
     const int p = blockIdx.x, t = threadIdx.x;
     if (ctl[p].lay.nc > kOneCams || ctl[p].done) return;
@@ -2582,8 +2609,8 @@ __global__ void __launch_bounds__(kOneThreads, 1)
         }
     } else {
         const int n_eff = L.n_eff, sz = L.sz;
-        double* ph = phip + L.phoff;
-        float2* dp = reinterpret_cast<float2*>(dpinv) + int64_t(p) * mi1 * kMaxDirs * kMaxDirs;
+        double* ph = reinterpret_cast<double*>(phip + L.phoff);   // values here, not slots
+        double* dp = dpinv + int64_t(p) * mi1 * kMaxDirs * kMaxDirs;
         float* bt = beta + L.boff * kMaxDirs;
         int* cb = colblk + L.boff;
         const int* bo = blk_off + int64_t(p) * mi1;
@@ -2630,19 +2657,9 @@ __global__ void __launch_bounds__(kOneThreads, 1)
                 }
                 __syncthreads();
             }
-            solve_block(&m.c, m.s, w, nullptr);
+            solve_block(&m.c, m.s, w, dp + int64_t(it) * kMaxDirs * kMaxDirs);
             __syncthreads();
-            if (t < kMaxDirs * kMaxDirs) {   // Delta^+ in double-float for the reorthogonalisation
-                const int a = t / kMaxDirs, b = t % kMaxDirs;
-                if (a < w && b < w) {
-                    const double v = m.s.X[a][b];
-                    const float h = __double2float_rn(v);
-                    dp[int64_t(it) * kMaxDirs * kMaxDirs + t] = make_float2(h, __double2float_rn(v - double(h)));
-                }
-            } else if (t < kMaxDirs * kMaxDirs + kMaxDirs) {
-                const int b = t - kMaxDirs * kMaxDirs;
-                m.al[b] = b < w ? float(m.c.alpha_v[b]) : 0.f;
-            }
+            if (t < kMaxDirs) m.al[t] = t < w ? float(m.c.alpha_v[t]) : 0.f;
             __syncthreads();
             // update
             ExactSum<float> v[2];
@@ -2679,23 +2696,7 @@ __global__ void __launch_bounds__(kOneThreads, 1)
             // Phi: column c of the history against z over subset s, slot s hc + c
             for (int u = t; u < hc * n_eff; u += kOneThreads) {
                 const int s = u / hc, c = u - hc * s;
-                const int i0 = 9 * s * sz, i1 = min(9 * (s + 1) * sz, n);
-                const float* q = Qp + hist_at(n, 0, c);
-                ExactSum<float> a0, a1, a2;
-                for (int i = i0; i < i1; i += 9) {   // a camera's rows
-                    float qv[9];
-#pragma unroll
-                    for (int e = 0; e < 9; ++e) qv[e] = q[(i + e) * kOneTile];
-#pragma unroll
-                    for (int e = 0; e < 9; e += 3) {
-                        a0.add(qv[e], m.z[i + e]);
-                        a1.add(qv[e + 1], m.z[i + e + 1]);
-                        a2.add(qv[e + 2], m.z[i + e + 2]);
-                    }
-                }
-                combine(a0, a1);
-                combine(a0, a2);
-                store_partial(ph + u, a0);
+                ph[u] = one_phi<kOneTile>(Qp + hist_at(n, 0, c), m.z, 9 * s * sz, min(9 * (s + 1) * sz, n));
             }
             __syncthreads();
             if (!local) {   // a global step: over every subset, into the first one's slots
@@ -2703,37 +2704,36 @@ __global__ void __launch_bounds__(kOneThreads, 1)
                     double v[kMaxDirs];
 #pragma unroll
                     for (int s = 0; s < kMaxDirs; ++s) v[s] = s < n_eff ? ph[s * hc + c] : 0.0;
-                    ExactSum<float> a;
+                    double a0 = 0.0, a1 = 0.0;
 #pragma unroll
-                    for (int s = 0; s < kMaxDirs; ++s)
-                        if (s < n_eff) add_slot(a, v[s]);
-                    store_partial(ph + c, a);
+                    for (int s = 0; s < kMaxDirs; s += 2) {
+                        if (s < n_eff) a0 += v[s];
+                        if (s + 1 < n_eff) a1 += v[s + 1];
+                    }
+                    ph[c] = a0 + a1;
                 }
                 __syncthreads();
             }
-            // beta = Delta_j^+ Phi_j, entry (column c, new column s), products in double-float
+            // beta = Delta_j^+ Phi_j, entry (column c, new column s), in float64 rounded once
             for (int u = t; u < hc * wn; u += kOneThreads) {
                 const int s = u / hc, c = u - hc * s, jb = cb[c], o = bo[jb], wj = bw[jb];
-                const float2* Dr = dp + (int64_t(jb) * kMaxDirs + (c - o)) * kMaxDirs;
+                const double* Dr = dp + (int64_t(jb) * kMaxDirs + (c - o)) * kMaxDirs;
                 const double* phs = ph + s * hc + o;
-                df64 acc(0.f);
+                double acc0 = 0.0, acc1 = 0.0;
                 for (int b0 = 0; b0 < wj; b0 += 8) {   // eight terms' loads in flight
-                    double v[8];
-                    float2 dv[8];
+                    double v[8], dv[8];
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
                         v[e] = b0 + e < wj ? phs[b0 + e] : 0.0;
-                        dv[e] = b0 + e < wj ? Dr[b0 + e] : make_float2(0.f, 0.f);
+                        dv[e] = b0 + e < wj ? Dr[b0 + e] : 0.0;
                     }
 #pragma unroll
-                    for (int e = 0; e < 8; ++e)
-                        if (b0 + e < wj) {
-                            ExactSum<float> f;
-                            add_slot(f, v[e]);
-                            acc += df64(dv[e].x, dv[e].y) * df_fast_two_sum(f.hi, f.lo);
-                        }
+                    for (int e = 0; e < 8; e += 2) {
+                        if (b0 + e < wj) acc0 = fma(dv[e], v[e], acc0);
+                        if (b0 + e + 1 < wj) acc1 = fma(dv[e + 1], v[e + 1], acc1);
+                    }
                 }
-                bt[int64_t(c) * kMaxDirs + s] = __fadd_rn(acc.hi, acc.lo);
+                bt[int64_t(c) * kMaxDirs + s] = float(acc0 + acc1);
             }
             __syncthreads();
             // P_new = Z - P_hist beta: thread = (three rows, four new columns, an eighth of every 32 columns)
@@ -3757,7 +3757,7 @@ static int enqueue_small(Solver* w, const Structure& s, const System& y, bool mc
     }
     k_one_cta<<<w->nb, kOneThreads, one_smem(w->one_cams), st>>>(
         mcg, s.row_ptr, s.tile_ptr, s.col, y.S32, y.Dhat, ptr<float>(w->xw), ptr<float>(w->r), ptr<float>(w->z),
-        ptr<float>(w->P), ptr<float>(w->Q), ptr<double>(w->phip), ptr<double>(w->dpinv), ptr<float>(w->beta),
+        ptr<float>(w->P), ptr<float>(w->Q), ptr<WideSlot<float>>(w->phip), ptr<double>(w->dpinv), ptr<float>(w->beta),
         ptr<int>(w->colblk), ptr<double>(w->hist), ptr<int>(w->blk_off), ptr<int>(w->blk_w), w->mi1, ptr<Ctl>(w->ctl));
     return 1;
 }
@@ -4196,6 +4196,10 @@ __global__ void __launch_bounds__(kUpdThreads) k_test_update(const float* a, con
     if (i < n) v[0].add(a[i], b[i]);
     cta_publish<float, 1>(v, slots);
 }
+// a^T b as k_one_cta adds it: 9 n9 values by one thread
+__global__ void k_test_one_phi(const float* a, const float* b, int n9, double* out) {
+    if (threadIdx.x == 0) *out = one_phi<1>(a, b, 0, 9 * n9);
+}
 __global__ void k_test_update_total(const WideSlot<float>* slots, int np, double* out) {
     const WideSum<float> s = total_of<float, 1>(slots, np, 0);
     if (threadIdx.x == 0) *out = s.value();
@@ -4206,7 +4210,7 @@ void test_float_sums(const float* a, const float* b, int n, int chunk, double* o
     Buf ab, slots;
     grow(ab, sizeof(float) * 2 * size_t(n) + sizeof(double));
     const int ctas = (n + kUpdThreads - 1) / kUpdThreads, most = std::max(chunks, ctas);
-    grow(slots, sizeof(WideSlot<float>) * size_t(most) + 2 * sizeof(double));
+    grow(slots, sizeof(WideSlot<float>) * size_t(most) + 3 * sizeof(double));
     float* da = ptr<float>(ab);
     double* d = reinterpret_cast<double*>(ptr<WideSlot<float>>(slots) + most);
     cudaError_t e = cudaMemcpy(da, a, sizeof(float) * n, cudaMemcpyDefault);
@@ -4216,7 +4220,8 @@ void test_float_sums(const float* a, const float* b, int n, int chunk, double* o
         k_test_phi_block<<<1, 32>>>(ptr<WideSlot<float>>(slots), chunks, d);
         k_test_update<<<ctas, kUpdThreads>>>(da, da + n, n, ptr<WideSlot<float>>(slots));
         k_test_update_total<<<1, 32>>>(ptr<WideSlot<float>>(slots), ctas, d + 1);
-        e = cudaMemcpy(out, d, 2 * sizeof(double), cudaMemcpyDefault);
+        k_test_one_phi<<<1, 32>>>(da, da + n, n / 9, d + 2);
+        e = cudaMemcpy(out, d, 3 * sizeof(double), cudaMemcpyDefault);
     }
     free_buf(ab);
     free_buf(slots);

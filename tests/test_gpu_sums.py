@@ -46,7 +46,7 @@ def _within(got, a, b):
 def test_phi_sums_are_as_accurate_as_float64(n, chunk):
     for seed in range(4):
         a, b = _cancelling(n, seed)
-        out = (ctypes.c_double * 2)()
+        out = (ctypes.c_double * 3)()
         assert binding.lib().ba_test_float_sums(_ptr(a), _ptr(b), n, chunk, out) == 0
         assert _within(out[0], a, b), (seed, out[0])
 
@@ -56,6 +56,16 @@ def test_phi_sums_are_as_accurate_as_float64(n, chunk):
 def test_update_sums_are_as_accurate_as_float64(n):
     for seed in range(3):
         a, b = _cancelling(n, seed)
-        out = (ctypes.c_double * 2)()
+        out = (ctypes.c_double * 3)()
         assert binding.lib().ba_test_float_sums(_ptr(a), _ptr(b), n, 32, out) == 0
         assert _within(out[1], a, b), (seed, out[1])
+
+
+# Q^T z in the one-CTA sweep: a thread per column and subset, up to 20 cameras of 9 rows
+@pytest.mark.parametrize("cams", [1, 2, 3, 7, 13, 20])
+def test_one_cta_sums_are_as_accurate_as_float64(cams):
+    for seed in range(4):
+        a, b = _cancelling(9 * cams, seed)
+        out = (ctypes.c_double * 3)()
+        assert binding.lib().ba_test_float_sums(_ptr(a), _ptr(b), 9 * cams, 32, out) == 0
+        assert _within(out[2], a, b), (seed, out[2])
