@@ -2397,13 +2397,22 @@ __global__ void __launch_bounds__(PqShape<T>::kSlices * 32, RL == 1 ? 2 : 1) k_m
 // 13 cameras: PCG 7.5 us per iteration (launched kernels 14.5), MCG with 8 directions to 1e-9 18.8 us (35.2).
 //
 // The rule: float32 sweeps of problems with nc <= kOneCams (S takes 324 nc^2 bytes: 130 KB of shared memory
-// at 20 cameras), whatever else is in the batch, so a problem's result does not depend on the others.
+// at 20 cameras), by MCG with up to kOneDirs local directions, whatever else is in the batch, so a problem's
+// result does not depend on the others.  Delta_j^+ Phi_j costs w w' w float64 multiply-adds per pair of
+// blocks on this SM's float64 pipe alone, and a rank-deficient block's eigen-decomposition shares it:
+// to 1e-9 with 8 directions 19 to 26 us per iteration against 31 to 35 us in the kernels, with 10 directions
+// (20 cameras) 33.4 against 33.6 us, with 16 directions (16 cameras) 92 against 60 us.
 // Larger problems run the kernels above; a handle whose tile waits give up at once (wait_polls = -1) does
 // too, since there is no tile wait here.
 constexpr int kOneCams = 20;
+constexpr int kOneDirs = 10;
 constexpr int kOneRows = 9 * kOneCams;
 constexpr int kOneTile = 64;
 constexpr int kOneThreads = 512;   // solve_block uses as many; more would leave 64 registers a thread
+
+__host__ __device__ __forceinline__ bool one_cta_takes(const Layout& L, bool mcg) {
+    return L.nc <= kOneCams && (!mcg || L.n_eff <= kOneDirs);
+}
 
 struct OneSmem {
     Ctl c;
@@ -2534,7 +2543,7 @@ __global__ void __launch_bounds__(kOneThreads, 1)
               WideSlot<float>* phip, double* dpinv, float* beta, int* __restrict__ colblk, double* __restrict__ hist,
               int* blk_off, int* blk_w, int mi1, Ctl* ctl) {
     const int p = blockIdx.x, t = threadIdx.x;
-    if (ctl[p].lay.nc > kOneCams || ctl[p].done) return;
+    if (!one_cta_takes(ctl[p].lay, mcg) || ctl[p].done) return;
     extern __shared__ __align__(16) unsigned char smem_one[];
     OneSmem& m = *reinterpret_cast<OneSmem*>(smem_one);
     float* S = reinterpret_cast<float*>(smem_one + (sizeof(OneSmem) + 15) / 16 * 16);
@@ -3463,7 +3472,7 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
         L.phoff = phoff;
         L.boff = boff;
         // (a problem that one CTA solves keeps its history in whole tiles of columns; 16-byte aligned)
-        const int64_t cols = fp32 && L.nc <= kOneCams ? (cap + kOneTile - 1) / kOneTile * kOneTile : cap;
+        const int64_t cols = fp32 && one_cta_takes(L, a.mcg != 0) ? (cap + kOneTile - 1) / kOneTile * kOneTile : cap;
         hoff += (cols * 9 * int64_t(L.nc) + 3) / 4 * 4;
         phoff += cap * L.n_eff * L.K;
         boff += cap;
@@ -3512,9 +3521,9 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     // the largest problem that k_one_cta (float32) or k_pcg_cluster (float64 PCG) solves
     w->one_cams = 0;
     w->all_small = true;
-    const int small = fp32 ? kOneCams : (a.mcg ? 0 : kCluCams);
     for (const Layout& L : lay) {
-        if (L.nc <= small && a.wait_polls > 0) w->one_cams = std::max(w->one_cams, L.nc);
+        const bool small = fp32 ? one_cta_takes(L, a.mcg != 0) : !a.mcg && L.nc <= kCluCams;
+        if (small && a.wait_polls > 0) w->one_cams = std::max(w->one_cams, L.nc);
         else w->all_small = false;
     }
     if (fp32 && w->one_cams > 0) grow(w->colblk, size_t(boff) * sizeof(int));

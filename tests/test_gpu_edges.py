@@ -131,3 +131,38 @@ def test_one_cta_solves_launch_no_product():
             sweeps = _solve(p, args, 1e-6)["refinements"]
             per_sweep.append((p.ba_get_launch_count() - before - 3) / sweeps)
         assert per_sweep[0] == per_sweep[1] == per_sweep[2], per_sweep
+
+
+# Direction counts on both sides of 10, up to which one CTA runs MCG on up to 20 cameras (16 cameras: subsets of
+# one and two cameras), every step local and none, alone and beside problems that the other path takes.
+@pytest.mark.parametrize("dirs", [2, 5, 8, 10, 11, 15, 16])
+def test_direction_counts_around_the_one_cta_limit(dirs):
+    scenes = [sy.tiny(n, n_cams=n, n_pts=60 * n) for n in (10, 11, 16, 20, 30)]
+    solo = []
+    for sc in scenes:
+        with problem.from_scene(sc, precision="mixed") as p:
+            p.ba_build_normal(1e-4)
+            for tau in (1e9, 0.0):
+                st = p.ba_solve_mcg(1e-9, 5000, dirs, tau)
+                assert st["status"] == 0 and st["true_rel_residual"] <= 1e-9, (sc.n_cams, tau, st)
+                solo.append(p.ba_get_delta().copy())
+    off = np.cumsum([0] + [sc.n_cams for sc in scenes])
+    with problem.from_scenes(scenes, precision="mixed") as b:
+        b.ba_build_normal(1e-4)
+        for k, tau in enumerate((1e9, 0.0)):
+            assert b.ba_solve_mcg(1e-9, 5000, dirs, tau)["status"] == 0
+            x = b.ba_get_delta()
+            for q in range(len(scenes)):
+                assert np.array_equal(x[off[q]:off[q + 1]], solo[2 * q + k]), (tau, scenes[q].n_cams)
+
+
+# A full history ends a float32 sweep; one CTA keeps its history in tiles of 64 columns, so capacities around them.
+@pytest.mark.parametrize("cap", [9, 40, 63, 64, 65, 130])
+def test_full_histories_of_one_cta_sweeps(cap):
+    sc, m, _ = _system(13, 777)
+    with binding.Problem(sc.cams0, sc.pts0, sc.obs_cam, sc.obs_pt, m, precision="mixed", max_history=cap,
+                         max_refine=2000) as p:
+        p.ba_build_normal(1e-2)
+        for args in ((8, 3.0), (4, 1e9), (10, 0.0)):
+            st = p.ba_solve_mcg(1e-8, 20000, *args)
+            assert st["status"] == 0 and st["true_rel_residual"] <= 1e-8 and st["history_cols"] <= cap, (args, st)
