@@ -1494,7 +1494,8 @@ __global__ void __launch_bounds__(kThreads) k_pcg_dir(const T* __restrict__ z, T
 // The n rows of a problem fall into gram_parts runs of consecutive rows with a partial each, so the
 // partition depends on the problem alone.
 constexpr int kGramRows = 64;
-constexpr int kGramThreads = 1024;
+constexpr int kGramThreads = 1024;     // threads that the work of a CTA is divided over
+constexpr int kGramFew = 256;          // threads of a CTA when a batch has many problems
 __device__ __forceinline__ int gram_parts(int n, int gmax) { return min((n + kGramRows - 1) / kGramRows, gmax); }
 
 // A CTA takes the runs blockIdx.x, blockIdx.x + gridDim.x, ... and stages kGramRows rows at a time, the
@@ -1504,10 +1505,14 @@ __device__ __forceinline__ int gram_parts(int n, int gmax) { return min((n + kGr
 // float-pair additions (10 instructions a term): with one thread per entry over 128 rows the kernel took
 // 9 us on 1000 cameras (15.4k of its cycles staging and adding), now 4.7 us; more CTAs than SMs made a
 // batch of 16 problems pay each CTA's start in turn (14.1 us; looping CTAs 13.0 us).
-template <typename T>
-__global__ void __launch_bounds__(kGramThreads) k_mcg_gram(const T* __restrict__ P, const T* __restrict__ Q,
-                                                           const T* __restrict__ r, double* __restrict__ partial,
-                                                           int gmax, const Ctl* __restrict__ ctl) {
+// NT threads do the work of kGramThreads, kGramThreads / NT each, in the same order.  A CTA of 1024 threads
+// leaves no room for another on its SM, so many problems of a few runs each went through loads and barriers
+// in turn (64 problems of 60 cameras, one direction: 79.1 us per iteration, 75.1 with 256 threads).
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT, NT < kGramThreads ? 3 : 1) k_mcg_gram(const T* __restrict__ P, const T* __restrict__ Q,
+                                                                           const T* __restrict__ r,
+                                                                           double* __restrict__ partial, int gmax,
+                                                                           const Ctl* __restrict__ ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const int p = blockIdx.y;
     const Ctl& c = ctl[p];
@@ -1521,7 +1526,8 @@ __global__ void __launch_bounds__(kGramThreads) k_mcg_gram(const T* __restrict__
     __shared__ T sP[TR][kMaxDirs + 1], sQ[TR][kMaxDirs + 1], sr[TR];
     __shared__ double st[kGramThreads];      // the groups' sums, slot g w w + e
     __shared__ double sg[NW][kMaxDirs];      // the warps' sums of gamma
-    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    constexpr int V = kGramThreads / NT;     // threads of the division that a thread stands for: t + NT v
+    const int t = threadIdx.x, lane = t & 31;
     const int w = c.w_cur, off = c.off_cur, ww = w * w;
     const T* Pp = P + c.lay.hoff + int64_t(off) * n;
     const T* Qp = Q + c.lay.hoff + int64_t(off) * n;
@@ -1529,24 +1535,31 @@ __global__ void __launch_bounds__(kGramThreads) k_mcg_gram(const T* __restrict__
     const int per = (nr + gp - 1) / gp;
     int NG = 4;   // row groups; a group has kGramThreads / NG threads
     while (NG < 16 && kGramThreads / (2 * NG) >= ww) NG *= 2;
-    const int gt = kGramThreads / NG, g = t / gt, e = t - g * gt, gr = TR / NG;
-    const int lr = t % TR, lc = t / TR;      // loads: a warp reads 32 rows of one column
-    T pn = T(0), qn = T(0), rn = T(0);
+    const int gt = kGramThreads / NG, gr = TR / NG;
+    const int lr = t % TR;                   // loads: a warp reads 32 rows of one column
+    T pn[V], qn[V], rn = T(0);
     auto load = [&](int base, int end) {
         const bool in = base + lr < end;
-        pn = in && lc < w ? Pp[lc * n + base + lr] : T(0);
-        qn = in && lc < w ? Qp[lc * n + base + lr] : T(0);
-        rn = in && lc == 0 ? rp[base + lr] : T(0);
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            const int lc = (t + NT * v) / TR;
+            pn[v] = in && lc < w ? Pp[lc * n + base + lr] : T(0);
+            qn[v] = in && lc < w ? Qp[lc * n + base + lr] : T(0);
+        }
+        rn = in && t < TR ? rp[base + lr] : T(0);
     };
     int part = blockIdx.x, base = part * per;
     load(base, min(base + per, nr));
     while (part < gp) {
-        ExactSum<T> a0, a1, ag;
+        ExactSum<T> a0[V], a1[V], ag[V];
         bool more = true;
         while (more) {
-            sP[lr][lc] = pn;
-            sQ[lr][lc] = qn;
-            if (lc == 0) sr[lr] = rn;
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                sP[lr][(t + NT * v) / TR] = pn[v];
+                sQ[lr][(t + NT * v) / TR] = qn[v];
+            }
+            if (t < TR) sr[lr] = rn;
             __syncthreads();
             // the next rows of this run, or the first of the CTA's next run
             base += TR;
@@ -1554,33 +1567,40 @@ __global__ void __launch_bounds__(kGramThreads) k_mcg_gram(const T* __restrict__
             if (!more) base = (part + int(gridDim.x)) * per;
             const int np = more ? part : part + int(gridDim.x);
             if (np < gp) load(base, min((np + 1) * per, nr));
-            if (e < ww) {   // rows past the last one are zeros
-                const T* x = &sQ[g * gr][e / w];
-                const T* y = &sP[g * gr][e % w];
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const int g = (t + NT * v) / gt, e = t + NT * v - g * gt;
+                if (e < ww) {   // rows past the last one are zeros
+                    const T* x = &sQ[g * gr][e / w];
+                    const T* y = &sP[g * gr][e % w];
 #pragma unroll 4
-                for (int k = 0; k < gr; k += 2) {
-                    a0.add(x[k * (kMaxDirs + 1)], y[k * (kMaxDirs + 1)]);
-                    a1.add(x[(k + 1) * (kMaxDirs + 1)], y[(k + 1) * (kMaxDirs + 1)]);
+                    for (int k = 0; k < gr; k += 2) {
+                        a0[v].add(x[k * (kMaxDirs + 1)], y[k * (kMaxDirs + 1)]);
+                        a1[v].add(x[(k + 1) * (kMaxDirs + 1)], y[(k + 1) * (kMaxDirs + 1)]);
+                    }
                 }
-            }
-            {
-                const int row = 2 * wid + (lane >> 4);
-                ag.add(sP[row][lane & 15], sr[row]);
+                const int row = 2 * ((t + NT * v) >> 5) + (lane >> 4);
+                ag[v].add(sP[row][lane & 15], sr[row]);
             }
             __syncthreads();
         }
-        combine(a0, a1);
-        combine_shfl(ag, 16);
-        if (e < ww) store_partial(&st[g * ww + e], a0);
-        if (lane < kMaxDirs) store_partial(&sg[wid][lane], ag);
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            const int g = (t + NT * v) / gt, e = t + NT * v - g * gt;
+            combine(a0[v], a1[v]);
+            combine_shfl(ag[v], 16);
+            if (e < ww) store_partial(&st[g * ww + e], a0[v]);
+            if (lane < kMaxDirs) store_partial(&sg[(t + NT * v) >> 5][lane], ag[v]);
+        }
         __syncthreads();
         double* out = partial + (int64_t(p) * gmax + part) * kGramMax;
-        if (t < ww) {
+        for (int e = t; e < ww; e += NT) {
             ExactSum<T> a;
-            for (int k = 0; k < NG; ++k) load_partial(a, &st[k * ww + t]);
-            store_partial(out + t, a);
-        } else if (t >= kGramThreads - kMaxDirs && t - (kGramThreads - kMaxDirs) < w) {
-            const int cc = t - (kGramThreads - kMaxDirs);
+            for (int k = 0; k < NG; ++k) load_partial(a, &st[k * ww + e]);
+            store_partial(out + e, a);
+        }
+        if (t >= NT - kMaxDirs && t - (NT - kMaxDirs) < w) {
+            const int cc = t - (NT - kMaxDirs);
             ExactSum<T> a, b;
 #pragma unroll
             for (int k = 0; k < NW; k += 2) {
@@ -3684,6 +3704,10 @@ static int enqueue_product(Solver* w, const Structure& s, const T* S, const T* S
     return 1;
 }
 
+// A batch of this many problems fills the chip with small CTAs; fewer problems are spread over large CTAs and
+// clusters.  The results are the same bits.
+static bool many_problems(int nb) { return kSmallCtas * nb > num_sms(); }
+
 // Enqueue one iteration of the chosen algorithm for every problem on `st`; returns the launches.
 template <typename T>
 static int enqueue_iteration(Solver* w, const Structure& s, const T* S, const T* Su, const double* Dinv, T* x,
@@ -3703,8 +3727,12 @@ static int enqueue_iteration(Solver* w, const Structure& s, const T* S, const T*
                        ptr<double>(w->dtot), ptr<double>(w->hist), ctl);
         return np + 2;
     } else {
-        launch_chained(k_mcg_gram<T>, dim3(std::min(w->gg, std::max(1, 2 * num_sms() / nb)), nb), dim3(kGramThreads), 0,
-                       st, P, Q, r, ptr<double>(w->part_a), w->gg, ctl);
+        if (many_problems(nb))
+            launch_chained(k_mcg_gram<T, kGramFew>, dim3(w->gg, nb), dim3(kGramFew), 0, st, P, Q, r,
+                           ptr<double>(w->part_a), w->gg, ctl);
+        else
+            launch_chained(k_mcg_gram<T, kGramThreads>, dim3(std::min(w->gg, std::max(1, 2 * num_sms() / nb)), nb),
+                           dim3(kGramThreads), 0, st, P, Q, r, ptr<double>(w->part_a), w->gg, ctl);
         launch_chained(k_mcg_small<T>, dim3(nb * kSmallCtas), dim3(kSmallThreads), 0, st, ctl, ptr<double>(w->part_a), w->gg,
                        ptr<double>(w->dpinv), w->mi1);
         launch_chained(k_mcg_update<T>, dim3(w->gu, nb), dim3(kUpdThreads), 0, st, Dinv, P, Q, x, r, z,

@@ -166,3 +166,27 @@ def test_full_histories_of_one_cta_sweeps(cap):
         for args in ((8, 3.0), (4, 1e9), (10, 0.0)):
             st = p.ba_solve_mcg(1e-8, 20000, *args)
             assert st["status"] == 0 and st["true_rel_residual"] <= 1e-8 and st["history_cols"] <= cap, (args, st)
+
+
+# Batches of more than 19 problems run small CTAs where fewer problems have large ones and clusters: the same bits
+# as alone.  With a problem of 230 cameras in it the small solves keep their clusters.
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("largest", [70, 230])
+def test_many_problems_give_their_solo_bits(precision, largest):
+    sizes = [9, 16, 21, 30, 45, largest]
+    scenes = [sy.tiny(n, n_cams=n, n_pts=40 * n) for n in sizes]
+    solves = ((3, 3.0), (8, 1e9), (16, 10.0), (5, 0.0))
+    solo = []
+    for sc in scenes:
+        with problem.from_scene(sc, precision=precision) as p:
+            p.ba_build_normal(1e-3)
+            solo.append([(p.ba_solve_mcg(1e-6, 2000, *a), p.ba_get_delta().copy())[1] for a in solves])
+    batch = scenes * 4   # 24 problems
+    off = np.cumsum([0] + [sc.n_cams for sc in batch])
+    with problem.from_scenes(batch, precision=precision) as b:
+        b.ba_build_normal(1e-3)
+        for k, a in enumerate(solves):
+            assert b.ba_solve_mcg(1e-6, 2000, *a)["status"] == 0
+            x = b.ba_get_delta()
+            for q in range(len(batch)):
+                assert np.array_equal(x[off[q]:off[q + 1]], solo[q % len(scenes)][k]), (a, batch[q].n_cams, q)
