@@ -2116,14 +2116,16 @@ __device__ void mcg_decide(Ctl* c, const double* tot, double* hist, int* blk_off
 // row chunk of up to kPhiCols columns at once, 8 rows of each in flight (32 loads a lane), and reads z
 // once for all of them.  A column at a time with float64 shuffle trees ran at 2.1 TB/s (34 us on
 // 2000 columns of 9000 rows; now 21 us).  Fewer columns at once when there are not enough chunks for
-// the warps; a column's sum does not depend on it.  The problem's first CTA runs the decide step
-// beside them.
+// the warps; a column's sum does not depend on it.  Chunks of at most 64 (128) rows take 2 (4) steps of rows at
+// once: the registers of eight steps leave room for 24 warps an SM only (200 float64 problems of 16 cameras, 9 or
+// 18 rows a chunk: 1004 -> 943 us per iteration with 16 directions, 233 -> 213 with 8).  The problem's first CTA
+// runs the decide step beside them.
 constexpr int kPhiCols = 4;
-template <typename T, int NC>
+constexpr int phi_ctas(int steps) { return steps == 8 ? 3 : steps == 4 ? 4 : 5; }   // per SM
+template <typename T, int NC, int U = 8>
 __device__ __forceinline__ void phi_columns(const T* __restrict__ qc, int64_t n, const T* __restrict__ zp, int r0, int r1,
                                             WideSlot<T>* __restrict__ out, int64_t ostride) {
     const int lane = threadIdx.x & 31;
-    constexpr int U = 8;
     ExactSum<T> acc[NC];
     for (int base = r0 + lane; base < r1; base += 32 * U) {
         T zv[U], qv[NC][U];
@@ -2147,8 +2149,8 @@ __device__ __forceinline__ void phi_columns(const T* __restrict__ qc, int64_t n,
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k_mcg_phi(const T* __restrict__ Q, const T* __restrict__ z,
+template <typename T, int U>
+__global__ void __launch_bounds__(kThreads, phi_ctas(U)) k_mcg_phi(const T* __restrict__ Q, const T* __restrict__ z,
                                                       WideSlot<T>* __restrict__ phip,
                                                       const WideSlot<T>* __restrict__ dpart, int gu, double* __restrict__ hist_out, int* __restrict__ blk_off,
                                                       int* __restrict__ blk_w, int mi1, Ctl* ctl) {
@@ -2187,9 +2189,9 @@ __global__ void __launch_bounds__(kThreads) k_mcg_phi(const T* __restrict__ Q, c
         const T* qc = Qp + int64_t(c0) * n;
         WideSlot<T>* out = ph + int64_t(c0) * chunks + ch;
         const int m = hist - c0 < nb ? hist - c0 : nb;
-        if (m == kPhiCols) phi_columns<T, kPhiCols>(qc, n, zp, 9 * j0, 9 * j1, out, chunks);
+        if (m == kPhiCols) phi_columns<T, kPhiCols, U>(qc, n, zp, 9 * j0, 9 * j1, out, chunks);
         else
-            for (int u = 0; u < m; ++u) phi_columns<T, 1>(qc + u * n, n, zp, 9 * j0, 9 * j1, out + int64_t(u) * chunks, chunks);
+            for (int u = 0; u < m; ++u) phi_columns<T, 1, U>(qc + u * n, n, zp, 9 * j0, 9 * j1, out + int64_t(u) * chunks, chunks);
     }
 }
 
@@ -3215,12 +3217,13 @@ struct GraphKey {
     int lanes = -1;                   // column lanes of k_spmm
     int one = -1;                     // cameras of the largest problem that one CTA or cluster solves
     int all = -1;                     // one of them solves every problem
+    int phi = -1;                     // rows of the largest Phi chunk
     uint64_t allocs = ~uint64_t(0);   // buffer generation (any reallocation invalidates the graph)
     const void* ptrs[4] = {};
     bool operator==(const GraphKey& o) const {
         if (mcg != o.mcg || fp32 != o.fp32 || chunk != o.chunk || mi1 != o.mi1 || use_l != o.use_l ||
             epoch != o.epoch || polls != o.polls || nb != o.nb || host != o.host || cfg != o.cfg ||
-            lanes != o.lanes || one != o.one || all != o.all || allocs != o.allocs)
+            lanes != o.lanes || one != o.one || all != o.all || phi != o.phi || allocs != o.allocs)
             return false;
         for (int i = 0; i < 4; ++i) if (ptrs[i] != o.ptrs[i]) return false;
         return true;
@@ -3254,6 +3257,7 @@ struct Solver {
     int gq = 1;               // grid width of the per-row kernels
     int gpq = 1;              // grid width of the reorthogonalisation (32-row blocks)
     int gphi = 1, gb = 1;     // Phi and beta grid widths
+    int phi_rows = 1;         // rows of the largest Phi chunk
     int one_cams = 0;         // cameras of the largest problem that k_one_cta or k_pcg_cluster solves (0: none)
     bool all_small = false;   // one of those two solves every problem
     int gcol = 1;             // grid width of the column pass of the symmetric product (a CTA per camera)
@@ -3564,6 +3568,8 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     w->gpq = int(std::max<int64_t>(1, std::min<int64_t>((9 * int64_t(nc_max) + 31) / 32, 4 * G / nb)));
     w->gphi = std::max(1, 4 * G / nb);
     w->gb = std::max(1, G / nb);
+    w->phi_rows = 1;
+    for (const Layout& L : lay) w->phi_rows = std::max(w->phi_rows, 9 * ((L.sz + L.K - 1) / L.K));
     w->gcol = std::min(nc_max, std::max(1, 16 * G / nb));
     if (!w->h_ctl || int(w->lay.size()) != nb) {
         if (w->h_ctl) cudaFreeHost(w->h_ctl);
@@ -3794,7 +3800,8 @@ static int enqueue_iteration(Solver* w, const Structure& s, const T* S, const T*
                            w->gg, ptr<double>(w->dpinv), w->mi1);
         launch_chained(k_mcg_update<T>, dim3(w->gu, nb), dim3(kUpdThreads), 0, st, Dinv, P, Q, x, r, z,
                        ptr<WideSlot<T>>(w->dpart), ctl);
-        launch_chained(k_mcg_phi<T>, dim3(w->gphi + 1, nb), dim3(kThreads), 0, st, Q, z, ptr<WideSlot<T>>(w->phip),
+        auto phi = w->phi_rows <= 64 ? k_mcg_phi<T, 2> : w->phi_rows <= 128 ? k_mcg_phi<T, 4> : k_mcg_phi<T, 8>;
+        launch_chained(phi, dim3(w->gphi + 1, nb), dim3(kThreads), 0, st, Q, z, ptr<WideSlot<T>>(w->phip),
                        ptr<WideSlot<T>>(w->dpart), w->gu, ptr<double>(w->hist), ptr<int>(w->blk_off),
                        ptr<int>(w->blk_w), w->mi1, ctl);
         T* betat = ptr<T>(w->beta);
@@ -4104,6 +4111,7 @@ static cudaGraphExec_t solve_graph(Solver* w, const Structure& s, const System& 
     key.cfg = a.spmv_cfg;
     key.one = w->one_cams;
     key.all = w->all_small;
+    key.phi = w->phi_rows;
     key.lanes = w->col_lanes;
     key.allocs = g_allocs.load();
     const void* ptrs[4] = {x, fp32 ? (const void*)y.S32 : (const void*)y.S, w->items_g.items, w->items_l.items};
