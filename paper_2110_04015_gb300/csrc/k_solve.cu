@@ -2315,20 +2315,28 @@ template <typename T>
 struct PqShape;
 template <> struct PqShape<float> { static constexpr int kSlices = 16, kTile = 256; };
 template <> struct PqShape<double> { static constexpr int kSlices = 8, kTile = 128; };
+constexpr int kPqFew = 4;   // warps of a CTA when a batch has many problems
 
 // RL rows per lane: a column's 16 betas are read from shared memory once for 32 RL rows.  With one row
 // that read (16 words a lane for 16 multiply-adds) slows the kernel once every SM has work (17.7 us on average
 // over a 1000-camera solve, 15.5 us with two rows); with fewer rows than that, more CTAs count for more.
-template <typename T, int RL>
-__global__ void __launch_bounds__(PqShape<T>::kSlices * 32, RL == 1 ? 2 : 1) k_mcg_pq(T* __restrict__ P, T* __restrict__ Q,
-                                                                     const T* __restrict__ z, const T* __restrict__ beta,
-                                                                     T* __restrict__ PT, const Ctl* __restrict__ ctl) {
+// NW warps a CTA, kSlices / NW slices a warp, summed in the same order: with 16 warps two CTAs fit an SM, and a
+// batch of many problems, each of several row blocks and a short history, goes through their barriers and
+// loads in turn.  With four warps 64 problems of 60 cameras take 59.2 instead of 65.6 us per iteration (one
+// direction); with more than 8 directions the sums of four slices cost more than that gains (48 problems of 100
+// to 400 cameras, 16 directions: 411 -> 432 us), so the rule stops there.
+template <typename T, int RL, int NW = PqShape<T>::kSlices>
+__global__ void __launch_bounds__(NW * 32, NW < PqShape<T>::kSlices ? 4 : RL == 1 ? 2 : 1)
+    k_mcg_pq(T* __restrict__ P, T* __restrict__ Q, const T* __restrict__ z, const T* __restrict__ beta,
+             T* __restrict__ PT, const Ctl* __restrict__ ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const Ctl& c = ctl[blockIdx.y];
     if (c.done) return;
     constexpr bool kUpdQ = sizeof(T) == 8;
     constexpr int NS = PqShape<T>::kSlices, TC = PqShape<T>::kTile;
-    constexpr int U = kUpdQ ? 4 : 8;                   // columns in flight (of P, and of Q)
+    constexpr int SP = NS / NW;                        // slices of a warp: k, k + NW, ...
+    constexpr int U = (kUpdQ ? 4 : 8) / SP;            // columns of a slice in flight (of P, and of Q)
+    static_assert(SP * NW == NS && U > 0, "whole slices");
     // two beta tiles during the loop over the history, then the slices' sums
     __shared__ __align__(16) T smem[NS * 32 * (kMaxDirs + 1)];
     static_assert(2 * TC * kMaxDirs <= NS * 32 * (kMaxDirs + 1), "beta tiles fit");
@@ -2344,13 +2352,15 @@ __global__ void __launch_bounds__(PqShape<T>::kSlices * 32, RL == 1 ? 2 : 1) k_m
     static_assert(!kUpdQ || RL == 1, "two rows per lane in the float32 sweeps only");
     for (int64_t base = int64_t(blockIdx.x) * (32 * RL); base < n; base += int64_t(gridDim.x) * (32 * RL)) {
         const int64_t row = base + lane;   // and row + 32
-        T ap[RL][kMaxDirs], aq[kUpdQ ? kMaxDirs : 1];
+        T ap[RL][SP][kMaxDirs], aq[SP][kUpdQ ? kMaxDirs : 1];
 #pragma unroll
-        for (int s = 0; s < kMaxDirs; ++s) {
+        for (int j = 0; j < SP; ++j)
 #pragma unroll
-            for (int h = 0; h < RL; ++h) ap[h][s] = T(0);
-            if constexpr (kUpdQ) aq[s] = T(0);
-        }
+            for (int s = 0; s < kMaxDirs; ++s) {
+#pragma unroll
+                for (int h = 0; h < RL; ++h) ap[h][j][s] = T(0);
+                if constexpr (kUpdQ) aq[j][s] = T(0);
+            }
         // beta tile t + 1 is copied while tile t is used (rows of 16 values; past w they may hold
         // anything, which reaches only sums that are not used)
         auto copy_b = [&](int c0n) {
@@ -2371,64 +2381,75 @@ __global__ void __launch_bounds__(PqShape<T>::kSlices * 32, RL == 1 ? 2 : 1) k_m
             const T* pc = Pp + int64_t(c0) * n + row;
             const T* qc = Qp + int64_t(c0) * n + row;
             for (int cl = k; cl < tc; cl += NS * U) {
-                T pv[RL][U], qv[U];
+                T pv[RL][SP][U], qv[SP][U];
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int cu = cl + u * NS;
+                for (int j = 0; j < SP; ++j)
 #pragma unroll
-                    for (int h = 0; h < RL; ++h)
-                        pv[h][u] = row + 32 * h < n && cu < tc ? pc[int64_t(cu) * n + 32 * h] : T(0);
-                    if constexpr (kUpdQ) qv[u] = row < n && cu < tc ? qc[int64_t(cu) * n] : T(0);
-                }
+                    for (int u = 0; u < U; ++u) {
+                        const int cu = cl + NW * j + u * NS;
+#pragma unroll
+                        for (int h = 0; h < RL; ++h)
+                            pv[h][j][u] = row + 32 * h < n && cu < tc ? pc[int64_t(cu) * n + 32 * h] : T(0);
+                        if constexpr (kUpdQ) qv[j][u] = row < n && cu < tc ? qc[int64_t(cu) * n] : T(0);
+                    }
                 if (w == 1) {
 #pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int cu = cl + u * NS;
-                        const T b0 = cu < tc ? sB[cu][0] : T(0);
+                    for (int j = 0; j < SP; ++j)
 #pragma unroll
-                        for (int h = 0; h < RL; ++h) ap[h][0] += pv[h][u] * b0;
-                        if constexpr (kUpdQ) aq[0] += qv[u] * b0;
-                    }
+                        for (int u = 0; u < U; ++u) {
+                            const int cu = cl + NW * j + u * NS;
+                            const T b0 = cu < tc ? sB[cu][0] : T(0);
+#pragma unroll
+                            for (int h = 0; h < RL; ++h) ap[h][j][0] += pv[h][j][u] * b0;
+                            if constexpr (kUpdQ) aq[j][0] += qv[j][u] * b0;
+                        }
                 } else {
 #pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int cu = cl + u * NS;
-                        if (cu >= tc) break;
+                    for (int j = 0; j < SP; ++j)
 #pragma unroll
-                        for (int s = 0; s < kMaxDirs; s += 2) {
-                            if constexpr (kUpdQ) {
-                                ap[0][s] += pv[0][u] * sB[cu][s];
-                                ap[0][s + 1] += pv[0][u] * sB[cu][s + 1];
-                                aq[s] += qv[u] * sB[cu][s];
-                                aq[s + 1] += qv[u] * sB[cu][s + 1];
-                            } else {   // packed: each half rounds like a scalar fused multiply-add
-                                const float2 b2 = *reinterpret_cast<const float2*>(&sB[cu][s]);
+                        for (int u = 0; u < U; ++u) {
+                            const int cu = cl + NW * j + u * NS;
+                            if (cu >= tc) break;
 #pragma unroll
-                                for (int h = 0; h < RL; ++h) {
-                                    const float2 v = __ffma2_rn(make_float2(pv[h][u], pv[h][u]), b2,
-                                                                make_float2(ap[h][s], ap[h][s + 1]));
-                                    ap[h][s] = v.x;
-                                    ap[h][s + 1] = v.y;
+                            for (int s = 0; s < kMaxDirs; s += 2) {
+                                if constexpr (kUpdQ) {
+                                    ap[0][j][s] += pv[0][j][u] * sB[cu][s];
+                                    ap[0][j][s + 1] += pv[0][j][u] * sB[cu][s + 1];
+                                    aq[j][s] += qv[j][u] * sB[cu][s];
+                                    aq[j][s + 1] += qv[j][u] * sB[cu][s + 1];
+                                } else {   // packed: each half rounds like a scalar fused multiply-add
+                                    const float2 b2 = *reinterpret_cast<const float2*>(&sB[cu][s]);
+#pragma unroll
+                                    for (int h = 0; h < RL; ++h) {
+                                        const float2 v = __ffma2_rn(make_float2(pv[h][j][u], pv[h][j][u]), b2,
+                                                                    make_float2(ap[h][j][s], ap[h][j][s + 1]));
+                                        ap[h][j][s] = v.x;
+                                        ap[h][j][s + 1] = v.y;
+                                    }
                                 }
                             }
                         }
-                    }
                 }
             }
             __syncthreads();
         }
-        // column s of the new block is added by warp s mod NS, over the slices in order
-        auto slices = [&](const T* acc, auto&& put) {
+        // column s of the new block is added by warp s mod NW, over the slices in order
+        auto slices = [&](const auto& acc, auto&& put) {
             __syncthreads();
 #pragma unroll
-            for (int s = 0; s < kMaxDirs; ++s) red[k][lane][s] = acc[s];
+            for (int j = 0; j < SP; ++j)
+#pragma unroll
+                for (int s = 0; s < kMaxDirs; ++s)
+                    if (s < w) red[k + NW * j][lane][s] = acc[j][s];
             __syncthreads();
-            for (int s = k; s < kMaxDirs; s += NS) {
+#pragma unroll
+            for (int i = 0; i < (kMaxDirs + NW - 1) / NW; ++i) {
+                const int s = k + NW * i;
                 T sum = T(0);
                 if (s < w)
 #pragma unroll
                     for (int kk = 0; kk < NS; ++kk) sum += red[kk][lane][s];
-                put(s, sum);
+                put(i, s, sum);
             }
         };
 #pragma unroll
@@ -2437,23 +2458,26 @@ __global__ void __launch_bounds__(PqShape<T>::kSlices * 32, RL == 1 ? 2 : 1) k_m
             const bool act = rh < n;
             const int sub = act ? int(rh / 9) / sz : 0;
             const T zr = act ? z[r0g + rh] : T(0);
-            T pn = T(0);
-            slices(ap[h], [&](int s, T sum) {
-                pn = s < w ? (s == (local ? sub : 0) ? zr : T(0)) - sum : T(0);
-                if (act && s < w) Pp[int64_t(off + s) * n + rh] = pn;
+            T pn[kMaxDirs / NW];
+            slices(ap[h], [&](int i, int s, T sum) {
+                pn[i] = s < w ? (s == (local ? sub : 0) ? zr : T(0)) - sum : T(0);
+                if (act && s < w) Pp[int64_t(off + s) * n + rh] = pn[i];
             });
             if constexpr (kUpdQ) {
-                slices(aq, [&](int s, T sum) {
+                slices(aq, [&](int, int s, T sum) {
                     if (act && s < w) Qp[int64_t(off + s) * n + rh] -= sum;
                 });
             } else {
                 // row-major copy of the new block for the multi-column product (zero past w)
-                static_assert(kUpdQ || NS == kMaxDirs, "one column per warp");
                 __syncthreads();
-                red[0][lane][k] = pn;
+#pragma unroll
+                for (int i = 0; i < kMaxDirs / NW; ++i) red[0][lane][k + NW * i] = pn[i];
                 __syncthreads();
-                const int rr = threadIdx.x / kMaxDirs, ss = threadIdx.x % kMaxDirs;
-                if (base + 32 * h + rr < n) PT[(r0g + base + 32 * h) * kMaxDirs + threadIdx.x] = red[0][rr][ss];
+#pragma unroll
+                for (int x = threadIdx.x; x < 32 * kMaxDirs; x += 32 * NW) {
+                    const int rr = x / kMaxDirs, ss = x % kMaxDirs;
+                    if (base + 32 * h + rr < n) PT[(r0g + base + 32 * h) * kMaxDirs + x] = red[0][rr][ss];
+                }
             }
         }
         __syncthreads();
@@ -3821,8 +3845,10 @@ static int enqueue_iteration(Solver* w, const Structure& s, const T* S, const T*
         } else {
             // Algorithm 2: Q_{i+1} = S P_{i+1}
             // two rows per lane once they still give nearly every SM a CTA (a row's sum is the same either way)
-            auto pq = w->n >= int64_t(48) * Gt ? k_mcg_pq<T, 2> : k_mcg_pq<T, 1>;
-            launch_chained(pq, dim3(w->gpq, nb), dim3(PqShape<T>::kSlices * 32), 0, st, P, Q, z, betat, ptr<T>(w->PT), ctl);
+            const bool many = many_problems(nb) && w->col_lanes == 2;   // up to 8 directions
+            auto pq = many ? k_mcg_pq<T, 1, kPqFew> : w->n >= int64_t(48) * Gt ? k_mcg_pq<T, 2> : k_mcg_pq<T, 1>;
+            launch_chained(pq, dim3(w->gpq, nb), dim3((many ? kPqFew : PqShape<T>::kSlices) * 32), 0, st, P, Q, z, betat,
+                           ptr<T>(w->PT), ctl);
             const int np = enqueue_product<T, 2>(w, s, S, Su, P, kSelW1, Q, nullptr, st);
             auto mm = w->col_lanes == 2 ? k_spmm<T, 2> : k_spmm<T, 4>;
             launch_chained(mm, dim3(Gt), dim3(SpmmCfg::kWarps * 32), spmm_smem<T>(), st, s.row_ptr, s.tile_ptr,
