@@ -1301,8 +1301,10 @@ __global__ void k_df_to_double(double* __restrict__ buf, int64_t n) {
 // A warp per camera: lane l owns the entries l and l + 32 of the 45 of the lower triangle, which meet in
 // shared memory.  A sweep's chain is the pivot's reciprocal (four dependent float64 operations of about
 // 150 cycles) and one multiply-add, the entries' products formed meanwhile; a thread per camera took 34 us
-// for its Cholesky factor, triangular inverse and product, whatever the camera count (now 8 us).
+// for its Cholesky factor, triangular inverse and product, whatever the camera count; now 8 us, from a few hundred
+// cameras on more (17 us for 1000, the float64 pipe then three quarters busy).
 constexpr int kBjThreads = 64;
+constexpr int kBjWarpCams = 3600;   // more cameras: k_block_jacobi_cams
 __global__ void __launch_bounds__(kBjThreads) k_block_jacobi(int32_t n_c, const double* __restrict__ Sd,
                                                             double* __restrict__ Dinv, double* __restrict__ lam,
                                                             float* __restrict__ lam32, int* status) {
@@ -1371,6 +1373,89 @@ __global__ void __launch_bounds__(kBjThreads) k_block_jacobi(int32_t n_c, const 
         }
         __syncwarp();
     }
+}
+
+// The same with a thread per camera, the blocks staged in shared memory: the same operations per entry, so the
+// same bits.  A warp per camera pays a warp-wide float64 operation (19 cycles of the SM's float64 pipe) for
+// lanes of which 13 to 32 hold an entry, and fills the pipe from about 1000 cameras on; here every lane works,
+// in one long chain.  Mixed, 2000 / 4000 / 20,000 cameras: 29 / 51 / 222 us by warps, 49 / 49 / 69 us by threads; the
+// two meet at 3400 (float64) to 3900 cameras.
+constexpr int kBjCams = 32;
+__global__ void __launch_bounds__(kBjCams) k_block_jacobi_cams(int32_t n_c, const double* __restrict__ Sd,
+                                                               double* __restrict__ Dinv, double* __restrict__ lam,
+                                                               float* __restrict__ lam32, int* status) {
+    __shared__ double sb[kBjCams * 81];
+    const int t = threadIdx.x;
+    for (int64_t j0 = int64_t(blockIdx.x) * kBjCams; j0 < n_c; j0 += int64_t(gridDim.x) * kBjCams) {
+        const int nj = int(n_c - j0 < kBjCams ? n_c - j0 : kBjCams);
+#pragma unroll 27   // loads in flight
+        for (int u = 0; u < 81; ++u) {
+            const int e = t + kBjCams * u;
+            sb[e] = e < 81 * nj ? Sd[81 * j0 + e] : 0.0;
+        }
+        __syncthreads();
+        if (t < nj) {
+            double* B = sb + 81 * t;
+            double x[45], sc[9];
+            if (lam) {
+#pragma unroll
+                for (int a = 0; a < 9; ++a) {
+                    const double d = B[10 * a];
+                    sc[a] = d > 0.0 ? 1.0 / sqrt(d) : 1.0;
+                    lam[9 * (j0 + t) + a] = sc[a];
+                    lam32[9 * (j0 + t) + a] = float(sc[a]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 9; ++i)
+#pragma unroll
+                for (int j = 0; j <= i; ++j) {
+                    double v = B[9 * i + j];
+                    if (lam) v *= sc[i] * sc[j];
+                    x[i * (i + 1) / 2 + j] = v;
+                }
+            bool ok = true;
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                double col[9];   // column k before the sweep
+#pragma unroll
+                for (int i = 0; i < 9; ++i) col[i] = i >= k ? x[i * (i + 1) / 2 + k] : x[k * (k + 1) / 2 + i];
+                ok = ok && col[k] > 0.0;
+                const double r = rcp_fast(col[k] > 0.0 ? col[k] : 1.0);
+#pragma unroll
+                for (int i = 0; i < 9; ++i)
+#pragma unroll
+                    for (int j = 0; j <= i; ++j) {
+                        double& v = x[i * (i + 1) / 2 + j];
+                        const double a = i == k || j == k ? (i == j ? 1.0 : -v) : col[i] * col[j];
+                        v = fma(-a, r, i == k || j == k ? 0.0 : v);
+                    }
+            }
+            if (!ok) atomicExch(status, BA_ERR_SINGULAR);
+#pragma unroll
+            for (int i = 0; i < 9; ++i)
+#pragma unroll
+                for (int j = 0; j <= i; ++j) {   // the sweeps leave the negative of the inverse
+                    double v = -x[i * (i + 1) / 2 + j];
+                    if (lam) {
+                        const df64 d = df_from(v);
+                        v = __hiloint2double(__float_as_int(d.lo), __float_as_int(d.hi));   // the pair (hi, lo)
+                    }
+                    B[9 * i + j] = B[9 * j + i] = v;
+                }
+        }
+        __syncthreads();
+        for (int e = t; e < 81 * nj; e += kBjCams) Dinv[81 * j0 + e] = sb[e];
+        __syncthreads();
+    }
+}
+
+static void launch_bj(const Structure& s, const System& y, double* Dinv, double* lam, float* lam32, cudaStream_t st) {
+    if (s.n_c > kBjWarpCams)
+        k_block_jacobi_cams<<<grid_for(s.n_c, kBjCams), kBjCams, 0, st>>>(s.n_c, y.Sd, Dinv, lam, lam32, y.status);
+    else
+        k_block_jacobi<<<grid_for(int64_t(s.n_c) * 32, kBjThreads), kBjThreads, 0, st>>>(s.n_c, y.Sd, Dinv, lam, lam32,
+                                                                                       y.status);
 }
 
 __global__ void k_to_float(const double* __restrict__ in, float* __restrict__ out, int64_t n) {
@@ -1611,12 +1696,12 @@ void launch_cam_prep(const Structure& s, System& y, cudaStream_t st) {
 // Float64: D^{-1}.  Mixed precision: Lam and the inverse blocks of the scaled system only (its solves
 // use no other; launch_block_jacobi_plain forms D^{-1} when it is asked for).
 void launch_block_jacobi(const Structure& s, System& y, cudaStream_t st) {
-    if (y.S32) k_block_jacobi<<<grid_for(int64_t(s.n_c) * 32, kBjThreads), kBjThreads, 0, st>>>(s.n_c, y.Sd, y.Dhat, y.lam, y.lam32, y.status);
+    if (y.S32) launch_bj(s, y, y.Dhat, y.lam, y.lam32, st);
     else launch_block_jacobi_plain(s, y, st);
 }
 
 void launch_block_jacobi_plain(const Structure& s, System& y, cudaStream_t st) {
-    k_block_jacobi<<<grid_for(int64_t(s.n_c) * 32, kBjThreads), kBjThreads, 0, st>>>(s.n_c, y.Sd, y.Dinv, nullptr, nullptr, y.status);
+    launch_bj(s, y, y.Dinv, nullptr, nullptr, st);
 }
 
 

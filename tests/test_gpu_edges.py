@@ -190,3 +190,24 @@ def test_many_problems_give_their_solo_bits(precision, largest):
             x = b.ba_get_delta()
             for q in range(len(batch)):
                 assert np.array_equal(x[off[q]:off[q + 1]], solo[q % len(scenes)][k]), (a, batch[q].n_cams, q)
+
+
+# Handles of more than 3600 cameras form the preconditioner with a thread per camera instead of a warp: the same bits
+# as each problem alone, on both sides of the limit and with a last CTA that is not full.
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("problems", [225, 226, 229])
+def test_preconditioner_of_many_cameras_gives_the_solo_bits(precision, problems):
+    scenes = [sy.tiny(i, n_cams=16, n_pts=200) for i in range(3)]
+    solo = []
+    for sc in scenes:
+        with problem.from_scene(sc, precision=precision) as p:
+            p.ba_build_normal(1e-3)
+            p.ba_solve_pcg(1e-6, 1000)
+            solo.append((p.ba_get_preconditioner().copy(), p.ba_get_delta().copy()))
+    with problem.from_scenes([scenes[b % 3] for b in range(problems)], precision=precision) as b:
+        b.ba_build_normal(1e-3)
+        b.ba_solve_pcg(1e-6, 1000)
+        D, x = b.ba_get_preconditioner(), b.ba_get_delta()
+        for q in range(problems):
+            assert np.array_equal(D[16 * q:16 * q + 16], solo[q % 3][0]), q
+            assert np.array_equal(x[16 * q:16 * q + 16], solo[q % 3][1]), q
