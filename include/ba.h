@@ -89,7 +89,8 @@ typedef struct ba_options {
     int32_t max_refine;        /* MIXED: maximum outer refinement sweeps (default 64) */
     int32_t item_blocks;       /* stored 9x9 blocks of S per work item of the block-sparse products
                                   (longer rows are split): 0 (default) = 512, or 256 below 1200
-                                  cameras (float64: 256 below 800, 128 below 450, 64 below 200);
+                                  cameras (float64: 256 below 800, 128 below 450, 64 below 200; with
+                                  spmv_config 2 512 from 200 on);
                                   else a multiple of 32 in [32, 4096]; ba_autotune sets it */
     int32_t wait_polls;        /* bounded device waits: polls of a tile copy's barrier before the
                                   solve gives up with BA_ERR_TIMEOUT (the kernel then waits for its
@@ -98,7 +99,7 @@ typedef struct ba_options {
                                   wait gives up at once (tests the timeout path; the smallest problems
                                   then run the kernels that wait, like all others) */
     int32_t spmv_config;       /* warps x copy stages per CTA of the tile-streaming one-column product:
-                                  0 (default) = float32 16 x 1, float64 8 x 1; 1 = 8 x 2 / 4 x 2;
+                                  0 (default) = float32 16 x 1, float64 8 x 1; 1 = 8 x 2 / 8 x 1;
                                   2 = 10 x 2 / 2 x 4; ba_autotune sets it */
     int32_t host_loop;         /* 1: drive the iteration and refinement loops from the host (a plain
                                   graph of chunk_iters iterations per launch, the stop flags read back

@@ -566,7 +566,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int po
 // float32 16 warps x 1 stage (measured faster than 8 x 2 for the full-pattern product: more warps
 // cover the gathers of p), float64 8 x 1: two warps per scheduler keep the float64 pipe busy while one
 // waits for its copy (1936 cameras: 0.566 ms, 0.94 of the pipe's rate, against 0.824 ms for 4 x 2 and
-// 1.59 ms for 2 x 4; 601 cameras 85 us against 129 us).  The symmetric product does twice the
+// 1.59 ms for 2 x 4; 601 cameras 85 us against 129 us).  Shape 1 has always been 8 x 1 in float64; 4 x 2, the
+// default before, is slower from 300 cameras on and no faster below.  The symmetric product does twice the
 // arithmetic per tile, so a second stage per warp keeps the next copy in flight during it (shapes 1
 // and 2).  Every shape keeps its stages within 207 KB.
 template <typename T, int CFG>
@@ -575,7 +576,7 @@ template <> struct SpmvShape<float, 0> { static constexpr int kWarps = 16, kStag
 template <> struct SpmvShape<float, 1> { static constexpr int kWarps = 8, kStages = 2; };
 template <> struct SpmvShape<float, 2> { static constexpr int kWarps = 10, kStages = 2; };
 template <> struct SpmvShape<double, 0> { static constexpr int kWarps = 8, kStages = 1; };
-template <> struct SpmvShape<double, 1> { static constexpr int kWarps = 4, kStages = 2; };
+template <> struct SpmvShape<double, 1> { static constexpr int kWarps = 8, kStages = 1; };
 template <> struct SpmvShape<double, 2> { static constexpr int kWarps = 2, kStages = 4; };
 constexpr int kSpmvShapes = 3;
 // Shared memory of k_spmv: the warps' tile stages, the stages' barriers, then the warps' row sums.
@@ -3345,11 +3346,13 @@ static T* ptr(const Buf& b) {
 // faster), 1000 cameras 43.4 / 41.9 us, 1936 cameras 118.1 / 119.1 us (MCG 2.5 % slower); float64 601
 // cameras 82.0 / 71.1 us, 1000 cameras 166 / 174 us.  Float64 below that, at 256 / 128 / 64 blocks: 300
 // cameras 46.8 / 33.3 / 41.3 us, 150 cameras 30.9 / 28.7 / 20.9 us (a float64 tile takes about 3 us, so a
-// row in one warp is a long chain); a float64 batch of 48 problems of 100 to 400 cameras pays for it
+// row in one warp is a long chain), but with shape 2, which has a quarter of the warps, 61.0 us at 128 for 300
+// cameras and 53.3 us at 512, so that shape keeps 512 from 200 cameras on; a float64 batch of 48 problems of 100 to 400 cameras pays for it
 // (530 / 580 / 697 us).  Float32 keeps 256 there: 128 gains 14 % of a PCG solve at 300 cameras and
 // nothing at 150, and costs a batch 5 %.
-static int default_item_blocks(int n_cams, bool fp32) {
+static int default_item_blocks(int n_cams, bool fp32, int cfg) {
     if (fp32) return n_cams < 1200 ? 256 : 512;
+    if (cfg == 2 && n_cams >= 200) return 512;
     return n_cams < 200 ? 64 : (n_cams < 450 ? 128 : (n_cams < 800 ? 256 : 512));
 }
 
@@ -3359,12 +3362,13 @@ static int default_item_blocks(int n_cams, bool fp32) {
 // whose column camera lies in [c0 + s sz, c0 + (s + 1) sz), for s < n_eff (empty segments get
 // one empty item, which writes zeros).
 static std::vector<SpItem> build_items(const std::vector<int64_t>& h_row_ptr, const std::vector<int32_t>& h_col,
-                                       const std::vector<Layout>& lay, bool split, int forced_cb, bool fp32) {
+                                       const std::vector<Layout>& lay, bool split, int forced_cb, bool fp32,
+                                       int cfg) {
     std::vector<SpItem> out;
     int grp = 0;
     for (size_t b = 0; b < lay.size(); ++b) {
         const Layout& L = lay[b];
-        const int cb = forced_cb > 0 ? forced_cb : default_item_blocks(L.nc, fp32);
+        const int cb = forced_cb > 0 ? forced_cb : default_item_blocks(L.nc, fp32, cfg);
         const int nseg = split ? L.n_eff : 1;
         for (int32_t j = L.c0; j < L.c0 + L.nc; ++j) {
             const int64_t rj = h_row_ptr[j], nj = h_row_ptr[j + 1] - rj;
@@ -3517,14 +3521,14 @@ static void ensure_items(Solver* w, const Structure& s, int n_dirs, int forced_c
     const int64_t wg = sms * ng, wu = sms * nu, wl = sms * nl;
     const bool fresh = !w->items_g.items || w->items_cb != cb;
     if (fresh || w->items_g.nw != wg) {
-        upload_items(w->items_g, build_items(s.h_row_ptr, s.h_col, w->lay, false, cb, fp32), wg, ng);
+        upload_items(w->items_g, build_items(s.h_row_ptr, s.h_col, w->lay, false, cb, fp32, cfg), wg, ng);
         if (w->mm_part) cudaFree(w->mm_part);
         w->mm_part = nullptr;
         BA_CUDA_TRY(cudaMalloc(&w->mm_part, sizeof(double) * kMaxDirs * 9 * size_t(w->items_g.n > 0 ? w->items_g.n : 1)));
         ++w->epoch;
     }
     if (!s.h_row_ptr_u.empty() && (fresh || w->items_u.nw != wu)) {
-        upload_items(w->items_u, build_items(s.h_row_ptr_u, s.h_col_u, w->lay, false, cb, fp32), wu, nu);
+        upload_items(w->items_u, build_items(s.h_row_ptr_u, s.h_col_u, w->lay, false, cb, fp32, cfg), wu, nu);
         ++w->epoch;
     }
     if (fresh) {
@@ -3532,7 +3536,7 @@ static void ensure_items(Solver* w, const Structure& s, int n_dirs, int forced_c
         w->items_cb = cb;
     }
     if (n_dirs > 1 && (w->items_l_dirs != n_dirs || w->items_l.nw != wl)) {
-        upload_items(w->items_l, build_items(s.h_row_ptr, s.h_col, w->lay, true, cb, fp32), wl, nl);
+        upload_items(w->items_l, build_items(s.h_row_ptr, s.h_col, w->lay, true, cb, fp32, cfg), wl, nl);
         w->items_l_dirs = n_dirs;
         ++w->epoch;
     }
@@ -4411,6 +4415,7 @@ void solver_autotune(Solver* w, const Structure& s, const System& y, bool fp32, 
     double bms = 0.0;
     for (int cfg = 0; cfg < kSpmvShapes; ++cfg)
         for (int cb : cands) {
+            if (cfg == 1 && !fp32) break;   // the same shape as 0
             const double ms = solver_time_spmv(w, s, y, fp32, reps, cb, cfg, st);
             if (bcb == 0 || ms < bms) {
                 bcfg = cfg;

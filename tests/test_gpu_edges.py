@@ -211,3 +211,20 @@ def test_preconditioner_of_many_cameras_gives_the_solo_bits(precision, problems)
         for q in range(problems):
             assert np.array_equal(D[16 * q:16 * q + 16], solo[q % 3][0]), q
             assert np.array_equal(x[16 * q:16 * q + 16], solo[q % 3][1]), q
+
+
+# spmv_config 1 means 8 warps x 1 stage in float64, today's default shape too: the same product in the same time
+# (the other shapes take 1.4 and 2.8 times as long here).
+def test_float64_shape_1_is_8_warps():
+    sc = sy.dense(1, n_cams=1000, n_pts=100000, n_clusters=33)
+    xy = problem.device_measurements(sc)
+    ms, x = [], []
+    for cfg in (0, 1):
+        with problem.from_scene(sc, xy=xy, spmv_config=cfg) as p:
+            p.ba_build_normal(1e-4)
+            p.ba_time_kernel("spmv", 5)
+            ms.append(min(p.ba_time_kernel("spmv", 10) for _ in range(3)))
+            p.ba_solve_pcg(1e-6, 1000)
+            x.append(p.ba_get_delta().copy())
+    assert ms[1] < 1.2 * ms[0], ms
+    assert np.array_equal(x[0], x[1])
