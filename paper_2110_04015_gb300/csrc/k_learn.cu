@@ -170,12 +170,14 @@ __global__ void k_gnn_features(int32_t n_c, const double* __restrict__ aux, cons
 
 // standardise the centre (per axis: mean removed, divided by the axis' root mean square) and
 // log(1 + d) (mean removed, divided by its standard deviation); one CTA, a quarter of its threads per
-// column (the columns in turn took 18 us)
+// column (the columns in turn took 18 us).  A column is scaled by a power of two to below two first, which
+// changes no bit of the result but keeps the double-float squares in range in any length unit.
 constexpr int kStdThreads = 1024;
 __global__ void __launch_bounds__(kStdThreads) k_gnn_standardize(int32_t n_c, float* __restrict__ X) {
     constexpr int NT = kStdThreads / 4;
     __shared__ float2 red[kStdThreads / 32];
     __shared__ float2 stat[4];
+    __shared__ float top[kStdThreads / 32];
     const int grp = threadIdx.x / NT, t = threadIdx.x % NT, f = grp < 3 ? grp : 6;
     // f(the sum of v over the threads of this quarter), computed once per quarter: a float64 division by
     // every thread would queue on the float64 pipe
@@ -193,17 +195,26 @@ __global__ void __launch_bounds__(kStdThreads) k_gnn_standardize(int32_t n_c, fl
         __syncthreads();
         return df_ld(&stat[grp]);
     };
+    float m = 0.f;
+    for (int64_t j = t; j < n_c; j += NT) m = fmaxf(m, fabsf(X[kF * j + f]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) top[threadIdx.x >> 5] = m;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) m = fmaxf(m, top[grp * (NT / 32) + w]);
+    const float unit = m > 0.f && !isinf(m) ? ldexpf(1.f, -max(ilogbf(m), -126)) : 1.f;
     df64 s(0.f);
-    for (int64_t j = t; j < n_c; j += NT) s += df64(X[kF * j + f]);
+    for (int64_t j = t; j < n_c; j += NT) s += df64(X[kF * j + f] * unit);
     const df64 mean = quarter(s, [&](double v) { return v / n_c; });
     df64 q(0.f);
     for (int64_t j = t; j < n_c; j += NT) {
-        const df64 v = df64(X[kF * j + f]) - mean;
+        const df64 v = df64(X[kF * j + f] * unit) - mean;
         q += v * v;
     }
     const df64 inv = quarter(q, [&](double v) { return v > 0.0 ? 1.0 / sqrt(v / n_c) : 1.0; });
     for (int64_t j = t; j < n_c; j += NT) {
-        const df64 v = (df64(X[kF * j + f]) - mean) * inv;
+        const df64 v = (df64(X[kF * j + f] * unit) - mean) * inv;
         X[kF * j + f] = __fadd_rn(v.hi, v.lo);
     }
 }

@@ -228,3 +228,26 @@ def test_float64_shape_1_is_8_warps():
             x.append(p.ba_get_delta().copy())
     assert ms[1] < 1.2 * ms[0], ms
     assert np.array_equal(x[0], x[1])
+
+
+# The network's centre features are standardised per axis, so a power of two as the length unit changes no bit of them,
+# however far the squares of the coordinates are from float32's range.
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("k", [-70, -20, 20, 62])
+def test_network_features_do_not_depend_on_the_length_unit(k, precision):
+    sc, m, _ = _system(24, 1200)
+    X = []
+    for s in (1.0, 2.0 ** k):
+        cams = sc.cams0.copy()
+        cams[:, 3:6] *= s
+        with binding.Problem(cams, sc.pts0 * s, sc.obs_cam, sc.obs_pt, m, precision=precision) as p:
+            if k == -70 and precision == "mixed" and s < 1.0:   # the float32 build has no such range
+                with pytest.raises(binding.BAError) as e:
+                    p.ba_build_normal(1e-4)
+                assert e.value.code == binding.BA_ERR_SINGULAR
+                return
+            p.ba_build_normal(1e-4)
+            g = binding.GNN(np.zeros(17537, np.float32))
+            X.append(g.ba_gnn_graph(p)[0])
+            g.close()
+    assert np.array_equal(X[0][:, :6], X[1][:, :6])
