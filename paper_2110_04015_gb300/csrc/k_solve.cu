@@ -86,6 +86,7 @@ struct Ctl {
     int off_cur;
     double rr0, rr, rz, ga, tol2, tau;
     double rr0_inv;    // 1 / rr0: the residual history stores rr / rr0 without a division per step
+    int alone;         // k_one_cta or k_pcg_cluster solves the problem; done is set for everyone else
     int live;          // the problem was not done at this iteration's update (read by the kernel whose
                        // first CTA runs the decide step, which may set done meanwhile)
     double alpha_v[kMaxDirs];
@@ -1200,12 +1201,19 @@ __global__ void __launch_bounds__(kUpdThreads) k_init_vec(const Layout* __restri
     cta_publish<T, 1>(v, partial + int64_t(blockIdx.y) * gridDim.x);
 }
 
+// Which problems k_one_cta (mixed precision) and k_pcg_cluster (float64 PCG) solve; their comments say why.
+constexpr int kOneCams = 20, kOneDirs = 10, kCluCams = 24;
+__host__ __device__ __forceinline__ bool solved_alone(const Layout& L, bool fp32, bool mcg) {
+    return fp32 ? L.nc <= kOneCams && (!mcg || L.n_eff <= kOneDirs) : L.nc <= kCluCams && !mcg;
+}
+
 // One warp per problem.  outer (mixed precision, may be null) supplies the sweep's tolerance and
-// iteration budget and leaves the problems that are not refined any more done from the start.
+// iteration budget and leaves the problems that are not refined any more done from the start.  small: mark the
+// problems that are solved alone; they are done for the kernels of the iterations.
 template <typename T>
 __global__ void k_init_ctl(Ctl* ctl, const Layout* __restrict__ lay, const WideSlot<T>* __restrict__ partial, int np,
                            const Params* __restrict__ prm, double stag, int direct_q,
-                           const Outer* __restrict__ outer, int* blk_off, int* blk_w, int mi1) {
+                           const Outer* __restrict__ outer, int* blk_off, int* blk_w, int mi1, int small) {
     const int p = blockIdx.x;
     const double rr0 = warp_sum_slots<T>(partial + int64_t(p) * np, np).value();
     if (threadIdx.x == 0) {
@@ -1248,6 +1256,7 @@ __global__ void k_init_ctl(Ctl* ctl, const Layout* __restrict__ lay, const WideS
         if (!act) { c.done = 1; }
         else if (!(rr0 == rr0) || isinf(rr0)) { c.done = 1; c.status = BA_ERR_BREAKDOWN; }
         else if (rr0 == 0.0 || mi <= 0) { c.done = 1; c.status = rr0 == 0.0 ? BA_OK : BA_ERR_NOT_CONVERGED; }
+        if (small && !c.done && solved_alone(c.lay, sizeof(T) == 4, prm->mcg != 0)) c.alone = c.done = 1;
         ctl[p] = c;
         blk_off[int64_t(p) * mi1] = 0;
         blk_w[int64_t(p) * mi1] = 1;
@@ -2504,15 +2513,9 @@ __global__ void __launch_bounds__(NW * 32, NW < PqShape<T>::kSlices ? 4 : RL == 
 // (20 cameras) 33.4 against 33.6 us, with 16 directions (16 cameras) 92 against 60 us.
 // Larger problems run the kernels above; a handle whose tile waits give up at once (wait_polls = -1) does
 // too, since there is no tile wait here.
-constexpr int kOneCams = 20;
-constexpr int kOneDirs = 10;
 constexpr int kOneRows = 9 * kOneCams;
 constexpr int kOneTile = 64;
 constexpr int kOneThreads = 512;   // solve_block uses as many; more would leave 64 registers a thread
-
-__host__ __device__ __forceinline__ bool one_cta_takes(const Layout& L, bool mcg) {
-    return L.nc <= kOneCams && (!mcg || L.n_eff <= kOneDirs);
-}
 
 struct OneSmem {
     Ctl c;
@@ -2643,13 +2646,16 @@ __global__ void __launch_bounds__(kOneThreads, 1)
               WideSlot<float>* phip, double* dpinv, float* beta, int* __restrict__ colblk, double* __restrict__ hist,
               int* blk_off, int* blk_w, int mi1, Ctl* ctl) {
     const int p = blockIdx.x, t = threadIdx.x;
-    if (!one_cta_takes(ctl[p].lay, mcg) || ctl[p].done) return;
+    if (!ctl[p].alone) return;
     extern __shared__ __align__(16) unsigned char smem_one[];
     OneSmem& m = *reinterpret_cast<OneSmem*>(smem_one);
     float* S = reinterpret_cast<float*>(smem_one + (sizeof(OneSmem) + 15) / 16 * 16);
     const Layout L = ctl[p].lay;
     const int nc = L.nc, n = 9 * nc, c0 = L.c0;
-    if (t == 0) m.c = ctl[p];
+    if (t == 0) {
+        m.c = ctl[p];
+        m.c.alone = m.c.done = 0;   // running, for this CTA
+    }
     for (int u = t; u < nc * nc * 81; u += kOneThreads) S[u] = 0.f;
     for (int u = t; u < kOneRows * kMaxDirs + 4 * kOneCams; u += kOneThreads) m.PT[u] = m.QT[u] = 0.f;
     __syncthreads();
@@ -2924,7 +2930,6 @@ constexpr size_t one_smem(int nc) { return (sizeof(OneSmem) + 15) / 16 * 16 + si
 // rows' vectors live in the registers of its first warp, and the CTAs exchange the sums and the direction
 // through distributed shared memory, three cluster barriers per iteration (16 cameras: 6 us).  The rule is
 // the camera count alone, as for k_one_cta, and so is the exception (wait_polls = -1).
-constexpr int kCluCams = 24;
 constexpr int kCluThreads = 256;
 constexpr int kCluOwn = kCluCams / kSmallCtas;   // cameras of a CTA, 27 rows: one warp
 static_assert(9 * kCluOwn <= 32 && kCluCams % kSmallCtas == 0, "a CTA's rows in one warp");
@@ -2937,7 +2942,7 @@ __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kCluThreads
     cluster_arrive();   // waited for before the first store to another CTA: every CTA has started by then
     const int p = blockIdx.x / kSmallCtas, rank = blockIdx.x % kSmallCtas;
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    if (ctl[p].lay.nc > kCluCams || ctl[p].done) {   // the same in every CTA: the first one writes ctl after barriers
+    if (!ctl[p].alone) {   // the same in every CTA: the first one writes ctl after barriers
         cluster_wait();
         return;
     }
@@ -2947,7 +2952,10 @@ __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kCluThreads
     __shared__ int stop;
     const Layout L = ctl[p].lay;
     const int nc = L.nc, c0 = L.c0, own = rank < nc ? (nc - rank + kSmallCtas - 1) / kSmallCtas : 0;
-    if (t == 0) sc = ctl[p];
+    if (t == 0) {
+        sc = ctl[p];
+        sc.alone = sc.done = 0;   // running, for this cluster
+    }
     for (int u = t; u < own * nc * 81; u += kCluThreads) S[u] = 0.0;
     for (int u = t; u < 9 * nc; u += kCluThreads) sp[u] = zg[9 * c0 + u];
     __syncthreads();
@@ -3298,6 +3306,8 @@ struct Solver {
     std::vector<std::vector<double>> host_hist;   // per problem, residual history of the last solve
     int64_t launches = 0;     // kernel executions issued by the current solve
     cudaStream_t cap_stream = nullptr, cap2 = nullptr, cap3 = nullptr;   // capture streams (nested loops)
+    cudaStream_t cap_side = nullptr;                  // and of the branch of problems solved alone
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     std::vector<SolveExec*> execs;   // instantiated solve graphs
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;   // around a solve
     // work lists of the block-sparse products: whole rows, rows split by pose subset, and whole rows of
@@ -3577,7 +3587,7 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
         L.phoff = phoff;
         L.boff = boff;
         // (a problem that one CTA solves keeps its history in whole tiles of columns; 16-byte aligned)
-        const int64_t cols = fp32 && one_cta_takes(L, a.mcg != 0) ? (cap + kOneTile - 1) / kOneTile * kOneTile : cap;
+        const int64_t cols = fp32 && solved_alone(L, true, a.mcg != 0) ? (cap + kOneTile - 1) / kOneTile * kOneTile : cap;
         hoff += (cols * 9 * int64_t(L.nc) + 3) / 4 * 4;
         phoff += cap * L.n_eff * L.K;
         boff += cap;
@@ -3610,6 +3620,9 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     if (!w->cap_stream) BA_CUDA_TRY(cudaStreamCreateWithFlags(&w->cap_stream, cudaStreamNonBlocking));
     if (!w->cap2) BA_CUDA_TRY(cudaStreamCreateWithFlags(&w->cap2, cudaStreamNonBlocking));
     if (!w->cap3) BA_CUDA_TRY(cudaStreamCreateWithFlags(&w->cap3, cudaStreamNonBlocking));
+    if (!w->cap_side) BA_CUDA_TRY(cudaStreamCreateWithFlags(&w->cap_side, cudaStreamNonBlocking));
+    if (!w->ev_fork) BA_CUDA_TRY(cudaEventCreateWithFlags(&w->ev_fork, cudaEventDisableTiming));
+    if (!w->ev_join) BA_CUDA_TRY(cudaEventCreateWithFlags(&w->ev_join, cudaEventDisableTiming));
     if (!w->h_params) BA_CUDA_TRY(cudaMallocHost(&w->h_params, sizeof(Params)));
     if (!w->h_loops) BA_CUDA_TRY(cudaMallocHost(&w->h_loops, sizeof(Loops)));
     grow(w->P, size_t(hoff) * elt);
@@ -3629,8 +3642,7 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     w->one_cams = 0;
     w->all_small = true;
     for (const Layout& L : lay) {
-        const bool small = fp32 ? one_cta_takes(L, a.mcg != 0) : !a.mcg && L.nc <= kCluCams;
-        if (small && a.wait_polls > 0) w->one_cams = std::max(w->one_cams, L.nc);
+        if (solved_alone(L, fp32, a.mcg != 0) && a.wait_polls > 0) w->one_cams = std::max(w->one_cams, L.nc);
         else w->all_small = false;
     }
     if (fp32 && w->one_cams > 0) grow(w->colblk, size_t(boff) * sizeof(int));
@@ -3717,6 +3729,9 @@ void solver_destroy(Solver* w) {
     if (w->cap_stream) cudaStreamDestroy(w->cap_stream);
     if (w->cap2) cudaStreamDestroy(w->cap2);
     if (w->cap3) cudaStreamDestroy(w->cap3);
+    if (w->cap_side) cudaStreamDestroy(w->cap_side);
+    if (w->ev_fork) cudaEventDestroy(w->ev_fork);
+    if (w->ev_join) cudaEventDestroy(w->ev_join);
     delete w;
 }
 
@@ -3862,17 +3877,18 @@ static int enqueue_iteration(Solver* w, const Structure& s, const T* S, const T*
     }
 }
 
-// x = 0, r = sign * rhs, z = D^{-1} r, P_0 = z and the control blocks; returns the launches.
+// x = 0, r = sign * rhs, z = D^{-1} r, P_0 = z and the control blocks (small: of problems solved alone too);
+// returns the launches.
 template <typename T>
 static int krylov_init(Solver* w, const Structure& s, const T* S, const T* Su, const double* Dinv, const double* rhs,
-                       double sign, const double* scale, T* x, const Outer* outer, cudaStream_t st) {
+                       double sign, const double* scale, T* x, const Outer* outer, cudaStream_t st, bool small) {
     const int nb = w->nb;
     k_init_vec<T><<<dim3(w->gu, nb), kUpdThreads, 0, st>>>(ptr<Layout>(w->lay_d), rhs, sign, scale, Dinv, outer, x,
                                                             ptr<T>(w->r), ptr<T>(w->z), ptr<T>(w->P),
                                                             ptr<WideSlot<T>>(w->part_b));
     k_init_ctl<T><<<nb, 32, 0, st>>>(ptr<Ctl>(w->ctl), ptr<Layout>(w->lay_d), ptr<WideSlot<T>>(w->part_b), w->gu,
                                   ptr<Params>(w->params), sizeof(T) == 4 ? kStagnation : 0.0, sizeof(T) == 4 ? 1 : 0,
-                                  outer, ptr<int>(w->blk_off), ptr<int>(w->blk_w), w->mi1);
+                                  outer, ptr<int>(w->blk_off), ptr<int>(w->blk_w), w->mi1, small);
     return 2;
 }
 
@@ -3893,16 +3909,31 @@ static int enqueue_small(Solver* w, const Structure& s, const System& y, bool mc
     return 1;
 }
 
+// problems solved alone in a batch with others
+static bool beside(const Solver* w) { return w->one_cams > 0 && !w->all_small; }
+static void join_small(Solver* w, cudaStream_t st) {
+    if (beside(w)) BA_CUDA_TRY(cudaStreamWaitEvent(st, w->ev_join));
+}
+
 // The start of a sweep: krylov_init, the problems that are solved whole, and Q_0 = S P_0 of the others, from
 // which Algorithm 2 starts its iterations (Algorithm 1 forms Q = S P first in every one).  Problems that are
-// solved whole form their own Q_0 and are done by then: they take part in no tile-streaming product,
-// so no tile wait can end them.  Returns the launches.
+// solved whole form their own Q_0 and are done for everyone else: they take part in no tile-streaming
+// product, so no tile wait can end them.  In a batch with larger problems they run on a branch of the graph
+// (stream side, joined by join_small) beside the others' iterations: one after the other, 8 problems of 20
+// cameras and 8 of 300 took 11.8 ms to 1e-9 (MCG, 8 directions), beside each other 9.9 ms; the 300s alone 8.9.
+// Returns the launches.
 template <typename T>
 static int krylov_start(Solver* w, const Structure& s, const System& y, const T* S, const T* Su, const double* Dinv,
                         const double* rhs, double sign, const double* scale, T* x, const Outer* outer, bool mcg,
-                        cudaStream_t st) {
-    int n = krylov_init<T>(w, s, S, Su, Dinv, rhs, sign, scale, x, outer, st);
-    n += enqueue_small(w, s, y, mcg, sizeof(T) == 8 ? reinterpret_cast<double*>(x) : nullptr, st);
+                        cudaStream_t st, cudaStream_t side) {
+    int n = krylov_init<T>(w, s, S, Su, Dinv, rhs, sign, scale, x, outer, st, w->one_cams > 0);
+    if (!beside(w)) side = nullptr;
+    if (side) {
+        BA_CUDA_TRY(cudaEventRecord(w->ev_fork, st));
+        BA_CUDA_TRY(cudaStreamWaitEvent(side, w->ev_fork));
+    }
+    n += enqueue_small(w, s, y, mcg, sizeof(T) == 8 ? reinterpret_cast<double*>(x) : nullptr, side ? side : st);
+    if (side) BA_CUDA_TRY(cudaEventRecord(w->ev_join, side));
     if (mcg && !w->all_small) n += enqueue_product<T, 0>(w, s, S, Su, ptr<T>(w->P), kSelLive, ptr<T>(w->Q), nullptr, st);
     return n;
 }
@@ -3963,7 +3994,7 @@ static void capture_krylov(Solver* w, const Structure& s, const System& y, const
                            const double* rhs, double sign, const double* scale, T* x, const Outer* outer, bool mcg,
                            int chunk, cudaStream_t cs, cudaStream_t cb, int* pre, int* per_pass) {
     const cudaGraphConditionalHandle h = capture_handle(cs);
-    *pre = krylov_start<T>(w, s, y, S, Su, Dinv, rhs, sign, scale, x, outer, mcg, cs) + 1;
+    *pre = krylov_start<T>(w, s, y, S, Su, Dinv, rhs, sign, scale, x, outer, mcg, cs, w->cap_side) + 1;
     k_loop_cond<<<1, kThreads, 0, cs>>>(h, 1, ptr<Ctl>(w->ctl), w->nb, ptr<Loops>(w->loops), 1, chunk,
                                         ptr<Params>(w->params));
     cudaGraph_t body = capture_while(cs, h);
@@ -3975,6 +4006,7 @@ static void capture_krylov(Solver* w, const Structure& s, const System& y, const
     cudaGraph_t done = nullptr;
     cudaError_t e = cudaStreamEndCapture(cb, &done);
     if (e != cudaSuccess) throw Error(BA_ERR_CUDA, std::string("loop body capture: ") + cudaGetErrorString(e));
+    join_small(w, cs);
 }
 
 
@@ -4091,7 +4123,8 @@ static void run_host_loops(Solver* w, const Structure& s, const System& y, const
     const cudaGraphConditionalHandle none = cudaGraphConditionalHandle();
     int64_t launches = 0;
     if (!fp32) {
-        launches += krylov_start<double>(w, s, y, y.S, nullptr, y.Dinv, y.bt, -1.0, nullptr, x, nullptr, a.mcg != 0, st);
+        launches += krylov_start<double>(w, s, y, y.S, nullptr, y.Dinv, y.bt, -1.0, nullptr, x, nullptr, a.mcg != 0, st,
+                                         nullptr);
         k_loop_cond<<<1, kThreads, 0, st>>>(none, 0, ptr<Ctl>(w->ctl), nb, lp, 1, a.chunk, prm);
         launches += 1 + host_krylov_loop(w, chunk_exec, gc, a, st, waits);
         launches += true_residual(w, s, y, x, nullptr, st);
@@ -4108,7 +4141,7 @@ static void run_host_loops(Solver* w, const Structure& s, const System& y, const
             for (int b = 0; b < nb && !any; ++b) any = w->h_outer[b].swept != 0;
             if (!any) break;
             launches += krylov_start<float>(w, s, y, y.S32, y.S32u, y.Dhat, ptr<double>(w->rt), 1.0, y.lam,
-                                            ptr<float>(w->xw), ptr<Outer>(w->outer), a.mcg != 0, st);
+                                            ptr<float>(w->xw), ptr<Outer>(w->outer), a.mcg != 0, st, nullptr);
             k_loop_cond<<<1, kThreads, 0, st>>>(none, 0, ptr<Ctl>(w->ctl), nb, lp, 1, a.chunk, prm);
             launches += 1 + host_krylov_loop(w, chunk_exec, gc, a, st, waits);
             k_accumulate<<<dim3(w->gx, nb), kThreads, 0, st>>>(ptr<Layout>(w->lay_d), ptr<Outer>(w->outer),
@@ -4377,9 +4410,9 @@ double solver_time_spmv(Solver* w, const Structure& s, const System& y, bool fp3
     hp->max_iters = 1;
     BA_CUDA_TRY(cudaMemcpyAsync(w->params.p, hp, sizeof(Params), cudaMemcpyHostToDevice, st));
     if (fp32)
-        krylov_init<float>(w, s, y.S32, y.S32u, y.Dhat, y.bt, -1.0, y.lam, ptr<float>(w->xw), nullptr, st);
+        krylov_init<float>(w, s, y.S32, y.S32u, y.Dhat, y.bt, -1.0, y.lam, ptr<float>(w->xw), nullptr, st, false);
     else
-        krylov_init<double>(w, s, y.S, nullptr, y.Dinv, y.bt, -1.0, nullptr, ptr<double>(w->xw), nullptr, st);
+        krylov_init<double>(w, s, y.S, nullptr, y.Dinv, y.bt, -1.0, nullptr, ptr<double>(w->xw), nullptr, st, false);
     BA_CUDA_TRY(cudaGetLastError());
     cudaEvent_t e0, e1;
     BA_CUDA_TRY(cudaEventCreate(&e0));

@@ -251,3 +251,17 @@ def test_network_features_do_not_depend_on_the_length_unit(k, precision):
             X.append(g.ba_gnn_graph(p)[0])
             g.close()
     assert np.array_equal(X[0][:, :6], X[1][:, :6])
+
+
+# In a batch with larger problems the small ones run beside their iterations, not before them: the batch takes less than
+# the larger problems and the small ones one after the other (measured 9.9 against 8.9 + 2.6 ms).
+def test_small_problems_run_beside_larger_ones():
+    small = [sy.tiny(i, n_cams=20, n_pts=1500) for i in range(8)]
+    large = [sy.dense(i, n_cams=300, n_pts=30000, n_clusters=10) for i in range(8)]
+    ms = []
+    for scenes in (small, large, small + large):
+        with problem.from_scenes(scenes, precision="mixed") as b:
+            b.ba_build_normal(1e-4)
+            t = [b.ba_solve_mcg(1e-9, 1000, 8, 3.0)["ms"] for _ in range(7)]
+            ms.append(float(np.median(t)))
+    assert ms[2] < ms[1] + 0.75 * ms[0], ms
