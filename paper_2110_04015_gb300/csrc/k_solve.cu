@@ -641,6 +641,16 @@ __device__ __forceinline__ void camera_dots(int lane, T q, T p, T r, double* cam
     }
 }
 
+// A warp that gives up at item i leaves it and its later ones undone: their problems (of a batch, possibly
+// others than the one whose copy was waited for) end with the status at their next decide step.
+__device__ __forceinline__ void report_timeout(Ctl* ctl, const ItemList& L, int sel, int64_t i, const WarpItems& wi) {
+    if (threadIdx.x & 31) return;
+    for (; i < wi.end; i += wi.step) {
+        const int prob = L.items[i].prob;
+        if (selected(ctl, prob, sel)) atomicExch(&ctl[prob].status, BA_ERR_TIMEOUT);
+    }
+}
+
 // Tile cursor of a warp: the tiles of its selected items (WarpItems) in order, skipping empty
 // items.  The consumer loop selects items with the same predicate, which no kernel changes while
 // it runs.
@@ -729,8 +739,8 @@ __global__ void __launch_bounds__(SpmvShape<T, CFG>::kWarps * 32, 1) k_spmv(
     }
     int stage = 0;
     bool bad = false;
-    int bad_prob = 0;
-    for (int64_t i = wi.i0; i < wi.end && !bad; i += wi.step) {
+    int64_t i = wi.i0;
+    for (; i < wi.end; i += wi.step) {
         const SpItem it = L.items[i];
         if (!selected(ctl, it.prob, sel)) continue;
         const Ctl& c = ctl[it.prob];
@@ -777,7 +787,6 @@ __global__ void __launch_bounds__(SpmvShape<T, CFG>::kWarps * 32, 1) k_spmv(
                 const bool ok = mbar_wait(&bars[stage], (parity >> stage) & 1u, L.polls);
                 if (!__all_sync(0xffffffffu, ok)) {
                     bad = true;
-                    bad_prob = it.prob;
                     break;
                 }
                 parity ^= 1u << stage;
@@ -860,7 +869,7 @@ __global__ void __launch_bounds__(SpmvShape<T, CFG>::kWarps * 32, 1) k_spmv(
     if (bad) {
         // a copy did not land in time: report, then wait (bounded) for this warp's copies in flight;
         // the problem's next decide step ends it with the status
-        if (lane == 0) atomicExch(&ctl[bad_prob].status, BA_ERR_TIMEOUT);
+        report_timeout(ctl, L, sel, i, wi);
         for (int st = 0; st < NS; ++st)
             if (inflight & (1u << st)) mbar_wait(&bars[st], (parity >> st) & 1u, kDefaultWaitPolls);
     }
@@ -1021,8 +1030,8 @@ __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
     }
     int stage = 0;
     bool bad = false;
-    int bad_prob = 0;
-    for (int64_t i = wi.i0; i < wi.end && !bad; i += wi.step) {
+    int64_t i = wi.i0;
+    for (; i < wi.end; i += wi.step) {
         const SpItem it = L.items[i];
         if (!selected(ctl, it.prob, sel)) continue;
         const Ctl& c = ctl[it.prob];
@@ -1058,7 +1067,6 @@ __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
                 const bool ok = mbar_wait(&bars[stage], (parity >> stage) & 1u, L.polls);
                 if (!__all_sync(0xffffffffu, ok)) {
                     bad = true;
-                    bad_prob = it.prob;
                     break;
                 }
                 parity ^= 1u << stage;
@@ -1154,7 +1162,7 @@ __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
         __syncwarp();
     }
     if (bad) {
-        if (lane == 0) atomicExch(&ctl[bad_prob].status, BA_ERR_TIMEOUT);
+        report_timeout(ctl, L, sel, i, wi);
         for (int st = 0; st < NS; ++st)
             if (inflight & (1u << st)) mbar_wait(&bars[st], (parity >> st) & 1u, kDefaultWaitPolls);
     }

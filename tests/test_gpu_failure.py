@@ -11,6 +11,7 @@ import numpy as np
 import pytest
 
 from paper_2110_04015_gb300 import binding, problem
+from paper_2110_04015_gb300 import synthetic as sy
 from tests._gpu import scene
 
 pytestmark = pytest.mark.gpu
@@ -90,3 +91,17 @@ def test_counters_of_an_interrupted_product_are_cleared(precision):
             assert binding.lib().ba_test_interrupt_products(p.h) == 0
             assert solve()["status"] == 0
             assert np.array_equal(p.ba_get_delta(), x)
+
+
+# A warp whose wait gives up leaves the later items of its list too, and in a batch of more rows than warps those can be
+# another problem's: every problem that lost an item must end with TIMEOUT, none go on with what is left of its product.
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_every_problem_of_a_timed_out_batch_reports_it(precision):
+    scenes = [sy.tiny(i % 3, n_cams=25, n_pts=500) for i in range(240)]
+    with problem.from_scenes(scenes, precision=precision, wait_polls=-1) as b:
+        b.ba_build_normal(1e-4)
+        for solve in (lambda: b.ba_solve_pcg(1e-6, 50), lambda: b.ba_solve_mcg(1e-6, 50, 8, 1e9)):
+            with pytest.raises(binding.BAError) as e:
+                solve()
+            assert e.value.code == binding.BA_ERR_TIMEOUT
+            assert all(s["status"] == binding.BA_ERR_TIMEOUT for s in b.ba_get_batch_stats())
