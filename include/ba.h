@@ -79,8 +79,9 @@ typedef struct ba_options {
     int32_t chunk_iters;       /* Krylov iterations per pass of the solve graph's device-side loop
                                   between checks of the stop flags (default 8, 1..256); a solve is
                                   one graph launch and the host waits once, at its end (problems of
-                                  up to 20 cameras in MIXED, 24 in FP64 PCG, run a whole sweep in
-                                  one launch instead) */
+                                  up to 20 cameras in MIXED, by MCG with up to 10 subsets, and of up
+                                  to 24 in FP64 PCG run a whole sweep in one launch instead, in a
+                                  batch beside the larger ones) */
     int32_t max_history;       /* MCG: maximum stored direction columns (default 0 = max_iters * n_dirs + 1);
                                   when it is full FP64 stops with OOM, while MIXED ends the float32
                                   sweep and the refinement starts another from the true residual */

@@ -10,8 +10,8 @@
 // float64 iterative refinement of mixed precision is an outer WHILE node around it), so the host
 // launches the graph once and reads the results once; nothing inside a solve waits on the host.
 // A problem whose Ctl::done is set is skipped by every later launch while the others go on.
-// Problems of a few cameras run their whole sweep in one launch before that loop (k_one_cta,
-// k_pcg_cluster).
+// Problems of a few cameras run their whole sweep in one launch (k_one_cta, k_pcg_cluster), beside that
+// loop where a batch has larger ones too.
 //
 // Batches: problem b owns the cameras [c0, c0 + nc) of the handle (S is block-diagonal over the
 // problems, since no landmark is seen by two of them).  Per-problem kernels take the problem from
@@ -52,10 +52,11 @@ constexpr int kGramMax = kMaxDirs * kMaxDirs + kMaxDirs;   // Delta (w x w) and 
 constexpr int kChunkCams = 112;                             // cameras per Phi partial
 constexpr double kStagnation = 1e-4;                        // float32 sweep stop on t_i (see Ctl::stag)
 // Cameras and threads per CTA of the update kernels (126 rows).  Their time is a chain of latencies
-// (the camera sums, D^{-1} r, the CTA sum, the arrival of the last CTA), so the CTAs are small: 72 of
-// them for 1000 cameras; with 252 rows each, half as many SMs carried twice the arithmetic.
+// (the camera sums, D^{-1} r, the CTA sum), so the CTAs are small: 72 of them for 1000 cameras; with 252
+// rows each, half as many SMs carried twice the arithmetic.
 constexpr int kUpdCams = 14;
 constexpr int kUpdThreads = 128;
+constexpr int kMaxProblemCams = 28 * 65535;   // accepted in one problem (no grid is near its limit there)
 
 // Where one problem of the batch lives (fixed for a solve).
 struct Layout {           // no padding (compared as bytes)
@@ -963,10 +964,11 @@ __global__ void __launch_bounds__(kColWarps * 32, 12) k_spmv_col(const int64_t* 
 // used by the float32 sweeps, where the Eq. 18 update cancels).  Tiles stream through
 // shared memory as in k_spmv; CL lanes share a block (CL = 4, or 2 when no block is wider than 8
 // columns): lane = CL qi + g takes tile-local blocks qi, qi + 32 / CL, ... and columns
-// 4g .. 4g + 3, so each 9x9 block multiplies up to 4 CL columns per read from shared memory.  The kernel
-// is bound by what its lanes read from shared memory and L1 (81 words of S and 36 of P per 324
-// multiply-adds), so lanes left without columns cost as much as the others: N = 8 on 1000 dense cameras
-// took 94 us per local step with four lanes a block and takes 75 us with two (one lane for N = 4: 76 us).  PT is the row-major copy (9 n_c x 16, all problems) of the new blocks.
+// 4g .. 4g + 3, so each 9x9 block multiplies up to 4 CL columns per read from shared memory.  No unit is at
+// its limit (1000 dense cameras: L1 and shared memory 62 %, DRAM 42 %, issue 34 %); a warp waits most for its P
+// gathers, then for its 81 words of S and 36 of P per 324 multiply-adds.  Lanes left without columns wait like
+// the others: N = 8 on 1000 dense cameras took 94 us per local step with four lanes a block and takes 75 us
+// with two (one lane for N = 4: 76 us).  PT is the row-major copy (9 n_c x 16, all problems) of the new blocks.
 // The multi-column product waits on L2 gathers of PT more than on its tiles, so it runs twice
 // the warps of k_spmv with one tile stage each (the other warps' copies and arithmetic cover a
 // warp's wait for its next tile); at most 128 registers a thread.
@@ -1384,8 +1386,10 @@ __device__ __forceinline__ void sum_camdot(const double* cd, int nc, ExactSum<T>
 // partition depends on the problem alone (the grid has a CTA for every chunk of the largest).
 // Bound by latency: on 1000 cameras 12 us of a 22 us iteration when the sums ran in float64 (whose
 // pipe does 1.7 lanes per clock and SM, so each warp-wide addition of a shuffle tree costs as much as
-// a full one); 8.6 us with the float32 sweeps' sums as float pairs; 3.3 us with the camera sums' loads in
+// a full one); 8.6 us with the float32 sweeps' sums on the float32 pipe; 3.4 us with the camera sums' loads in
 // flight together and the decide step in k_pcg_dir.
+// Every CTA reads all camera sums, 16 n ceil(n / 14) bytes an iteration: 4 MB of L2 reads at 1936 cameras and
+// 1 GB at 30,000, where an iteration on a banded S takes 193 us (311 us with 28 cameras a CTA and float64 sums).
 template <typename T>
 __global__ void __launch_bounds__(kUpdThreads) k_pcg_update(const double* __restrict__ Dinv, const T* __restrict__ P,
                                                             const T* __restrict__ Q, T* __restrict__ x,
@@ -1527,10 +1531,9 @@ __device__ __forceinline__ int gram_parts(int n, int gmax) { return min((n + kGr
 // leaves no room for another on its SM, so many problems of a few runs each went through loads and barriers
 // in turn (64 problems of 60 cameras, one direction: 79.1 us per iteration, 75.1 with 256 threads).
 template <typename T, int NT>
-__global__ void __launch_bounds__(NT, NT < kGramThreads ? 3 : 1) k_mcg_gram(const T* __restrict__ P, const T* __restrict__ Q,
-                                                                           const T* __restrict__ r,
-                                                                           double* __restrict__ partial, int gmax,
-                                                                           const Ctl* __restrict__ ctl) {
+__global__ void __launch_bounds__(NT, NT < kGramThreads ? 3 : 1)
+    k_mcg_gram(const T* __restrict__ P, const T* __restrict__ Q, const T* __restrict__ r,
+               double* __restrict__ partial, int gmax, const Ctl* __restrict__ ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const int p = blockIdx.y;
     const Ctl& c = ctl[p];
@@ -2168,10 +2171,10 @@ __device__ __forceinline__ void phi_columns(const T* __restrict__ qc, int64_t n,
 }
 
 template <typename T, int U>
-__global__ void __launch_bounds__(kThreads, phi_ctas(U)) k_mcg_phi(const T* __restrict__ Q, const T* __restrict__ z,
-                                                      WideSlot<T>* __restrict__ phip,
-                                                      const WideSlot<T>* __restrict__ dpart, int gu, double* __restrict__ hist_out, int* __restrict__ blk_off,
-                                                      int* __restrict__ blk_w, int mi1, Ctl* ctl) {
+__global__ void __launch_bounds__(kThreads, phi_ctas(U))
+    k_mcg_phi(const T* __restrict__ Q, const T* __restrict__ z, WideSlot<T>* __restrict__ phip,
+              const WideSlot<T>* __restrict__ dpart, int gu, double* __restrict__ hist_out,
+              int* __restrict__ blk_off, int* __restrict__ blk_w, int mi1, Ctl* ctl) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const int p = blockIdx.y;
     const Ctl& c = ctl[p];
@@ -2209,7 +2212,8 @@ __global__ void __launch_bounds__(kThreads, phi_ctas(U)) k_mcg_phi(const T* __re
         const int m = hist - c0 < nb ? hist - c0 : nb;
         if (m == kPhiCols) phi_columns<T, kPhiCols, U>(qc, n, zp, 9 * j0, 9 * j1, out, chunks);
         else
-            for (int u = 0; u < m; ++u) phi_columns<T, 1, U>(qc + u * n, n, zp, 9 * j0, 9 * j1, out + int64_t(u) * chunks, chunks);
+            for (int u = 0; u < m; ++u)
+                phi_columns<T, 1, U>(qc + u * n, n, zp, 9 * j0, 9 * j1, out + int64_t(u) * chunks, chunks);
     }
 }
 
@@ -2218,8 +2222,8 @@ __global__ void __launch_bounds__(kThreads, phi_ctas(U)) k_mcg_phi(const T* __re
 // (t = 0 .. nt - 1, whole warps): G of them share an entry, each adds every G-th partial into two
 // interleaved sums, and the group's sums meet in a fixed shuffle tree.
 template <typename T>
-__device__ __forceinline__ void phi_block(const WideSlot<T>* ph, int off, int w, int ne, int m, int n_eff, int K, bool local,
-                                          int t, int nt, double* sphi) {
+__device__ __forceinline__ void phi_block(const WideSlot<T>* ph, int off, int w, int ne, int m, int n_eff, int K,
+                                          bool local, int t, int nt, double* sphi) {
     int G = 1;
     while (G < 32 && 2 * G * ne <= nt) G *= 2;
     const int e = t / G, g = t % G;
@@ -2259,9 +2263,9 @@ __device__ __forceinline__ double beta_entry(const double* Dp, const double* sph
 // thread per entry), smaller ones a warp each.  With a warp per 16 x 16 block the 128 float64
 // multiply-adds of a warp were a chain of 13 us (2000 columns); 4.8 us with the CTA.
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_mcg_beta(const WideSlot<T>* __restrict__ phip, const double* __restrict__ dpinv,
-                                                       const int* __restrict__ blk_off, const int* __restrict__ blk_w,
-                                                       T* __restrict__ beta, const Ctl* __restrict__ ctl, int mi1) {
+__global__ void __launch_bounds__(kThreads)
+    k_mcg_beta(const WideSlot<T>* __restrict__ phip, const double* __restrict__ dpinv, const int* __restrict__ blk_off,
+               const int* __restrict__ blk_w, T* __restrict__ beta, const Ctl* __restrict__ ctl, int mi1) {
     wait_prior_grid();   // chained launch: the previous kernel's results are visible from here
     const int p = blockIdx.y;
     const Ctl& c = ctl[p];
@@ -2293,7 +2297,8 @@ __global__ void __launch_bounds__(kThreads) k_mcg_beta(const WideSlot<T>* __rest
                 if (e0 == 0 && part == ne) phi_block<T>(ph, off, w, ne, m, n_eff, K, local, lane, 32, swarp[wid]);
                 else if (lane < part) {
                     const int e = e0 + lane, a = e / w, s2 = e - w * (e / w);
-                    const WideSlot<T>* sp = local ? ph + (int64_t(off + a) * n_eff + s2) * K : ph + int64_t(off + a) * n_eff * K;
+                    const int64_t cc = int64_t(off + a) * n_eff;
+                    const WideSlot<T>* sp = local ? ph + (cc + s2) * K : ph + cc * K;
                     WideSum<T> a0;
                     for (int k = 0; k < m; ++k) a0.add(sp[k]);
                     swarp[wid][e] = a0.value();
@@ -3365,8 +3370,10 @@ static T* ptr(const Buf& b) {
 // cameras 82.0 / 71.1 us, 1000 cameras 166 / 174 us.  Float64 below that, at 256 / 128 / 64 blocks: 300
 // cameras 46.8 / 33.3 / 41.3 us, 150 cameras 30.9 / 28.7 / 20.9 us (a float64 tile takes about 3 us, so a
 // row in one warp is a long chain), but with shape 2, which has a quarter of the warps, 61.0 us at 128 for 300
-// cameras and 53.3 us at 512, so that shape keeps 512 from 200 cameras on; a float64 batch of 48 problems of 100 to 400 cameras pays for it
-// (530 / 580 / 697 us).  Float32 keeps 256 there: 128 gains 14 % of a PCG solve at 300 cameras and
+// cameras and 53.3 us at 512, so that shape keeps 512 from 200 cameras on.  What decides is the tiles of a row
+// against the warps of the launch, which a batch shares: 48 float64 problems of 100 to 400 cameras pay for the
+// rule (530 / 580 / 697 us), the price of summing like a solo solve; ba_autotune sets the size for a handle.
+// Float32 keeps 256 there: 128 gains 14 % of a PCG solve at 300 cameras and
 // nothing at 150, and costs a batch 5 %.
 static int default_item_blocks(int n_cams, bool fp32, int cfg) {
     if (fp32) return n_cams < 1200 ? 256 : 512;
@@ -3607,7 +3614,7 @@ static void prepare(Solver* w, const Structure& s, const SolveArgs& a, int n_dir
     w->n = n;
     w->mi1 = std::max(w->mi1, a.max_iters + 1);
     w->gx = int(std::min<int64_t>(std::max(1, 4 * G / nb), (9 * int64_t(nc_max) + kThreads - 1) / kThreads));
-    if ((int64_t(nc_max) + 27) / 28 > 65535) throw Error(BA_ERR_INVALID_ARG, "too many cameras in one problem");
+    if (nc_max > kMaxProblemCams) throw Error(BA_ERR_INVALID_ARG, "too many cameras in one problem");
     w->gu = (nc_max + kUpdCams - 1) / kUpdCams;
     w->gg = int(std::min<int64_t>(G, (9 * int64_t(nc_max) + kGramRows - 1) / kGramRows));
     w->gq = std::max(1, G / nb);
@@ -3784,11 +3791,14 @@ static void launch_spmv(int cfg, cudaStream_t st, const int64_t* row_ptr, const 
                         const T* S, const T* z, const ItemList& L, int sel, T* out, const T* rvec, double* camdot,
                         Ctl* ctl, T* tb, T* tb8 = nullptr, const int32_t* cslot = nullptr) {
     if (cfg == 1)
-        launch_spmv_cfg<T, MODE, ZH, SYM, 1>(st, row_ptr, tile_ptr, col, S, z, L, sel, out, rvec, camdot, ctl, tb, tb8, cslot);
+        launch_spmv_cfg<T, MODE, ZH, SYM, 1>(st, row_ptr, tile_ptr, col, S, z, L, sel, out, rvec, camdot, ctl, tb, tb8,
+                                             cslot);
     else if (cfg == 2)
-        launch_spmv_cfg<T, MODE, ZH, SYM, 2>(st, row_ptr, tile_ptr, col, S, z, L, sel, out, rvec, camdot, ctl, tb, tb8, cslot);
+        launch_spmv_cfg<T, MODE, ZH, SYM, 2>(st, row_ptr, tile_ptr, col, S, z, L, sel, out, rvec, camdot, ctl, tb, tb8,
+                                             cslot);
     else
-        launch_spmv_cfg<T, MODE, ZH, SYM, 0>(st, row_ptr, tile_ptr, col, S, z, L, sel, out, rvec, camdot, ctl, tb, tb8, cslot);
+        launch_spmv_cfg<T, MODE, ZH, SYM, 0>(st, row_ptr, tile_ptr, col, S, z, L, sel, out, rvec, camdot, ctl, tb, tb8,
+                                             cslot);
 }
 
 // A one-column product y = S z, z a column of the direction history (modes of k_spmv).  With the upper
@@ -4363,7 +4373,8 @@ __global__ void k_test_phi_block(const WideSlot<float>* slots, int chunks, doubl
 }
 
 // a^T b as k_pcg_update and k_pcg_dir add it: a product per thread, kUpdThreads a CTA
-__global__ void __launch_bounds__(kUpdThreads) k_test_update(const float* a, const float* b, int n, WideSlot<float>* slots) {
+__global__ void __launch_bounds__(kUpdThreads) k_test_update(const float* a, const float* b, int n,
+                                                             WideSlot<float>* slots) {
     const int i = blockIdx.x * kUpdThreads + threadIdx.x;
     ExactSum<float> v[1];
     if (i < n) v[0].add(a[i], b[i]);
