@@ -178,9 +178,18 @@ void launch_cam_rhs(const Structure& s, System& y, int damping, double lambda, c
 void launch_schur_diag32(const Structure& s, System& y, cudaStream_t st);
 void launch_schur(const Structure& s, System& y, cudaStream_t st);
 void launch_schur_mixed(const Structure& s, System& y, cudaStream_t st);
+// Exponent of a b to within one, from the bits (no float64 operation); kNoExponent for a zero (or subnormal) factor.
+constexpr int kNoExponent = -5000;
+#ifdef __CUDACC__
+__device__ __forceinline__ int product_exponent(double a, double b) {
+    const int ea = (__double2hiint(a) >> 20) & 0x7ff, eb = (__double2hiint(b) >> 20) & 0x7ff;
+    return ea == 0 || eb == 0 ? kNoExponent : ea + eb - 2 * 1023;
+}
+#endif
 // out = -b~ - S x with the implicit float64 operator (mixed precision, no explicit S)
 // S x = sum_o J_p^T (J_p x - J_l V^-1 sum J_l^T J_p x) + lambda D_p x;
-// partial[3 j] .. partial[3 j + 2] receive camera j's sums of out^2, b~^2 and (Lam out)^2 (3 n_c values)
+// partial[3 j], [3 j + 1] receive camera j's sums of out^2 and b~^2, [3 j + 2] (as int) the largest exponent of
+// Lam out (3 n_c values)
 int launch_implicit_residual(const Structure& s, const System& y, const double* x, double* out, double* partial,
                               cudaStream_t st);
 void launch_block_jacobi(const Structure& s, System& y, cudaStream_t st);

@@ -1198,7 +1198,8 @@ __global__ void k_jres_land_df(int32_t n_l, const int64_t* __restrict__ pt_ptr, 
 }
 
 // True residual, camera pass: out_j = -b~_j - (S x)_j with (S x)_j = sum_{o in j} J_p^T v_o (double-float)
-// + lambda D_p x_j (float64); camera j's |out_j|^2, |b~_j|^2 and |Lam out_j|^2 into partial[3 j] ..
+// + lambda D_p x_j (float64); camera j's |out_j|^2, |b~_j|^2 and the largest exponent of Lam out_j (an int in the
+// value's place) into partial[3 j] ..
 __global__ void __launch_bounds__(kCamThreads) k_jres_cam_df(
     int32_t n_c, const int64_t* __restrict__ cam_ptr, const int32_t* __restrict__ cam_obs,
     const float2* __restrict__ Jc, const float2* __restrict__ uv, const double* __restrict__ dadd,
@@ -1218,7 +1219,8 @@ __global__ void __launch_bounds__(kCamThreads) k_jres_cam_df(
             for (int a = 0; a < 9; ++a) acc[a] += jc[a] * u[0] + jc[9 + a] * u[1];
         }
         cta_sum_df<9>(acc, red);
-        double tt = 0.0, bb = 0.0, ss = 0.0;
+        double tt = 0.0, bb = 0.0;
+        int top = kNoExponent;
         if (threadIdx.x < 9) {
             const int a = threadIdx.x;
             const int64_t i = 9 * int64_t(j) + a;
@@ -1226,19 +1228,18 @@ __global__ void __launch_bounds__(kCamThreads) k_jres_cam_df(
             const double b_ = bt[i];
             const double rv = -b_ - sx;
             if (out) out[i] = rv;
-            const double sv = lam[i] * rv;
             tt = rv * rv;
             bb = b_ * b_;
-            ss = sv * sv;
+            top = product_exponent(lam[i], rv);
         }
         if (threadIdx.x < 32) {
             tt = warp_sum(tt);
             bb = warp_sum(bb);
-            ss = warp_sum(ss);
+            top = __reduce_max_sync(0xffffffffu, top);
             if (threadIdx.x == 0) {
                 partial[3 * int64_t(j)] = tt;
                 partial[3 * int64_t(j) + 1] = bb;
-                partial[3 * int64_t(j) + 2] = ss;
+                *reinterpret_cast<int*>(partial + 3 * int64_t(j) + 2) = top;
             }
         }
         __syncthreads();

@@ -92,7 +92,7 @@ struct Ctl {
                        // first CTA runs the decide step, which may set done meanwhile)
     double alpha_v[kMaxDirs];
     double true_rr, bb;                 // true residual and |rhs|^2
-    double scaled_rr;  // mixed precision: |Lam (true residual)|^2
+    int scaled_exp;    // mixed precision: the largest exponent of Lam (true residual)
     double stag;       // float32 sweeps: stop when t_i (energy decrease / r^T D^-1 r) falls below this
     int direct_q;      // 1: Q_{i+1} = S P_{i+1} (Algorithm 2); 0: the Q update of Eq. 18
     int pinv_steps;    // steps whose Delta_i took the eigen-decomposition pseudo-inverse
@@ -119,9 +119,10 @@ struct Outer {
     double bb;         // |b~|^2
     double tr;         // |-b~ - S x|^2 of the current x
     double tr_prev;    // the same before the last sweep (scales that sweep's residual history)
-    double sr;         // |Lam (-b~ - S x)|^2 of the current x: the residual of the sweeps' scaled system
     double tol_in;     // relative tolerance of the next inner sweep
-    double unit;       // power of two near sqrt(sr): the sweep solves for Lam (-b~ - S x) divided by it
+    double unit;       // power of two near the largest value of Lam (-b~ - S x), the residual of the sweeps'
+                       // scaled system: the sweep solves for that residual divided by it
+    int se;            // its exponent
     int status;
     int active;        // still refining
     int swept;         // takes part in the sweep being run
@@ -1173,8 +1174,8 @@ __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
 // ---------------------------------------------------------------------------------------
 // initialisation shared by both algorithms: x = 0, r = sign * rhs, z = D^{-1} r, P_0 = z
 // (grid: update CTAs x problems; thread = row, as in the update kernels; partial: one slot per CTA).
-// outer (mixed precision, may be null): r is divided by the sweep's unit, a power of two near |r|, so that
-// a sweep starts with |r| in [1, 2) whatever the residual's size and the units of the cameras and
+// outer (mixed precision, may be null): r is divided by the sweep's unit, a power of two near its largest value,
+// so that a sweep starts with that in [1, 4) whatever the residual's size and the units of the cameras and
 // landmarks (the error terms of its float32 sums, and Delta^+ in double-float, would otherwise leave the
 // float32 range on late sweeps, or on the first one of a scene with coordinates of 1e-9).
 
@@ -3121,13 +3122,22 @@ __global__ void k_true_residual(int32_t n_c, const int64_t* __restrict__ row_ptr
     }
 }
 
-// per problem: ctl.true_rr, ctl.bb and (ns = 3) ctl.scaled_rr from the ns per-camera partials (camera
-// order); a warp per sum
+// per problem: ctl.true_rr, ctl.bb and (ns = 3) ctl.scaled_exp from the ns per-camera partials (camera
+// order); a warp each
 __global__ void k_true_reduce(Ctl* ctl, const double* __restrict__ partial, int ns) {
     Ctl* c = ctl + blockIdx.x;
-    const int k = threadIdx.x >> 5;
-    const double v = sum_partials(partial + ns * int64_t(c->lay.c0), c->lay.nc, ns, k);
-    if ((threadIdx.x & 31) == 0) (k == 0 ? c->true_rr : k == 1 ? c->bb : c->scaled_rr) = v;
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double* pp = partial + ns * int64_t(c->lay.c0);
+    if (k < 2) {
+        const double v = sum_partials(pp, c->lay.nc, ns, k);
+        if (lane == 0) (k == 0 ? c->true_rr : c->bb) = v;
+    } else {
+        int top = kNoExponent;
+        for (int p = lane; p < c->lay.nc; p += 32)
+            top = max(top, *reinterpret_cast<const int*>(pp + int64_t(p) * ns + k));
+        top = __reduce_max_sync(0xffffffffu, top);
+        if (lane == 0) c->scaled_exp = top;
+    }
 }
 
 // mixed precision: x += unit Lam d, a float32 sweep's correction mapped back from the scaled system,
@@ -3156,27 +3166,32 @@ __global__ void k_start_refine(int64_t n, const double* __restrict__ bt, double*
     }
 }
 
-// One CTA per problem: |b~|^2 and |Lam b~|^2 (fixed order) and the refinement state at x = 0.
+// One CTA per problem: |b~|^2 (fixed order), the largest exponent of Lam b~ and the refinement state at x = 0.
 __global__ void k_outer_init(const Layout* __restrict__ lay, const double* __restrict__ bt,
                              const double* __restrict__ lam, Outer* outer) {
     const Layout L = lay[blockIdx.x];
     const int64_t n = int64_t(L.nc) * 9;
     const double* b = bt + 9 * int64_t(L.c0);
-    double v[2] = {0.0, 0.0};
+    __shared__ double s[1];
+    __shared__ int top;
+    if (threadIdx.x == 0) top = kNoExponent;
+    double v[1] = {0.0};
+    int e = kNoExponent;
     for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-        const double sb = lam[9 * int64_t(L.c0) + i] * b[i];
         v[0] += b[i] * b[i];
-        v[1] += sb * sb;
+        e = max(e, product_exponent(lam[9 * int64_t(L.c0) + i], b[i]));
     }
-    __shared__ double s[2];
-    cta_sum_write<2>(v, s);
+    cta_sum_write<1>(v, s);
+    e = __reduce_max_sync(0xffffffffu, e);
+    if ((threadIdx.x & 31) == 0) atomicMax(&top, e);
+    __syncthreads();
     if (threadIdx.x == 0) {
         Outer o;
         memset(&o, 0, sizeof(o));
         o.bb = s[0];
         o.tr = s[0];
         o.tr_prev = s[0];
-        o.sr = s[1];
+        o.se = top;
         o.unit = 1.0;
         o.status = s[0] == 0.0 ? BA_OK : BA_ERR_NOT_CONVERGED;
         o.active = s[0] == 0.0 ? 0 : 1;
@@ -3207,7 +3222,7 @@ __global__ void k_refine_plan(Outer* outer, int nb, const Params* __restrict__ p
         double t = need > 0.1 * inner_tol ? fmax(0.3 * need, 0.1 * inner_tol) : inner_tol;
         if (t >= 1.0) t = 0.5;
         o->tol_in = t;
-        o->unit = o->sr > 0.0 ? ldexp(1.0, max(-900, min(900, ilogb(sqrt(o->sr))))) : 1.0;
+        o->unit = o->se > kNoExponent ? ldexp(1.0, max(-900, min(900, o->se))) : 1.0;
         o->max_in = prm->max_iters - o->iters;
         o->swept = 1;
         mine = 1;
@@ -3234,7 +3249,7 @@ __global__ void k_refine_after(const Ctl* __restrict__ ctl, Outer* outer, const 
     o->cols = mcg ? c.cols : 1;
     o->tr_prev = o->tr;
     o->tr = c.true_rr;
-    o->sr = c.scaled_rr;
+    o->se = c.scaled_exp;
     if (c.status == BA_ERR_BREAKDOWN || c.status == BA_ERR_OOM || c.status == BA_ERR_TIMEOUT) {
         o->status = c.status;
         o->active = 0;
