@@ -645,10 +645,12 @@ __device__ __forceinline__ void camera_dots(int lane, T q, T p, T r, double* cam
 
 // A warp that gives up at item i leaves it and its later ones undone: their problems (of a batch, possibly
 // others than the one whose copy was waited for) end with the status at their next decide step.
-__device__ __forceinline__ void report_timeout(Ctl* ctl, const ItemList& L, int sel, int64_t i, const WarpItems& wi) {
+// (Not inlined, with the list position found again: k_spmm has no register to spare for this path.)
+__device__ __noinline__ void report_timeout(Ctl* ctl, const SpItem* items, int sel, int64_t item, int64_t end,
+                                            int64_t step) {
     if (threadIdx.x & 31) return;
-    for (; i < wi.end; i += wi.step) {
-        const int prob = L.items[i].prob;
+    for (int64_t i = item; i < end; i += step) {
+        const int prob = items[i].prob;
         if (selected(ctl, prob, sel)) atomicExch(&ctl[prob].status, BA_ERR_TIMEOUT);
     }
 }
@@ -741,8 +743,8 @@ __global__ void __launch_bounds__(SpmvShape<T, CFG>::kWarps * 32, 1) k_spmv(
     }
     int stage = 0;
     bool bad = false;
-    int64_t i = wi.i0;
-    for (; i < wi.end; i += wi.step) {
+    int bad_item = 0;
+    for (int64_t i = wi.i0; i < wi.end && !bad; i += wi.step) {
         const SpItem it = L.items[i];
         if (!selected(ctl, it.prob, sel)) continue;
         const Ctl& c = ctl[it.prob];
@@ -789,6 +791,7 @@ __global__ void __launch_bounds__(SpmvShape<T, CFG>::kWarps * 32, 1) k_spmv(
                 const bool ok = mbar_wait(&bars[stage], (parity >> stage) & 1u, L.polls);
                 if (!__all_sync(0xffffffffu, ok)) {
                     bad = true;
+                    bad_item = int(i);
                     break;
                 }
                 parity ^= 1u << stage;
@@ -871,7 +874,8 @@ __global__ void __launch_bounds__(SpmvShape<T, CFG>::kWarps * 32, 1) k_spmv(
     if (bad) {
         // a copy did not land in time: report, then wait (bounded) for this warp's copies in flight;
         // the problem's next decide step ends it with the status
-        report_timeout(ctl, L, sel, i, wi);
+        const WarpItems left = warp_items(L, NW, wid);
+        report_timeout(ctl, L.items, sel, bad_item, left.end, left.step);
         for (int st = 0; st < NS; ++st)
             if (inflight & (1u << st)) mbar_wait(&bars[st], (parity >> st) & 1u, kDefaultWaitPolls);
     }
@@ -1033,8 +1037,8 @@ __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
     }
     int stage = 0;
     bool bad = false;
-    int64_t i = wi.i0;
-    for (; i < wi.end; i += wi.step) {
+    int bad_item = 0;
+    for (int64_t i = wi.i0; i < wi.end && !bad; i += wi.step) {
         const SpItem it = L.items[i];
         if (!selected(ctl, it.prob, sel)) continue;
         const Ctl& c = ctl[it.prob];
@@ -1070,6 +1074,7 @@ __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
                 const bool ok = mbar_wait(&bars[stage], (parity >> stage) & 1u, L.polls);
                 if (!__all_sync(0xffffffffu, ok)) {
                     bad = true;
+                    bad_item = int(i);
                     break;
                 }
                 parity ^= 1u << stage;
@@ -1165,7 +1170,8 @@ __global__ void __launch_bounds__(SpmmCfg::kWarps * 32, 1) k_spmm(
         __syncwarp();
     }
     if (bad) {
-        report_timeout(ctl, L, sel, i, wi);
+        const WarpItems left = warp_items(L, NW, wid);
+        report_timeout(ctl, L.items, sel, bad_item, left.end, left.step);
         for (int st = 0; st < NS; ++st)
             if (inflight & (1u << st)) mbar_wait(&bars[st], (parity >> st) & 1u, kDefaultWaitPolls);
     }
