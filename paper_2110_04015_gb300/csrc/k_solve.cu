@@ -226,10 +226,9 @@ __device__ __forceinline__ float two_sum(float a, float b, float& e) {   // fl(a
 // on the integer pipe.  Subnormals (below 1e-38 of sums that start near one) become zero.
 __device__ __forceinline__ double widen(float f) {
     const int b = __float_as_int(f), e = b & 0x7f800000;
-    if (e == 0x7f800000) return double(f);   // infinities and NaN
-    if (e == 0) return 0.0;
-    return __longlong_as_double(((static_cast<long long>(b & 0x7fffffff) + (896ll << 23)) << 29) |
-                                (static_cast<long long>(b & int(0x80000000)) << 32));
+    // exponent 255 (infinities and NaN) becomes 2047
+    const long long m = (static_cast<long long>(b & 0x7fffffff) << 29) + (e == 0x7f800000 ? 1792ll << 52 : 896ll << 52);
+    return __longlong_as_double((e == 0 ? 0ll : m) | (static_cast<long long>(b & int(0x80000000)) << 32));
 }
 template <typename T>
 struct WideSum;
@@ -2608,13 +2607,39 @@ __device__ __forceinline__ void one_product(const float* S, OneSmem& m, int nc, 
     }
 }
 
-// Sums of NV values over the rows (threads 0 .. kOneRows - 1 hold a product each, zeros past the problem), the
-// same in every thread.  Contains a barrier before and after the sums are read.
+// Sums of NV values over the rows (threads 0 .. kOneRows - 1 hold a product each, zeros past the problem).
+// one_sums: float pairs, the same in every thread (Delta and gamma); a barrier before and after they are read.
+// one_wide: the warps' wide sums into st and a barrier; one_total adds them, in the threads that need a value.
+constexpr int kOneRowWarps = (kOneRows + 31) / 32;
+static_assert(kOneRowWarps % 2 == 0, "pairs of warps");
 template <int NV>
-__device__ __forceinline__ void one_sums(const ExactSum<float> (&v)[NV], WideSum<float> (&sum)[NV], float4* st) {
-    constexpr int NWR = (kOneRows + 31) / 32;
+__device__ __forceinline__ void one_sums(ExactSum<float> (&v)[NV], double* st) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (wid < NWR) {
+    if (wid < kOneRowWarps) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            v[k] = warp_total(v[k]);
+            if (lane == 0) store_partial(&st[NV * wid + k], v[k]);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        ExactSum<float> a, b;
+#pragma unroll
+        for (int q = 0; q < kOneRowWarps; q += 2) {
+            load_partial(a, &st[NV * q + k]);
+            load_partial(b, &st[NV * (q + 1) + k]);
+        }
+        combine(a, b);
+        v[k] = a;
+    }
+    __syncthreads();
+}
+template <int NV>
+__device__ __forceinline__ void one_wide(const ExactSum<float> (&v)[NV], float4* st) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (wid < kOneRowWarps) {
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
             const WideSum<float> s = warp_total(WideSum<float>(v[k]));
@@ -2622,19 +2647,19 @@ __device__ __forceinline__ void one_sums(const ExactSum<float> (&v)[NV], WideSum
         }
     }
     __syncthreads();
+}
+template <int NV>
+__device__ __forceinline__ double one_total(const float4* st, int k) {
+    WideSum<float> a, b;
+    a.set(st[k]);
+    b.set(st[NV + k]);
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        WideSum<float> a, b;
-        static_assert(NWR % 2 == 0, "pairs of warps");
-#pragma unroll
-        for (int q = 0; q < NWR; q += 2) {
-            a.add(st[NV * q + k]);
-            b.add(st[NV * (q + 1) + k]);
-        }
-        a.add(b);
-        sum[k] = a;
+    for (int q = 2; q < kOneRowWarps; q += 2) {
+        a.add(st[NV * q + k]);
+        b.add(st[NV * (q + 1) + k]);
     }
-    __syncthreads();
+    a.add(b);
+    return a.value();
 }
 
 // q^T z over the rows [i0, i1) of whole cameras (QS apart in q), by one thread: as accurate as float64.  (With
@@ -2709,9 +2734,8 @@ __global__ void __launch_bounds__(kOneThreads, 1)
                 d[0].add(m.QT[own_at], m.PT[own_at]);
                 d[1].add(m.PT[own_at], m.r[t]);
             }
-            WideSum<float> dg[2];
-            one_sums<2>(d, dg, reinterpret_cast<float4*>(m.st));
-            const float alpha = __fdiv_rn(__fadd_rn(dg[1].hi, dg[1].lo), __fadd_rn(dg[0].hi, dg[0].lo));
+            one_sums<2>(d, m.st);
+            const float alpha = __fdiv_rn(__fadd_rn(d[1].hi, d[1].lo), __fadd_rn(d[0].hi, d[0].lo));
             ExactSum<float> v[3];
             float rv = 0.f, qv = 0.f;
             if (act) {
@@ -2728,14 +2752,13 @@ __global__ void __launch_bounds__(kOneThreads, 1)
                 v[1].add(qv, zs);
                 v[2].add(rv, zs);
             }
-            WideSum<float> vs[3];
-            one_sums<3>(v, vs, reinterpret_cast<float4*>(m.st));
-            if (t == 0) m.scal[0] = float(vs[1].value() * fast_rcp<2>(dg[0].value()));
+            float4* st = reinterpret_cast<float4*>(m.st);
+            one_wide<3>(v, st);
+            if (t == 0) m.scal[0] = float(one_total<3>(st, 1) * fast_rcp<2>(d[0].value()));
             if (t == 32) {   // the stop test beside it
-                m.tot[0] = vs[0].value();
-                m.tot[1] = vs[1].value();
-                m.tot[2] = vs[2].value();
-                pcg_decide(&m.c, dg[0].value(), dg[1].value(), m.tot, hist, p, gridDim.x);
+                m.tot[0] = one_total<3>(st, 0);
+                m.tot[2] = one_total<3>(st, 2);
+                pcg_decide(&m.c, d[0].value(), d[1].value(), m.tot, hist, p, gridDim.x);
             }
             __syncthreads();
             if (m.c.done) break;
@@ -2816,11 +2839,11 @@ __global__ void __launch_bounds__(kOneThreads, 1)
                 m.z[t] = zs;
                 v[1].add(m.r[t], zs);
             }
-            WideSum<float> vs[2];
-            one_sums<2>(v, vs, reinterpret_cast<float4*>(m.st));
+            float4* st = reinterpret_cast<float4*>(m.st);
+            one_wide<2>(v, st);
             if (t == 0) {
-                m.tot[0] = vs[0].value();
-                m.tot[1] = vs[1].value();
+                m.tot[0] = one_total<2>(st, 0);
+                m.tot[1] = one_total<2>(st, 1);
                 m.c.hist_cols = m.c.cols;
                 mcg_decide(&m.c, m.tot, hist, blk_off, blk_w, mi1, p, gridDim.x);
             }
