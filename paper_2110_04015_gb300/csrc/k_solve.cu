@@ -2522,13 +2522,13 @@ __global__ void __launch_bounds__(NW * 32, NW < PqShape<T>::kSlices ? 4 : RL == 
 // tiles of 64 columns stored row by row (hist_at), so that threads on neighbouring columns read
 // neighbouring words.  It does what the kernels above do, step by step: exact-product sums, the float64 small
 // solve and Delta^+ Phi, the same decide steps.
-// 13 cameras: PCG 7.5 us per iteration (launched kernels 14.5), MCG with 8 directions to 1e-9 18.8 us (35.2).
+// 13 cameras: PCG 5.4 us per iteration (launched kernels 14.5), MCG with 8 directions to 1e-9 17.9 us (35.2).
 //
 // The rule: float32 sweeps of problems with nc <= kOneCams (S takes 324 nc^2 bytes: 130 KB of shared memory
 // at 20 cameras), by MCG with up to kOneDirs local directions, whatever else is in the batch, so a problem's
 // result does not depend on the others.  Delta_j^+ Phi_j costs w w' w float64 multiply-adds per pair of
 // blocks on this SM's float64 pipe alone, and a rank-deficient block's eigen-decomposition shares it:
-// to 1e-9 with 8 directions 19 to 26 us per iteration against 31 to 35 us in the kernels, with 10 directions
+// to 1e-9 with 8 directions 18 to 25 us per iteration against 31 to 35 us in the kernels, with 10 directions
 // (20 cameras) 33.4 against 33.6 us, with 16 directions (16 cameras) 92 against 60 us.
 // Larger problems run the kernels above; a handle whose tile waits give up at once (wait_polls = -1) does
 // too, since there is no tile wait here.
