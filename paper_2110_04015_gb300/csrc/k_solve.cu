@@ -969,7 +969,7 @@ __global__ void __launch_bounds__(kColWarps * 32, 12) k_spmv_col(const int64_t* 
 // shared memory as in k_spmv; CL lanes share a block (CL = 4, or 2 when no block is wider than 8
 // columns): lane = CL qi + g takes tile-local blocks qi, qi + 32 / CL, ... and columns
 // 4g .. 4g + 3, so each 9x9 block multiplies up to 4 CL columns per read from shared memory.  No unit is at
-// its limit (1000 dense cameras: L1 and shared memory 62 %, DRAM 42 %, issue 34 %); a warp waits most for its P
+// its limit (1000 dense cameras: L1 and shared memory 65 %, DRAM 43 %, issue 36 %); a warp waits most for its P
 // gathers, then for its 81 words of S and 36 of P per 324 multiply-adds.  Lanes left without columns wait like
 // the others: N = 8 on 1000 dense cameras took 94 us per local step with four lanes a block and takes 75 us
 // with two (one lane for N = 4: 76 us).  PT is the row-major copy (9 n_c x 16, all problems) of the new blocks.
